@@ -290,7 +290,7 @@ int gcamb_interp_sources(const gcamb_grid *g, const double *k_in, int nk_in, con
  * Cross spectrum, Eq. (1) with X, Y in {T, E}:
  *   C^XY[m][l] = 4 pi sum_k w_k P[m][k] DX[m][k][l] DY[m][k][l]
  * DX, DY [M][nk][nl] device, both of d_dtype (GCAMB_F64 or GCAMB_F32);
- * Pk[M][nk], Cl[M][nl] device double.  Summed in FP64 in increasing k.
+ * Pk[M][nk], Cl[M][nl] device double.  Summed in FP64 in an order fixed by nk (deterministic).
  */
 int gcamb_cl_cross(const gcamb_grid *g, const void *DX, const void *DY, int d_dtype, const double *Pk, int M,
                    double *Cl, void *stream);
@@ -300,7 +300,7 @@ int gcamb_cl_cross(const gcamb_grid *g, const void *DX, const void *DY, int d_dt
  *   Delta[M][nk][nl]   device, d_dtype = GCAMB_F64 or GCAMB_F32
  *   Pk[M][nk]          device double, P_R(k) per source
  *   Cl[M][nl]          device double, C_l for l = lmin..lmax
- * Summed in FP64 in increasing k (deterministic).
+ * Summed in FP64 in an order fixed by nk (deterministic).
  */
 int gcamb_cl(const gcamb_grid *g, const void *Delta, int d_dtype, const double *Pk, int M,
              double *Cl, void *stream);

@@ -376,89 +376,138 @@ int launch_los_tensor(const gcamb_grid *g, const void *ST, const void *SP, int M
   return launch_los_plain_k<2, true>(g, ST, M, mode, DT, st);
 }
 
-// C_l[m][l] = 4 pi sum_k w_k P[m][k] Delta[m][k][l]^2 in FP64, increasing k.
-template <typename TD>
-__global__ void __launch_bounds__(256) cl_kernel(const TD *__restrict__ Delta, const double *__restrict__ Pk,
-                                                 const double *__restrict__ wk, int nk, int nl,
-                                                 double *__restrict__ Cl) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  const int m = blockIdx.y;
-  if (l >= nl) return;
-  const TD *d = Delta + (size_t)m * nk * nl + l;
-  const double *p = Pk + (size_t)m * nk;
+// C^XY_l[m] = 4 pi sum_k w_k P[m][k] DX[m][k][l] DY[m][k][l] in FP64 (kCross;
+// else Y = X and only DX is read).  kPrefix (the uneven FP32 plan): source
+// m0 + m of the chunk on its own k prefix [0, nk_m) with the trapezoid in ln k
+// of that prefix (the last node of a shorter prefix takes half its interval)
+// and zero above its own l_max; rows of DX beyond the prefix are not read.
+//
+// A serial walk over k by one thread per (m, l) is bound by the latency of
+// its loads (l_max = 5000, 3000 k, one model: 1097 us for 120 MB).  Here the
+// k range is cut into kClParts contiguous parts, summed in eight groups of
+// eight: a warp sums one part (or 2, 4, 8 of them in turn) for 32 adjacent
+// multipoles with eight loads in flight; the CTAs of a cluster (grid y) share
+// out the groups and the first one adds the eight group sums it gets through
+// distributed shared memory.  The order of the additions is fixed by nk
+// alone: it does not depend on the cluster size, the batch or the block.  The
+// weight 4 pi w_k P is formed once per (k, CTA), not per element, which leaves
+// two FP64 operations an element (GB300's FP64 pipe runs at 1/64 of the FP32
+// one).  Measured, one model: l_max 5000 x 3000 k 1097 -> 68 us, l_max 500 x
+// 300 k 116 -> 7.8 us; cross spectra, l_max 1500 x 1000 k 528 -> 11.9 us.
+constexpr int kClParts = 64, kClGroups = 8;
+enum ClKind { kAuto = 0, kCross = 1, kPrefix = 2 };
+
+struct ClPrefix {
+  const double *kk;
+  const int *lrow, *lmax_m, *nk_m;
+  int m0;
+};
+
+template <typename TD, int KIND>
+__global__ void __launch_bounds__(256) cl_sum_kernel(const TD *__restrict__ DX, const TD *__restrict__ DY,
+                                                     const double *__restrict__ Pk, const double *__restrict__ wk,
+                                                     int nk, int nl, double *__restrict__ Cl, ClPrefix px) {
+  __shared__ double fw[8][32];               // weights of a warp's next 32 k
+  __shared__ double part[kClParts][32];      // this CTA's parts (the first kClParts / cluster size rows)
+  __shared__ double gsum[kClGroups][32];     // the first CTA of the cluster: every group's sum
+  const int cs = gridDim.y, rank = blockIdx.y;  // cluster size (1, 2, 4, 8) and rank: the cluster spans grid y
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int l = blockIdx.x * 32 + lane;
+  const size_t m = blockIdx.z;                            // source within DX
+  const size_t mg = KIND == kPrefix ? px.m0 + m : m;      // source within Pk and Cl
+  const TD *dx = DX + m * nk * nl + l, *dy = DY + m * nk * nl + l;
+  const double *p = Pk + mg * nk;
   const double four_pi = 4.0 * 3.14159265358979323846;
-  double acc = 0.0;
-  for (int q = 0; q < nk; ++q) {
-    const double v = (double)d[(size_t)q * nl];
-    const double f = four_pi * wk[q] * p[q];
-    acc = fma(f, v * v, acc);
+  const int nkm = KIND == kPrefix ? px.nk_m[mg] : nk;
+  const bool live = l < nl && (KIND != kPrefix || px.lrow[l] <= px.lmax_m[mg]);
+  const int pc = (nk + kClParts - 1) / kClParts;  // k per part
+  const int ppw = 8 / cs;                         // parts per warp
+  for (int j = 0; j < ppw; ++j) {
+    const int lp = warp * ppw + j;  // part within the CTA
+    const int qb = min(nkm, (rank * (kClParts / cs) + lp) * pc), qe = min(nkm, qb + pc);
+    double acc = 0.0;
+    for (int q0 = qb; q0 < qe; q0 += 32) {
+      __syncwarp();
+      const int q = q0 + lane;
+      if (q < qe) {
+        double w = wk[q];
+        if (KIND == kPrefix && nkm < nk && q + 1 == nkm) w = q > 0 ? 0.5 * (log(px.kk[q]) - log(px.kk[q - 1])) : 0.0;
+        fw[warp][lane] = four_pi * w * p[q];
+      }
+      __syncwarp();
+      const int n = min(32, qe - q0);
+      if (live) {
+#pragma unroll 1
+        for (int i = 0; i < n; i += 8) {
+          TD x[8], y[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const size_t o = (size_t)(q0 + i + u) * nl;
+            x[u] = i + u < n ? dx[o] : TD(0);
+            if constexpr (KIND == kCross) y[u] = i + u < n ? dy[o] : TD(0);
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (i + u < n) acc = fma(fw[warp][i + u], (double)x[u] * (double)(KIND == kCross ? y[u] : x[u]), acc);
+        }
+      }
+    }
+    part[lp][lane] = acc;
   }
-  Cl[(size_t)m * nl + l] = acc;
+  __syncthreads();
+  const int ng = kClGroups / cs;  // groups of this CTA
+  if (warp < ng) {
+    double s = part[warp * 8][lane];
+#pragma unroll
+    for (int j = 1; j < 8; ++j) s += part[warp * 8 + j][lane];
+    // into the first CTA's gsum
+    uint32_t dst = (uint32_t)__cvta_generic_to_shared(&gsum[rank * ng + warp][lane]);
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, 0;\n\tst.shared::cluster.f64 [a], %1;\n\t}\n" ::"r"(dst),
+                 "d"(s)
+                 : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank == 0 && warp == 0 && l < nl) {
+    double s = gsum[0][lane];
+#pragma unroll
+    for (int g = 1; g < kClGroups; ++g) s += gsum[g][lane];
+    Cl[mg * nl + l] = s;
+  }
 }
 
-// C^XY_l[m] = 4 pi sum_k w_k P[m][k] DX[m][k][l] DY[m][k][l] in FP64, increasing k.
-template <typename TD>
-__global__ void __launch_bounds__(256) cl_cross_kernel(const TD *__restrict__ DX, const TD *__restrict__ DY,
-                                                       const double *__restrict__ Pk, const double *__restrict__ wk,
-                                                       int nk, int nl, double *__restrict__ Cl) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  const int m = blockIdx.y;
-  if (l >= nl) return;
-  const size_t base = (size_t)m * nk * nl + l;
-  const double *p = Pk + (size_t)m * nk;
-  const double four_pi = 4.0 * 3.14159265358979323846;
-  double acc = 0.0;
-  for (int q = 0; q < nk; ++q) {
-    const double f = four_pi * wk[q] * p[q];
-    acc = fma(f, (double)DX[base + (size_t)q * nl] * (double)DY[base + (size_t)q * nl], acc);
-  }
-  Cl[(size_t)m * nl + l] = acc;
+template <typename TD, int KIND>
+static cudaError_t launch_cl_sum(const gcamb_grid *g, const void *DX, const void *DY, const double *Pk, int M,
+                                 double *Cl, cudaStream_t st, const ClPrefix &px = ClPrefix()) {
+  // cluster size: the smallest that gives every SM six CTAs of 256 threads
+  // (of the eight that fit), up to the portable eight: with one model even
+  // l_max = 5000 has only 157 blocks of 32 multipoles
+  const unsigned lb = (unsigned)((g->nl + 31) / 32);
+  unsigned cs = 1;
+  while (cs < 8 && (size_t)lb * M * cs < 152 * 6) cs *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(lb, cs, (unsigned)M);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 1;
+  at.val.clusterDim.y = cs;
+  at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, cl_sum_kernel<TD, KIND>, static_cast<const TD *>(DX), static_cast<const TD *>(DY),
+                            Pk, static_cast<const double *>(g->d_wk), g->nk, g->nl, Cl, px);
 }
 
 int launch_cl_cross(const gcamb_grid *g, const void *DX, const void *DY, int d_dtype, const double *Pk, int M,
                     double *Cl, cudaStream_t st) {
   if (M > 65535) return fail(GCAMB_EINVAL, "cl_cross: too many sources for one launch");
-  dim3 grid((g->nl + 255) / 256, M);
   ProfScope prof(GCAMB_K_CL, st);
-  if (d_dtype == GCAMB_F64)
-    cl_cross_kernel<double><<<grid, 256, 0, st>>>(static_cast<const double *>(DX), static_cast<const double *>(DY), Pk,
-                                                  g->d_wk, g->nk, g->nl, Cl);
-  else
-    cl_cross_kernel<float><<<grid, 256, 0, st>>>(static_cast<const float *>(DX), static_cast<const float *>(DY), Pk,
-                                                 g->d_wk, g->nk, g->nl, Cl);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = d_dtype == GCAMB_F64 ? launch_cl_sum<double, kCross>(g, DX, DY, Pk, M, Cl, st)
+                                       : launch_cl_sum<float, kCross>(g, DX, DY, Pk, M, Cl, st);
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "cl_cross: launch");
   return GCAMB_OK;
-}
-
-// Uneven batch in FP32 on the CUDA cores: C_l[m][row] of one chunk of
-// sources (m0 .. m0 + mc), each on its own k prefix [0, nk_m) with the
-// trapezoid in ln k of that prefix (the last node of a shorter prefix takes
-// half its interval) and zero above its own l_max; Delta [mc][nk][nl] FP32 of
-// the chunk (rows beyond the chunk's l-tiles and k beyond its longest prefix
-// are not read: they belong to no source's sum).  FP64 sum in increasing k.
-__global__ void __launch_bounds__(256) cl_prefix_kernel(const float *__restrict__ Delta, const double *__restrict__ Pk,
-                                                        const double *__restrict__ wk, const double *__restrict__ kk,
-                                                        int nk, int nl, const int *__restrict__ lrow,
-                                                        const int *__restrict__ lmax_m, const int *__restrict__ nk_m,
-                                                        int m0, double *__restrict__ Cl) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  const int mi = blockIdx.y, m = m0 + mi;
-  if (row >= nl) return;
-  double acc = 0.0;
-  if (lrow[row] <= lmax_m[m]) {
-    const int nkm = nk_m[m];
-    const float *d = Delta + (size_t)mi * nk * nl + row;
-    const double *p = Pk + (size_t)m * nk;
-    const double four_pi = 4.0 * 3.14159265358979323846;
-    for (int q = 0; q < nkm; ++q) {
-      // trapezoid in ln k on the prefix [0, nkm)
-      const double w = (nkm == nk || q + 1 < nkm) ? wk[q] : (q > 0 ? 0.5 * (log(kk[q]) - log(kk[q - 1])) : 0.0);
-      const double v = (double)d[(size_t)q * nl];
-      acc = fma(four_pi * w * p[q], v * v, acc);
-    }
-  }
-  Cl[(size_t)m * nl + row] = acc;
 }
 
 // Sources per launch pair of the FP32 plan (the Delta buffer of a chunk).
@@ -503,10 +552,9 @@ int launch_plain_plan(const gcamb_grid *g, const float *S, const double *Pk, int
     }
     {
       ProfScope prof(GCAMB_K_CL, st);
-      dim3 grid((g->nl + 255) / 256, mc);
-      cl_prefix_kernel<<<grid, 256, 0, st>>>(D, Pk, g->d_wk, g->d_k, g->nk, g->nl, g->d_lrow, d_lmax, d_nk, m0, Cl);
+      e = launch_cl_sum<float, kPrefix>(g, D, D, Pk, mc, Cl, st, ClPrefix{g->d_k, g->d_lrow, d_lmax, d_nk, m0});
     }
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "plan_launch: FP32 launch");
   }
   return GCAMB_OK;
@@ -515,13 +563,10 @@ int launch_plain_plan(const gcamb_grid *g, const float *S, const double *Pk, int
 int launch_cl(const gcamb_grid *g, const void *Delta, int d_dtype, const double *Pk, int M, double *Cl,
               cudaStream_t st) {
   if (M > 65535) return fail(GCAMB_EINVAL, "cl: too many sources for one launch");
-  dim3 grid((g->nl + 255) / 256, M);
   ProfScope prof(GCAMB_K_CL, st);
-  if (d_dtype == GCAMB_F64)
-    cl_kernel<double><<<grid, 256, 0, st>>>(static_cast<const double *>(Delta), Pk, g->d_wk, g->nk, g->nl, Cl);
-  else
-    cl_kernel<float><<<grid, 256, 0, st>>>(static_cast<const float *>(Delta), Pk, g->d_wk, g->nk, g->nl, Cl);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = d_dtype == GCAMB_F64 ? launch_cl_sum<double, kAuto>(g, Delta, Delta, Pk, M, Cl, st)
+                                       : launch_cl_sum<float, kAuto>(g, Delta, Delta, Pk, M, Cl, st);
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "cl: launch");
   return GCAMB_OK;
 }
