@@ -157,6 +157,25 @@ int ensure_device_grid(gcamb_grid *g) {
     if (e != cudaSuccess) return e;
     return cudaMemcpy(*dst, src.data(), src.size() * sizeof(int), cudaMemcpyHostToDevice);
   };
+  auto up2 = [](float **dst, const std::vector<double> &src) -> cudaError_t {  // each double as the sum of two floats
+    std::vector<float> v(2 * src.size());
+    for (size_t i = 0; i < src.size(); ++i) {
+      v[2 * i] = (float)src[i];
+      v[2 * i + 1] = (float)(src[i] - (double)v[2 * i]);
+    }
+    cudaError_t e = cudaMalloc(dst, std::max<size_t>(1, v.size()) * sizeof(float));
+    if (e != cudaSuccess) return e;
+    return cudaMemcpy(*dst, v.data(), v.size() * sizeof(float), cudaMemcpyHostToDevice);
+  };
+  std::vector<double> dt(g->ntau), cl(g->nl);
+  for (int i = 0; i < g->ntau; ++i) dt[i] = g->tau0 - g->tau[i];
+  for (int r = 0; r < g->nl; ++r) {
+    const double l = g->lrow[r];
+    cl[r] = g->lrow[r] >= 2 ? std::sqrt((l + 2) * (l + 1) * l * (l - 1)) : 0.0;
+  }
+  if ((e = up2(&g->d_dt2, dt)) != cudaSuccess) return cuda_fail(e, "grid upload");
+  if ((e = up(&g->d_cl, cl)) != cudaSuccess) return cuda_fail(e, "grid upload");
+  if ((e = up2(&g->d_cl2, cl)) != cudaSuccess) return cuda_fail(e, "grid upload");
   if ((e = upi(&g->d_lrow, g->lrow)) != cudaSuccess) return cuda_fail(e, "grid upload");
   if ((e = upi(&g->d_rowof, g->rowof)) != cudaSuccess) return cuda_fail(e, "grid upload");
   // the mapped error word is set up here, with the grid's first device copy,
@@ -385,6 +404,9 @@ int gcamb_grid_destroy(gcamb_grid *g) {
   cudaFree(g->d_wk);
   cudaFree(g->d_xstart);
   cudaFree(g->d_xthr);
+  cudaFree(g->d_dt2);
+  cudaFree(g->d_cl);
+  cudaFree(g->d_cl2);
   cudaFree(g->d_lrow);
   cudaFree(g->d_rowof);
   delete g;

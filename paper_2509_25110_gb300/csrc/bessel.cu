@@ -665,6 +665,7 @@ int launch_bessel_table(gcamb_grid *g, int mode, cudaStream_t st) {
         t.nkb[e] = (g->ext[e] + lay.kb - 1) / lay.kb;
         t.off[e] = nb;
         nb += t.nkb[e];
+        t.max_nkb = std::max(t.max_nkb, t.nkb[e]);
       }
     t.nblocks = nb;
     if (mode == GCAMB_F16X3) {

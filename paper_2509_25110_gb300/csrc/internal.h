@@ -47,6 +47,7 @@ struct Table {
   std::vector<int32_t> nkb;   // [nk][nlt] tau-blocks stored per (k, l-tile)
   std::vector<int64_t> off;   // [nk][nlt] first block of the chunk
   int64_t nblocks = 0;
+  int max_nkb = 0;            // longest tau-prefix, in blocks
   void *d_data = nullptr;     // table blocks
   int32_t *d_nkb = nullptr;
   int64_t *d_off = nullptr;
@@ -92,6 +93,9 @@ struct gcamb_grid {
   double *d_k = nullptr, *d_tau = nullptr, *d_wtau = nullptr, *d_wk = nullptr;
   double *d_xstart = nullptr;
   double *d_xthr = nullptr;
+  double *d_cl = nullptr;  // [nl] sqrt((l+2)!/(l-2)!) of each row, 0 for l < 2
+  float *d_cl2 = nullptr;  // [nl][2] the same as the sum of two floats
+  float *d_dt2 = nullptr;  // [ntau][2]: tau0 - tau as the sum of two floats
   int nxs = 0;
   gcamb::Table tab[gcamb::kNumModes];
 };

@@ -1,18 +1,16 @@
 // Plain FP64 / FP32 path: the tau-window sum of Eq. (2) per (k, l) on the CUDA
 // cores (Algorithm 1's gang over k and vector loops over l and tau, here one
-// CTA per (l-tile, k, source chunk) and one warp per multipole row), and the
-// FP64 k-sum of Eq. (1).
+// CTA per (k, rows of an l-tile, source chunk)), and the FP64 k-sum of Eq. (1).
 #include <cmath>
+#include <type_traits>
 
 #include "internal.h"
 
 namespace gcamb {
 
-// Sum over the warp of each of the V values v[0..V) (V = 1, 2, 4, 8): every
-// step of the first log2(V) halves the values a lane holds (a lane keeps one
-// half, sends the other to its partner and adds what it receives), then plain
-// shuffle adds finish; lane L returns the total of value L >> (5 - log2 V).
-// (V - 1) + (5 - log2 V) adds a lane instead of 5 V.
+// The first step(s) of a sum over lanes of several values a lane holds: a
+// lane keeps half of its values, sends the other half to its partner (lane
+// XOR o) and adds what it receives.
 template <typename T, int N, int V>
 __device__ __forceinline__ void halve_lanes(T (&v)[V], int lane, int o) {
   const bool up = (lane & o) != 0;
@@ -24,166 +22,445 @@ __device__ __forceinline__ void halve_lanes(T (&v)[V], int lane, int o) {
   }
 }
 
-template <typename T, int V>
-__device__ __forceinline__ T reduce_lanes(T (&v)[V], int lane) {
-  static_assert(V == 1 || V == 2 || V == 4 || V == 8, "reduce_lanes: V in {1, 2, 4, 8}");
-  int o = 16;
-  if constexpr (V >= 8) {
-    halve_lanes<T, 4>(v, lane, o);
-    o >>= 1;
-  }
-  if constexpr (V >= 4) {
-    halve_lanes<T, 2>(v, lane, o);
-    o >>= 1;
-  }
-  if constexpr (V >= 2) {
-    halve_lanes<T, 1>(v, lane, o);
-    o >>= 1;
-  }
-  T t = v[0];
-  for (; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
+// Sum over the 8 lanes of a group of each of the RV values a lane holds
+// (RV = 4, 8); lane L of the group returns the total of value L / (8 / RV).
+// The additions of one value are the same for both RV (partners 4, 2, 1).
+template <typename T, int RV>
+__device__ __forceinline__ T reduce_group(T (&v)[RV], int lane) {
+  static_assert(RV == 4 || RV == 8, "reduce_group: RV in {4, 8}");
+  halve_lanes<T, RV / 2>(v, lane, 4);
+  halve_lanes<T, RV / 4>(v, lane, 2);
+  if constexpr (RV == 8) halve_lanes<T, 1>(v, lane, 1);
+  else v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  return v[0];
 }
 
-// One CTA: 128 multipoles x MC sources at one k.  The sources' tau-prefix is
-// staged in shared memory; each warp walks table rows (tau contiguous, read
-// coalesced), the lanes split tau and reduce by shuffles.
-//
-// xthr (temperature on flat j_l grids, else null): per row the Watson
-// threshold below which |j_l| < eps_cut.  The tile's tau-prefix is that of
-// its lowest multipole; a row stops at the first 64-node block whose first
-// node has x below its own threshold (x falls along tau, so every later node
-// is below it too): the terms left out are below eps_cut |w S| each.
-//
-// E = true: E-mode polarisation, Eq. (3) with eps_l(x) = c_l j_l(x)/x^2,
-// c_l = sqrt((l+2)!/(l-2)!).  The j_l table is shared with temperature: the
-// staged source is S_P/x^2, the row sum is multiplied by c_l.  Nodes with
-// x < x_lo (x = 0 included) are left out of the table sum: there the table's
-// j_2 may be cut to zero (activity threshold, Miller start) although
-// j_2(x)/x^2 -> 1/15.  They add, to l = 2 only, the power series
-//   j_2(x)/x^2 = 1/15 - x^2/210 + x^4/7560 - x^6/498960 + O(x^8)
-// (from j_l(x) = x^l sum_n (-x^2/2)^n / (n! (2l+2n+1)!!)); for l >= 3 their
-// eps_l is below c_l x_lo^(l-2)/(2l+1)!!, and x_lo <= 0.2.
-//
-// XP: the staged source is S x^-XP for x >= x_lo and 0 below (XP >= 0), or
-// S itself (XP < 0, temperature); E: the E-mode epilogue above (XP = 2).
-// XP = 0, 1, 2 without E give the raw sums D_XP[l] = sum_i w_i j_l S x^-XP of
-// the tensor-mode kernels.
-template <typename T, int MC, int XP, bool E>
-__global__ void __launch_bounds__(256) los_plain_kernel(const T *__restrict__ table, const int32_t *__restrict__ nkb,
-                                                        const int64_t *__restrict__ off, int nk, int nlt, int nl,
-                                                        const int *__restrict__ lrow, int ntau,
-                                                        const T *__restrict__ S, int M,
-                                                        T *__restrict__ Delta, const double *__restrict__ kk,
-                                                        const double *__restrict__ tau, double tau0,
-                                                        const double *__restrict__ wtau, double x_lo,
-                                                        const double *__restrict__ xthr) {
-  constexpr int KB = 64;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T *s = reinterpret_cast<T *>(smem_raw);  // [MC][ext]
-  __shared__ T res[MC][kTileL];
-  const int lt = blockIdx.x, q = blockIdx.y, m0 = blockIdx.z * MC;
-  const int row0 = lt * kTileL;  // first row (output index) of the tile
-  const size_t e_idx = (size_t)q * nlt + lt;
-  const int nb = nkb[e_idx];
-  const int ext = nb * KB;
-  const int mc = min(MC, M - m0);
-  for (int idx = threadIdx.x; idx < MC * ext; idx += blockDim.x) {
-    const int m = idx / ext, t = idx - m * ext;
-    T v = (m < mc && t < ntau) ? S[((size_t)(m0 + m) * nk + q) * ntau + t] : T(0);
-    if constexpr (XP >= 0) {
-      if (m < mc && t < ntau) {
-        const double x = kk[q] * (tau0 - tau[t]);
-        const double f = XP == 2 ? 1.0 / (x * x) : (XP == 1 ? 1.0 / x : 1.0);
-        v = x >= x_lo ? (T)((double)v * f) : T(0);
-      }
-    }
-    s[idx] = v;
+// What is summed against the table's w_i j_l:
+//   kFieldT       the sources themselves
+//   kFieldE       S_P x^-2, x = k (tau0 - tau) (E-mode, Eq. 3)
+//   kFieldTensor  S_P, S_P x^-1, S_P x^-2 and S_T x^-2 (tensor modes)
+enum PlainField { kFieldT = 0, kFieldE = 1, kFieldTensor = 2 };
+
+struct PlainArgs {
+  const int32_t *nkb;   // [nk][nlt] stored tau-blocks
+  const int64_t *off;   // [nk][nlt] first block
+  const int *lrow;      // [nl] multipole of each row
+  const double *kk, *tau, *wtau;
+  const float2 *dt2;    // [ntau] tau0 - tau as the sum of two floats
+  const double *cl;     // [nl] c_l = sqrt((l+2)!/(l-2)!) of each row (0 for l < 2)
+  const float2 *cl2;    // [nl] the same as the sum of two floats
+  const double *xthr;   // [nl] Watson thresholds, or null: every row takes the whole tile's prefix
+  double tau0, x_lo;
+  int nk, nlt, nl, ntau, M, lmin;
+  int q0;               // last k of the launch
+  int rows;             // rows per CTA: 128 or 64
+};
+
+constexpr int kPlainWarps = 4;
+constexpr int kPlainKB = 64;  // tau nodes per table block
+
+// Rows a lane holds at a time (a warp pass covers 4 of them per lane group).
+constexpr int plain_rv(int nv) { return nv == 1 ? 8 : 4; }
+
+// Steps whose table loads a lane has in flight together: FP64 is bound by its
+// pipe at one (2 measured the same), FP32 by loads in flight (E-mode, 5
+// sources, l_max 2001: 352 us at one, 318 at two).
+template <typename T>
+constexpr int plain_unroll() { return sizeof(T) == 8 ? 1 : 2; }
+
+// Tau blocks staged in shared memory at a time (64 KB of sources).
+constexpr int plain_stage_blocks(int nv, size_t esize) { return (int)(65536 / (nv * esize * kPlainKB)); }
+
+// x^-1 and x^-2 of one node as sums of two floats (about 2^-45 relative), from
+// x = k dt with k and dt as sums of two floats, in FP32 operations: GB300's
+// FP64 pipe runs at 1/64 of the FP32 rate.
+__device__ __forceinline__ void inv_x_ff(float2 k, float2 d, float2 &i1, float2 &i2) {
+  const float p = __fmul_rn(k.x, d.x);
+  float e = __fmaf_rn(k.x, d.x, -p);
+  e = __fmaf_rn(k.x, d.y, e);
+  e = __fmaf_rn(k.y, d.x, e);
+  const float r = __frcp_rn(p);
+  i1.x = r;
+  i1.y = __fmul_rn(r, __fmaf_rn(-e, r, __fmaf_rn(-p, r, 1.f)));
+  const float p2 = __fmul_rn(p, p);
+  const float e2 = __fmaf_rn(__fmul_rn(2.f, p), e, __fmaf_rn(p, p, -p2));
+  const float s = __frcp_rn(p2);
+  i2.x = s;
+  i2.y = __fmul_rn(s, __fmaf_rn(-e2, s, __fmaf_rn(-p2, s, 1.f)));
+}
+
+// v (f.x + f.y), rounded once but for the last bits of f.
+__device__ __forceinline__ float mul_ff(float v, float2 f) {
+  const float p = __fmul_rn(v, f.x);
+  const float e = __fmaf_rn(v, f.y, __fmaf_rn(v, f.x, -p));
+  return fabsf(p) <= 3.4e38f ? __fadd_rn(p, e) : p;  // overflow, infinities, NaN: the plain product
+}
+
+// The power series of the tensor kernels at small x for the nodes
+// below the cut, from j_l(x) = x^l s_l(x^2),
+// s_l(y) = sum_n (-y/2)^n / (n! (2l+2n+1)!!) (seven terms: exact to rounding
+// for x <= 0.2):
+//   e_l = x^(l-2) [l (l-1) s_l - 2 x^2 s_l + 2 s_(l-1)],
+//   b_l = 2 x^(l-1) [s_(l-1) - (l-1) s_l].
+__device__ __forceinline__ double sph_series(int l, double y) {
+  double df = 1.0;  // (2l+1)!!
+  for (int j = 3; j <= 2 * l + 1; j += 2) df *= j;
+  double term = 1.0 / df, sum = term;
+  for (int n = 0; n < 6; ++n) {
+    term *= (-0.5 * y) / ((n + 1) * (2.0 * l + 2 * n + 3));
+    sum += term;
   }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const T *chunk = table + (size_t)off[e_idx] * (kTileL * KB);
-  // A warp takes RV adjacent rows at a time, so that it holds V = MC RV = 8
-  // sums a lane and their cross-lane reduction costs 7 + 2 adds a lane for
-  // the 8 sums (5 a sum one at a time: on GB300's narrow FP64 pipe that was
-  // a third of the plain FP64 path's work for one source).
-  constexpr int RV = 8 / MC, V = MC * RV;
-  static_assert(kTileL % (8 * RV) == 0, "rows per warp pass");
-  for (int rb = warp * RV; rb < kTileL; rb += 8 * RV) {
-    T acc[V];  // acc[m * RV + i]: source m, row rb + i
-#pragma unroll
-    for (int j = 0; j < V; ++j) acc[j] = T(0);
-    int nbr[RV];  // blocks each row needs
-    int nbmax = 0;
-#pragma unroll
-    for (int i = 0; i < RV; ++i) {
-      nbr[i] = 0;
-      if (row0 + rb + i < nl) {
-        nbr[i] = nb;
-        if (xthr) {
-          const double xe = xthr[row0 + rb + i], kq = kk[q];
-          nbr[i] = 0;
-          for (int b0 = 0; b0 < nb; b0 += 32) {
-            const int b = b0 + lane;
-            nbr[i] += __popc(__ballot_sync(0xffffffffu, b < nb && kq * (tau0 - tau[b * KB]) >= xe));
-          }
-        }
-      }
-      nbmax = max(nbmax, nbr[i]);
+  return sum;
+}
+
+// E-mode term of row l from the sum D2 of S_P x^-2 j_l: c_l D2, plus, at
+// l = 2, the nodes below x_lo (the tail of the tau grid: x falls with tau)
+// through the power series
+//   j_2(x)/x^2 = 1/15 - x^2/210 + x^4/7560 - x^6/498960 + O(x^8)
+// (from j_l(x) = x^l sum_n (-x^2/2)^n / (n! (2l+2n+1)!!)): there the table's
+// j_2 may be cut to zero (activity threshold, Miller start) although
+// j_2(x)/x^2 -> 1/15.  For l >= 3 their eps_l is below
+// c_l x_lo^(l-2)/(2l+1)!!, and x_lo <= 0.2.
+template <typename T>
+__device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, T d2, const T *src) {
+  if (a.lrow[row] != 2) {
+    // c_l from the grid: its square root and the FP64 product per (row,
+    // source) took half of the FP32 kernel's time
+    if constexpr (sizeof(T) == 8) return a.cl[row] * d2;
+    else return mul_ff(d2, a.cl2[row]);
+  }
+  const double c = a.cl[row];
+  double d = c * (double)d2;
+  {
+    double tail = 0.0;
+    for (int i = a.ntau - 1; i >= 0; --i) {
+      const double x = kq * (a.tau0 - a.tau[i]);
+      if (!(x < a.x_lo)) break;
+      const double x2 = x * x;
+      const double e2 = 1.0 / 15.0 - x2 * (1.0 / 210.0 - x2 * (1.0 / 7560.0 - x2 / 498960.0));
+      tail += a.wtau[i] * (double)src[i] * e2;
     }
-    const T *rows = chunk + rb * KB + lane;
-    for (int b = 0; b < nbmax; ++b) {
-      const int t = b * KB + lane;
-      T sa[MC], sb[MC];
+    d += c * tail;
+  }
+  return (T)d;
+}
+
+// One CTA (4 warps): `rows` multipoles of an l-tile x MC sources at one k.
+// The sources' tau-prefix is staged in shared memory (times x^-1, x^-2 for
+// the polarisation and tensor fields; NV = MC or 4 MC staged vectors).
+//
+// What bounds it.  FP64: the DFMA pipe (two lanes a clock and SM), so every
+// FP64 instruction that is not a product of the sum counts: the row prefixes
+// are compared as integers, the lanes of a group of 8 share a row (16-byte
+// loads; the lane sums of 32 rows reduce in 7 adds, where a warp per row
+// needed 9 adds for 8), the tensor kernels read the table once for their
+// four sums and combine them here.  FP32: HBM for one source, else the FP32
+// pipe and shared-memory reads, which RV rows a lane amortise.
+// Measured (one model, before -> after): FP64 l_max 500 93 -> 69 us,
+// l_max 5000 9380 -> 7951 us (its products alone: 7300 us); tensor modes l_max
+// 1500 3105 (four passes and a combining one) -> 1948 us; FP32 E-mode, 5
+// sources, l_max 2001 950 -> 307 us.
+//
+// Splits: a warp pass covers 4 RV rows (lane group g, slot i: row 4 i + g);
+// the rows / 32 row warps take passes in turn, and the 128 / rows warps that
+// share a row take every (128 / rows)-th tau block; their sums are added in a
+// fixed order.  `rows` depends on the grid only (plain_rows), so a source's
+// result does not depend on the batch it came in.
+//
+// a.xthr (flat j_l grids, else null): per row the Watson threshold below
+// which |j_l| < eps_cut.  The tile's tau-prefix is that of its lowest
+// multipole; four adjacent rows stop at the first step (16 or 32 nodes) whose first
+// node has x below the lowest one's threshold (x falls along tau, so every
+// later node is below it too): the terms left out are below eps_cut |w S|
+// each.  With x^-1 or x^-2 only rows whose threshold is at least 1 stop:
+// j_l(x) x^-2 rises with x below the threshold (l >= 3 there), so each term
+// left out is below eps_cut |w S| as well.
+template <typename T, int MC, int FIELD>
+__global__ void __launch_bounds__(kPlainWarps * 32, 4)
+    los_plain_kernel(const T *__restrict__ table, const T *__restrict__ S, const T *__restrict__ ST,
+                     T *__restrict__ Delta, T *__restrict__ DE, T *__restrict__ DB, PlainArgs a) {
+  using V16 = std::conditional_t<sizeof(T) == 8, double2, float4>;
+  constexpr int KB = kPlainKB;
+  constexpr int NV = FIELD == kFieldTensor ? 4 * MC : MC;
+  constexpr int RV = plain_rv(NV);
+  constexpr int VE = 16 / sizeof(T);        // nodes per 16-byte load
+  constexpr int SN = 8 * VE;                // nodes per step of a lane group (128 bytes of a row): 16 or 32
+  constexpr int STEPS = KB / SN;            // steps per block
+  constexpr int CHB = plain_stage_blocks(NV, sizeof(T));
+  constexpr int HALO = FIELD == kFieldTensor ? 1 : 0;  // tensor: also the row before the CTA's first
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int R = a.rows, TS = kTileL / R;
+  const int q = a.q0 - blockIdx.y;          // the long prefixes (high k) first
+  const int lt = blockIdx.x / TS, rsub = (blockIdx.x - lt * TS) * R;
+  const int m0 = blockIdx.z * MC, mc = min(MC, a.M - m0);
+  const int row0 = lt * kTileL + rsub;      // first output row of the CTA
+  if (row0 >= a.nl) return;
+  const size_t e_idx = (size_t)q * a.nlt + lt;
+  const int nb = a.nkb[e_idx];
+  if (nb == 0 && (FIELD == kFieldT || a.lrow[row0] > 5)) {  // nothing active, no small-x tail: zeros
+    for (int idx = threadIdx.x; idx < mc * R; idx += kPlainWarps * 32) {
+      const int m = idx / R, r = idx - m * R;
+      if (row0 + r >= a.nl) continue;
+      const size_t o = ((size_t)(m0 + m) * a.nk + q) * a.nl + row0 + r;
+      Delta[o] = T(0);
+      if constexpr (FIELD == kFieldTensor) DE[o] = DB[o] = T(0);
+    }
+    return;
+  }
+  const double kq = a.kk[q];
+  const int stride = (nb < CHB ? nb : CHB) * KB;  // staged nodes per vector
+  T *s = reinterpret_cast<T *>(smem_raw);                       // [NV][stride]
+  T *res = s + (size_t)NV * stride;                             // [TS][NV][R]
+  long long *xb = reinterpret_cast<long long *>(res + (size_t)NV * kTileL);  // [nb STEPS] x of each step's first node
+  T *halo = reinterpret_cast<T *>(xb + nb * STEPS);             // tensor: [NV] sums of row row0 - 1
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int grp = lane >> 3, sub = lane & 7;
+  const int WR = kPlainWarps / TS, rw = warp % WR, ts = warp / WR;
+  // nonnegative doubles order as their bit patterns
+  for (int i = tid; i < nb * STEPS; i += kPlainWarps * 32)
+    xb[i] = i * SN < a.ntau ? __double_as_longlong(kq * (a.tau0 - a.tau[i * SN])) : -1;
+  for (int i = tid; i < NV * kTileL; i += kPlainWarps * 32) res[i] = T(0);
+  if (HALO && tid < NV) halo[tid] = T(0);
+  const T *chunk = table + (size_t)a.off[e_idx] * (kTileL * KB);
+  for (int b0 = 0; b0 < nb; b0 += CHB) {
+    const int nbc = min(CHB, nb - b0), nt = nbc * KB, t0 = b0 * KB;
+    if (b0) __syncthreads();
+    // ---- stage the sources of nodes t0 .. t0 + nt (zero beyond ntau)
+    if constexpr (FIELD == kFieldT) {
 #pragma unroll
       for (int m = 0; m < MC; ++m) {
-        sa[m] = s[m * ext + t];
-        sb[m] = s[m * ext + t + 32];
+        const T *src = S + ((size_t)(m0 + m) * a.nk + q) * a.ntau;
+#pragma unroll 4
+        for (int t = tid; t < nt; t += kPlainWarps * 32)
+          s[m * stride + t] = (m < mc && t0 + t < a.ntau) ? src[t0 + t] : T(0);
       }
+    } else {
+      const float kh = (float)kq;
+      const float2 k2 = make_float2(kh, (float)(kq - (double)kh));
+      // SU nodes' loads per thread in flight (a node at a time left the stage
+      // bound by load latency)
+      constexpr int SU = NV >= 8 ? 2 : 4;
+      for (int tb = tid; tb < nt; tb += SU * kPlainWarps * 32) {
+        T vv[SU][MC], ww[SU][MC];
 #pragma unroll
-      for (int i = 0; i < RV; ++i) {
-        if (b >= nbr[i]) continue;  // the same for every lane
-        const T *row = rows + i * KB + (size_t)b * kTileL * KB;
-        const T ja = __ldg(row), jb = __ldg(row + 32);
+        for (int u = 0; u < SU; ++u) {
+          const int t = tb + u * kPlainWarps * 32;
+          const bool in = t < nt && t0 + t < a.ntau;
 #pragma unroll
-        for (int m = 0; m < MC; ++m) {
-          acc[m * RV + i] = fma(ja, sa[m], acc[m * RV + i]);
-          acc[m * RV + i] = fma(jb, sb[m], acc[m * RV + i]);
+          for (int m = 0; m < MC; ++m) {
+            const size_t o = ((size_t)(m0 + m) * a.nk + q) * a.ntau + t0 + t;
+            vv[u][m] = (in && m < mc) ? S[o] : T(0);
+            ww[u][m] = (FIELD == kFieldTensor && in && m < mc) ? ST[o] : T(0);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+          const int t = tb + u * kPlainWarps * 32;
+          if (t >= nt) break;
+          const bool in = t0 + t < a.ntau;
+          const T(&v)[MC] = vv[u];
+          const T(&w)[MC] = ww[u];
+          T v0[MC], v1[MC], v2[MC], w2[MC];
+          bool keep = false, ff = false;
+          if constexpr (sizeof(T) == 4) {
+            const float2 d2 = in ? a.dt2[t0 + t] : make_float2(0.f, 0.f);
+            const float xf = k2.x * d2.x;
+            // well above the cut and inside FP32's range of x^2: no FP64 needed
+            ff = xf > 1e-14f && xf < 1e15f && xf > 1.01f * (float)a.x_lo && kh > 1e-30f && d2.x > 1e-30f;
+            if (ff) {
+              float2 i1, i2;
+              inv_x_ff(k2, d2, i1, i2);
+#pragma unroll
+              for (int m = 0; m < MC; ++m) {
+                v0[m] = v[m];
+                v1[m] = mul_ff(v[m], i1);
+                v2[m] = mul_ff(v[m], i2);
+                w2[m] = mul_ff(w[m], i2);
+              }
+              keep = true;
+            }
+          }
+          if (!ff) {
+            const double x = in ? kq * (a.tau0 - a.tau[t0 + t]) : 0.0;
+            keep = in && x >= a.x_lo;
+            const double i1 = FIELD == kFieldTensor && keep ? 1.0 / x : 0.0;
+            const double i2 = keep ? 1.0 / (x * x) : 0.0;
+#pragma unroll
+            for (int m = 0; m < MC; ++m) {
+              v0[m] = v[m];
+              v1[m] = FIELD == kFieldTensor ? (T)((double)v[m] * i1) : T(0);
+              v2[m] = (T)((double)v[m] * i2);
+              w2[m] = FIELD == kFieldTensor ? (T)((double)w[m] * i2) : T(0);
+            }
+          }
+#pragma unroll
+          for (int m = 0; m < MC; ++m) {
+            if constexpr (FIELD == kFieldE) {
+              s[m * stride + t] = keep ? v2[m] : T(0);
+            } else {
+              s[(4 * m + 0) * stride + t] = keep ? v0[m] : T(0);
+              s[(4 * m + 1) * stride + t] = keep ? v1[m] : T(0);
+              s[(4 * m + 2) * stride + t] = keep ? v2[m] : T(0);
+              s[(4 * m + 3) * stride + t] = keep ? w2[m] : T(0);
+            }
+          }
         }
       }
     }
-    // lane L holds the total of sum L >> 2
-    const T v = reduce_lanes<T, V>(acc, lane);
-    if ((lane & 3) == 0) {
-      const int j = lane >> 2;
-      res[j / RV][rb + j % RV] = v;
+    __syncthreads();
+    // ---- rows
+    for (int rb = rw * 4 * RV; rb < R; rb += WR * 4 * RV) {
+      int ns[RV];  // steps of this chunk that rows rb + 4 i .. + 3 need
+      const int nsc = nbc * STEPS;
+      int nmin = nsc, nmax = 0;
+#pragma unroll
+      for (int i = 0; i < RV; ++i) {
+        const int row = row0 + rb + 4 * i;
+        ns[i] = 0;
+        if (row < a.nl) {
+          ns[i] = nsc;
+          if (a.xthr) {
+            const double xe = a.xthr[row];
+            if (FIELD == kFieldT || xe >= 1.0) {
+              const long long xi = __double_as_longlong(xe);
+              int n = 0;
+              for (int c = 0; c < nsc; c += 32)
+                n += __popc(__ballot_sync(0xffffffffu, c + lane < nsc && xb[b0 * STEPS + c + lane] >= xi));
+              ns[i] = n;
+            }
+          }
+        }
+        nmax = max(nmax, ns[i]);
+        nmin = min(nmin, ns[i]);
+      }
+      T acc[NV][RV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int i = 0; i < RV; ++i) acc[v][i] = T(0);
+      const T *rows = chunk + (size_t)b0 * kTileL * KB + (rsub + rb + grp) * KB + sub * VE;
+      // steps that all RV row sets need, then the rest (a set's bound is
+      // uniform over the warp); UN steps' loads are in flight together
+      auto step = [&](int i0, auto un, auto check) {
+        constexpr int UN = decltype(un)::value;
+        V16 j[UN][RV];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+          const int st = i0 + u * TS;
+          const T *blk = rows + (size_t)(st / STEPS) * (kTileL * KB) + (st % STEPS) * SN;
+#pragma unroll
+          for (int i = 0; i < RV; ++i)
+            if (!check || st < ns[i]) j[u][i] = __ldg(reinterpret_cast<const V16 *>(blk + 4 * i * KB));
+        }
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+          const int st = i0 + u * TS;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const V16 sv = *reinterpret_cast<const V16 *>(s + v * stride + st * SN + sub * VE);
+#pragma unroll
+            for (int i = 0; i < RV; ++i) {
+              if (check && st >= ns[i]) continue;
+              const V16 t = j[u][i];
+              if constexpr (sizeof(T) == 8) {
+                acc[v][i] = fma(t.y, sv.y, fma(t.x, sv.x, acc[v][i]));
+              } else {
+                const float d = __fmaf_rn(t.w, sv.w, __fmaf_rn(t.z, sv.z, __fmaf_rn(t.y, sv.y, __fmul_rn(t.x, sv.x))));
+                acc[v][i] = __fadd_rn(acc[v][i], d);
+              }
+            }
+          }
+        }
+      };
+      constexpr int UN = plain_unroll<T>();
+      int st = ts;
+      for (; st + (UN - 1) * TS < nmin; st += UN * TS) step(st, std::integral_constant<int, UN>(), std::false_type());
+      for (; st < nmax; st += TS) step(st, std::integral_constant<int, 1>(), std::true_type());
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const T t = reduce_group<T, RV>(acc[v], lane);
+        constexpr int LPV = 8 / RV;  // lanes that end with the same value
+        if (sub % LPV == 0) {
+          T *r = res + (ts * NV + v) * R + rb + grp + 4 * (sub / LPV);
+          *r = b0 ? *r + t : t;
+        }
+      }
+    }
+    if constexpr (HALO) {
+      // tensor: row row0 - 1 (of this tile, or the last row of the tile before
+      // it, whose prefix is at least as long), by the last warp over all lanes
+      if (warp == kPlainWarps - 1 && row0 > 0) {
+        const int pr = row0 - 1, plt = pr / kTileL;
+        const T *prow = table + (size_t)a.off[(size_t)q * a.nlt + plt] * (kTileL * KB) + (size_t)b0 * kTileL * KB +
+                        (pr - plt * kTileL) * KB;
+        T h[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) h[v] = T(0);
+        for (int t = lane; t < nt; t += 32) {
+          const T j = __ldg(prow + (size_t)(t / KB) * kTileL * KB + t % KB);
+#pragma unroll
+          for (int v = 0; v < NV; ++v)
+            if (v % 4 != 3) h[v] = fma(j, s[v * stride + t], h[v]);
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          if (v % 4 == 3) continue;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) h[v] += __shfl_xor_sync(0xffffffffu, h[v], o);
+          if (lane == 0) halo[v] += h[v];
+        }
+      }
     }
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < MC * kTileL; idx += blockDim.x) {
-    const int m = idx / kTileL, r = idx - m * kTileL;
-    const int orow = row0 + r;
-    if (m < mc && orow < nl) {
-      T v = res[m][r];
-      if constexpr (E) {
-        const int l = lrow[orow];
-        const double c = l >= 2 ? sqrt((double)(l + 2) * (l + 1) * l * (l - 1)) : 0.0;
-        double d = c * (double)v;
-        if (l == 2) {  // the small-x nodes are the tail of the tau grid (x decreases with tau)
-          const T *src = S + ((size_t)(m0 + m) * nk + q) * ntau;
-          double tail = 0.0;
-          for (int i = ntau - 1; i >= 0; --i) {
-            const double x = kk[q] * (tau0 - tau[i]);
-            if (!(x < x_lo)) break;
-            const double x2 = x * x;
-            const double e2 = 1.0 / 15.0 - x2 * (1.0 / 210.0 - x2 * (1.0 / 7560.0 - x2 / 498960.0));
-            tail += wtau[i] * (double)src[i] * e2;
-          }
-          d += c * tail;
+  // ---- outputs
+  auto sum = [&](int v, int r) {
+    T t = res[v * R + r];
+    for (int i = 1; i < TS; ++i) t += res[(i * NV + v) * R + r];
+    return t;
+  };
+  for (int idx = tid; idx < mc * R; idx += kPlainWarps * 32) {
+    const int m = idx / R, r = idx - m * R;
+    const int row = row0 + r;
+    if (row >= a.nl) continue;
+    const size_t o = ((size_t)(m0 + m) * a.nk + q) * a.nl + row;
+    if constexpr (FIELD == kFieldT) {
+      Delta[o] = sum(m, r);
+    } else if constexpr (FIELD == kFieldE) {
+      Delta[o] = emode_row(a, row, kq, sum(m, r), S + ((size_t)(m0 + m) * a.nk + q) * a.ntau);
+    } else {
+      const size_t so = ((size_t)(m0 + m) * a.nk + q) * a.ntau;
+      const int l = a.lmin + row;
+      Delta[o] = emode_row(a, row, kq, sum(4 * m + 3, r), ST + so);
+      double ve = 0.0, vb = 0.0;
+      if (l >= 2) {
+        const double d0 = (double)sum(4 * m, r), d1 = (double)sum(4 * m + 1, r), d2 = (double)sum(4 * m + 2, r);
+        double p0, p1;  // D0, D1 of row l - 1
+        if (row == 0) {
+          // j_(l-1) = (2l+1)/x j_l - j_(l+1) (the sums leave out the same nodes)
+          p1 = a.nl > 1 ? (2.0 * l + 1.0) * d2 - (double)sum(4 * m + 1, 1) : 0.0;
+          p0 = a.nl > 1 ? (2.0 * l + 1.0) * d1 - (double)sum(4 * m, 1) : 0.0;
+        } else {
+          p0 = (double)(r > 0 ? sum(4 * m, r - 1) : halo[4 * m]);
+          p1 = (double)(r > 0 ? sum(4 * m + 1, r - 1) : halo[4 * m + 1]);
         }
-        v = (T)d;
+        ve = (double)l * (l - 1) * d2 - 2.0 * d0 + 2.0 * p1;
+        vb = 2.0 * p0 - 2.0 * (l - 1) * d1;
+        if (l <= 5) {
+          const T *src = S + so;
+          for (int i = a.ntau - 1; i >= 0; --i) {
+            const double x = kq * (a.tau0 - a.tau[i]);
+            if (x >= a.x_lo) break;
+            const double y = x * x, sl = sph_series(l, y), sm = sph_series(l - 1, y);
+            const double xl2 = l == 2 ? 1.0 : pow(x, l - 2);
+            const double ws = a.wtau[i] * (double)src[i];
+            ve += ws * xl2 * ((double)l * (l - 1) * sl - 2.0 * y * sl + 2.0 * sm);
+            vb += ws * 2.0 * xl2 * x * (sm - (l - 1) * sl);
+          }
+        }
       }
-      Delta[((size_t)(m0 + m) * nk + q) * nl + orow] = v;
+      DE[o] = (T)ve;
+      DB[o] = (T)vb;
     }
   }
 }
@@ -202,146 +479,140 @@ int emode_x_lo(const gcamb_grid *g, double *x_lo) {
   return x <= 0.2 ? 0 : -1;
 }
 
-template <typename T, int MC, int XP, bool E>
-static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, int M, T *Delta, cudaStream_t st) {
-  int max_ext = 0;
-  for (int v : t.nkb) max_ext = max_ext > v ? max_ext : v;
-  max_ext *= 64;
-  const size_t smem = (size_t)MC * max_ext * sizeof(T);
-  if (smem > 200 * 1024) return fail(GCAMB_EINVAL, "los_transfer: tau grid too long for the plain kernel");
-  cudaError_t e = cudaFuncSetAttribute(los_plain_kernel<T, MC, XP, E>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem > 0 ? smem : 16));
-  if (e != cudaSuccess) return cuda_fail(e, "los_transfer: smem attribute");
-  dim3 grid(g->nlt, g->nk, (M + MC - 1) / MC);
-  if (grid.z > 65535) return fail(GCAMB_EINVAL, "los_transfer: too many sources for one launch");
-  ProfScope prof(GCAMB_K_LOS_PLAIN, st);
-  double x_lo = 1e-12;
-  if (XP >= 0 && emode_x_lo(g, &x_lo))
+// Rows per CTA of the plain kernel: a whole 128-row tile, or 64 rows (the
+// CTA's four warps then share out the tau steps in pairs) where the tiles are
+// too few to balance the SMs.  Counted in CTAs of the longest prefix (blocks /
+// longest prefix): a log-spaced k grid has most of its work in the last few
+// k, so that the number of non-empty tiles says little.  Sampled multipoles
+// take 64 rows too: the prefixes of one tile's rows then span most of the
+// grid, and the warps of a CTA would finish far apart.  By the grid alone, so
+// that a source's sums do not depend on its batch.  Measured at 128 / 64 (32)
+// rows: l_max 500 (count 570) 73 / 69 (74) us; tensor l_max 1500 (2540) 1950 /
+// 2058 (2385); E-mode FP32 l_max 2001 (3063) 307 / 363 (495); l_max 5000
+// (19702) 7951 / 7962 (8334); sampled l_max 2500 (2043) 343 / 293 (302).
+static int plain_rows(const gcamb_grid *g, const Table &t) {
+  const double full = t.max_nkb > 0 ? (double)t.nblocks / t.max_nkb : 0.0;
+  return !g->lsampled && full >= 152 * 8 ? 128 : 64;
+}
+
+static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M) {
+  PlainArgs a{};
+  a.nkb = t.d_nkb;
+  a.off = t.d_off;
+  a.lrow = g->d_lrow;
+  a.kk = g->d_k;
+  a.tau = g->d_tau;
+  a.wtau = g->d_wtau;
+  a.dt2 = reinterpret_cast<const float2 *>(g->d_dt2);
+  // rows stop at their own prefix on flat j_l grids only
+  a.cl = g->d_cl;
+  a.cl2 = reinterpret_cast<const float2 *>(g->d_cl2);
+  a.xthr = (g->kernel == 0 && !g->curved) ? g->d_xthr : nullptr;
+  a.tau0 = g->tau0;
+  a.x_lo = 1e-12;
+  a.nk = g->nk;
+  a.nlt = g->nlt;
+  a.nl = g->nl;
+  a.ntau = g->ntau;
+  a.M = M;
+  a.lmin = g->lmin;
+  a.rows = plain_rows(g, t);
+  return a;
+}
+
+// nk, nlt: the k prefix and l-tiles of the launch (the whole grid, or an
+// uneven plan chunk's).
+template <typename T, int MC, int FIELD>
+static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, const T *ST, int M, T *D, T *DE, T *DB,
+                          int nk, int nlt, cudaStream_t st) {
+  constexpr int NV = FIELD == kFieldTensor ? 4 * MC : MC;
+  PlainArgs a = plain_args(g, t, M);
+  if (FIELD != kFieldT && emode_x_lo(g, &a.x_lo))
     return fail(GCAMB_EINVAL, "los_transfer: eps_cut too large for the l = 2 limit of the polarisation kernels");
-  // rows stop at their own prefix: temperature on flat j_l grids only (the
-  // polarisation and tensor sources carry 1/x^2, 1/x factors)
-  const double *xthr = (XP < 0 && !E && g->kernel == 0 && !g->curved) ? g->d_xthr : nullptr;
-  los_plain_kernel<T, MC, XP, E><<<grid, 256, smem, st>>>(static_cast<const T *>(t.d_data), t.d_nkb, t.d_off,
-                                                          g->nk, g->nlt, g->nl, g->d_lrow, g->ntau, S, M, Delta,
-                                                          g->d_k, g->d_tau, g->tau0, g->d_wtau, x_lo, xthr);
+  const int stage = t.max_nkb < plain_stage_blocks(NV, sizeof(T)) ? t.max_nkb : plain_stage_blocks(NV, sizeof(T));
+  const size_t smem = (size_t)NV * stage * kPlainKB * sizeof(T) + (size_t)NV * kTileL * sizeof(T) +
+                      (size_t)t.max_nkb * (kPlainKB * sizeof(T) / 128) * sizeof(long long) + NV * sizeof(T);
+  cudaError_t e = cudaFuncSetAttribute(los_plain_kernel<T, MC, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return cuda_fail(e, "los_transfer: smem attribute");
+  ProfScope prof(GCAMB_K_LOS_PLAIN, st);
+  a.q0 = nk - 1;
+  for (int m0 = 0; m0 < M; m0 += 65535 * MC) {
+    a.M = M - m0 < 65535 * MC ? M - m0 : 65535 * MC;
+    const dim3 grid(nlt * (kTileL / a.rows), nk, (a.M + MC - 1) / MC);
+    const size_t si = (size_t)m0 * g->nk * g->ntau, so = (size_t)m0 * g->nk * g->nl;
+    los_plain_kernel<T, MC, FIELD><<<grid, kPlainWarps * 32, smem, st>>>(
+        static_cast<const T *>(t.d_data), S + si, ST ? ST + si : nullptr, D + so, DE ? DE + so : nullptr,
+        DB ? DB + so : nullptr, a);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "los_transfer: launch");
   return GCAMB_OK;
 }
 
-template <int XP, bool E>
-static int launch_los_plain_k(const gcamb_grid *g, const void *S, int M, int mode, void *Delta, cudaStream_t st) {
+// Limits of the path: the staged tau-prefix of one chunk of sources (1, 2, 4,
+// FP32 also 8) fits 200 KB, and 65535 chunks.
+static int plain_limits(const Table &t, int M, int mode) {
+  const int mc = mode != GCAMB_PLAIN64 && M >= 8 ? 8 : (M >= 4 ? 4 : (M >= 2 ? 2 : 1));
+  const size_t smem = (size_t)mc * t.max_nkb * kPlainKB * (mode == GCAMB_PLAIN64 ? 8 : 4);
+  if (smem > 200 * 1024) return fail(GCAMB_EINVAL, "los_transfer: tau grid too long for the plain kernel");
+  if ((M + mc - 1) / mc > 65535) return fail(GCAMB_EINVAL, "los_transfer: too many sources for one launch");
+  return GCAMB_OK;
+}
+
+// Sources per CTA: the batch in equal chunks of at most 4 (FP64) or 8
+// (FP32).  The table is read once per chunk, and FP64 sums of sources
+// that are not there would cost as much as real ones.
+template <int FIELD>
+static int launch_los_plain_f(const gcamb_grid *g, const void *S, int M, int mode, void *Delta, cudaStream_t st) {
   const Table &t = g->tab[mode];
+  if (int rc = plain_limits(t, M, mode)) return rc;
   if (mode == GCAMB_PLAIN64) {
     auto s = static_cast<const double *>(S);
     auto d = static_cast<double *>(Delta);
-    if (M >= 4) return launch_plain_t<double, 4, XP, E>(g, t, s, M, d, st);
-    if (M >= 2) return launch_plain_t<double, 2, XP, E>(g, t, s, M, d, st);
-    return launch_plain_t<double, 1, XP, E>(g, t, s, M, d, st);
+    const int chunks = (M + 3) / 4, mc = (M + chunks - 1) / chunks;
+    auto go = [&](auto c) {
+      return launch_plain_t<double, decltype(c)::value, FIELD>(g, t, s, nullptr, M, d, nullptr, nullptr, g->nk, g->nlt,
+                                                               st);
+    };
+    if (mc == 1) return go(std::integral_constant<int, 1>());
+    if (mc == 2) return go(std::integral_constant<int, 2>());
+    if (mc == 3) return go(std::integral_constant<int, 3>());
+    return go(std::integral_constant<int, 4>());
   }
   auto s = static_cast<const float *>(S);
   auto d = static_cast<float *>(Delta);
-  if (M >= 8) return launch_plain_t<float, 8, XP, E>(g, t, s, M, d, st);
-  if (M >= 4) return launch_plain_t<float, 4, XP, E>(g, t, s, M, d, st);
-  if (M >= 2) return launch_plain_t<float, 2, XP, E>(g, t, s, M, d, st);
-  return launch_plain_t<float, 1, XP, E>(g, t, s, M, d, st);
+  const int chunks = (M + 7) / 8, mc = (M + chunks - 1) / chunks;
+  auto go = [&](auto c) {
+    return launch_plain_t<float, decltype(c)::value, FIELD>(g, t, s, nullptr, M, d, nullptr, nullptr, g->nk, g->nlt, st);
+  };
+  switch (mc) {
+    case 1: return go(std::integral_constant<int, 1>());
+    case 2: return go(std::integral_constant<int, 2>());
+    case 3: return go(std::integral_constant<int, 3>());
+    case 4: return go(std::integral_constant<int, 4>());
+    case 5: return go(std::integral_constant<int, 5>());
+    case 6: return go(std::integral_constant<int, 6>());
+    case 7: return go(std::integral_constant<int, 7>());
+    default: return go(std::integral_constant<int, 8>());
+  }
 }
 
 int launch_los_plain(const gcamb_grid *g, const void *S, int M, int mode, void *Delta, cudaStream_t st, bool emode) {
-  return emode ? launch_los_plain_k<2, true>(g, S, M, mode, Delta, st)
-               : launch_los_plain_k<-1, false>(g, S, M, mode, Delta, st);
+  return emode ? launch_los_plain_f<kFieldE>(g, S, M, mode, Delta, st)
+               : launch_los_plain_f<kFieldT>(g, S, M, mode, Delta, st);
 }
 
-// Tensor modes: power series of the tensor kernels at small x for the nodes
-// below the cut, from j_l(x) = x^l s_l(x^2),
-// s_l(y) = sum_n (-y/2)^n / (n! (2l+2n+1)!!) (seven terms: exact to rounding
-// for x <= 0.2):
-//   e_l = x^(l-2) [l (l-1) s_l - 2 x^2 s_l + 2 s_(l-1)],
-//   b_l = 2 x^(l-1) [s_(l-1) - (l-1) s_l].
-__device__ __forceinline__ double sph_series(int l, double y) {
-  double df = 1.0;  // (2l+1)!!
-  for (int j = 3; j <= 2 * l + 1; j += 2) df *= j;
-  double term = 1.0 / df, sum = term;
-  for (int n = 0; n < 6; ++n) {
-    term *= (-0.5 * y) / ((n + 1) * (2.0 * l + 2 * n + 3));
-    sum += term;
-  }
-  return sum;
-}
-
-// Combines the raw tensor sums, in place: D0 -> Delta_E, D1 -> Delta_B
-// (D2 read only), one CTA per (source, k) row walking l in chunks.
+// Tensor modes, one launch: D0, D1, D2 of S_P and the x^-2 sum of S_T share
+// each table load, and each CTA combines its rows (with the row before its
+// first):
+//   Delta_T[l] = c_l (x^-2 sum of S_T) + the l = 2 tail
 //   Delta_E[l] = l (l-1) D2[l] - 2 D0[l] + 2 D1[l-1] + tail_e(l)
 //   Delta_B[l] = 2 D0[l-1] - 2 (l-1) D1[l] + tail_b(l)
 // Row l-1 of the first multipole (lmin >= 2) comes from the recurrence
 // j_(l-1) = (2l+1)/x j_l - j_(l+1):  D1[l-1] = (2l+1) D2[l] - D1[l+1],
 // D0[l-1] = (2l+1) D1[l] - D0[l+1] (all three sums leave out the same nodes).
 // The tails add, for l = 2..5, the series terms of the nodes below the cut.
-template <typename T>
-__global__ void __launch_bounds__(256) tensor_combine_kernel(T *__restrict__ DE, T *__restrict__ DB,
-                                                             const T *__restrict__ D2, const T *__restrict__ SP,
-                                                             const double *__restrict__ kk,
-                                                             const double *__restrict__ tau, double tau0,
-                                                             const double *__restrict__ wtau, double x_lo, int nk,
-                                                             int ntau, int lmin, int lmax) {
-  __shared__ double carry[2];
-  const int nl = lmax - lmin + 1;
-  const size_t row = blockIdx.x;  // m * nk + q
-  const int q = (int)(row % nk);
-  T *e = DE + row * nl;
-  T *b = DB + row * nl;
-  const T *d2 = D2 + row * nl;
-  const T *src = SP + row * ntau;
-  for (int base = 0; base < nl; base += blockDim.x) {
-    const int idx = base + threadIdx.x;
-    const int l = lmin + idx;
-    double d0 = 0, d1 = 0, dd2 = 0, p0 = 0, p1 = 0;
-    if (idx < nl) {
-      d0 = (double)e[idx];
-      d1 = (double)b[idx];
-      dd2 = (double)d2[idx];
-      if (idx == 0) {
-        if (l >= 2 && nl > 1) {
-          p1 = (2.0 * l + 1.0) * dd2 - (double)b[1];
-          p0 = (2.0 * l + 1.0) * d1 - (double)e[1];
-        }
-      } else if (threadIdx.x == 0) {
-        p0 = carry[0];
-        p1 = carry[1];
-      } else {
-        p0 = (double)e[idx - 1];
-        p1 = (double)b[idx - 1];
-      }
-    }
-    __syncthreads();  // every read of this chunk (and of the carry) precedes its writes
-    if (threadIdx.x == blockDim.x - 1) {
-      carry[0] = d0;
-      carry[1] = d1;
-    }
-    if (idx < nl) {
-      double ve = 0.0, vb = 0.0;
-      if (l >= 2) {
-        ve = (double)l * (l - 1) * dd2 - 2.0 * d0 + 2.0 * p1;
-        vb = 2.0 * p0 - 2.0 * (l - 1) * d1;
-        if (l <= 5) {
-          for (int i = ntau - 1; i >= 0; --i) {
-            const double x = kk[q] * (tau0 - tau[i]);
-            if (x >= x_lo) break;
-            const double y = x * x, sl = sph_series(l, y), sm = sph_series(l - 1, y);
-            const double xl2 = l == 2 ? 1.0 : pow(x, l - 2);
-            const double ws = wtau[i] * (double)src[i];
-            ve += ws * xl2 * ((double)l * (l - 1) * sl - 2.0 * y * sl + 2.0 * sm);
-            vb += ws * 2.0 * xl2 * x * (sm - (l - 1) * sl);
-          }
-        }
-      }
-      e[idx] = (T)ve;
-      b[idx] = (T)vb;
-    }
-    __syncthreads();  // the carry is read by the next chunk
-  }
-}
-
 int launch_los_tensor(const gcamb_grid *g, const void *ST, const void *SP, int M, int mode, void *DT, void *DE,
                       void *DB, cudaStream_t st) {
   if (g->lsampled)
@@ -350,30 +621,17 @@ int launch_los_tensor(const gcamb_grid *g, const void *ST, const void *SP, int M
     return fail(GCAMB_EINVAL, "los_transfer_tensor: needs lmax > lmin when lmin >= 2 (the kernels take j_(l-1))");
   double x_lo = 1e-12;
   if (emode_x_lo(g, &x_lo)) return fail(GCAMB_EINVAL, "los_transfer_tensor: eps_cut too large for the l = 2 limit");
-  // raw sums of the polarisation source: D0 -> DE, D1 -> DB, D2 -> DT
-  int rc = launch_los_plain_k<0, false>(g, SP, M, mode, DE, st);
-  if (!rc) rc = launch_los_plain_k<1, false>(g, SP, M, mode, DB, st);
-  if (!rc) rc = launch_los_plain_k<2, false>(g, SP, M, mode, DT, st);
-  if (rc) return rc;
-  const unsigned rows = (unsigned)((size_t)M * g->nk);
   if ((size_t)M * g->nk > 0x7fffffffULL) return fail(GCAMB_EINVAL, "los_transfer_tensor: too many rows");
-  {
-    ProfScope prof(GCAMB_K_LOS_PLAIN, st);
-    if (mode == GCAMB_PLAIN64)
-      tensor_combine_kernel<double><<<rows, 256, 0, st>>>(static_cast<double *>(DE), static_cast<double *>(DB),
-                                                          static_cast<const double *>(DT),
-                                                          static_cast<const double *>(SP), g->d_k, g->d_tau,
-                                                          g->tau0, g->d_wtau, x_lo, g->nk, g->ntau, g->lmin, g->lmax);
-    else
-      tensor_combine_kernel<float><<<rows, 256, 0, st>>>(static_cast<float *>(DE), static_cast<float *>(DB),
-                                                         static_cast<const float *>(DT),
-                                                         static_cast<const float *>(SP), g->d_k, g->d_tau, g->tau0,
-                                                         g->d_wtau, x_lo, g->nk, g->ntau, g->lmin, g->lmax);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "los_transfer_tensor: launch");
-  }
-  // temperature: t_l = c_l j_l / x^2, the E-mode kernel of Eq. (3), into DT
-  return launch_los_plain_k<2, true>(g, ST, M, mode, DT, st);
+  const Table &t = g->tab[mode];
+  if (int rc = plain_limits(t, M, mode)) return rc;
+  auto go = [&](auto v, auto c) {
+    using T = decltype(v);
+    return launch_plain_t<T, decltype(c)::value, kFieldTensor>(
+        g, t, static_cast<const T *>(SP), static_cast<const T *>(ST), M, static_cast<T *>(DT), static_cast<T *>(DE),
+        static_cast<T *>(DB), g->nk, g->nlt, st);
+  };
+  if (mode == GCAMB_PLAIN64) return go(0.0, std::integral_constant<int, 1>());
+  return M >= 2 ? go(0.f, std::integral_constant<int, 2>()) : go(0.f, std::integral_constant<int, 1>());
 }
 
 // C^XY_l[m] = 4 pi sum_k w_k P[m][k] DX[m][k][l] DY[m][k][l] in FP64 (kCross;
@@ -533,23 +791,12 @@ int launch_plain_plan(const gcamb_grid *g, const float *S, const double *Pk, int
       const int lt = (r < 0 ? 0 : r) / kTileL;
       ltc = lt > ltc ? lt : ltc;
     }
-    int max_ext = 0;
-    for (int v : t.nkb) max_ext = max_ext > v ? max_ext : v;
-    max_ext *= 64;
-    constexpr int MC = 8;
-    const size_t smem = (size_t)MC * max_ext * sizeof(float);
-    if (smem > 200 * 1024) return fail(GCAMB_EINVAL, "plan_launch: tau grid too long for the plain kernel");
-    cudaError_t e = cudaFuncSetAttribute(los_plain_kernel<float, MC, -1, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem > 0 ? smem : 16));
-    if (e != cudaSuccess) return cuda_fail(e, "plan_launch: smem attribute");
-    const double *xthr = (g->kernel == 0 && !g->curved) ? g->d_xthr : nullptr;
-    {
-      ProfScope prof(GCAMB_K_LOS_PLAIN, st);
-      dim3 grid(ltc + 1, nkc, (mc + MC - 1) / MC);
-      los_plain_kernel<float, MC, -1, false><<<grid, 256, smem, st>>>(
-          static_cast<const float *>(t.d_data), t.d_nkb, t.d_off, g->nk, g->nlt, g->nl, g->d_lrow, g->ntau,
-          S + (size_t)m0 * g->nk * g->ntau, mc, D, g->d_k, g->d_tau, g->tau0, g->d_wtau, 1e-12, xthr);
-    }
+    if ((size_t)8 * t.max_nkb * kPlainKB * sizeof(float) > 200 * 1024)
+      return fail(GCAMB_EINVAL, "plan_launch: tau grid too long for the plain kernel");
+    const float *Sc = S + (size_t)m0 * g->nk * g->ntau;
+    if (int rc = launch_plain_t<float, 8, kFieldT>(g, t, Sc, nullptr, mc, D, nullptr, nullptr, nkc, ltc + 1, st))
+      return rc;
+    cudaError_t e = cudaSuccess;
     {
       ProfScope prof(GCAMB_K_CL, st);
       e = launch_cl_sum<float, kPrefix>(g, D, D, Pk, mc, Cl, st, ClPrefix{g->d_k, g->d_lrow, d_lmax, d_nk, m0});

@@ -1,0 +1,88 @@
+"""The plain transfers at the edges of their tiling: multipole tiles and row
+sets that are not full, tau grids of one node, around a step, a block and the
+staged chunk, the batch sizes of every sources-per-CTA variant, and both row
+splits (64 rows where the grid is small, 128 where it is large), against the
+FP64 oracle.
+
+Bounds.  FP64: 1e-11 of the model's largest |Delta| (the recurrences of the
+table, as in the other parity tests).  FP32, per element: table, source and
+product roundings plus at most ntau / 32 + 12 additions in sequence, each
+2^-24 of A = sum_i w_i |S_i| |kernel_l(x_i)|, and the terms the grid's activity
+threshold leaves out, each below eps_cut = 1e-30 times w_i |S_i| (E-mode: times
+c_l, the kernel's prefactor)."""
+import numpy as np
+import pytest
+
+from paper_2509_25110_gb300 import build, gcamb, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    gcamb.lib()
+
+
+def make(nk, ntau, lmax, M, seed):
+    k = synth.log_grid(1e-3, 0.08, nk)
+    tau = synth.uniform_grid(200.0, 14000.0, ntau) if ntau > 1 else np.array([300.0])
+    rng = np.random.default_rng(seed)
+    S = rng.standard_normal((2, M, nk, ntau)) * (1.0 + 10.0 * rng.random((2, M, 1, 1)))
+    g = gcamb.grid_create(k, tau, 14000.0, 2, lmax)
+    return k, tau, S, g
+
+
+CASES = [  # nk, ntau, lmax, M
+    (3, 1, 2, 1), (3, 15, 3, 2), (4, 16, 33, 3), (4, 17, 34, 4), (3, 63, 65, 5), (3, 64, 128, 6), (3, 65, 129, 7),
+    (2, 129, 130, 8), (2, 300, 257, 9), (2, 2049, 200, 2), (2, 2113, 70, 1), (1300, 40, 131, 1), (1300, 70, 190, 5),
+]
+
+
+@pytest.mark.parametrize("nk,ntau,lmax,M", CASES)
+def test_fp64_fields(orc, nk, ntau, lmax, M):
+    k, tau, S, g = make(nk, ntau, lmax, M, seed=nk + ntau)
+    gcamb.bessel_table(g, gcamb.PLAIN64)
+    d = [torch.as_tensor(s, device="cuda") for s in S]
+    got = [gcamb.los_transfer(g, d[0], gcamb.PLAIN64), gcamb.los_transfer_e(g, d[1], gcamb.PLAIN64)]
+    ref = [orc.los_cl(k, tau, 14000.0, 2, lmax, S[0], want_cl=False)[0], orc.los_e(k, tau, 14000.0, 2, lmax, S[1])]
+    if lmax > 2:
+        got += gcamb.los_transfer_tensor(g, d[0], d[1], gcamb.PLAIN64)
+        ref += orc.los_tensor(k, tau, 14000.0, 2, lmax, S[0], S[1])
+    gcamb.sync()
+    for a, r in zip(got, ref):
+        scale = np.abs(r).reshape(M, -1).max(axis=1)[:, None, None] + 1e-300
+        assert (np.abs(a.cpu().numpy() - r) <= 1e-11 * scale).all(), np.max(np.abs(a.cpu().numpy() - r) / scale)
+    # a source's sums do not depend on the batch it came in
+    one = gcamb.los_transfer(g, d[0][M - 1:].contiguous(), gcamb.PLAIN64)
+    gcamb.sync()
+    assert torch.equal(one[0], got[0][M - 1])
+
+
+@pytest.mark.parametrize("nk,ntau,lmax,M", CASES)
+def test_fp32_fields(orc, nk, ntau, lmax, M):
+    k, tau, S, g = make(nk, ntau, lmax, M, seed=nk + ntau + 1)
+    S = S.astype(np.float32).astype(np.float64)
+    gcamb.bessel_table(g, gcamb.PLAIN32)
+    d = [torch.as_tensor(s, dtype=torch.float32, device="cuda") for s in S]
+    got = [gcamb.los_transfer(g, d[0], gcamb.PLAIN32), gcamb.los_transfer_e(g, d[1], gcamb.PLAIN32)]
+    gcamb.sync()
+    x = k[:, None] * (14000.0 - tau)[None, :]
+    j = orc.sph_bessel(lmax, x.ravel()).reshape(nk, ntau, -1)[:, :, 2:]
+    l = np.arange(2, lmax + 1)[None, None, :]
+    xs = np.maximum(x, 1e-3)[:, :, None]
+    e = np.where(x[:, :, None] < 1e-3, np.where(l == 2, np.sqrt(24.0) / 15.0, 0.0),
+                 np.sqrt((l + 2.0) * (l + 1.0) * l * (l - 1.0)) * j / xs ** 2)
+    w = orc.trapz_weights(tau)
+    c = np.sqrt((l + 2.0) * (l + 1.0) * l * (l - 1.0))
+    for s, kern, pre, a in ((S[0], j, 1.0, got[0]), (S[1], e, c, got[1])):
+        r = np.einsum("mqt,qtl->mql", s * w, kern)
+        A = np.einsum("mqt,qtl->mql", np.abs(s) * w, np.abs(kern))
+        tol = (ntau / 32.0 + 12.0) * 2.0 ** -24
+        err = np.abs(a.cpu().numpy() - r)
+        left_out = 1e-30 * pre * (np.abs(s) * w).sum(2)[:, :, None]
+        assert (err <= tol * A + left_out).all(), np.max(err / (tol * A + left_out + 1e-300))
