@@ -656,6 +656,12 @@ int gcamb_probe_flops(int what, double *flops) {
   return run_probe_flops(what, flops);
 }
 
+int gcamb_probe_mma(const float *A, const float *B, int K, float *C, void *stream) {
+  if (!A || !B || !C) return fail(GCAMB_EINVAL, "probe_mma: NULL pointer");
+  if (K < 1 || K > (1 << 20)) return fail(GCAMB_EINVAL, "probe_mma: K must be in [1, 2^20]");
+  return run_probe_mma(A, B, K, C, (cudaStream_t)stream);
+}
+
 int gcamb_selftest_wait(int *status, void *stream) { return run_wait_selftest(status, (cudaStream_t)stream); }
 
 }  // extern "C"

@@ -4,9 +4,10 @@
 // (l = lmin..lmax of a grid).  It is trained on the device by the library's
 // own kernels: tcgen05 GEMMs with bf16 operands and FP32 accumulation
 // (emu_gemm.cuh) for the forward pass, the input and weight gradients, and
-// small kernels for GELU, the loss, bias gradients and Adam.  Parameters and
-// Adam moments are FP32; every matrix-product operand is rounded to bf16 at
-// load time.  A held-out check (spectra from the projection path) marks cells
+// small kernels for the loss, bias gradients and Adam.  Parameters and Adam
+// moments are FP32, as are pre-activations and gradients; every matrix-product
+// operand is rounded to bf16 once, by the kernel that produces it (Adam writes
+// the weights' bf16 copies beside the FP32 ones).  A held-out check (spectra from the projection path) marks cells
 // of parameter space as trusted; gcamb_emulate answers trusted requests from
 // the network and the rest from the batched projection (gcamb_los_cl) on
 // sources regenerated from the features.
@@ -32,12 +33,20 @@ struct gcamb_emu {
   size_t n_params = 0;
   float *theta = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
   float *mu_x = nullptr, *isd_x = nullptr, *mu_y = nullptr, *sd_y = nullptr;
-  float *xs = nullptr, *out = nullptr, *d0 = nullptr, *d1 = nullptr, *loss_part = nullptr, *loss = nullptr;
-  std::vector<float *> Z, H;             // hidden pre-activations and activations [B][width]
-  // feature-major copies, so that every GEMM operand is contiguous along its
-  // contraction index: xs^T, H^T [width][B], the gradients' (d)^T, W^T
-  float *xsT = nullptr, *dT0 = nullptr, *dT1 = nullptr, *WT = nullptr, *splitk = nullptr;
-  std::vector<float *> HT;
+  float *loss_part = nullptr;             // the last layer's warps' sums of squared errors
+  // bf16 operands, rows padded to 8 elements (the copies' 16-byte strides):
+  // weights [out][in], standardised features and activations [B][in] (act[l]
+  // is the input of layer l), gradients wrt the pre-activations [B][out]
+  std::vector<__nv_bfloat16 *> W, act, dB;
+  std::vector<float *> Z, dF;            // FP32 [B][padded width]: hidden pre-activations, gradients wrt the pre-activations
+  unsigned long long *exp_tab = nullptr; // exp2 tables of exp_q53
+  int *flags_host = nullptr, *flags_dev = nullptr;  // mapped host copy of emulate's fallback flags
+  // tensor maps of those buffers for the last batch size
+  struct Maps {
+    CUtensorMap act_k, act_mn, d_k, d_mn, w_k, w_mn;
+  };
+  std::vector<Maps> maps;
+  int maps_B = 0;
   int64_t step = 0;
   int *err = nullptr;
   // trust cells: bit d of a cell is (x[cell_dim[d]] > cell_mid[d])
@@ -62,7 +71,6 @@ static int amp_col(const gcamb_emu *e) { return e->n_in == 9 ? 8 : -1; }
 
 namespace {
 
-constexpr int kLossBlocks = 256;
 constexpr uint32_t kEmuMagic = 0x47454D55u;  // "GEMU"
 
 int ck(cudaError_t e, const char *what) { return e == cudaSuccess ? GCAMB_OK : cuda_fail(e, what); }
@@ -94,97 +102,144 @@ __global__ void init_uniform_kernel(float *p, size_t n, float bound, uint64_t se
   }
 }
 
+// Standardised features, rounded to the bf16 operand of the first layer.
 __global__ void standardize_kernel(const float *__restrict__ X, const int *__restrict__ idx, int B, int n,
-                                   const float *__restrict__ mu, const float *__restrict__ isd, float *__restrict__ xs,
-                                   float *__restrict__ xsT) {
+                                   const float *__restrict__ mu, const float *__restrict__ isd,
+                                   __nv_bfloat16 *__restrict__ xs, int ld) {
+  pdl_start();
+  pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= B * n) return;
   const int b = e / n, j = e - b * n;
   const int r = idx ? idx[b] : b;
-  const float v = (X[(size_t)r * n + j] - mu[j]) * isd[j];
-  xs[e] = v;
-  if (xsT) xsT[(size_t)j * B + b] = v;
+  xs[(size_t)b * ld + j] = __float2bfloat16_rn((X[(size_t)r * n + j] - mu[j]) * isd[j]);
 }
 
-// dOut = 2 (out - y) / (B N); per-block partial sums of (out - y)^2
-__global__ void __launch_bounds__(256) loss_kernel(const float *__restrict__ out, const float *__restrict__ Y,
-                                                   const int *__restrict__ idx, int B, int N, float *__restrict__ dout,
-                                                   float *__restrict__ doutT, float *__restrict__ part) {
-  __shared__ float red[256];
-  const size_t total = (size_t)B * N;
-  const float scale = 2.f / (float)total;
-  float acc = 0.f;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t b = e / N, n = e - b * N;
-    const size_t r = idx ? (size_t)idx[b] : b;
-    const float d = out[e] - Y[r * N + n];
-    dout[e] = scale * d;
-    doutT[n * B + b] = scale * d;
-    acc += d * d;
-  }
-  red[threadIdx.x] = acc;
+constexpr int kSumCols = 16;    // columns of a block of bias_kernel
+constexpr int kSumClasses = 32;
+
+// Column sums by rows mod 32: thread (column c, class r) holds the sum of its
+// rows b = r, r + 32, ... in increasing order; the classes are added as a
+// balanced tree (16, 8, 4, 2, 1 apart).  Fixed order: deterministic.
+__device__ __forceinline__ void class_sum(float (*s)[kSumCols + 1], int c, int r, float v, float *out) {
+  s[r][c] = v;
   __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+#pragma unroll
+  for (int o = kSumClasses / 2; o > 0; o >>= 1) {
+    if (r < o) s[r][c] += s[r + o][c];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  if (r == 0 && out) *out = s[0][c];
 }
 
-__global__ void loss_final_kernel(const float *__restrict__ part, int nb, float inv_total, float *__restrict__ loss) {
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < nb; ++i) s += part[i];
-    *loss = (float)(s * inv_total);
-  }
-}
+// Bias gradients of every layer (grid y): column sums of d [B][ld], all of a
+// thread's next 32 rows in flight.  The grid's last block adds up the loss
+// from the warps' partial sums, in order.
+constexpr int kMaxLayers = 9;
+struct BiasSums {
+  const float *d[kMaxLayers];
+  float *db[kMaxLayers];
+  int N[kMaxLayers], ld[kMaxLayers];
+  const float *part;
+  int nparts;
+  float inv_total;
+  float *loss;
+};
 
-// db[n] = sum_b DT[n][b]: one warp per row, lanes in a fixed order then a
-// fixed shuffle tree (deterministic)
-__global__ void rowsum_kernel(const float *__restrict__ DT, int B, int N, float *__restrict__ db) {
-  const int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (n >= N) return;
-  float s = 0.f;
-  for (int b = lane; b < B; b += 32) s += DT[(size_t)n * B + b];
+__global__ void __launch_bounds__(kSumCols *kSumClasses) bias_kernel(const __grid_constant__ BiasSums a, int B, int L) {
+  __shared__ float s[kSumClasses][kSumCols + 1];
+  __shared__ double red[kSumCols * kSumClasses / 32];
+  const int c = threadIdx.x % kSumCols, r = threadIdx.x / kSumCols, l = blockIdx.y;
+  pdl_start();
+  pdl_wait();
+  if (l == L) {
+    if (blockIdx.x > 0 || !a.loss) return;
+    double t = 0.0;
+    for (int i = threadIdx.x; i < a.nparts; i += kSumCols * kSumClasses) t += (double)a.part[i];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) db[n] = s;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int i = 1; i < kSumCols * kSumClasses / 32; ++i) t += red[i];
+      *a.loss = (float)(t * a.inv_total);
+    }
+    return;
+  }
+  const int n = blockIdx.x * kSumCols + c, N = a.N[l];
+  if (blockIdx.x * kSumCols >= (unsigned)N) return;  // the whole block
+  const float *d = a.d[l];
+  const size_t ld = a.ld[l];
+  float sum = 0.f;
+  if (n < N) {
+    int b = r;
+    for (; b + 31 * kSumClasses < B; b += 32 * kSumClasses) {
+      float v[32];
+#pragma unroll
+      for (int u = 0; u < 32; ++u) v[u] = __ldcg(d + (size_t)(b + u * kSumClasses) * ld + n);
+#pragma unroll
+      for (int u = 0; u < 32; ++u) sum += v[u];
+    }
+    for (; b < B; b += kSumClasses) sum += d[(size_t)b * ld + n];
+  }
+  class_sum(s, c, r, sum, n < N ? a.db[l] + n : nullptr);
 }
 
-// WT[i][o] = W[o][i]
-__global__ void transpose_kernel(const float *__restrict__ W, int nout, int nin, float *__restrict__ WT) {
-  __shared__ float t[32][33];
-  const int o0 = blockIdx.y * 32, i0 = blockIdx.x * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int o = o0 + r, i = i0 + threadIdx.x;
-    if (o < nout && i < nin) t[r][threadIdx.x] = W[(size_t)o * nin + i];
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int i = i0 + r, o = o0 + threadIdx.x;
-    if (o < nout && i < nin) WT[(size_t)i * nout + o] = t[threadIdx.x][r];
-  }
-}
-
-// C[e] = sum_z part[z][e], increasing z
-__global__ void splitk_reduce_kernel(const float *__restrict__ part, int nz, size_t n, float *__restrict__ C) {
+// bf16 copies of the weights from the FP32 parameters.
+__global__ void weights_bf16_kernel(const float *__restrict__ W, int nout, int nin, __nv_bfloat16 *__restrict__ Wb,
+                                    int ld) {
+  const size_t n = (size_t)nout * nin;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < nz; ++z) s += part[(size_t)z * n + e];
-    C[e] = s;
+    const size_t o = e / nin;
+    Wb[o * ld + (e - o * nin)] = __float2bfloat16_rn(W[e]);
   }
 }
+
+// Adam on the flat parameters; layer grid y writes its weights' bf16 copy too.
+struct AdamLayers {
+  size_t w_off[kMaxLayers], end[kMaxLayers];  // the layer's first weight, one past its last bias
+  unsigned int nw[kMaxLayers];                // weights
+  int nin[kMaxLayers], ld[kMaxLayers];
+  __nv_bfloat16 *Wb[kMaxLayers];
+};
 
 __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                            float *__restrict__ v, size_t n, float lr, float b1, float b2, float eps, float bc1,
+                            float *__restrict__ v, AdamLayers L, float lr, float b1, float b2, float eps, float bc1,
                             float bc2) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+  constexpr int U = 4;  // parameters a thread, all loads in flight
+  pdl_start();
+  const int l = blockIdx.y;
+  const size_t base = L.w_off[l];
+  const unsigned int n = (unsigned int)(L.end[l] - base), nw = L.nw[l], nin = L.nin[l];
+  pdl_wait();
+  for (unsigned int e0 = blockIdx.x * (blockDim.x * U) + threadIdx.x; e0 < n; e0 += gridDim.x * (blockDim.x * U)) {
+    float gi[U], mo[U], vo[U], po[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned int e = e0 + u * blockDim.x;
+      if (e < n) {
+        gi[u] = g[base + e];
+        mo[u] = m[base + e];
+        vo[u] = v[base + e];
+        po[u] = p[base + e];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned int e = e0 + u * blockDim.x;
+      if (e >= n) break;
+      // one rounding order, whatever the compiler contracts
+      const float mi = __fmaf_rn(1.f - b1, gi[u], __fmul_rn(b1, mo[u]));
+      const float vi = __fmaf_rn(__fmul_rn(1.f - b2, gi[u]), gi[u], __fmul_rn(b2, vo[u]));
+      m[base + e] = mi;
+      v[base + e] = vi;
+      const float pi = po[u] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+      p[base + e] = pi;
+      if (e < nw) {
+        const unsigned int o = e / nin;
+        L.Wb[l][(size_t)o * L.ld[l] + (e - o * nin)] = __float2bfloat16_rn(pi);
+      }
+    }
   }
 }
 
@@ -233,27 +288,17 @@ __global__ void inv_sd_kernel(const float *__restrict__ sd, int n, float *__rest
   if (j < n) isd[j] = sd[j] > 1e-12f ? 1.f / sd[j] : 0.f;
 }
 
-// C_l = exp(out sd + mu + (x_amp - mu_amp))
-__global__ void exp_kernel(const float *__restrict__ out, size_t B, int n, const float *__restrict__ mu,
-                           const float *__restrict__ sd, const float *__restrict__ X, int n_in, int amp,
-                           const float *__restrict__ mu_x, double *__restrict__ C) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < B * n; i += (size_t)gridDim.x * blockDim.x) {
-    const int j = (int)(i % n);
-    C[i] = exp((double)out[i] * (double)(sd[j] > 0.f ? sd[j] : 1.f) + (double)mu[j] +
-               amp_shift(X, n_in, amp, mu_x, i / n));
-  }
-}
-
 __global__ void cell_kernel(const float *__restrict__ X, int B, int n_in, const int *__restrict__ dims,
                             const float *__restrict__ mids, int nd, const unsigned char *__restrict__ trusted,
-                            int *__restrict__ cell, int *__restrict__ fallback) {
+                            int *__restrict__ fallback, int *__restrict__ fallback_host) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   int c = 0;
   for (int d = 0; d < nd; ++d)
     if (X[(size_t)b * n_in + dims[d]] > mids[d]) c |= 1 << d;
-  if (cell) cell[b] = c;
-  if (fallback) fallback[b] = trusted ? (trusted[c] ? 0 : 1) : 1;
+  const int f = trusted ? (trusted[c] ? 0 : 1) : 1;
+  fallback[b] = f;
+  fallback_host[b] = f;
 }
 
 // per-sample max |C_emu / C_ref - 1|
@@ -330,59 +375,170 @@ __global__ void __launch_bounds__(256) synth_kernel(const float *__restrict__ X,
 
 // ---------------------------------------------------------------- GEMM launcher
 
-template <int EPI>
-int gemm(const GemmArgs &a, cudaStream_t st, int nz = 1) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
-    if (e != cudaSuccess) return cuda_fail(e, "emu: gemm smem attribute");
-    attr = true;
-  }
-  dim3 grid((a.M + 127) / 128, (a.N + 127) / 128, nz);
-  gemm_kernel<EPI><<<grid, 128, kGemmSmem, st>>>(a);
-  return ck(cudaGetLastError(), "emu: gemm launch");
+// Launch of a kernel of the chain behind the one before it (see pdl_wait).
+template <typename... P, typename... A>
+cudaError_t chain_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
-View rowmajor(const float *p, int R, int K, long long ld, const int *rows = nullptr) {
-  return View{p, ld, 1, rows, R, K};
+template <int EPI, bool AMN, bool BMN, int NP, int ST>
+int gemm_st(const GemmArgs<NP> &a, int tiles, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(gemm_kernel<EPI, AMN, BMN, NP, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       gemm_smem(ST));
+  if (e != cudaSuccess) return cuda_fail(e, "emu: gemm smem attribute");
+  return ck(chain_launch(gemm_kernel<EPI, AMN, BMN, NP, ST>, dim3(tiles), dim3(kGemmThreads), gemm_smem(ST), st, a),
+            "emu: gemm launch");
 }
 
-int forward_pass(gcamb_emu *e, const float *X, const int *idx, int B, cudaStream_t st) {
+// Six stages where every tile has an SM to itself, else three and two CTAs an
+// SM (see emu_gemm.cuh).
+template <int EPI, bool AMN, bool BMN, int NP>
+int gemm(const GemmArgs<NP> &a, int tiles, cudaStream_t st) {
+  return tiles <= 152 ? gemm_st<EPI, AMN, BMN, NP, 6>(a, tiles, st) : gemm_st<EPI, AMN, BMN, NP, 3>(a, tiles, st);
+}
+
+// Rows and tiles of a problem: C[M][N] over K.
+int set_prob(Prob &p, int M, int N, int K, int first_tile) {
+  p.M = M;
+  p.N = N;
+  p.K = K;
+  p.tiles_n = (N + 127) / 128;
+  p.tile_end = first_tile + (M + 127) / 128 * p.tiles_n;
+  return p.tile_end;
+}
+
+int pad8(int n) { return (n + 7) & ~7; }
+
+// Tensor map of a bf16 matrix [rows][cols] with padded rows of ld elements:
+// boxes of 64 columns by `box` rows, 128-byte swizzle, zero beyond its extents.
+int encode_bf16(CUtensorMap *tm, const __nv_bfloat16 *p, int rows, int cols, int ld, int box) {
+  auto fn = reinterpret_cast<CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                          const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
+                                          CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                                          CUtensorMapFloatOOBfill)>(tensor_map_encoder());
+  if (!fn) return fail(GCAMB_ECUDA, "emu: cuTensorMapEncodeTiled is not available from the driver");
+  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+  const cuuint32_t boxes[2] = {64, (cuuint32_t)box};
+  const cuuint32_t es[2] = {1, 1};
+  const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(p), dims, strides, boxes, es,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(GCAMB_ECUDA, "emu: tensor map rejected (" + std::to_string((int)r) + ")");
+  return GCAMB_OK;
+}
+
+// The handle's tensor maps for batch size B.  K-major operands are copied in
+// boxes of 128 rows x 64 k, MN-major ones in boxes of 64 k x 64 rows.
+int ensure_maps(gcamb_emu *e, int B) {
+  if (e->maps_B == B) return GCAMB_OK;
   const int L = e->depth + 1;
+  e->maps.resize(L);
+  e->maps_B = 0;
+  for (int l = 0; l < L; ++l) {
+    auto &m = e->maps[l];
+    const int nin = e->sizes[l], nout = e->sizes[l + 1];
+    int rc;
+    if ((rc = encode_bf16(&m.act_k, e->act[l], B, nin, pad8(nin), 128)) ||
+        (rc = encode_bf16(&m.act_mn, e->act[l], B, nin, pad8(nin), 64)) ||
+        (rc = encode_bf16(&m.d_k, e->dB[l], B, nout, pad8(nout), 128)) ||
+        (rc = encode_bf16(&m.d_mn, e->dB[l], B, nout, pad8(nout), 64)) ||
+        (rc = encode_bf16(&m.w_k, e->W[l], nout, nin, pad8(nin), 128)) ||
+        (rc = encode_bf16(&m.w_mn, e->W[l], nout, nin, pad8(nin), 64)))
+      return rc;
+  }
+  e->maps_B = B;
+  return GCAMB_OK;
+}
+
+// bf16 copies of all weights (after the parameters were written as a whole).
+int refresh_weights(gcamb_emu *e, cudaStream_t st) {
+  for (size_t l = 0; l + 1 < e->sizes.size(); ++l) {
+    const int nin = e->sizes[l], nout = e->sizes[l + 1];
+    weights_bf16_kernel<<<512, 256, 0, st>>>(e->theta + e->w_off[l], nout, nin, e->W[l], pad8(nin));
+  }
+  return ck(cudaGetLastError(), "emu: weight copies");
+}
+
+// Forward pass of B rows, the output as FP32 to out [B][n_out], as C_l to CD
+// [B][n_out], or (Y: training) as the loss gradient and its partial sums, with
+// the hidden pre-activations kept.
+int forward_pass(gcamb_emu *e, const float *X, const int *idx, int B, const float *Y, float *out, double *CD,
+                 cudaStream_t st) {
+  const int L = e->depth + 1;
+  if (int rc = ensure_maps(e, B)) return rc;
   {
     const int n = B * e->n_in;
-    standardize_kernel<<<(n + 255) / 256, 256, 0, st>>>(X, idx, B, e->n_in, e->mu_x, e->isd_x, e->xs, e->xsT);
+    standardize_kernel<<<(n + 255) / 256, 256, 0, st>>>(X, idx, B, e->n_in, e->mu_x, e->isd_x, e->act[0],
+                                                        pad8(e->n_in));
   }
-  const float *h = e->xs;
-  int hin = e->n_in;
   for (int l = 0; l < L; ++l) {
-    const int nout = e->sizes[l + 1];
-    GemmArgs a{};
-    a.A = rowmajor(h, B, hin, hin);
-    a.B = rowmajor(e->theta + e->w_off[l], nout, hin, hin);
-    a.M = B;
-    a.N = nout;
-    a.K = hin;
-    a.bias = e->theta + e->b_off[l];
+    const int nin = e->sizes[l], nout = e->sizes[l + 1];
+    GemmArgs<1> a{};
+    Prob &p = a.p[0];
+    p.ta = e->maps[l].act_k;
+    p.tb = e->maps[l].w_k;
+    const int tiles = set_prob(p, B, nout, nin, 0);
+    a.np = 1;
+    p.bias = e->theta + e->b_off[l];
     a.err = e->err;
     int rc;
     if (l < L - 1) {
-      a.C = e->Z[l];
-      a.ldc = nout;
-      a.H = e->H[l];
-      a.CT = e->HT[l];
-      a.ldct = B;
-      rc = gemm<kBiasGelu>(a, st);
-      h = e->H[l];
+      p.C = Y ? e->Z[l] : nullptr;
+      p.ldc = pad8(nout);
+      p.Cb = e->act[l + 1];
+      p.ldb = pad8(nout);
+      rc = gemm<kGelu, false, false, 1>(a, tiles, st);
+    } else if (CD) {
+      a.ex = ExpArgs{CD, e->mu_y, e->sd_y, X, e->mu_x, e->n_in, amp_col(e), e->exp_tab};
+      rc = gemm<kExp, false, false, 1>(a, tiles, st);
+    } else if (Y) {
+      p.C = e->dF[l];
+      p.ldc = p.ldb = pad8(nout);
+      p.Cb = e->dB[l];
+      a.ls = LossArgs{Y, idx, 2.f / (float)((size_t)B * nout), e->loss_part};
+      rc = gemm<kLoss, false, false, 1>(a, tiles, st);
     } else {
-      a.C = e->out;
-      a.ldc = nout;
-      rc = gemm<kBias>(a, st);
+      p.C = out;
+      p.ldc = nout;
+      rc = gemm<kBias, false, false, 1>(a, tiles, st);
     }
     if (rc) return rc;
-    hin = nout;
   }
   return GCAMB_OK;
+}
+
+// 2^(i/64), i < 64, then 2^(j/8192), j < 128, as Q1.63, from the series of
+// exp(x ln 2) in double-double arithmetic (products by fused multiply-add).
+void exp2_tables(unsigned long long *tab) {
+  const double ln2h = 0x1.62e42fefa39efp-1, ln2l = 0x1.abc9e3b39803fp-56;
+  for (int i = 0; i < 192; ++i) {
+    const double f = i < 64 ? i / 64.0 : (i - 64) / 8192.0;  // exact
+    const double xh = f * ln2h, xl = std::fma(f, ln2h, -xh) + f * ln2l;
+    double sh = 1.0, sl = 0.0;  // Horner: s = 1 + x/n s
+    for (int n = 26; n >= 1; --n) {
+      // t = x s
+      const double th = xh * sh, tl = std::fma(xh, sh, -th) + (xh * sl + xl * sh);
+      // t / n
+      const double qh = th / n, ql = (std::fma(-qh, (double)n, th) + tl) / n;
+      // 1 + q
+      const double uh = 1.0 + qh, ul = (1.0 - uh) + qh + ql;
+      sh = uh + ul;
+      sl = ul - (sh - uh);
+    }
+    const double scale = 9223372036854775808.0;  // 2^63: sh in [1, 2) is an integer of at most 2^64 there
+    tab[i] = (unsigned long long)(sh * scale) + (unsigned long long)(long long)std::nearbyint(sl * scale);
+  }
 }
 
 int check_emu(const gcamb_emu *e, int B) {
@@ -394,28 +550,6 @@ int check_emu(const gcamb_emu *e, int B) {
 }  // namespace
 
 extern "C" {
-
-// One 128 x 128 tile C = A B^T over K through the library's tcgen05 GEMM
-// (operands rounded to bf16 by its loaders, FP32 accumulation in TMEM): the
-// self-test of the tensor cores' accumulation.
-int gcamb_probe_mma(const float *A, const float *B, int K, float *C, void *stream) {
-  if (!A || !B || !C) return fail(GCAMB_EINVAL, "probe_mma: NULL pointer");
-  if (K < 1 || K > (1 << 20)) return fail(GCAMB_EINVAL, "probe_mma: K must be in [1, 2^20]");
-  int *err = device_error_flag();
-  if (!err) return fail(GCAMB_ECUDA, "probe_mma: error flag allocation");
-  GemmArgs a{};
-  a.A = rowmajor(A, 128, K, K);
-  a.B = rowmajor(B, 128, K, K);
-  a.M = 128;
-  a.N = 128;
-  a.K = K;
-  a.C = C;
-  a.ldc = 128;
-  a.CT = nullptr;
-  a.kchunks = 0;
-  a.err = err;
-  return gemm<kStore>(a, (cudaStream_t)stream);
-}
 
 int gcamb_emu_create(gcamb_grid *g, int n_in, int width, int depth, int max_batch, uint64_t seed, gcamb_emu **out) {
   if (!out) return fail(GCAMB_EINVAL, "emu_create: out is NULL");
@@ -445,37 +579,44 @@ int gcamb_emu_create(gcamb_grid *g, int n_in, int width, int depth, int max_batc
     o += e->sizes[l + 1];
   }
   e->n_params = o;
-  const size_t mx = std::max(width, e->n_out);
-  if ((rc = dalloc(&e->theta, o)) || (rc = dalloc(&e->grad, o)) || (rc = dalloc(&e->m, o)) || (rc = dalloc(&e->v, o)) ||
-      (rc = dalloc(&e->mu_x, n_in)) || (rc = dalloc(&e->isd_x, n_in)) || (rc = dalloc(&e->mu_y, e->n_out)) ||
-      (rc = dalloc(&e->sd_y, e->n_out)) || (rc = dalloc(&e->xs, (size_t)max_batch * n_in)) ||
-      (rc = dalloc(&e->out, (size_t)max_batch * e->n_out)) || (rc = dalloc(&e->d0, (size_t)max_batch * mx)) ||
-      (rc = dalloc(&e->d1, (size_t)max_batch * mx)) || (rc = dalloc(&e->loss_part, kLossBlocks)) ||
-      (rc = dalloc(&e->loss, 1)) || (rc = dalloc(&e->err, 1)) || (rc = dalloc(&e->xsT, (size_t)max_batch * n_in)) ||
-      (rc = dalloc(&e->dT0, (size_t)max_batch * mx)) || (rc = dalloc(&e->dT1, (size_t)max_batch * mx)) ||
-      (rc = dalloc(&e->WT, o))) {
+  const size_t mb = (size_t)max_batch;
+  rc = GCAMB_OK;
+  auto bf16_buf = [&](std::vector<__nv_bfloat16 *> &v, size_t n) {
+    __nv_bfloat16 *q = nullptr;
+    if (!rc) rc = dalloc(&q, n);
+    v.push_back(q);
+  };
+  auto f32_buf = [&](std::vector<float *> &v, size_t n) {
+    float *q = nullptr;
+    if (!rc) rc = dalloc(&q, n);
+    v.push_back(q);
+  };
+  for (int l = 0; l <= depth; ++l) {
+    const int nin = e->sizes[l], nout = e->sizes[l + 1];
+    bf16_buf(e->W, (size_t)nout * pad8(nin));
+    bf16_buf(e->act, mb * pad8(nin));
+    bf16_buf(e->dB, mb * pad8(nout));
+    f32_buf(e->dF, mb * pad8(nout));
+    if (l < depth) f32_buf(e->Z, mb * pad8(nout));
+  }
+  if (rc || (rc = dalloc(&e->theta, o)) || (rc = dalloc(&e->grad, o)) || (rc = dalloc(&e->m, o)) ||
+      (rc = dalloc(&e->v, o)) || (rc = dalloc(&e->mu_x, n_in)) || (rc = dalloc(&e->isd_x, n_in)) ||
+      (rc = dalloc(&e->mu_y, e->n_out)) || (rc = dalloc(&e->sd_y, e->n_out)) ||
+      (rc = dalloc(&e->loss_part, ((mb + 127) / 128) * ((e->n_out + 127) / 128) * 8)) ||
+      (rc = dalloc(&e->err, 1)) || (rc = dalloc(&e->exp_tab, 192))) {
     gcamb_emu_destroy(e);
     return rc;
   }
-  for (int d = 0; d < depth; ++d) {
-    float *z = nullptr, *h = nullptr, *ht = nullptr;
-    if ((rc = dalloc(&z, (size_t)max_batch * width)) || (rc = dalloc(&h, (size_t)max_batch * width)) ||
-        (rc = dalloc(&ht, (size_t)max_batch * width))) {
-      cudaFree(z);
-      cudaFree(h);
-      gcamb_emu_destroy(e);
-      return rc;
-    }
-    e->Z.push_back(z);
-    e->H.push_back(h);
-    e->HT.push_back(ht);
+  if (cudaHostAlloc(reinterpret_cast<void **>(&e->flags_host), mb * sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer(reinterpret_cast<void **>(&e->flags_dev), e->flags_host, 0) != cudaSuccess) {
+    cudaGetLastError();
+    gcamb_emu_destroy(e);
+    return fail(GCAMB_ENOMEM, "emu_create: mapped flags");
   }
   {
-    // split-K partials of the weight gradients: (ceil(max_batch / 256)) slices of the largest W
-    size_t wmax = 0;
-    for (size_t l = 0; l + 1 < e->sizes.size(); ++l) wmax = std::max(wmax, (size_t)e->sizes[l + 1] * e->sizes[l]);
-    const size_t nzmax = ((size_t)max_batch + 255) / 256;
-    if ((rc = dalloc(&e->splitk, nzmax * wmax))) {
+    unsigned long long tab[192];
+    exp2_tables(tab);
+    if ((rc = ck(cudaMemcpy(e->exp_tab, tab, sizeof tab, cudaMemcpyHostToDevice), "emu_create: tables"))) {
       gcamb_emu_destroy(e);
       return rc;
     }
@@ -486,6 +627,10 @@ int gcamb_emu_create(gcamb_grid *g, int n_in, int width, int depth, int max_batc
     const size_t nw = (size_t)e->sizes[l + 1] * e->sizes[l];
     init_uniform_kernel<<<256, 256>>>(e->theta + e->w_off[l], nw, bound, seed, e->w_off[l]);
     init_uniform_kernel<<<64, 256>>>(e->theta + e->b_off[l], e->sizes[l + 1], bound, seed, e->b_off[l]);
+  }
+  if ((rc = refresh_weights(e, nullptr))) {
+    gcamb_emu_destroy(e);
+    return rc;
   }
   cudaMemset(e->m, 0, o * sizeof(float));
   cudaMemset(e->v, 0, o * sizeof(float));
@@ -506,15 +651,16 @@ int gcamb_emu_create(gcamb_grid *g, int n_in, int width, int depth, int max_batc
 int gcamb_emu_destroy(gcamb_emu *e) {
   if (!e) return GCAMB_OK;
   for (void *p : {(void *)e->theta, (void *)e->grad, (void *)e->m, (void *)e->v, (void *)e->mu_x, (void *)e->isd_x,
-                  (void *)e->mu_y, (void *)e->sd_y, (void *)e->xs, (void *)e->out, (void *)e->d0, (void *)e->d1,
-                  (void *)e->loss_part, (void *)e->loss, (void *)e->err, (void *)e->d_cell_dim,
-                  (void *)e->d_cell_mid, (void *)e->d_trusted, (void *)e->fb_x, (void *)e->fb_S, (void *)e->fb_P,
-                  (void *)e->fb_C, (void *)e->fb_idx, e->fb_ws, (void *)e->xsT, (void *)e->dT0, (void *)e->dT1,
-                  (void *)e->WT, (void *)e->splitk})
+                  (void *)e->mu_y, (void *)e->sd_y, (void *)e->loss_part,
+                  (void *)e->err, (void *)e->exp_tab, (void *)e->d_cell_dim, (void *)e->d_cell_mid,
+                  (void *)e->d_trusted, (void *)e->fb_x, (void *)e->fb_S, (void *)e->fb_P, (void *)e->fb_C,
+                  (void *)e->fb_idx, e->fb_ws})
     cudaFree(p);
-  for (float *p : e->Z) cudaFree(p);
-  for (float *p : e->H) cudaFree(p);
-  for (float *p : e->HT) cudaFree(p);
+  for (auto *v : {&e->W, &e->act, &e->dB})
+    for (__nv_bfloat16 *p : *v) cudaFree(p);
+  for (auto *v : {&e->Z, &e->dF})
+    for (float *p : *v) cudaFree(p);
+  if (e->flags_host) cudaFreeHost(e->flags_host);
   delete e;
   return GCAMB_OK;
 }
@@ -530,6 +676,8 @@ int gcamb_emu_params(gcamb_emu *e, float *host_out, const float *host_in) {
   const size_t bytes = e->n_params * sizeof(float);
   if (host_in) {
     int rc = ck(cudaMemcpy(e->theta, host_in, bytes, cudaMemcpyHostToDevice), "emu_params: upload");
+    if (!rc) rc = refresh_weights(e, nullptr);
+    if (!rc) rc = ck(cudaStreamSynchronize(nullptr), "emu_params: weight copies");
     if (rc) return rc;
   }
   if (host_out) return ck(cudaMemcpy(host_out, e->theta, bytes, cudaMemcpyDeviceToHost), "emu_params: download");
@@ -583,7 +731,6 @@ int gcamb_emu_fit_norm(gcamb_emu *e, const float *X, const double *Cl, int N, in
   if (rc) return rc;
   colstats_kernel<<<1, 32, 0, st>>>(X, N, e->n_in, e->mu_x, sdx);
   inv_sd_kernel<<<1, 32, 0, st>>>(sdx, e->n_in, e->isd_x);
-  const size_t n = (size_t)N * e->n_out;
   log_kernel<<<1024, 256, 0, st>>>(Cl, (size_t)N, e->n_out, X, e->n_in, amp_col(e), e->mu_x, Y);
   colstats_kernel<<<(e->n_out + 127) / 128, 128, 0, st>>>(Y, N, e->n_out, e->mu_y, e->sd_y);
   if (!per_l) global_scale_kernel<<<1, 32, 0, st>>>(e->sd_y, e->n_out);
@@ -599,9 +746,7 @@ int gcamb_emu_forward(gcamb_emu *e, const float *X, int B, float *Y, void *strea
   if (rc) return rc;
   if (!X || !Y) return fail(GCAMB_EINVAL, "emu_forward: NULL pointer");
   cudaStream_t st = (cudaStream_t)stream;
-  if ((rc = forward_pass(e, X, nullptr, B, st))) return rc;
-  return ck(cudaMemcpyAsync(Y, e->out, (size_t)B * e->n_out * sizeof(float), cudaMemcpyDeviceToDevice, st),
-            "emu_forward: copy");
+  return forward_pass(e, X, nullptr, B, nullptr, Y, nullptr, st);
 }
 
 int gcamb_emu_train_step(gcamb_emu *e, const float *X, const float *Y, const int *idx, int B, float lr, float *loss,
@@ -611,64 +756,77 @@ int gcamb_emu_train_step(gcamb_emu *e, const float *X, const float *Y, const int
   if (!X || !Y) return fail(GCAMB_EINVAL, "emu_train_step: NULL pointer");
   cudaStream_t st = (cudaStream_t)stream;
   const int L = e->depth + 1;
-  if ((rc = forward_pass(e, X, idx, B, st))) return rc;
-  loss_kernel<<<kLossBlocks, 256, 0, st>>>(e->out, Y, idx, B, e->n_out, e->d0, e->dT0, e->loss_part);
-  loss_final_kernel<<<1, 32, 0, st>>>(e->loss_part, kLossBlocks, 1.f / ((float)B * e->n_out), e->loss);
-  // W^T of every layer (the input-gradient GEMMs read it along the output index)
-  for (int l = 1; l < L; ++l) {
+  if ((rc = forward_pass(e, X, idx, B, Y, nullptr, nullptr, st))) return rc;
+  // d of layer l-1 [b][i] = (sum_o d_l[b][o] W_l[o][i]) GELU'(Z_{l-1}[b][i])
+  for (int l = L - 1; l >= 1; --l) {
     const int nin = e->sizes[l], nout = e->sizes[l + 1];
-    dim3 tg((nin + 31) / 32, (nout + 31) / 32);
-    transpose_kernel<<<tg, dim3(32, 8), 0, st>>>(e->theta + e->w_off[l], nout, nin, e->WT + e->w_off[l]);
+    GemmArgs<1> a{};
+    Prob &p = a.p[0];
+    p.ta = e->maps[l].d_k;
+    p.tb = e->maps[l].w_mn;
+    const int tiles = set_prob(p, B, nin, nout, 0);
+    a.np = 1;
+    p.C = e->dF[l - 1];
+    p.ldc = pad8(nin);
+    p.Cb = e->dB[l - 1];
+    p.ldb = pad8(nin);
+    p.Z = e->Z[l - 1];
+    a.err = e->err;
+    if ((rc = gemm<kDGelu, false, true, 1>(a, tiles, st))) return rc;
   }
-  // d / dT: gradient wrt the current layer's pre-activation, [B][out] and [out][B]
-  float *d = e->d0, *dn = e->d1, *dT = e->dT0, *dnT = e->dT1;
-  const int nkc = (B + 63) / 64;
-  const int kpc = 4;                       // K-chunks per CTA of the weight-gradient GEMMs
-  const int nz = (nkc + kpc - 1) / kpc;
-  for (int l = L - 1; l >= 0; --l) {
-    const int nin = e->sizes[l], nout = e->sizes[l + 1];
-    const float *hT = l == 0 ? e->xsT : e->HT[l - 1];
-    // dW_l[o][i] = sum_b dT[o][b] hT[i][b], split over b, summed in a fixed order
-    GemmArgs w{};
-    w.A = rowmajor(dT, nout, B, B);
-    w.B = rowmajor(hT, nin, B, B);
-    w.M = nout;
-    w.N = nin;
-    w.K = B;
-    w.C = e->splitk;
-    w.ldc = nin;
-    w.kchunks = kpc;
-    w.err = e->err;
-    if ((rc = gemm<kStore>(w, st, nz))) return rc;
-    const size_t nw = (size_t)nout * nin;
-    splitk_reduce_kernel<<<(unsigned)std::min<size_t>(4096, (nw + 255) / 256), 256, 0, st>>>(
-        e->splitk, nz, nw, e->grad + e->w_off[l]);
-    rowsum_kernel<<<(nout + 7) / 8, 256, 0, st>>>(dT, B, nout, e->grad + e->b_off[l]);
-    if (l > 0) {
-      // dn[b][i] = (sum_o d[b][o] W_l[o][i]) GELU'(Z_{l-1}[b][i]), and its transpose
-      GemmArgs x{};
-      x.A = rowmajor(d, B, nout, nout);
-      x.B = rowmajor(e->WT + e->w_off[l], nin, nout, nout);
-      x.M = B;
-      x.N = nin;
-      x.K = nout;
-      x.C = dn;
-      x.ldc = nin;
-      x.CT = dnT;
-      x.ldct = B;
-      x.Zprev = e->Z[l - 1];
-      x.err = e->err;
-      if ((rc = gemm<kDGelu>(x, st))) return rc;
-      std::swap(d, dn);
-      std::swap(dT, dnT);
+  // dW_l[o][i] = sum_b d_l[b][o] h_l[b][i], every layer in one launch
+  {
+    GemmArgs<kMaxLayers> a{};
+    int tiles = 0;
+    for (int l = L - 1; l >= 0; --l) {
+      const int nin = e->sizes[l], nout = e->sizes[l + 1];
+      Prob &p = a.p[a.np++];
+      p.ta = e->maps[l].d_mn;
+      p.tb = e->maps[l].act_mn;
+      tiles = set_prob(p, nout, nin, B, tiles);
+      p.C = e->grad + e->w_off[l];
+      p.ldc = nin;
     }
+    a.err = e->err;
+    if ((rc = gemm<kSliced, true, true, kMaxLayers>(a, tiles, st))) return rc;
+  }
+  {
+    BiasSums bs{};
+    int nmax = 0;
+    for (int l = 0; l < L; ++l) {
+      bs.d[l] = e->dF[l];
+      bs.db[l] = e->grad + e->b_off[l];
+      bs.N[l] = e->sizes[l + 1];
+      bs.ld[l] = pad8(e->sizes[l + 1]);
+      nmax = std::max(nmax, bs.N[l]);
+    }
+    bs.part = e->loss_part;
+    bs.nparts = ((B + 127) / 128) * ((e->n_out + 127) / 128) * 8;
+    bs.inv_total = 1.f / ((float)B * e->n_out);
+    bs.loss = loss;
+    if ((rc = ck(chain_launch(bias_kernel, dim3((nmax + kSumCols - 1) / kSumCols, L + 1), dim3(kSumCols * kSumClasses),
+                              0, st, bs, B, L),
+                 "emu_train_step: bias gradients")))
+      return rc;
   }
   ++e->step;
   const float b1 = 0.9f, b2 = 0.999f;
   const float bc1 = 1.f - powf(b1, (float)e->step), bc2 = 1.f - powf(b2, (float)e->step);
-  adam_kernel<<<1024, 256, 0, st>>>(e->theta, e->grad, e->m, e->v, e->n_params, lr, b1, b2, 1e-8f, bc1, bc2);
-  if (loss) cudaMemcpyAsync(loss, e->loss, sizeof(float), cudaMemcpyDeviceToDevice, st);
-  return ck(cudaGetLastError(), "emu_train_step: launch");
+  AdamLayers al{};
+  for (int l = 0; l < L; ++l) {
+    al.w_off[l] = e->w_off[l];
+    al.end[l] = e->b_off[l] + e->sizes[l + 1];
+    al.nw[l] = (unsigned)((size_t)e->sizes[l + 1] * e->sizes[l]);
+    al.nin[l] = e->sizes[l];
+    al.ld[l] = pad8(e->sizes[l]);
+    al.Wb[l] = e->W[l];
+  }
+  size_t most = 0;
+  for (int l = 0; l < L; ++l) most = std::max(most, al.end[l] - al.w_off[l]);
+  const unsigned blocks = (unsigned)std::min<size_t>(4096, (most + 1023) / 1024);
+  return ck(chain_launch(adam_kernel, dim3(blocks, L), dim3(256), 0, st, e->theta, e->grad, e->m, e->v, al, lr, b1, b2,
+                         1e-8f, bc1, bc2),
+            "emu_train_step: Adam");
 }
 
 int gcamb_synth_sources(const gcamb_grid *g, const float *X, int M, float *S, double *Pk, void *stream) {
@@ -702,9 +860,7 @@ int gcamb_emu_check(gcamb_emu *e, const float *X, const double *Cl_ref, int N, d
       cudaFree(d_err);
       return rc;
     }
-    if (!(rc = forward_pass(e, X, nullptr, N, st))) {
-      exp_kernel<<<1024, 256, 0, st>>>(e->out, N, e->n_out, e->mu_y, e->sd_y, X, e->n_in, amp_col(e), e->mu_x,
-                                       d_ce);
+    if (!(rc = forward_pass(e, X, nullptr, N, nullptr, nullptr, d_ce, st))) {
       maxrel_kernel<<<N, 256, 0, st>>>(d_ce, Cl_ref, e->n_out, d_err);
       rc = ck(cudaStreamSynchronize(st), "emu_check: kernels");
       if (!rc) rc = ck(cudaMemcpy(he.data(), d_err, N * sizeof(double), cudaMemcpyDeviceToHost), "emu_check: errors");
@@ -800,17 +956,14 @@ int gcamb_emulate(gcamb_emu *e, const float *X, int B, double *Cl, int *used_fal
   if (rc) return rc;
   if (!X || !Cl || !used_fallback) return fail(GCAMB_EINVAL, "emulate: NULL pointer");
   cudaStream_t st = (cudaStream_t)stream;
-  if ((rc = forward_pass(e, X, nullptr, B, st))) return rc;
-  exp_kernel<<<1024, 256, 0, st>>>(e->out, B, e->n_out, e->mu_y, e->sd_y, X, e->n_in, amp_col(e), e->mu_x, Cl);
+  // the cell of every request first: its flags land in mapped host memory while the network runs
   const int nd = (int)e->cell_dim.size();
-  cell_kernel<<<(B + 255) / 256, 256, 0, st>>>(X, B, e->n_in, e->d_cell_dim, e->d_cell_mid, nd, e->d_trusted, nullptr,
-                                               used_fallback);
-  if ((rc = ck(cudaGetLastError(), "emulate: launch"))) return rc;
-  // requests outside the trusted cells: the batched projection on regenerated sources
-  std::vector<int> hf(B);
-  if ((rc = ck(cudaMemcpyAsync(hf.data(), used_fallback, B * sizeof(int), cudaMemcpyDeviceToHost, st), "emulate")))
-    return rc;
+  cell_kernel<<<(B + 255) / 256, 256, 0, st>>>(X, B, e->n_in, e->d_cell_dim, e->d_cell_mid, nd, e->d_trusted,
+                                               used_fallback, e->flags_dev);
+  if ((rc = forward_pass(e, X, nullptr, B, nullptr, nullptr, Cl, st))) return rc;
   if ((rc = ck(cudaStreamSynchronize(st), "emulate: sync"))) return rc;
+  // requests outside the trusted cells: the batched projection on regenerated sources
+  const volatile int *hf = e->flags_host;
   std::vector<int> idx;
   for (int b = 0; b < B; ++b)
     if (hf[b]) idx.push_back(b);
@@ -954,6 +1107,7 @@ int gcamb_emu_load(gcamb_emu *e, const char *path) {
     if (!get(h.data(), h.size() * sizeof(float))) return fail(GCAMB_EINVAL, "emu_load: truncated");
     cudaMemcpy(dst, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice);
   }
+  if (int rc = refresh_weights(e, nullptr)) return rc;
   std::vector<float> nx(e->n_in), ny(e->n_out);
   for (float *dst : {e->mu_x, e->isd_x}) {
     if (!get(nx.data(), nx.size() * sizeof(float))) return fail(GCAMB_EINVAL, "emu_load: truncated");

@@ -156,6 +156,10 @@ int launch_los_cl_fixed(const gcamb_grid *g, const float *S, const double *Pk, i
 // Probes (probe.cu).
 int run_probe_flops(int what, double *flops);
 int run_wait_selftest(int *status, cudaStream_t st);
+int run_probe_mma(const float *A, const float *B, int K, float *C, cudaStream_t st);
+
+// The driver's cuTensorMapEncodeTiled (tc.cu), or null.
+void *tensor_map_encoder();
 
 // Event tracer: brackets one kernel launch when profiling is on.
 struct ProfScope {

@@ -2211,6 +2211,8 @@ int launch_tc_pair(const gcamb_grid *gx, const gcamb_grid *gy, const TcPlan &pl,
 
 }  // namespace
 
+void *tensor_map_encoder() { return reinterpret_cast<void *>(encode_tiled()); }
+
 int launch_los_cl_pair(const gcamb_grid *gx, const gcamb_grid *gy, const float *SX, const float *SY,
                        const double *Pk, int M, double *ClXX, double *ClYY, double *ClXY, void *ws, size_t ws_bytes,
                        cudaStream_t st) {
