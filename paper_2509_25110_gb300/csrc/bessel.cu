@@ -1,5 +1,5 @@
 // Spherical Bessel tables: w_i j_l(k (tau0 - tau_i)) over the active extents,
-// generated in FP64 per (k, tau) node by three-term recurrences in l.
+// generated per (k, tau) node by three-term recurrences in l.
 //
 // For x = k (tau0 - tau) the orders split at ls = min(floor(x), l_top):
 //   l <= ls  (x >= 1): forward recurrence from j_0 = sin x / x and
@@ -11,6 +11,28 @@
 //            j_0 for x < 1.  A first backward pass finds the scale, a second
 //            writes the scaled values, so no per-thread order buffer is kept.
 // Recurrence: j_{l-1} + j_{l+1} = (2l+1)/x j_l (both directions).
+//
+// Arithmetic (x >= 1): 64-bit integers.  GB300's FP64 pipe runs at 1/64 of
+// the FP32 rate (two lanes a clock and SM), so a recurrence step of a product,
+// a fused multiply-add and an addition in FP64 takes about ten times as long
+// as the same step in integers:
+//   forward   x j_l + 8 as an unsigned fixed-point number of 60 fraction bits
+//             (|x j_l| < 4 for every l <= x, l <= 20000), (2l+1)/x < 2 as one of 63
+//             with 32 further bits carried along, the upper half of their
+//             product: an error below 2^-60 a step, where an FP64 step of
+//             values near 1 makes 2^-54;
+//   backward  f_l and f_(l+1) as 64-bit mantissas with a common exponent.
+//             While (2l+1)/x >= 4 (x of a few units) they are renormalised
+//             every step; below, f grows by less than four a step and both
+//             are shifted by two bits where f passes 2^62: an error below
+//             2^-58 a step, and about 20 x^(1/3) steps.
+// Orders are converted to FP64 (and the row's weight applied) where they are
+// table rows, so a grid of sampled multipoles converts only those.
+// Measured: PLAIN64 table of 130 sampled multipoles to 2500, 2000 k x 1000
+// tau 6667 -> 1328 us; every multipole 7759 -> 3360 (PLAIN64),
+// 9209 -> 3854 (PLAIN32), 13660 -> 8216 (F16X3); l_max 5000, 3000 k x 2000 tau, PLAIN64
+// 41.5 -> 21.8 ms.  What is left is the integer pipes (59% of issue slots) and, for
+// every multipole, the stores.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -25,85 +47,263 @@
 namespace gcamb {
 
 // First order l >= lfrom whose start threshold exceeds x (|j_l(x)| < delta);
-// xs is increasing for l >= 1.
+// xs is increasing for l >= 1.  Nonnegative doubles compare as their bits.
 __device__ __forceinline__ int miller_start(const double *__restrict__ xs, int nxs, int lfrom, double x) {
+  const long long *xb = reinterpret_cast<const long long *>(xs);
+  const long long xi = __double_as_longlong(x);
   int lo = lfrom < 1 ? 1 : lfrom, hi = nxs - 1;
   if (lo >= hi) return hi > lo ? hi : lo;
-  if (xs[hi] <= x) return hi;
+  if (__ldg(xb + hi) <= xi) return hi;
   while (lo < hi) {
     int mid = (lo + hi) >> 1;
-    if (xs[mid] > x) hi = mid;
+    if (__ldg(xb + mid) > xi) hi = mid;
     else lo = mid + 1;
   }
   return lo;
 }
 
-// Calls put(l, j_l(x)) for the orders l in [lmin, ltop] that are not below
-// the Miller start; orders not passed to put are zero to within delta.
+// 96-bit unsigned fixed-point number (low word first).
+struct U96 {
+  unsigned int w0, w1, w2;
+  __device__ __forceinline__ explicit U96(unsigned __int128 v)
+      : w0((unsigned int)v), w1((unsigned int)(v >> 32)), w2((unsigned int)(v >> 64)) {}
+  __device__ __forceinline__ unsigned long long hi() const { return ((unsigned long long)w2 << 32) | w1; }
+  // (carried along: (2l+1) N by three products a step measured 23% slower)
+  __device__ __forceinline__ void add(const U96 &b) {
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(w0), "+r"(w1), "+r"(w2)
+        : "r"(b.w0), "r"(b.w1), "r"(b.w2));
+  }
+  __device__ __forceinline__ void sub(const U96 &b) {
+    asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %4;\n\tsubc.u32 %2, %2, %5;"
+        : "+r"(w0), "+r"(w1), "+r"(w2)
+        : "r"(b.w0), "r"(b.w1), "r"(b.w2));
+  }
+  __device__ __forceinline__ void shl1() {
+    w2 = (w2 << 1) | (w1 >> 31);
+    w1 = (w1 << 1) | (w0 >> 31);
+    w0 <<= 1;
+  }
+};
+
+// 1/x, x >= 1, as N 2^-95 (N < 2^96), from the FP64 quotient and its exact
+// remainder (about 2^-105 relative, or the 95 bits).
+__device__ __forceinline__ unsigned __int128 inv_fixed(double x) {
+  const double d = 1.0 / x;
+  const double r = fma(-x, d, 1.0) * d;  // 1/x - d
+  const long long b = __double_as_longlong(d);
+  const unsigned __int128 m = (unsigned long long)((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll);
+  const int sh = (int)(b >> 52) - 1075 + 95;
+  unsigned __int128 n = sh >= 0 ? m << sh : (sh > -53 ? m >> -sh : 0);
+  // r 2^95, |r| <= 2^-54: below 2^42
+  n += (unsigned __int128)(__int128)__double2ll_rn(r * 39614081257132168796771975168.0);
+  return n;
+}
+
+// A nonnegative double as g 2^e with the leading bit of g set (0: g = 0).
+__device__ __forceinline__ unsigned long long mantissa(double v, int *e) {
+  const long long b = __double_as_longlong(v);
+  *e = (int)(b >> 52) - 1086;
+  return b == 0 ? 0 : (unsigned long long)((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << 11;
+}
+
+// a g 2^e, leading bits of a and g set (or 0), rounded to FP64 (0 below its
+// normal range), in integers.
+__device__ __forceinline__ double mul_mantissas(unsigned long long a, unsigned long long g, int e) {
+  unsigned long long p = __umul64hi(a, g);
+  const int t = (long long)p < 0 ? 0 : 1;
+  p <<= t;
+  const unsigned long long m = (p >> 11) + ((p >> 10) & 1);  // up to 2^53: carries into the exponent
+  const int field = e - t + (75 + 52 + 1022);
+  return p == 0 || field < 0 ? 0.0 : __longlong_as_double((long long)(((unsigned long long)field << 52) + m));
+}
+
+// Calls put.store(r, w j_l(x)), w = put.weight() >= 0, for the rows r whose
+// order l = put.order(r) is in [lmin, ltop] and not below the Miller start;
+// rows not stored are zero to within delta.  put.order rises with r from
+// put.order(0) = lmin (a huge order past the last row); put.last(l) is the last
+// row of order <= l.  A sink that can hold FP64 numbers (kRaw) takes the
+// backward orders unscaled, put.raw(r, v), from one pass, and then
+// put.rescale(r, s) for each of them; the others get a second pass.
 template <class Sink>
 __device__ __forceinline__ void bessel_orders(double x, int lmin, int ltop, const double *__restrict__ xs, int nxs,
                                               Sink &put) {
   if (ltop < lmin) return;
-  if (x == 0.0) {
-    if (lmin == 0) put(0, 1.0);
-    return;
-  }
+  const double w = put.weight();
   if (x < 1e-150) {  // j_1 = x/3, j_l < 1e-300 for l >= 2
-    if (lmin == 0) put(0, 1.0);
-    if (lmin <= 1 && ltop >= 1) put(1, x / 3.0);
+    const int r1 = lmin == 0 ? 1 : 0;
+    if (lmin == 0) put.store(0, w);
+    if (x > 0.0 && ltop >= 1 && put.order(r1) == 1) put.store(r1, w * (x / 3.0));
     return;
   }
+  if (x < 1.0) {  // few orders, and (2l+1)/x has no useful bound: FP64
+    const double inv = 1.0 / x, j0 = sin(x) / x;
+    if (lmin == 0) put.store(0, w * j0);
+    const int L = miller_start(xs, nxs, 1, x);
+    double fh = 0.0, f = 1.0, dl = 2.0 * L + 1.0;
+    for (int l = L; l > 0; --l) {
+      const double fm = fma(dl * inv, f, -fh);
+      fh = f;
+      f = fm;
+      dl -= 2.0;
+    }
+    const double scale = w * (j0 / f);
+    const int rend = lmin == 0 ? 1 : 0;
+    int row = put.last(L < ltop ? L : ltop);
+    int want = row >= rend ? put.order(row) : -1;
+    fh = 0.0;
+    f = 1.0;
+    dl = 2.0 * L + 1.0;
+    for (int l = L; row >= rend; --l) {
+      if (l == want) {
+        put.store(row, scale * f);
+        if (--row >= rend) want = put.order(row);
+      }
+      const double fm = fma(dl * inv, f, -fh);
+      fh = f;
+      f = fm;
+      dl -= 2.0;
+    }
+    return;
+  }
+  const int ls = x >= (double)ltop ? ltop : (int)floor(x);
+  const unsigned __int128 N = inv_fixed(x);  // 2^95 / x
   const double inv = 1.0 / x;
-  int ls = 0;
-  double fa = 0.0, fb = 0.0;  // forward j_{ls-1}, j_{ls}
-  double j0 = 0.0;
-  if (x >= 1.0) {
-    ls = x >= (double)ltop ? ltop : (int)floor(x);
-    double s, c;
-    sincos(x, &s, &c);
-    double jm = s / x;
-    double j = (jm - c) / x;
-    if (lmin == 0) put(0, jm);
-    if (ls >= 1 && lmin <= 1) put(1, j);
-    double dl = 3.0;  // 2l+1 at l = 1
+  int row = 0;     // next row
+  double fa, fb;   // x j_(ls-1), x j_ls, times 2^60
+  {
+    double sx, cx;
+    sincos(x, &sx, &cx);
+    const double q = 1152921504606846976.0;  // 2^60
+    const double j1 = fma(sx, inv, -cx);     // x j_1
+    int want = put.order(0);
+    if (want == 0) {
+      put.store(0, w * (sx * inv));
+      want = put.order(++row);
+    }
+    if (want == 1 && ls >= 1) {
+      put.store(row, w * (j1 * inv));
+      want = put.order(++row);
+    }
+    // A = a + 2^63, a = x j_l 2^60
+    constexpr unsigned long long kOff = 1ull << 63;
+    unsigned long long Am = (unsigned long long)__double2ll_rn(sx * q) + kOff;
+    unsigned long long A = (unsigned long long)__double2ll_rn(j1 * q) + kOff;
+    int ge;
+    const unsigned long long gm = mantissa(w * inv * (1.0 / q), &ge);
+    // c = (2l+1)/x, 63 + 32 fraction bits; below 2 for every l < ls (3/x of ls = 1 is not used)
+    U96 c(3 * N), st(2 * N);
+#pragma unroll 2
     for (int l = 1; l < ls; ++l) {
-      const double jn = fma(dl * inv, j, -jm);
-      jm = j;
-      j = jn;
-      dl += 2.0;
-      if (l + 1 >= lmin) put(l + 1, j);
+      // a_(l+1) = c a_l - a_(l-1), c a = c A - 2^63 c: the product's upper half
+      // has 59 fraction bits (the half unit dropped on average added back)
+      const unsigned long long ch = c.hi();
+      const unsigned long long An = 2 * __umul64hi(A, ch) + 1 - ch - Am;
+      Am = A;
+      A = An;
+      c.add(st);
+      if (l + 1 == want) {
+        const long long a = (long long)(A - kOff);
+        const unsigned long long ua = (unsigned long long)(a < 0 ? -a : a);
+        const int n = __clzll((long long)ua);
+        const double v = mul_mantissas(ua << (n & 63), gm, ge - n);
+        put.store(row, a < 0 ? -v : v);
+        want = put.order(++row);
+      }
     }
     if (ls >= ltop) return;
-    fa = jm;
-    fb = j;
+    fa = (double)(long long)(Am - kOff);
+    fb = (double)(long long)(A - kOff);
+  }
+  // ---- backward from L (here ltop > ls = floor(x) >= 1), to the rows from `row` on
+  int L = miller_start(xs, nxs, ls + 1, x);
+  const int top = put.last(L < ltop ? L : ltop);
+  if (top < row) return;
+  {
+    // Neighbouring nodes start at the highest of their orders (a higher start
+    // only lowers the truncation), so that the lanes of a warp come to a row's
+    // order together: one by one, the rows' stores cost more than the steps
+    // added.  Where the orders lie far apart, or the exponent of f (below 1000
+    // from the Miller start) could grow by more than 400, each keeps its own.
+    const int Lw = __reduce_max_sync(__activemask(), L);
+    if ((Lw - L) * (32 - __clz((2 * Lw + 1) / ls)) <= 400) L = Lw;
+  }
+  // c_L = (2L+1)/x = C 2^(K-64) with C's leading bit set, 32 further bits
+  const unsigned __int128 P = N * (unsigned)(2 * L + 1);                          // above 2^96: c_L > 2
+  const int sh = 64 - __clzll((long long)(unsigned long long)(P >> 64));          // P >> sh has 64 bits
+  unsigned long long f, fh;
+  int E;
+  // Runs l = L .. lstop + 1, calling at(l, f, E) (f_l = f 2^E) before the step
+  // to f_(l-1) = c_l f_l - f_(l+1); ends with f_lstop, f_(lstop+1) = fh 2^E.
+  auto descend = [&](int lstop, auto at) {
+    f = 1ull << 60;
+    fh = 0;
+    E = 0;
+    U96 c(P >> (sh - 32)), st((2 * N) >> (sh - 32));
+    int K = sh - 31, l = L;
+    for (; l > lstop && K > 2; --l) {  // c >= 4: renormalise every step
+      at(l);
+      const unsigned long long fn = __umul64hi(f, c.hi()) - (fh >> K);  // in units of 2^K
+      const int s = min(__clzll((long long)fn) - 3, K);                  // leading bit to bit 60 (fn < f)
+      fh = f >> (K - s);
+      f = fn << s;
+      E += K - s;
+      c.sub(st);
+      if ((int)c.w2 >= 0) {
+        c.shl1();
+        st.shl1();
+        --K;
+      }
+    }
+#pragma unroll 2
+    for (; l > lstop; --l) {  // c < 4: 62 fraction bits
+      at(l);
+      const unsigned long long fn = 4 * __umul64hi(f, c.hi()) - fh;
+      fh = f;
+      f = fn;
+      c.sub(st);
+      if (f >> 62) {
+        f >>= 2;
+        fh >>= 2;
+        E += 2;
+      }
+    }
+  };
+  const bool low = fabs(fb) < fabs(fa);  // match at ls - 1 where that is the larger
+  const int lm = low ? ls - 1 : ls;
+  int r = top, want = put.order(top);
+  if constexpr (Sink::kRaw) {
+    descend(lm, [&](int l) {
+      if (l == want) {
+        // f 2^(E-500) as FP64 (E stays below 1400)
+        const int n = __clzll((long long)f);
+        const unsigned long long m = f << n;
+        const unsigned long long m53 = (m >> 11) + ((m >> 10) & 1);
+        put.raw(r, __longlong_as_double((long long)(((unsigned long long)(63 - n + E - 500 + 1022) << 52) + m53)));
+        want = --r >= row ? put.order(r) : -1;
+      }
+    });
   } else {
-    j0 = sin(x) / x;
-    if (lmin == 0) put(0, j0);
+    descend(lm, [](int) {});
   }
-  const int L = miller_start(xs, nxs, ls + 1, x);
-  const int lstop = x >= 1.0 ? ls - 1 : 0;  // pass 1 ends with f at this order
-  // pass 1: scale
-  double fh = 0.0, f = 1.0, dl = 2.0 * L + 1.0;
-  for (int l = L; l > lstop; --l) {
-    const double fm = fma(dl * inv, f, -fh);
-    fh = f;
-    f = fm;
-    dl -= 2.0;
-  }
-  double scale;
-  if (x >= 1.0) scale = (fabs(fb) >= fabs(fa)) ? fb / fh : fa / f;  // fh = f_ls, f = f_{ls-1}
-  else scale = j0 / f;                                                // f = f_0
-  // pass 2: scaled values above ls
-  const int lwrite_hi = L < ltop ? L : ltop;
-  fh = 0.0;
-  f = 1.0;
-  dl = 2.0 * L + 1.0;
-  for (int l = L; l > ls; --l) {
-    if (l <= lwrite_hi && l >= lmin) put(l, scale * f);
-    const double fm = fma(dl * inv, f, -fh);
-    fh = f;
-    f = fm;
-    dl -= 2.0;
+  // w j_l = (w matched value 2^-60 / x / f) f_l, the power of two apart (f_l spans 1/delta)
+  const double sc = (low ? fa : fb) * inv * w / (double)f;
+  if constexpr (Sink::kRaw) {
+    // times 2^(500 - 60 - E): in range, the matched value being below 1
+    const double scr = sc == 0.0 ? 0.0 : sc * __hiloint2double((1023 + 440 - E) << 20, 0);
+    for (int t = top; t >= row; --t) put.rescale(t, scr);
+  } else {
+    int ge;
+    const unsigned long long gm = mantissa(fabs(sc), &ge);
+    const int Em = E + 60;
+    descend(put.order(row) - 1, [&](int l) {
+      if (l == want) {
+        const int n = __clzll((long long)f);
+        const double v = mul_mantissas(f << n, gm, ge - n + E - Em);
+        put.store(r, sc < 0.0 ? -v : v);
+        want = --r >= row ? put.order(r) : -1;
+      }
+    });
   }
 }
 
@@ -253,15 +453,47 @@ struct TableSink {
   int cur_lt;
   char *base;
   const int *rowof;  // null: every order is a row
-  __device__ __forceinline__ void operator()(int l, double v) {
-    const int t = rowof ? rowof[l - lmin] : l - lmin;
-    if (t < 0) return;
-    const int lt = t >> 7, r = t & 127;
+  const int *lrow;   // sampled: the rows' orders
+  int nl;
+  static constexpr bool kRaw = MODE == GCAMB_PLAIN64;
+  __device__ __forceinline__ double weight() const { return w; }
+  __device__ __forceinline__ int order(int row) const {
+    return row >= nl ? 0x7fffffff : (lrow ? __ldg(lrow + row) : lmin + row);
+  }
+  __device__ __forceinline__ int last(int l) const {
+    if (!lrow) return l - lmin;
+    if (l < lmin) return -1;
+    int lo = 0, hi = nl - 1;  // last row of order <= l
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__ldg(lrow + mid) <= l) lo = mid;
+      else hi = mid - 1;
+    }
+    return lo;
+  }
+  __device__ __forceinline__ int locate(int row) {  // the row in its tile, whose base pointer is kept
+    const int lt = row >> 7;
     if (lt != cur_lt) {
       cur_lt = lt;
       base = table + (size_t)(off_q[lt] + kbi) * TableSink::block_bytes();
     }
-    const double wv = w * v;
+    return row & 127;
+  }
+  __device__ __forceinline__ void raw(int row, double v) {
+    const int r = locate(row);
+    reinterpret_cast<double *>(base)[r * 64 + c] = v;
+  }
+  __device__ __forceinline__ void rescale(int row, double f) {
+    const int r = locate(row);
+    reinterpret_cast<double *>(base)[r * 64 + c] *= f;
+  }
+  // order l, unweighted (orders that are no row are dropped)
+  __device__ __forceinline__ void operator()(int l, double v) {
+    const int row = rowof ? rowof[l - lmin] : l - lmin;
+    if (row >= 0) store(row, w * v);
+  }
+  __device__ __forceinline__ void store(int row, double wv) {
+    const int r = locate(row);
     if constexpr (MODE == GCAMB_PLAIN64) {
       reinterpret_cast<double *>(base)[r * 64 + c] = wv;
     } else if constexpr (MODE == GCAMB_PLAIN32) {
@@ -305,6 +537,12 @@ struct KernelSink {
   double ix, ix2;
   int pl, fl;
   double pv, fv;
+  static constexpr bool kRaw = false;  // every order from l0 = the order of "row" 0: each kernel takes two
+  int l0;
+  __device__ __forceinline__ double weight() const { return 1.0; }
+  __device__ __forceinline__ int order(int row) const { return l0 + row; }
+  __device__ __forceinline__ int last(int l) const { return l - l0; }
+  __device__ __forceinline__ void store(int row, double v) { (*this)(l0 + row, v); }
   __device__ __forceinline__ void emit(int l, double jl, double jm) {
     if (l < lmin || l < 2) return;
     const double dl = (double)l;
@@ -387,7 +625,7 @@ __global__ void __launch_bounds__(128) bessel_table_kernel(const double *__restr
   // the highest multipole of the last tile this node is active in
   const int ltop = lrow ? lrow[min((lt_last + 1) * kTileL, nl) - 1] : min(lmin + (lt_last + 1) * kTileL - 1, lmax);
   TableSink<MODE> sink{static_cast<char *>(table), off + (size_t)q * nlt, lmin, kbi, i % KB,
-                       ldexp(wtau[i], scale_exp), -1, nullptr, rowof};
+                       ldexp(wtau[i], scale_exp), -1, nullptr, rowof, lrow, nl};
   if (curved) {  // hyperspherical: beta = q / sqrt|K|, chi = sqrt|K| (tau0 - tau)
     hyper_orders(k[q] / rk, rk * (tau0 - tau[i]), curved == 2, lmin, ltop, sink, s_sh, is_sh, ns);
   } else if (kern) {
@@ -395,8 +633,9 @@ __global__ void __launch_bounds__(128) bessel_table_kernel(const double *__restr
     if (x < x_lo) {
       for (int l = max(lmin, 2); l <= min(ltop, 5); ++l) sink(l, small_x_kernel(kern, l, x));
     } else {
-      KernelSink<TableSink<MODE>> ks{sink, kern, lmin, 1.0 / x, 1.0 / (x * x), -10, -10, 0.0, 0.0};
-      bessel_orders(x, lmin > 0 ? lmin - 1 : 0, ltop, xs, nxs, ks);
+      const int l0 = lmin > 0 ? lmin - 1 : 0;
+      KernelSink<TableSink<MODE>> ks{sink, kern, lmin, 1.0 / x, 1.0 / (x * x), -10, -10, 0.0, 0.0, l0};
+      bessel_orders(x, l0, ltop, xs, nxs, ks);
     }
   } else {
     bessel_orders(k[q] * (tau0 - tau[i]), lmin, ltop, xs, nxs, sink);
@@ -501,7 +740,13 @@ int curved_extents(gcamb_grid *g, cudaStream_t st) {
 
 struct DenseSink {
   double *row;
-  __device__ __forceinline__ void operator()(int l, double v) { row[l] = v; }
+  static constexpr bool kRaw = true;
+  __device__ __forceinline__ double weight() const { return 1.0; }
+  __device__ __forceinline__ int order(int r) const { return r; }
+  __device__ __forceinline__ int last(int l) const { return l; }
+  __device__ __forceinline__ void store(int r, double v) { row[r] = v; }
+  __device__ __forceinline__ void raw(int r, double v) { row[r] = v; }
+  __device__ __forceinline__ void rescale(int r, double f) { row[r] *= f; }
 };
 
 __global__ void sph_bessel_kernel(const double *__restrict__ x, int n, int lmax, const double *__restrict__ xs, int nxs,

@@ -1,0 +1,69 @@
+"""The integer recurrences of the Bessel tables where they change branch: x at
+and around 1 and whole numbers, the match at ls or ls - 1, orders cut below,
+at and above x, x beyond every order, lanes of one warp whose orders lie far
+apart (each then keeps its own Miller start) or close together, tables of
+sampled multipoles, and activity thresholds down to the smallest the grid
+takes.  Against the FP64 oracle with the bars of the other parity tests:
+1e-11 of the order's envelope (sph_bessel), of the largest |Delta| (tables)."""
+import numpy as np
+import pytest
+
+from paper_2509_25110_gb300 import build, gcamb, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    gcamb.lib()
+
+
+def check_rows(orc, x, lmax):
+    out = gcamb.sph_bessel(torch.as_tensor(x, device="cuda"), lmax).cpu().numpy()
+    gcamb.sync()
+    ref = orc.sph_bessel(lmax, x)
+    l = np.arange(lmax + 1)[None, :]
+    env = np.where(l > x[:, None], np.abs(ref), np.maximum(np.abs(ref), 1.0 / np.maximum(x[:, None], 1e-300)))
+    err = np.abs(out - ref)
+    ok = err <= 1e-11 * env + 1e-40
+    assert ok.all(), (np.argwhere(~ok)[:5], x[np.argwhere(~ok)[:5, 0]], err[~ok][:5], ref[~ok][:5])
+
+
+@pytest.mark.parametrize("lmax", [0, 1, 2, 3, 7, 64, 700])
+def test_orders_at_branch_points(orc, lmax):
+    n = np.array([1.0, 2.0, 3.0, 4.0, 7.0, 8.0, 31.0, 63.0, 64.0, 65.0, 700.0, 701.0])
+    x = np.concatenate([[0.0, 1e-300, 1e-20, 1e-3, 0.5, np.nextafter(1.0, 0.0), np.pi, 2 * np.pi, 4.4934094579],
+                        n, np.nextafter(n, 0.0), np.nextafter(n, 1e9), n + 0.5, [5000.0, 20000.0, 3.0e5]])
+    check_rows(orc, x, lmax)
+    # the same nodes one to a warp neighbourhood of their own
+    check_rows(orc, np.repeat(x, 32)[:32 * 12], lmax)
+
+
+def test_orders_of_neighbouring_nodes(orc):
+    # as in a table: x falls along the lanes, in small and in large steps
+    for step in (0.01, 1.3, 4.1, 40.0):
+        x = np.maximum(1900.0 - step * np.arange(160), 0.3)
+        check_rows(orc, x, 2200)
+
+
+@pytest.mark.parametrize("ntau,eps_cut,boost", [(40, 0.0, 1.0), (40, 1e-200, 1.0), (300, 1e-200, 3.0), (300, 0.0, 50.0)])
+@pytest.mark.parametrize("mode", [gcamb.PLAIN64, gcamb.PLAIN32])
+def test_tables(orc, ntau, eps_cut, boost, mode):
+    k = synth.log_grid(1e-4, 0.1, 23)
+    tau = synth.uniform_grid(200.0, 14000.0, ntau)
+    lmax = 500
+    rows = gcamb.l_sampling(2, lmax, boost)
+    S = np.random.default_rng(ntau).standard_normal((2, k.size, ntau))
+    g = gcamb.grid_create_lsampled(k, tau, 14000.0, rows, eps_cut=eps_cut)
+    gcamb.bessel_table(g, mode)
+    dt = torch.float64 if mode == gcamb.PLAIN64 else torch.float32
+    D = gcamb.los_transfer(g, torch.as_tensor(S, dtype=dt, device="cuda"), mode).cpu().numpy()
+    gcamb.sync()
+    ref = orc.los_cl(k, tau, 14000.0, 2, lmax, S, want_cl=False)[0][:, :, rows - 2]
+    scale = np.abs(ref).reshape(2, -1).max(axis=1)[:, None, None]
+    assert (np.abs(D - ref) <= (1e-11 if mode == gcamb.PLAIN64 else 1e-5) * scale).all()
