@@ -274,7 +274,9 @@ int gcamb_cl_interp(const gcamb_grid *g, const double *Cl_s, int M, double *Cl, 
  * Source interpolation onto the grid's k nodes (the step that prepares the
  * sources before the projection, Sec. 3.3): the natural cubic spline in k of
  * every (source, tau) column (second derivatives zero at both ends), solved
- * and evaluated in the sources' precision (FP64 or FP32).
+ * and evaluated in the sources' precision (FP64 or FP32; in FP32 the nodes more
+ * than 24 away from a second derivative may be left out of it where their
+ * weight is below 2^-40, so a non-finite value need not reach its whole column).
  *   k_in[nk_in]          host, strictly increasing, nk_in >= 2; the grid's k
  *                        range must lie inside [k_in[0], k_in[nk_in-1]]
  *   S_in[M][nk_in][ntau] device, dtype GCAMB_F64 or GCAMB_F32 (ntau: the grid's)

@@ -9,13 +9,19 @@
 // (the cubic factors are evaluated in their factored forms, which do not
 // cancel next to a node).
 // The elimination coefficients and 1/h depend on the k nodes only and are
-// formed on the host; one thread per (source, tau) column runs the forward
-// sweep and the back substitution (reads along k are coalesced across tau),
-// then one thread per output element evaluates the spline.  The arithmetic
-// is that of the sources: FP64 for FP64 sources, FP32 for FP32 sources (the
-// GPU's FP64 rate would make the FP32 case ALU-bound).
+// formed on the host.  The arithmetic is that of the sources: FP64 for FP64
+// sources, FP32 for FP32 sources (the GPU's FP64 rate would make the FP32 case
+// ALU-bound).
+//
+// FP32: one kernel solves and evaluates, marching up the nodes
+// (spline_march_kernel).  FP64, and FP32 nodes so uneven that a segment's
+// neighbourhood does not decide its second derivatives (seg_halo_ok): one
+// thread per (source, tau) column runs the forward sweep and the back
+// substitution over all nodes (reads along k are coalesced across tau), then
+// one thread per output element evaluates the spline.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -71,113 +77,307 @@ __global__ void __launch_bounds__(256) spline_solve_kernel(const T *__restrict__
 // the interval's y and M only when the interval changes.
 constexpr int kQB = 64;
 
-template <typename T, typename A>
-__global__ void __launch_bounds__(256) spline_eval_kernel(const T *__restrict__ y, const A *__restrict__ Md,
-                                                          const int *__restrict__ jq, const A *__restrict__ tq,
-                                                          const A *__restrict__ hq, int n, int nq, int ntau, int ntc,
-                                                          T *__restrict__ out) {
+// An output node's factors: y = u y_j + s y_(j+1) + a M_j + b M_(j+1),
+// s = (k - k_j)/h, u = 1 - s, a = -h^2/6 s u (1 + u), b = -h^2/6 s u (1 + s)
+// (u^3 - u = -s u (1 + u) and s^3 - s = -s u (1 + s): no cancellation near the
+// nodes), each rounded once from FP64.
+template <typename A>
+struct __align__(4 * sizeof(A)) OutCoef {
+  A s, u, a, b;
+};
+
+// V adjacent columns of a thread, loaded and stored together.
+template <int V, typename T = float>
+struct __align__(sizeof(T) * V) FV {
+  T e[V];
+};
+
+template <typename T, int V>
+__global__ void __launch_bounds__(256) spline_eval_kernel(const T *__restrict__ y, const T *__restrict__ Md,
+                                                          const int *__restrict__ jq,
+                                                          const OutCoef<T> *__restrict__ qc, int n, int nq, int ntau,
+                                                          int ntc, T *__restrict__ out) {
   const int qb = (int)(blockIdx.x / (unsigned)ntc);
-  const int t = (int)(blockIdx.x - (unsigned)qb * ntc) * 256 + threadIdx.x;
+  const int t = ((int)(blockIdx.x - (unsigned)qb * ntc) * 256 + threadIdx.x) * V;
   if (t >= ntau) return;
   const size_t m = blockIdx.y;
   const int q0 = qb * kQB, q1 = min(nq, q0 + kQB);
   int jc = -1;
-  A y0 = A(0), y1 = A(0), m0 = A(0), m1 = A(0);
+  FV<V, T> y0{}, y1{}, m0{}, m1{};
   for (int q = q0; q < q1; ++q) {
     const int j = jq[q];
     if (j != jc) {
       const size_t i0 = (m * (size_t)n + j) * ntau + t, i1 = i0 + ntau;
-      y0 = (A)y[i0];
-      y1 = (A)y[i1];
-      m0 = Md[i0];
-      m1 = Md[i1];
+      y0 = *reinterpret_cast<const FV<V, T> *>(y + i0);
+      y1 = *reinterpret_cast<const FV<V, T> *>(y + i1);
+      m0 = *reinterpret_cast<const FV<V, T> *>(Md + i0);
+      m1 = *reinterpret_cast<const FV<V, T> *>(Md + i1);
       jc = j;
     }
-    const A s = tq[q], h = hq[q], u = A(1) - s;
-    // u^3 - u = -s u (1 + u) and s^3 - s = -s u (1 + s): no cancellation near the nodes
-    const A su = s * u;
-    const A v = u * y0 + s * y1 - h * h / A(6) * su * ((A(1) + u) * m0 + (A(1) + s) * m1);
-    out[(m * nq + q) * (size_t)ntau + t] = (T)v;
+    const OutCoef<T> c = qc[q];
+    FV<V, T> r;
+#pragma unroll
+    for (int v = 0; v < V; ++v) r.e[v] = c.u * y0.e[v] + c.s * y1.e[v] + (c.a * m0.e[v] + c.b * m1.e[v]);
+    *reinterpret_cast<FV<V, T> *>(out + (m * nq + q) * (size_t)ntau + t) = r;
   }
 }
 
-// FP32 sources with ntau % 4 == 0 and 16-byte aligned arrays: the same
-// arithmetic per element, four adjacent tau columns a thread (16-byte loads
-// and stores; the output is written in 512-byte runs per warp).
-__global__ void __launch_bounds__(256) spline_eval4_kernel(const float4 *__restrict__ y, const float4 *__restrict__ Md,
-                                                           const int *__restrict__ jq, const float *__restrict__ tq,
-                                                           const float *__restrict__ hq, int n, int nq, int nt4,
-                                                           int ntc, float4 *__restrict__ out) {
-  const int qb = (int)(blockIdx.x / (unsigned)ntc);
-  const int t = (int)(blockIdx.x - (unsigned)qb * ntc) * 256 + threadIdx.x;
-  if (t >= nt4) return;
+// FP32 sources: solve and evaluate in one pass.  A thread marches up the k
+// nodes of its tau columns in segments of kSegT intervals: the forward sweep
+// runs kSegH nodes ahead; the back substitution starts there, from zero,
+// reaches the segment, and each interval's outputs follow as its two second
+// derivatives are known.
+//
+// A value r_i changes d'_j of the forward sweep by the product of the factors
+// h_(k-1)/den_k between them, and d'_i changes M_j of the back substitution by
+// the product of the c'_k (0.27 a node on even nodes, at most 2/3 and 1/2 on
+// any).  So kSegH nodes decide a second derivative: what is left out is below
+// 2^-40 of the one at that distance (the host checks the products,
+// seg_halo_ok), where FP32 keeps 2^-24.  The k range is also cut into parts
+// whose forward sweeps start kSegH nodes early, in the same way.
+//
+// Bound by HBM: the sources are read once (1 GB of 256 x 1000 x 1000), the
+// outputs written once (8.2 GB on 8000 nodes).  The columns' values arrive by
+// asynchronous copies into a ring two segments ahead, the nodes' coefficients
+// and the outputs' factors likewise (read from global memory where they are
+// used, they missed the little L1 the rings leave: 2850 us).  The sweep over whole columns that this
+// replaces wrote and read the second derivatives and was one serial chain of
+// loads a column: 1099 us and 1585 us for the evaluation, now 1483 us (DRAM at
+// 80% of its peak cycles).  (Segments
+// solved by themselves, with both neighbourhoods loaded and swept for each:
+// 1927 us at best.)
+constexpr int kSegT = 8, kSegA = 3, kSegH = kSegA * kSegT;  // segment, segments ahead
+constexpr int kYSlots = kSegA + 3, kDSlots = kSegA + 1;     // rings of segments: values, d'
+constexpr int kSegPad = 2 * kSegH + 2 * kSegT;              // zero coefficients before and after the nodes'
+constexpr int kCSlots = kYSlots + 1, kQSlots = 3;           // rings shared by the block: coefficients, output factors
+constexpr int kSegQ = 96;                                   // output nodes staged per segment (more: read from global)
+constexpr int kSegSmem = (kYSlots + kDSlots) * kSegT * 128 * 4 + kQSlots * kSegQ * 16 + kCSlots * kSegT * 16 +
+                         kQSlots * (kSegT + 1) * 4;
+
+struct __align__(16) SegCoef {
+  float ih, hm, inv, cp;  // 1/h_j, h_(j-1), 1/den_j, c'_j (0 where the node has no equation)
+};
+
+// coef and qs start at node 0 (kSegPad zero coefficients before it; qs[j] = nq
+// from the last node on, for kSegPad nodes).
+template <int V>
+__global__ void __launch_bounds__(128 / V) spline_march_kernel(const float *__restrict__ y,
+                                                               const SegCoef *__restrict__ coef,
+                                                               const int *__restrict__ qs,
+                                                               const OutCoef<float> *__restrict__ qc, int n, int nq,
+                                                               int ntau, int ntc, int nseg, int spp,
+                                                               float *__restrict__ out) {
+  constexpr int NT = 128 / V, T = kSegT, A = kSegA;
+  extern __shared__ __align__(16) float ring[];
+  FV<V> *yr = reinterpret_cast<FV<V> *>(ring) + threadIdx.x;  // [slot][row]: stride NT
+  FV<V> *dr = yr + kYSlots * T * NT;
+  OutCoef<float> *qring = reinterpret_cast<OutCoef<float> *>(ring + (kYSlots + kDSlots) * T * 128);
+  float4 *cring = reinterpret_cast<float4 *>(qring + kQSlots * kSegQ);      // ih, hm, inv, cp
+  int *nring = reinterpret_cast<int *>(cring + kCSlots * T);                // first outputs of a segment's intervals
+  const int part = (int)(blockIdx.x / (unsigned)ntc);
+  const int t = (int)(blockIdx.x - (unsigned)part * ntc) * 128 + threadIdx.x * V;
+  const bool live = t < ntau;
   const size_t m = blockIdx.y;
-  const int q0 = qb * kQB, q1 = min(nq, q0 + kQB);
-  int jc = -1;
-  float4 y0{}, y1{}, m0{}, m1{};
-  for (int q = q0; q < q1; ++q) {
-    const int j = jq[q];
-    if (j != jc) {
-      const size_t i0 = (m * (size_t)n + j) * nt4 + t, i1 = i0 + nt4;
-      y0 = y[i0];
-      y1 = y[i1];
-      m0 = Md[i0];
-      m1 = Md[i1];
-      jc = j;
+  const int sa = part * spp, sb = min(nseg, sa + spp);
+  const float *src = y + m * (size_t)n * ntau + t;
+  float *oc = out + m * (size_t)nq * ntau + t;
+  auto yslot = [&](int seg) { return yr + (seg + kYSlots * 4) % kYSlots * (T * NT); };
+  auto dslot = [&](int seg) { return dr + (seg + kDSlots * 4) % kDSlots * (T * NT); };
+  auto cslot = [&](int seg) { return cring + (seg + kCSlots * 4) % kCSlots * T; };
+  auto copy16 = [](void *to, const void *from) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from)
+                 : "memory");
+  };
+  // values and coefficients of a segment
+  auto load = [&](int seg) {
+    if (live) {
+      FV<V> *to = yslot(seg);
+#pragma unroll
+      for (int r = 0; r < T; ++r) {
+        const float *p = src + (size_t)min(max(seg * T + r, 0), n - 1) * ntau;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to + r * NT)),
+                     "l"(p), "n"(4 * V)
+                     : "memory");
+      }
     }
-    const float s = tq[q], h = hq[q], u = 1.f - s;
-    const float su = s * u, c = h * h / 6.f * su, a = 1.f + u, b = 1.f + s;
-    float4 v;
-    v.x = u * y0.x + s * y1.x - c * (a * m0.x + b * m1.x);
-    v.y = u * y0.y + s * y1.y - c * (a * m0.y + b * m1.y);
-    v.z = u * y0.z + s * y1.z - c * (a * m0.z + b * m1.z);
-    v.w = u * y0.w + s * y1.w - c * (a * m0.w + b * m1.w);
-    out[(m * nq + q) * (size_t)nt4 + t] = v;
+    if (threadIdx.x < T) copy16(cslot(seg) + threadIdx.x, coef + seg * T + threadIdx.x);
+  };
+  const int s_first = sa - 2 * A;
+  load(s_first + A);
+  load(s_first + A + 1);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  int qa = 0, qb = 0;  // outputs of segment s + 1: [qa, qb)
+  int qs1 = qs[max(s_first + 1, sa) * T];
+  FV<V> s0{}, dp{};
+  for (int s = s_first; s < sb; ++s) {
+    // this iteration's copies: values two segments past the sweep, factors of the next segment's
+    // outputs.  A slot was last read before the barrier of the iteration before.
+    load(s + A + 2);
+    const int qs0 = qs1;  // first output of segment s + 1 (from the part's first segment on)
+    qs1 = __ldg(qs + max(s + 2, sa) * T);
+    const int na = qa, nb = qb;  // this segment's
+    qa = qs0;
+    qb = s + 1 >= sa ? qs1 : qs0;
+    if (s + 1 >= sa) {
+      OutCoef<float> *to = qring + (s + 1 + kQSlots) % kQSlots * kSegQ;
+      if (qb - qa <= kSegQ)
+        for (int i = threadIdx.x; i < qb - qa; i += NT) copy16(to + i, qc + qa + i);
+      if (threadIdx.x <= T)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(
+                         nring + (s + 1 + kQSlots) % kQSlots * (T + 1) + threadIdx.x)),
+                     "l"(qs + (s + 1) * T + threadIdx.x)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
+    __syncthreads();  // the copies of the iteration before, all threads' (segments up to s + A + 1)
+    if (!live) continue;
+    {
+      // forward sweep of segment s + A; nodes without an equation have zero coefficients, hence d' = 0
+      const int f = s + A;
+      const FV<V> *ya = yslot(f), *yb = yslot(f + 1);
+      const float4 *cf = cslot(f);
+      FV<V> *d = dslot(f);
+      FV<V> y1 = ya[0];
+#pragma unroll
+      for (int r = 0; r < T; ++r) {
+        const FV<V> y2 = r + 1 < T ? ya[(r + 1) * NT] : yb[0];
+        const float4 k = cf[r];
+        // the part's first node: the slope before it is not known, its equation is left out
+        const bool lead = s == s_first && r == 0;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const float s1 = (y2.e[v] - y1.e[v]) * k.x;
+          dp.e[v] = lead ? 0.f : (6.f * (s1 - s0.e[v]) - k.y * dp.e[v]) * k.z;
+          s0.e[v] = s1;
+        }
+        d[r * NT] = dp;
+        y1 = y2;
+      }
+    }
+    if (s < sa) continue;
+    // back substitution down to the segment
+    FV<V> next{};
+#pragma unroll
+    for (int g = A; g >= 1; --g) {
+      const FV<V> *d = dslot(s + g);
+      const float4 *cf = cslot(s + g);
+#pragma unroll
+      for (int r = T - 1; r >= 0; --r) {
+        const FV<V> x = d[r * NT];
+#pragma unroll
+        for (int v = 0; v < V; ++v) next.e[v] = x.e[v] - cf[r].w * next.e[v];
+      }
+    }
+    const FV<V> *d = dslot(s), *ya = yslot(s);
+    const float4 *cf = cslot(s);
+    const OutCoef<float> *qst = qring + (s + kQSlots) % kQSlots * kSegQ;
+    const int *nst = nring + (s + kQSlots) % kQSlots * (T + 1);
+    const bool staged = nb - na <= kSegQ;
+    FV<V> yn = yslot(s + 1)[0];
+#pragma unroll
+    for (int r = T - 1; r >= 0; --r) {
+      const FV<V> x = d[r * NT], y0 = ya[r * NT];
+      FV<V> cur;
+#pragma unroll
+      for (int v = 0; v < V; ++v) cur.e[v] = x.e[v] - cf[r].w * next.e[v];
+      int q = nst[r];
+      const int q1 = nst[r + 1];
+      float *o = oc + (size_t)q * ntau;
+      auto put = [&](const OutCoef<float> &w, float *op) {
+        FV<V> z;
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          z.e[v] = fmaf(w.u, y0.e[v], fmaf(w.s, yn.e[v], fmaf(w.a, cur.e[v], w.b * next.e[v])));  // small terms first
+        if constexpr (V == 2) __stcs(reinterpret_cast<float2 *>(op), make_float2(z.e[0], z.e[1]));
+        else __stcs(op, z.e[0]);
+      };
+      if (staged) {
+        for (; q + 4 <= q1; q += 4) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) put(qst[q + u - na], o + (size_t)u * ntau);
+          o += (size_t)4 * ntau;
+        }
+        for (; q < q1; ++q, o += ntau) put(qst[q - na], o);
+      } else {
+        for (; q < q1; ++q, o += ntau) put(qc[q], o);
+      }
+      next = cur;
+      yn = y0;
+    }
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Workspace regions (each 256-byte aligned): node coefficients in FP64
-// [4][n] and FP32 [4][n]; each output node's t and h in FP64 [2][nq] and FP32
-// [2][nq]; its interval [nq] (int); the second derivatives [M][n][ntau] in the
-// arithmetic's precision (sized for FP64).
+// Workspace regions (each 256-byte aligned): node coefficients [4][n], each
+// output node's factors [nq][4], its interval [nq] (int), the intervals' first
+// outputs [n] (int): sized for FP64; the second derivatives [M][n][ntau] in the
+// arithmetic's precision (sized for FP64).  One upload fills the regions
+// before the derivatives.
 struct InterpLayout {
-  size_t c64, c32, q64, q32, qj, md, total;
+  size_t coef, q, qj, qs, md, total;
   InterpLayout(int M, int n, int ntau, int nq) {
-    c64 = 0;
-    c32 = c64 + a256((size_t)n * 4 * sizeof(double));
-    q64 = c32 + a256((size_t)n * 4 * sizeof(float));
-    q32 = q64 + a256((size_t)nq * 2 * sizeof(double));
-    qj = q32 + a256((size_t)nq * 2 * sizeof(float));
-    md = qj + a256((size_t)nq * sizeof(int));
+    coef = 0;
+    q = coef + a256(((size_t)n + kSegPad) * 4 * sizeof(double));
+    qj = q + a256((size_t)nq * 4 * sizeof(double));
+    qs = qj + a256((size_t)nq * sizeof(int));
+    md = qs + a256(((size_t)n + kSegPad) * sizeof(int));
     total = md + a256((size_t)M * n * ntau * sizeof(double));
   }
 };
 
-template <typename T, typename A>
-int launch_interp_t(const InterpLayout &L, char *w, int n, int nq, int ntau, int M, const T *S_in, T *S_out,
-                    cudaStream_t st) {
-  const A *c = reinterpret_cast<const A *>(w + (sizeof(A) == 8 ? L.c64 : L.c32));
-  const A *qd = reinterpret_cast<const A *>(w + (sizeof(A) == 8 ? L.q64 : L.q32));
-  NodeCoef<A> nc{c, c + n, c + 2 * n, c + 3 * n};
-  A *Md = reinterpret_cast<A *>(w + L.md);
+template <typename T>
+void launch_interp_columns(const InterpLayout &L, char *w, int n, int nq, int ntau, int M, const T *S_in, T *S_out,
+                           cudaStream_t st) {
+  const T *c = reinterpret_cast<const T *>(w + L.coef);
+  NodeCoef<T> nc{c, c + n, c + 2 * n, c + 3 * n};
+  T *Md = reinterpret_cast<T *>(w + L.md);
   const size_t cols = (size_t)M * ntau;
-  const int ntc = (ntau + 255) / 256, nqb = (nq + kQB - 1) / kQB;
-  spline_solve_kernel<T, A><<<(unsigned)((cols + 255) / 256), 256, 0, st>>>(S_in, nc, n, ntau, M, Md);
-  if constexpr (sizeof(T) == 4 && sizeof(A) == 4) {
-    if (ntau % 4 == 0 && reinterpret_cast<uintptr_t>(S_in) % 16 == 0 && reinterpret_cast<uintptr_t>(S_out) % 16 == 0 &&
-        reinterpret_cast<uintptr_t>(Md) % 16 == 0) {
-      const int nt4 = ntau / 4, ntc4 = (nt4 + 255) / 256;
-      spline_eval4_kernel<<<dim3((unsigned)((size_t)nqb * ntc4), (unsigned)M), 256, 0, st>>>(
-          reinterpret_cast<const float4 *>(S_in), reinterpret_cast<const float4 *>(Md),
-          reinterpret_cast<const int *>(w + L.qj), qd, qd + nq, n, nq, nt4, ntc4, reinterpret_cast<float4 *>(S_out));
-      return GCAMB_OK;
+  const int nqb = (nq + kQB - 1) / kQB;
+  spline_solve_kernel<T, T><<<(unsigned)((cols + 255) / 256), 256, 0, st>>>(S_in, nc, n, ntau, M, Md);
+  auto eval = [&](auto v) {
+    constexpr int V = decltype(v)::value;
+    const int ntc = (ntau / V + 255) / 256;
+    spline_eval_kernel<T, V><<<dim3((unsigned)((size_t)nqb * ntc), (unsigned)M), 256, 0, st>>>(
+        S_in, Md, reinterpret_cast<const int *>(w + L.qj), reinterpret_cast<const OutCoef<T> *>(w + L.q), n, nq, ntau,
+        ntc, S_out);
+  };
+  // FP32: four columns a thread in 16-byte loads and stores where the rows are aligned
+  if (sizeof(T) == 4 && ntau % 4 == 0 &&
+      (reinterpret_cast<uintptr_t>(S_in) | reinterpret_cast<uintptr_t>(S_out) | reinterpret_cast<uintptr_t>(Md)) % 16 == 0)
+    eval(std::integral_constant<int, sizeof(T) == 4 ? 4 : 1>());
+  else
+    eval(std::integral_constant<int, 1>());
+}
+
+// Whether kSegH nodes decide a second derivative: every product of kSegH - 1
+// consecutive factors of either sweep is below 2^-40.  (The host
+// needs logarithms of n factors; sums over the window slide.)
+bool seg_halo_ok(const double *h, const double *cp, const double *inv, int n) {
+  const double bound = -40.0 * 0.69314718055994530942;
+  double fw = 0.0, bw = 0.0;
+  std::vector<double> lf(n, -1e30), lb(n, -1e30);  // ends of the system: a factor of zero
+  for (int j = 2; j < n - 1; ++j) lf[j] = std::log(h[j - 1] * inv[j]);
+  for (int j = 1; j < n - 2; ++j) lb[j] = std::log(cp[j]);
+  const int w = kSegH - 1;
+  for (int j = 0; j < n; ++j) {
+    double a = 0.0, b = 0.0;
+    if (j + w > n) break;  // a shorter window reaches the system's end
+    if (j == 0 || lf[j - 1] < -1e29 || lb[j - 1] < -1e29) {
+      for (int i = j; i < j + w; ++i) {
+        a += lf[i];
+        b += lb[i];
+      }
+      fw = a;
+      bw = b;
+    } else {
+      fw += lf[j + w - 1] - lf[j - 1];
+      bw += lb[j + w - 1] - lb[j - 1];
     }
+    if (fw > bound || bw > bound) return false;
   }
-  spline_eval_kernel<T, A><<<dim3((unsigned)((size_t)nqb * ntc), (unsigned)M), 256, 0, st>>>(
-      S_in, Md, reinterpret_cast<const int *>(w + L.qj), qd, qd + nq, n, nq, ntau, ntc, S_out);
-  return GCAMB_OK;
+  return true;
 }
 
 }  // namespace
@@ -194,8 +394,10 @@ int launch_interp_sources(const double *k_in, int nk_in, const void *S_in, int M
   if ((size_t)nq * ((ntau + 255) / 256) > 0x7fffffffULL || M > 65535 || (size_t)M * ntau / 256 > 0x7fffffffULL)
     return fail(GCAMB_EINVAL, "interp_sources: too many sources or nodes for one launch");
   // elimination coefficients (nodes only) and each output node's interval
-  std::vector<double> c64(4 * (size_t)n, 0.0), q64(2 * (size_t)nq);
-  std::vector<int> qj(nq);
+  std::vector<double> c64(4 * (size_t)n, 0.0);
+  std::vector<OutCoef<double>> q64(nq);
+  std::vector<char> up(L.md);
+  int *qj = reinterpret_cast<int *>(up.data() + L.qj), *qs = reinterpret_cast<int *>(up.data() + L.qs);
   double *h = c64.data(), *ih = h + n, *cp = ih + n, *inv = cp + n;
   for (int j = 0; j + 1 < n; ++j) {
     h[j] = k_in[j + 1] - k_in[j];
@@ -207,30 +409,62 @@ int launch_interp_sources(const double *k_in, int nk_in, const void *S_in, int M
     inv[j] = 1.0 / den;
     cp[j] = (j < n - 2 ? h[j] : 0.0) * inv[j];
   }
-  for (int q = 0; q < nq; ++q) {
+  for (int q = 0, jn = 0; q < nq; ++q) {
     const double k = g->k[q];
     int j = (int)(std::upper_bound(k_in, k_in + n, k) - k_in) - 1;
     j = j < 0 ? 0 : (j > n - 2 ? n - 2 : j);
     qj[q] = j;
-    q64[q] = (k - k_in[j]) / h[j];
-    q64[nq + q] = h[j];
+    // u from the upper node: exact where s is near 1
+    const double s = (k - k_in[j]) / h[j], u = (k_in[j + 1] - k) / h[j], f = -h[j] * h[j] / 6.0 * s * u;
+    q64[q] = {s, u, f * (1.0 + u), f * (1.0 + s)};
+    for (; jn <= j; ++jn) qs[jn] = q;  // the grid's k rise: first output of interval jn
+    if (q == nq - 1)
+      for (; jn < n + kSegPad; ++jn) qs[jn] = nq;
   }
-  std::vector<float> c32(c64.begin(), c64.end()), q32(q64.begin(), q64.end());
+  // segments of intervals, and the parts of the k range: at least 16 segments a
+  // part (its sweep starts three segments early), and enough of them for ten
+  // blocks of 128 columns a resident place (five an SM)
+  const size_t nchunk = ((size_t)ntau + 127) / 128, nseg = ((size_t)n - 2) / kSegT + 1;
+  const size_t want = (152 * 50 + nchunk * M - 1) / (nchunk * M);
+  const size_t spp = std::max<size_t>(16, (nseg + want - 1) / want), nparts = (nseg + spp - 1) / spp;
+  const bool seg = dtype == GCAMB_F32 && nparts * nchunk <= 0x7fffffffULL && seg_halo_ok(h, cp, inv, n);
+  if (dtype == GCAMB_F64) {
+    std::copy(c64.begin(), c64.end(), reinterpret_cast<double *>(up.data() + L.coef));
+    std::copy(q64.begin(), q64.end(), reinterpret_cast<OutCoef<double> *>(up.data() + L.q));
+  } else {
+    if (seg) {
+      SegCoef *sc = reinterpret_cast<SegCoef *>(up.data() + L.coef) + kSegPad;  // zeros around
+      for (int j = 0; j < n; ++j)
+        sc[j] = SegCoef{(float)ih[j], j > 0 ? (float)h[j - 1] : 0.f, (float)inv[j], (float)cp[j]};
+    } else {
+      std::copy(c64.begin(), c64.end(), reinterpret_cast<float *>(up.data() + L.coef));
+    }
+    OutCoef<float> *qc = reinterpret_cast<OutCoef<float> *>(up.data() + L.q);
+    for (int q = 0; q < nq; ++q) qc[q] = {(float)q64[q].s, (float)q64[q].u, (float)q64[q].a, (float)q64[q].b};
+  }
   char *w = static_cast<char *>(ws);
-  // pageable copies return once the host data is staged
-  cudaError_t e = cudaMemcpyAsync(w + L.c64, c64.data(), c64.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(w + L.c32, c32.data(), c32.size() * sizeof(float), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(w + L.q64, q64.data(), q64.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(w + L.q32, q32.data(), q32.size() * sizeof(float), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(w + L.qj, qj.data(), qj.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  // a pageable copy returns once the host data is staged
+  cudaError_t e = cudaMemcpyAsync(w, up.data(), L.md, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(e, "interp_sources: coefficient upload");
   ProfScope prof(GCAMB_K_INTERP, st);
   if (dtype == GCAMB_F64)
-    launch_interp_t<double, double>(L, w, n, nq, ntau, M, static_cast<const double *>(S_in),
-                                    static_cast<double *>(S_out), st);
-  else
-    launch_interp_t<float, float>(L, w, n, nq, ntau, M, static_cast<const float *>(S_in), static_cast<float *>(S_out),
+    launch_interp_columns<double>(L, w, n, nq, ntau, M, static_cast<const double *>(S_in), static_cast<double *>(S_out),
                                   st);
+  else if (seg) {
+    auto go = [&](auto v) {
+      constexpr int V = decltype(v)::value;
+      spline_march_kernel<V><<<dim3((unsigned)(nparts * nchunk), (unsigned)M), 128 / V, kSegSmem, st>>>(
+          static_cast<const float *>(S_in), reinterpret_cast<const SegCoef *>(w + L.coef) + kSegPad,
+          reinterpret_cast<const int *>(w + L.qs), reinterpret_cast<const OutCoef<float> *>(w + L.q), n, nq, ntau,
+          (int)nchunk, (int)nseg, (int)spp, static_cast<float *>(S_out));
+    };
+    if (ntau % 2 == 0 && (reinterpret_cast<uintptr_t>(S_in) | reinterpret_cast<uintptr_t>(S_out)) % 8 == 0)
+      go(std::integral_constant<int, 2>());
+    else
+      go(std::integral_constant<int, 1>());
+  } else
+    launch_interp_columns<float>(L, w, n, nq, ntau, M, static_cast<const float *>(S_in), static_cast<float *>(S_out),
+                                 st);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "interp_sources: launch");
   return GCAMB_OK;

@@ -98,3 +98,30 @@ def test_interp_errors():
         gcamb.interp_sources(g, np.array([1e-4]), S[:, :1])
     assert ei.value.code == gcamb.EINVAL
     gcamb.sync()
+
+
+@pytest.mark.parametrize("nk_in,ntau,uneven", [(33, 127, 0.3), (34, 128, 0.3), (60, 129, 0.3), (61, 1, 0.3), (65, 200, 0.3),
+                                               (89, 64, 0.3), (300, 40, 0.3), (257, 64, 3.0)])
+def test_fp32_segments(nk_in, ntau, uneven):
+    """FP32 nodes around the segments of the one-pass kernel (32 intervals, 28
+    nodes of neighbourhood, 128 columns); the last case's spacings differ by
+    factors of up to e^6.  (The 30 log-spaced nodes of test_interp_matches_oracle
+    take the whole-column path.)  Bar: that of test_interp_matches_oracle."""
+    g = grid(nk=400, ntau=ntau)
+    rng = np.random.default_rng(nk_in)
+    d = np.exp(rng.uniform(-uneven, uneven, nk_in - 1))
+    k_in = 1e-4 + (0.3 - 1e-4) * np.concatenate([[0.0], np.cumsum(d) / d.sum()])
+    k_in[-1] = 0.3
+    S32 = rng.normal(size=(3, nk_in, ntau)).astype(np.float32)
+    ref = ointerp.interp_sources(k_in, S32.astype(np.float64), g.k)
+    out = gcamb.interp_sources(g, k_in, torch.as_tensor(S32, device="cuda")).cpu().numpy()
+    gcamb.sync()
+    cols = np.moveaxis(S32.astype(np.float64), 1, -1)
+    Mo = ointerp.natural_second_derivatives(k_in, cols)
+    j = np.clip(np.searchsorted(k_in, g.k, side="right") - 1, 0, nk_in - 2)
+    h = k_in[j + 1] - k_in[j]
+    t = (g.k - k_in[j]) / h
+    u = 1.0 - t
+    env = (np.abs(u * cols[..., j]) + np.abs(t * cols[..., j + 1]) +
+           h * h / 6.0 * (np.abs(u ** 3 - u) * np.abs(Mo[..., j]) + np.abs(t ** 3 - t) * np.abs(Mo[..., j + 1])))
+    assert np.all(np.abs(out - ref) <= 64 * 2.0 ** -24 * np.moveaxis(env, -1, 1) + 1e-30)
