@@ -596,15 +596,86 @@ __global__ void __launch_bounds__(256) cl_spline_block_kernel(const double *__re
   }
 }
 
+// Up to kPcrSamples samples: the second derivatives by parallel cyclic
+// reduction.  Stage s adds multiples of the equations s = 1, 2, 4, ... away that
+// cancel the neighbours, the factors (of the nodes alone) from the host:
+//   d_j <- d_j + alpha_j d_(j-s) + gamma_j d_(j+s),  M_j = d_j / b_j at the end.
+// log2(nl) steps of two FP64 multiply-adds a thread instead of a serial sweep
+// of 2 nl steps, each several dependent FP64 operations long: 130 samples, one
+// model 64 -> 11 us (cold caches).
+constexpr int kPcrSamples = 1024;
+
+int pcr_stages(int nl) {
+  int k = 0;
+  while ((1 << k) < nl - 2) ++k;
+  return k;
+}
+
+__global__ void __launch_bounds__(256) cl_spline_pcr_kernel(const double *__restrict__ Cs, const int *__restrict__ lrow,
+                                                            const int *__restrict__ rowof,
+                                                            const double *__restrict__ ih,
+                                                            const double *__restrict__ fac, int stages,
+                                                            const int *__restrict__ jl, const double *__restrict__ sl,
+                                                            int nl, int lmin, int nout, double *__restrict__ out) {
+  __shared__ double y[kPcrSamples], da[kPcrSamples], db[kPcrSamples];
+  const int m = blockIdx.x;
+  const double *c = Cs + (size_t)m * nl;
+  for (int j = threadIdx.x; j < nl; j += blockDim.x) {
+    const double l = lrow[j];
+    y[j] = l * (l + 1.0) * c[j];
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < nl; j += blockDim.x)
+    da[j] = j > 0 && j < nl - 1 ? 6.0 * ((y[j + 1] - y[j]) * ih[j] - (y[j] - y[j - 1]) * ih[j - 1]) : 0.0;
+  double *d = da, *dn = db;
+  for (int s = 0; s < stages; ++s) {
+    __syncthreads();
+    const double *al = fac + (size_t)2 * s * nl, *ga = al + nl;
+    for (int j = threadIdx.x; j < nl; j += blockDim.x) {
+      double v = d[j];
+      if (j >= (1 << s)) v = fma(al[j], d[j - (1 << s)], v);
+      if (j + (1 << s) < nl) v = fma(ga[j], d[j + (1 << s)], v);
+      dn[j] = v;
+    }
+    double *t = d;
+    d = dn;
+    dn = t;
+  }
+  __syncthreads();
+  const double *ib = fac + (size_t)2 * stages * nl;  // 1 / b, zero at both ends
+  for (int j = threadIdx.x; j < nl; j += blockDim.x) d[j] *= ib[j];
+  __syncthreads();
+  double *o = out + (size_t)m * nout;
+  // grid y shares out the outputs (each block repeats the reduction, which is
+  // small against them: FP64 on one SM took most of the time)
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < nout; i += gridDim.y * blockDim.x) {
+    const int own = rowof[i];
+    if (own >= 0) {
+      o[i] = c[own];
+      continue;
+    }
+    const int l = lmin + i, lo = jl[i];
+    const double hh = (double)(lrow[lo + 1] - lrow[lo]), s = sl[i], u = 1.0 - s, su = s * u;
+    const double v = u * y[lo] + s * y[lo + 1] - hh * hh / 6.0 * su * ((1.0 + u) * d[lo] + (1.0 + s) * d[lo + 1]);
+    o[i] = v / ((double)l * (l + 1.0));
+  }
+}
+
 size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
-// Workspace: [h, 1/h, c', 1/den] (4 nl doubles) | [s] (nout doubles) |
-// [lo] (nout ints) | second derivatives [M][nl] (doubles).
+// Coefficients: [h, 1/h, c', 1/den], or (up to kPcrSamples samples) [h, 1/h]
+// and the reduction's factors.
+static size_t cl_interp_coefs(int nl) {
+  return (nl <= kPcrSamples ? 2 + 2 * (size_t)pcr_stages(nl) + 1 : 4) * (size_t)nl;
+}
+
+// Workspace: coefficients (doubles) | [s] (nout doubles) | [lo] (nout ints) |
+// second derivatives [M][nl] (doubles).
 size_t cl_interp_workspace_bytes(const gcamb_grid *g, int M) {
   const size_t nout = (size_t)(g->lmax - g->lmin + 1);
-  return al(4 * (size_t)g->nl * sizeof(double)) + al(nout * sizeof(double)) + al(nout * sizeof(int)) +
+  return al(cl_interp_coefs(g->nl) * sizeof(double)) + al(nout * sizeof(double)) + al(nout * sizeof(int)) +
          al((size_t)M * g->nl * sizeof(double));
 }
 
@@ -630,17 +701,50 @@ int gcamb_cl_interp(const gcamb_grid *g, const double *Cl_s, int M, double *Cl, 
   if (int rc = ensure_device_grid(const_cast<gcamb_grid *>(g))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   const int nl = g->nl, nout = g->lmax - g->lmin + 1;
-  std::vector<double> coef(4 * (size_t)nl, 0.0), sv(nout, 0.0);
-  std::vector<int> jv(nout, 0);
-  double *h = coef.data(), *ih = h + nl, *cp = ih + nl, *inv = cp + nl;
+  const bool pcr = nl <= kPcrSamples;
+  const size_t ncoef = cl_interp_coefs(nl);
+  const size_t o1 = al(ncoef * sizeof(double)), o2 = o1 + al((size_t)nout * sizeof(double));
+  const size_t o3 = o2 + al((size_t)nout * sizeof(int));
+  std::vector<char> up(o3, 0);  // coefficients, s, lo in one upload
+  double *coef = reinterpret_cast<double *>(up.data()), *sv = reinterpret_cast<double *>(up.data() + o1);
+  int *jv = reinterpret_cast<int *>(up.data() + o2);
+  double *h = coef, *ih = h + nl;
   for (int j = 0; j + 1 < nl; ++j) {
     h[j] = (double)(g->lrow[j + 1] - g->lrow[j]);
     ih[j] = 1.0 / h[j];
   }
-  for (int j = 1; j < nl - 1; ++j) {
-    const double den = 2.0 * (h[j - 1] + h[j]) - (j > 1 ? h[j - 1] * cp[j - 1] : 0.0);
-    inv[j] = 1.0 / den;
-    cp[j] = (j < nl - 2 ? h[j] : 0.0) * inv[j];
+  const int stages = pcr ? pcr_stages(nl) : 0;
+  if (pcr) {
+    std::vector<double> A(nl, 0.0), B(nl, 1.0), C(nl, 0.0), An(nl), Bn(nl), Cn(nl);
+    for (int j = 1; j < nl - 1; ++j) {
+      A[j] = j > 1 ? h[j - 1] : 0.0;
+      B[j] = 2.0 * (h[j - 1] + h[j]);
+      C[j] = j < nl - 2 ? h[j] : 0.0;
+    }
+    for (int s = 0; s < stages; ++s) {
+      double *fa = coef + (2 + 2 * (size_t)s) * nl, *fg = fa + nl;
+      const int w = 1 << s;
+      for (int j = 0; j < nl; ++j) {
+        const double al_ = j >= w ? -A[j] / B[j - w] : 0.0, ga_ = j + w < nl ? -C[j] / B[j + w] : 0.0;
+        fa[j] = al_;
+        fg[j] = ga_;
+        An[j] = j >= w ? al_ * A[j - w] : 0.0;
+        Cn[j] = j + w < nl ? ga_ * C[j + w] : 0.0;
+        Bn[j] = B[j] + (j >= w ? al_ * C[j - w] : 0.0) + (j + w < nl ? ga_ * A[j + w] : 0.0);
+      }
+      A.swap(An);
+      B.swap(Bn);
+      C.swap(Cn);
+    }
+    double *ib = coef + (2 + 2 * (size_t)stages) * nl;
+    for (int j = 1; j < nl - 1; ++j) ib[j] = 1.0 / B[j];
+  } else {
+    double *cp = ih + nl, *inv = cp + nl;
+    for (int j = 1; j < nl - 1; ++j) {
+      const double den = 2.0 * (h[j - 1] + h[j]) - (j > 1 ? h[j - 1] * cp[j - 1] : 0.0);
+      inv[j] = 1.0 / den;
+      cp[j] = (j < nl - 2 ? h[j] : 0.0) * inv[j];
+    }
   }
   for (int i = 0, j = 0; i < nout && nl > 1; ++i) {
     const int l = g->lmin + i;
@@ -649,19 +753,19 @@ int gcamb_cl_interp(const gcamb_grid *g, const double *Cl_s, int M, double *Cl, 
     sv[i] = (l - g->lrow[j]) * ih[j];
   }
   char *w = static_cast<char *>(ws);
-  const size_t o1 = al(4 * (size_t)nl * sizeof(double)), o2 = o1 + al((size_t)nout * sizeof(double));
-  const size_t o3 = o2 + al((size_t)nout * sizeof(int));
   double *d_coef = reinterpret_cast<double *>(w);
   double *d_s = reinterpret_cast<double *>(w + o1);
   int *d_j = reinterpret_cast<int *>(w + o2);
   double *Md = reinterpret_cast<double *>(w + o3);
-  // pageable copies return once the host data is staged
-  cudaError_t e = cudaMemcpyAsync(d_coef, coef.data(), coef.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_s, sv.data(), sv.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_j, jv.data(), jv.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  // a pageable copy returns once the host data is staged
+  cudaError_t e = cudaMemcpyAsync(w, up.data(), o3, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(e, "cl_interp: coefficient upload");
   ProfScope prof(GCAMB_K_INTERP, st);
-  if (nl <= kSmemSamples) {
+  if (pcr) {
+    const unsigned ny = (unsigned)std::max(1, std::min((nout + 255) / 256, 304 / std::min(M, 304)));
+    cl_spline_pcr_kernel<<<dim3((unsigned)M, ny), 256, 0, st>>>(Cl_s, g->d_lrow, g->d_rowof, d_coef + nl, d_coef + 2 * (size_t)nl, stages, d_j,
+                                            d_s, nl, g->lmin, nout, Cl);
+  } else if (nl <= kSmemSamples) {
     const size_t smem = (size_t)6 * nl * sizeof(double);
     e = cudaFuncSetAttribute(cl_spline_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cl_interp: smem attribute");

@@ -139,3 +139,24 @@ def test_cl_interp_shared_and_global_paths(nl_keep):
     ref = ointerp.natural_spline_eval(x, y, ointerp.natural_second_derivatives(x, y), l_all) / (l_all * (l_all + 1.0))
     assert np.all(np.abs(Cf - ref) <= 1e-12 * np.abs(y).max(axis=1, keepdims=True) / (l_all * (l_all + 1.0)))
     assert np.array_equal(Cf[:, lv - 2], Cs)
+
+
+@pytest.mark.parametrize("nl", [1, 2, 3, 4, 5, 6, 34, 35, 257, 1023, 1024, 1025])
+def test_cl_interp_reduction_edges(nl):
+    """Sample counts around the stages of the parallel reduction and its limit
+    (1024), on uneven samples; bar as in the module docstring."""
+    rng = np.random.default_rng(nl)
+    lv = np.sort(rng.choice(np.arange(2, 4000), nl, replace=False)).astype(np.int32)
+    g = gcamb.grid_create_lsampled(synth.log_grid(1e-4, 0.3, 4), synth.uniform_grid(200.0, 14000.0, 8), 14000.0, lv)
+    Cs = 1.0 / (lv * (lv + 1.0))[None, :] * (1.0 + 0.5 * rng.standard_normal((3, nl)))
+    Cf = gcamb.cl_interp(g, dev(Cs)).cpu().numpy()
+    gcamb.sync()
+    if nl == 1:
+        assert np.array_equal(Cf, Cs)
+        return
+    l_all = np.arange(lv[0], lv[-1] + 1, dtype=np.float64)
+    x = lv.astype(np.float64)
+    y = x * (x + 1.0) * Cs
+    ref = ointerp.natural_spline_eval(x, y, ointerp.natural_second_derivatives(x, y), l_all) / (l_all * (l_all + 1.0))
+    assert np.all(np.abs(Cf - ref) <= 1e-12 * np.abs(y).max(axis=1, keepdims=True) / (l_all * (l_all + 1.0)))
+    assert np.array_equal(Cf[:, lv - lv[0]], Cs)
