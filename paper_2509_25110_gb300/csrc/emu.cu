@@ -391,20 +391,22 @@ cudaError_t chain_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cu
   return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
-template <int EPI, bool AMN, bool BMN, int NP, int ST>
-int gemm_st(const GemmArgs<NP> &a, int tiles, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(gemm_kernel<EPI, AMN, BMN, NP, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       gemm_smem(ST));
+template <int EPI, bool AMN, bool BMN, int NP, bool PS>
+int gemm_ps(const GemmArgs<NP> &a, int grid, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(gemm_kernel<EPI, AMN, BMN, NP, PS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       gemm_smem(PS));
   if (e != cudaSuccess) return cuda_fail(e, "emu: gemm smem attribute");
-  return ck(chain_launch(gemm_kernel<EPI, AMN, BMN, NP, ST>, dim3(tiles), dim3(kGemmThreads), gemm_smem(ST), st, a),
+  return ck(chain_launch(gemm_kernel<EPI, AMN, BMN, NP, PS>, dim3(grid), dim3(kGemmThreads), gemm_smem(PS), st, a),
             "emu: gemm launch");
 }
 
-// Six stages where every tile has an SM to itself, else three and two CTAs an
-// SM (see emu_gemm.cuh).
+// One tile a CTA where every tile has an SM to itself, else persistent CTAs
+// (see emu_gemm.cuh).
 template <int EPI, bool AMN, bool BMN, int NP>
 int gemm(const GemmArgs<NP> &a, int tiles, cudaStream_t st) {
-  return tiles <= 152 ? gemm_st<EPI, AMN, BMN, NP, 6>(a, tiles, st) : gemm_st<EPI, AMN, BMN, NP, 3>(a, tiles, st);
+  constexpr int kSms = 152;
+  return tiles <= kSms ? gemm_ps<EPI, AMN, BMN, NP, false>(a, tiles, st)
+                       : gemm_ps<EPI, AMN, BMN, NP, true>(a, kSms, st);
 }
 
 // Rows and tiles of a problem: C[M][N] over K.
@@ -602,7 +604,7 @@ int gcamb_emu_create(gcamb_grid *g, int n_in, int width, int depth, int max_batc
   if (rc || (rc = dalloc(&e->theta, o)) || (rc = dalloc(&e->grad, o)) || (rc = dalloc(&e->m, o)) ||
       (rc = dalloc(&e->v, o)) || (rc = dalloc(&e->mu_x, n_in)) || (rc = dalloc(&e->isd_x, n_in)) ||
       (rc = dalloc(&e->mu_y, e->n_out)) || (rc = dalloc(&e->sd_y, e->n_out)) ||
-      (rc = dalloc(&e->loss_part, ((mb + 127) / 128) * ((e->n_out + 127) / 128) * 8)) ||
+      (rc = dalloc(&e->loss_part, ((mb + 127) / 128) * ((e->n_out + 127) / 128) * kEpiWarpsG)) ||
       (rc = dalloc(&e->err, 1)) || (rc = dalloc(&e->exp_tab, 192))) {
     gcamb_emu_destroy(e);
     return rc;
@@ -801,7 +803,7 @@ int gcamb_emu_train_step(gcamb_emu *e, const float *X, const float *Y, const int
       nmax = std::max(nmax, bs.N[l]);
     }
     bs.part = e->loss_part;
-    bs.nparts = ((B + 127) / 128) * ((e->n_out + 127) / 128) * 8;
+    bs.nparts = ((B + 127) / 128) * ((e->n_out + 127) / 128) * kEpiWarpsG;
     bs.inv_total = 1.f / ((float)B * e->n_out);
     bs.loss = loss;
     if ((rc = ck(chain_launch(bias_kernel, dim3((nmax + kSumCols - 1) / kSumCols, L + 1), dim3(kSumCols * kSumClasses),

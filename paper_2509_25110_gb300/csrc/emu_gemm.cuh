@@ -10,23 +10,29 @@
 // same activations, gradients and weights as the forward pass: no transposed
 // copies exist.  Whoever produces an operand rounds it to bf16 once.
 //
-// One CTA per 128 x 128 tile, K in chunks of 64 through a ring of 32 KB
-// stages: three where the tiles are more than the SMs (two CTAs fit an SM,
-// one's epilogue beside the other's main loop), six where one CTA has the SM
-// to itself (a stage's copy takes about 1.2 us from issue to use, and three
-// in flight give an SM 80 GB/s; the last layer's input gradient 38 -> 21 us, the
-// weight gradients 32 -> 28 us): warp 0 issues the copies, warp 1 the MMAs (M = 128, N = 128, K = 16 into one
-// TMEM accumulator, in increasing k), warps 2-9 the epilogue, which turns the
-// tile through shared memory so that every global access is along a row.
+// 128 x 128 tiles, K in chunks of 64 through a ring of 32 KB stages: warp 0
+// issues the copies, warp 1 the MMAs (M = 128, N = 128, K = 16 into a TMEM
+// accumulator, in increasing k), warps 2-17 the epilogue, 32 x 32 values each,
+// turned through shared memory so that every global access is along a row.
+// Sixteen epilogue warps: eight left the latency of erff, the exp of C_l and
+// the global loads bare.
+//
+// Up to 152 tiles: one tile a CTA, six stages (a stage's copy takes about 1.2
+// us from issue to use, and three in flight give an SM 80 GB/s; the last
+// layer's input gradient 38 -> 22 us with six), the epilogue's tiles over the
+// ring.  More tiles: 152 persistent CTAs with four stages, two TMEM accumulators and the
+// epilogue's tiles beside the ring, so that a tile's loads and MMAs run under
+// the epilogue of the one before.  640 tiles of the loss layer (batch 4096,
+// n_out 2499) took 46 us with one tile a CTA, two CTAs an SM, whose 2.1 waves
+// ran as three; now 34 us.
 //
 // What bounds it: at the emulator's sizes (4096 x 512 x 512 .. 4096 x 2499 x
 // 512) one tile's operands take longer from L2 than its MMAs; the GEMMs it
 // replaces converted FP32 operands in the loading threads, a row a thread,
 // without a copy in flight beside the MMAs.  Measured, batch 4096, width 512,
-// n_out 2499: forward
-// 412 -> 57 us, input gradients 554 -> 47 us, weight gradients 350 -> 28 us, a
-// whole training step 1600 -> 181 us, bit for bit the same parameters; 4096
-// served spectra 907 -> 129 us.
+// n_out 2499: forward 412 -> 47 us, input gradients 554 -> 44 us, weight
+// gradients 350 -> 28 us, a whole training step 1600 -> 164 us, bit for bit the
+// same parameters; 4096 served spectra 907 -> 126 us.
 //
 // Every wait is bounded; a timeout sets the error word and the CTA drains its
 // copies and MMAs and frees its TMEM.
@@ -57,9 +63,14 @@ enum Epi { kGelu = 0, kBias = 1, kExp = 2, kDGelu = 3, kSliced = 4, kLoss = 5 };
 constexpr int kChunkK = 64;
 constexpr int kSliceChunks = 4;  // chunks per slice (kSliced)
 constexpr int kStageG = 32768;
-constexpr int kGemmThreads = 320;
-constexpr int kPitch = 66;       // floats per row of the epilogue's tiles
-constexpr int gemm_smem(int stages) { return stages * kStageG + 1024 /*align*/ + 256 /*barriers*/ + 192 * 8 /*exp tables*/; }
+constexpr int kEpiWarpsG = 16;
+constexpr int kGemmThreads = 64 + 32 * kEpiWarpsG;
+constexpr int kPitch = 34;       // floats per row of the epilogue's tiles (32 x 32 a warp)
+constexpr int gemm_stages(bool ps) { return ps ? 4 : 6; }
+constexpr int gemm_smem(bool ps) {
+  return gemm_stages(ps) * kStageG + 1024 /*align*/ + 256 /*barriers*/ + 192 * 8 /*exp tables*/ +
+         (ps ? kEpiWarpsG * 32 * kPitch * 4 : 0);
+}
 
 struct Prob {
   CUtensorMap ta, tb;
@@ -87,7 +98,7 @@ struct LossArgs {
   const float *Y;       // [rows][N]
   const int *idx;       // target row of each batch row, or null
   float scale;
-  float *part;          // [tiles][8]
+  float *part;          // [tiles][kEpiWarpsG]
 };
 
 template <int NP>
@@ -155,30 +166,41 @@ __device__ __forceinline__ uint64_t g_desc(uint32_t saddr) {
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-template <int EPI, bool AMN, bool BMN, int NP, int ST>
-__global__ void __launch_bounds__(kGemmThreads, ST == 3 ? 2 : 1) gemm_kernel(const __grid_constant__ GemmArgs<NP> a) {
+template <int EPI, bool AMN, bool BMN, int NP, bool PS>
+__global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_constant__ GemmArgs<NP> a) {
   constexpr bool kSl = EPI == kSliced;
-  constexpr int kStagesG = ST;
-  constexpr uint32_t kCols = kSl ? 256 : 128;  // TMEM columns: one accumulator, sliced: two
+  constexpr int kStagesG = gemm_stages(PS);
+  constexpr uint32_t kCols = kSl || PS ? 256 : 128;  // TMEM columns: two accumulators, or one
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStagesG * kStageG);
   // full[ST], empty[ST], tfull[2], tempty[2], drain, slot, abort
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + ST), tfull0 = smem_u32(bars + 2 * ST),
-                 tempty0 = smem_u32(bars + 2 * ST + 2), drain = smem_u32(bars + 2 * ST + 4);
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * ST + 5);
-  volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 2 * ST + 6);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStagesG), tfull0 = smem_u32(bars + 2 * kStagesG),
+                 tempty0 = smem_u32(bars + 2 * kStagesG + 2), drain = smem_u32(bars + 2 * kStagesG + 4);
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStagesG + 5);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 2 * kStagesG + 6);
   unsigned long long *tab = reinterpret_cast<unsigned long long *>(bars + 32);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int pi = 0;
-  if constexpr (NP > 1)
-    while (pi + 1 < a.np && (int)blockIdx.x >= a.p[pi].tile_end) ++pi;
-  const Prob &p = a.p[pi];
-  const int tile = (int)blockIdx.x - (NP > 1 && pi > 0 ? a.p[pi - 1].tile_end : 0);
-  const int i0 = tile / p.tiles_n * 128, n0 = tile % p.tiles_n * 128;
-  const int nkc = (p.K + kChunkK - 1) / kChunkK;
-  const int per = kSl ? kSliceChunks : nkc;                  // chunks per accumulation
-  const int nsl = kSl ? (nkc + per - 1) / per : 1;
+  // tiles blockIdx.x, + gridDim.x, .. (PS; else one)
+  const int ntiles = a.p[NP > 1 ? a.np - 1 : 0].tile_end;
+  struct Tile {
+    const Prob *p;
+    int tile, i0, n0, nkc, per, nsl;  // per: chunks per accumulation, nsl: accumulations
+  };
+  auto get_tile = [&](int t) {
+    Tile r;
+    int pi = 0;
+    if constexpr (NP > 1)
+      while (pi + 1 < a.np && t >= a.p[pi].tile_end) ++pi;
+    r.p = &a.p[pi];
+    r.tile = t - (NP > 1 && pi > 0 ? a.p[pi - 1].tile_end : 0);
+    r.i0 = r.tile / r.p->tiles_n * 128;
+    r.n0 = r.tile % r.p->tiles_n * 128;
+    r.nkc = (r.p->K + kChunkK - 1) / kChunkK;
+    r.per = kSl ? kSliceChunks : r.nkc;
+    r.nsl = kSl ? (r.nkc + r.per - 1) / r.per : 1;
+    return r;
+  };
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStagesG; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -186,7 +208,7 @@ __global__ void __launch_bounds__(kGemmThreads, ST == 3 ? 2 : 1) gemm_kernel(con
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull0 + 8 * b, 1);
-      mbar_init(tempty0 + 8 * b, 8);
+      mbar_init(tempty0 + 8 * b, kEpiWarpsG);
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -211,27 +233,35 @@ __global__ void __launch_bounds__(kGemmThreads, ST == 3 ? 2 : 1) gemm_kernel(con
       uint32_t ph = 0;
 #pragma unroll
       for (int s = 0; s < kStagesG; ++s) last[s] = -1;
-      for (int kc = 0; kc < nkc; ++kc) {
-        if (!mbar_wait(empty0 + 8 * stage, ph ^ 1u, abort_flag, a.err)) break;
-        const uint32_t sa = smem_u32(smem + stage * kStageG), sb = sa + 16384, bar = full0 + 8 * stage;
-        const int k0 = kc * kChunkK;
-        mbar_expect_tx(bar, kStageG);
-        last[stage] = (int)ph;
-        if constexpr (AMN) {
-          tma_load_2d(sa, &p.ta, i0, k0, bar);
-          tma_load_2d(sa + 8192, &p.ta, i0 + 64, k0, bar);
-        } else {
-          tma_load_2d(sa, &p.ta, k0, i0, bar);
-        }
-        if constexpr (BMN) {
-          tma_load_2d(sb, &p.tb, n0, k0, bar);
-          tma_load_2d(sb + 8192, &p.tb, n0 + 64, k0, bar);
-        } else {
-          tma_load_2d(sb, &p.tb, k0, n0, bar);
-        }
-        if (++stage == kStagesG) {
-          stage = 0;
-          ph ^= 1u;
+      bool ok = true;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        const Tile tl = get_tile(t);
+        const CUtensorMap *ta = &tl.p->ta, *tb = &tl.p->tb;
+        for (int kc = 0; kc < tl.nkc; ++kc) {
+          if (!mbar_wait(empty0 + 8 * stage, ph ^ 1u, abort_flag, a.err)) {
+            ok = false;
+            break;
+          }
+          const uint32_t sa = smem_u32(smem + stage * kStageG), sb = sa + 16384, bar = full0 + 8 * stage;
+          const int k0 = kc * kChunkK;
+          mbar_expect_tx(bar, kStageG);
+          last[stage] = (int)ph;
+          if constexpr (AMN) {
+            tma_load_2d(sa, ta, tl.i0, k0, bar);
+            tma_load_2d(sa + 8192, ta, tl.i0 + 64, k0, bar);
+          } else {
+            tma_load_2d(sa, ta, k0, tl.i0, bar);
+          }
+          if constexpr (BMN) {
+            tma_load_2d(sb, tb, tl.n0, k0, bar);
+            tma_load_2d(sb + 8192, tb, tl.n0 + 64, k0, bar);
+          } else {
+            tma_load_2d(sb, tb, k0, tl.n0, bar);
+          }
+          if (++stage == kStagesG) {
+            stage = 0;
+            ph ^= 1u;
+          }
         }
       }
       // no copy may still be landing when the CTA exits
@@ -243,32 +273,45 @@ __global__ void __launch_bounds__(kGemmThreads, ST == 3 ? 2 : 1) gemm_kernel(con
     if (lane == 0) {
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((AMN ? 1u : 0u) << 15) | ((BMN ? 1u : 0u) << 16) |
                                  ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-      int stage = 0;
+      int stage = 0, un = 0;  // un: accumulations so far, in buffers 0, 1, 0, ..
       uint32_t ph = 0;
-      for (int kc = 0; kc < nkc; ++kc) {
-        const int sl = kc / per, buf = kSl ? sl & 1 : 0, first = kc - sl * per;
-        if (kSl && first == 0 && !mbar_wait(tempty0 + 8 * buf, ((uint32_t)(sl >> 1) & 1u) ^ 1u, abort_flag, a.err)) break;
-        if (!mbar_wait(full0 + 8 * stage, ph, abort_flag, a.err)) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sa = smem_u32(smem + stage * kStageG), sb = sa + 16384;
-        const uint32_t d = tmem + (uint32_t)(buf * 128);
+      bool ok = true;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        const Tile tl = get_tile(t);
+        int first = 0;
+        for (int kc = 0; kc < tl.nkc; ++kc) {
+          const int buf = un & 1;
+          if ((first == 0 && !mbar_wait(tempty0 + 8 * buf, ((uint32_t)(un >> 1) & 1u) ^ 1u, abort_flag, a.err)) ||
+              !mbar_wait(full0 + 8 * stage, ph, abort_flag, a.err)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t sa = smem_u32(smem + stage * kStageG), sb = sa + 16384;
+          const uint32_t d = tmem + (uint32_t)(buf * 128);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t da = g_desc<AMN>(sa + kk * (AMN ? 2048 : 32)), db = g_desc<BMN>(sb + kk * (BMN ? 2048 : 32));
-          const uint32_t acc = (first | kk) ? 1u : 0u;
-          asm volatile(
-              "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-              "l"(da), "l"(db), "r"(idesc), "r"(acc));
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty0 + 8 * stage)
-                     : "memory");
-        if (first == per - 1 || kc == nkc - 1)
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull0 + 8 * buf)
+          for (int kk = 0; kk < 4; ++kk) {
+            const uint64_t da = g_desc<AMN>(sa + kk * (AMN ? 2048 : 32)), db = g_desc<BMN>(sb + kk * (BMN ? 2048 : 32));
+            const uint32_t acc = (first | kk) ? 1u : 0u;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+                "l"(da), "l"(db), "r"(idesc), "r"(acc));
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty0 +
+                                                                                                         8 * stage)
                        : "memory");
-        if (++stage == kStagesG) {
-          stage = 0;
-          ph ^= 1u;
+          if (++first == tl.per || kc == tl.nkc - 1) {
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull0 +
+                                                                                                           8 * buf)
+                         : "memory");
+            first = 0;
+            ++un;
+          }
+          if (++stage == kStagesG) {
+            stage = 0;
+            ph ^= 1u;
+          }
         }
       }
       // every MMA this thread issued has completed before TMEM is freed
@@ -276,113 +319,98 @@ __global__ void __launch_bounds__(kGemmThreads, ST == 3 ? 2 : 1) gemm_kernel(con
       mbar_wait(drain, 0, nullptr, a.err);
     }
   } else {
-    // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns 64 half ..
-    const int sp = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t taddr = tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(half * 64);
-    float acc[kSl ? 64 : 1];
-    float2 gz[EPI == kDGelu || EPI == kLoss ? 32 : 1];
+    // ---- epilogue: warp w has TMEM lanes 32 (w % 4) .., columns 32 quarter ..
+    const int sp = warp & 3, cq = (warp - 2) >> 2;
+    const uint32_t taddr = tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(cq * 32);
+    // its 32 x 32 tile in shared memory (one tile a CTA: over the ring, which all MMAs have read)
+    float *st = reinterpret_cast<float *>(PS ? reinterpret_cast<unsigned char *>(tab + 192) : smem) +
+                (warp - 2) * 32 * kPitch;
+    const int c2 = 2 * (lane & 15), rp = lane >> 4;  // two adjacent columns of rows rp, rp + 2, ..
+    int un = 0;
     bool ok = true;
-    auto load32 = [&](uint32_t ad, uint32_t(&r)[32]) {
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-          "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-            "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-            "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-            "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-          : "r"(ad));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    };
-    if constexpr (kSl) {
-#pragma unroll
-      for (int j = 0; j < 64; ++j) acc[j] = 0.f;
-      for (int sl = 0; sl < nsl; ++sl) {
-        const int buf = sl & 1;
-        if (!mbar_wait(tfull0 + 8 * buf, (uint32_t)(sl >> 1) & 1u, abort_flag, a.err)) {
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {  // 16 columns at a time (registers)
-          uint32_t r[16];
-          const uint32_t ad = taddr + (uint32_t)(buf * 128 + h * 16);
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-              : "r"(ad));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int j = 0; j < 16; ++j) acc[h * 16 + j] += __uint_as_float(r[j]);
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
-      }
-    } else {
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      const Tile tl = get_tile(t);
+      const Prob &p = *tl.p;
+      const int ib = tl.i0 + sp * 32, nr = min(32, p.M - ib), nb = tl.n0 + cq * 32;
+      float acc[32];
+      float2 gz[EPI == kDGelu ? 16 : 1];
+      float yt[EPI == kLoss ? 32 : 1];
+      auto load32 = [&](uint32_t ad, uint32_t(&r)[32]) {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+              "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+              "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+            : "r"(ad));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      };
       if constexpr (EPI == kDGelu) {
-        // GELU' of the tile's pre-activations while the MMAs run: all 32 rows'
-        // loads in flight, two adjacent columns a lane
-        const int ib = i0 + sp * 32, n = n0 + half * 64 + 2 * lane;
+        // GELU' of the tile's pre-activations while the MMAs run, all loads in flight
+        const int n = nb + c2;
 #pragma unroll
-        for (int r = 0; r < 32; ++r)
-          gz[r] = (ib + r < p.M && n < p.N) ? *reinterpret_cast<const float2 *>(p.Z + (long long)(ib + r) * p.ldc + n)
-                                            : make_float2(0.f, 0.f);
+        for (int i = 0; i < 16; ++i) {
+          const int r = ib + 2 * i + rp;
+          gz[i] = (r < p.M && n < p.N) ? *reinterpret_cast<const float2 *>(p.Z + (long long)r * p.ldc + n)
+                                       : make_float2(0.f, 0.f);
+        }
 #pragma unroll
-        for (int r = 0; r < 32; ++r) gz[r] = make_float2(gelu_grad_f(gz[r].x), gelu_grad_f(gz[r].y));
+        for (int i = 0; i < 16; ++i) gz[i] = make_float2(gelu_grad_f(gz[i].x), gelu_grad_f(gz[i].y));
       }
       if constexpr (EPI == kLoss) {
-        // the targets of the tile while the MMAs run (lane's columns n, n + 32)
-        const int ib = i0 + sp * 32, n = n0 + half * 64 + lane;
+        // the targets of the tile while the MMAs run (lane's column)
+        const int n = nb + lane;
         const int tr = ib + lane < p.M ? (a.ls.idx ? a.ls.idx[ib + lane] : ib + lane) : 0;
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
           const float *y = a.ls.Y + (size_t)__shfl_sync(0xffffffffu, tr, r) * p.N;
-          gz[r].x = n < p.N ? __ldg(y + n) : 0.f;
-          gz[r].y = n + 32 < p.N ? __ldg(y + n + 32) : 0.f;
+          yt[r] = n < p.N ? __ldg(y + n) : 0.f;
         }
       }
-      ok = mbar_wait(tfull0, 0, abort_flag, a.err);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    }
-    // all MMAs have read the ring: it now holds the epilogue's tiles
-    float *st = reinterpret_cast<float *>(smem) + (warp - 2) * 32 * kPitch;
-    if (__all_sync(0xffffffffu, ok)) {
-      float2 *row = reinterpret_cast<float2 *>(st + lane * kPitch);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if constexpr (kSl) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) row[h * 16 + j] = make_float2(acc[h * 32 + 2 * j], acc[h * 32 + 2 * j + 1]);
-        } else {
-          uint32_t r[32];
-          load32(taddr + (uint32_t)(h * 32), r);
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            row[h * 16 + j] = make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+      for (int j = 0; j < 32; ++j) acc[j] = 0.f;
+      for (int sl = 0; sl < tl.nsl; ++sl, ++un) {
+        const int buf = un & 1;
+        if (!__all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * buf, (uint32_t)(un >> 1) & 1u, abort_flag, a.err))) {
+          ok = false;
+          break;
         }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        uint32_t r[32];
+        load32(taddr + (uint32_t)(buf * 128), r);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = kSl ? acc[j] + __uint_as_float(r[j]) : __uint_as_float(r[j]);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
+      }
+      if (!ok) break;
+      {
+        float2 *row = reinterpret_cast<float2 *>(st + lane * kPitch);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) row[j] = make_float2(acc[2 * j], acc[2 * j + 1]);
       }
       __syncwarp();
-      const int ib = i0 + sp * 32, nr = min(32, p.M - ib), nb = n0 + half * 64;
-      // body(r) for the warp's rows.  A full tile has no exit in the loop, so that
-      // the rows' chains (erff, expf, the exp of C_l) interleave: eight warps
-      // alone leave their latency bare.
-      auto rows = [&](auto un, auto body) {
+      // body(r) for the lane's rows: first, + step, ..  A full tile has no exit in
+      // the loop, so that the rows' chains (erff, the exp of C_l) interleave.
+      auto rows = [&](auto step, auto body) {
+        constexpr int S = decltype(step)::value;
         if (nr == 32) {
-#pragma unroll decltype(un)::value
-          for (int r = 0; r < 32; ++r) body(r);
+#pragma unroll 8
+          for (int i = 0; i < 32 / S; ++i) body(i * S + (S == 2 ? rp : 0));
         } else {
 #pragma unroll 1
-          for (int r = 0; r < nr; ++r) body(r);
+          for (int i = 0; i < 32 / S; ++i)
+            if (i * S + (S == 2 ? rp : 0) < nr) body(i * S + (S == 2 ? rp : 0));
         }
       };
       if constexpr (EPI == kGelu) {
-        const int n = nb + 2 * lane;  // two adjacent columns a lane; ldc, ldb even
+        const int n = nb + c2;  // ldc, ldb even
         const float2 b = make_float2(n < p.N ? p.bias[n] : 0.f, n + 1 < p.N ? p.bias[n + 1] : 0.f);
         if (n < p.N)
-          rows(std::integral_constant<int, 8>(), [&](int r) {
-            float2 v = *reinterpret_cast<const float2 *>(st + r * kPitch + 2 * lane);
+          rows(std::integral_constant<int, 2>(), [&](int r) {
+            float2 v = *reinterpret_cast<const float2 *>(st + r * kPitch + c2);
             v.x += b.x;
             v.y += b.y;
             if (p.C)  // the padding column holds nothing that is read
@@ -391,100 +419,81 @@ __global__ void __launch_bounds__(kGemmThreads, ST == 3 ? 2 : 1) gemm_kernel(con
                 __floats2bfloat162_rn(gelu_f(v.x), gelu_f(v.y));
           });
       } else if constexpr (EPI == kDGelu) {
-        const int n = nb + 2 * lane;
+        const int n = nb + c2;
         if (n < p.N) {
 #pragma unroll
-          for (int r = 0; r < 32; ++r) {
+          for (int i = 0; i < 16; ++i) {
+            const int r = 2 * i + rp;
             if (r < nr) {
-              float2 v = *reinterpret_cast<const float2 *>(st + r * kPitch + 2 * lane);
-              v.x *= gz[r].x;
-              v.y *= gz[r].y;
+              float2 v = *reinterpret_cast<const float2 *>(st + r * kPitch + c2);
+              v.x *= gz[i].x;
+              v.y *= gz[i].y;
               *reinterpret_cast<float2 *>(p.C + (long long)(ib + r) * p.ldc + n) = v;
               *reinterpret_cast<__nv_bfloat162 *>(p.Cb + (long long)(ib + r) * p.ldb + n) = __floats2bfloat162_rn(v.x, v.y);
             }
           }
         }
       } else if constexpr (EPI == kExp) {
-        // lane's columns nb + lane, + 32; the amplitude term of row `lane`
+        // lane's column nb + lane; the amplitude term of row `lane`
         const ExpArgs &x = a.ex;
-        float sd[2], mu[2], bs[2];
-        long long qmu[2];
-        int ms[2], es[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int n = nb + lane + 32 * u;
-          const bool c = n < p.N;
-          sd[u] = c ? x.sd[n] : 1.f;
-          sd[u] = sd[u] > 0.f ? sd[u] : 1.f;
-          mu[u] = c ? x.mu[n] : 0.f;
-          bs[u] = c ? p.bias[n] : 0.f;
-          qmu[u] = __double2ll_rn((double)mu[u] * 9007199254740992.0);
-          const unsigned int sbits = __float_as_uint(sd[u]);
-          ms[u] = (int)((sbits & 0x7fffffu) | 0x800000u);
-          es[u] = (int)(sbits >> 23) - 150;
-          if ((sbits >> 23) == 0) mu[u] = __int_as_float(0x7f800000);  // subnormal sd: take the FP64 path
-        }
+        const int n = nb + lane;
+        const bool cin = n < p.N;
+        float sd = cin ? x.sd[n] : 1.f;
+        sd = sd > 0.f ? sd : 1.f;
+        float mu = cin ? x.mu[n] : 0.f;
+        const float bs = cin ? p.bias[n] : 0.f;
+        const long long qmu = __double2ll_rn((double)mu * 9007199254740992.0);
+        const unsigned int sbits = __float_as_uint(sd);
+        const int ms = (int)((sbits & 0x7fffffu) | 0x800000u), es = (int)(sbits >> 23) - 150;
+        if ((sbits >> 23) == 0) mu = __int_as_float(0x7f800000);  // subnormal sd: take the FP64 path
         double sh = 0.0;
         if (x.amp >= 0 && lane < nr) sh = (double)x.X[(size_t)(ib + lane) * x.n_in + x.amp] - (double)x.mu_x[x.amp];
         const float shf_l = (float)sh;
         const long long qsh_l = __double2ll_rn(sh * 9007199254740992.0);
-        constexpr int RU = 4;  // rows whose chains interleave
+        constexpr int RU = 8;  // rows whose chains interleave
         for (int r0 = 0; r0 < nr; r0 += RU) {
-          double c[RU][2];
+          double c[RU];
           bool bad = false;
 #pragma unroll
           for (int i = 0; i < RU; ++i) {
             const int r = r0 + i;
             const float shf = __shfl_sync(0xffffffffu, shf_l, r);
             const long long qsh = __shfl_sync(0xffffffffu, qsh_l, r);
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              const float y = st[r * kPitch + lane + 32 * u] + bs[u];
-              const float fa = y * sd[u];
-              bad |= !(fabsf(fa) < 900.f && fabsf(mu[u]) < 900.f && fabsf(shf) < 900.f &&
-                       fabsf(fa + mu[u] + shf) < 690.f);
-              const unsigned int yb = __float_as_uint(y);
-              const int ye = (int)((yb >> 23) & 255u);
-              int my = ye ? (int)((yb & 0x7fffffu) | 0x800000u) : 0;  // a subnormal y adds less than 2^-53
-              my = (yb >> 31) ? -my : my;
-              const long long m = (long long)my * (long long)ms[u];
-              const int s = ye + es[u] - 97;  // y sd 2^53 = m 2^s
-              const unsigned long long q =
-                  s >= 0 ? (unsigned long long)m << min(s, 63) : (unsigned long long)(m >> min(-s, 63));
-              c[i][u] = exp_q53((long long)(q + (unsigned long long)qmu[u] + (unsigned long long)qsh), tab);
-            }
+            const float y = st[r * kPitch + lane] + bs;
+            const float fa = y * sd;
+            bad |= !(fabsf(fa) < 900.f && fabsf(mu) < 900.f && fabsf(shf) < 900.f && fabsf(fa + mu + shf) < 690.f);
+            const unsigned int yb = __float_as_uint(y);
+            const int ye = (int)((yb >> 23) & 255u);
+            int my = ye ? (int)((yb & 0x7fffffu) | 0x800000u) : 0;  // a subnormal y adds less than 2^-53
+            my = (yb >> 31) ? -my : my;
+            const long long m = (long long)my * (long long)ms;
+            const int s = ye + es - 97;  // y sd 2^53 = m 2^s
+            const unsigned long long q =
+                s >= 0 ? (unsigned long long)m << min(s, 63) : (unsigned long long)(m >> min(-s, 63));
+            c[i] = exp_q53((long long)(q + (unsigned long long)qmu + (unsigned long long)qsh), tab);
           }
           if (__any_sync(0xffffffffu, bad)) {  // out of the fixed-point range: FP64
 #pragma unroll
             for (int i = 0; i < RU; ++i) {
               const double shd = __shfl_sync(0xffffffffu, sh, r0 + i);
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                const int n = nb + lane + 32 * u;
-                const float y = st[(r0 + i) * kPitch + lane + 32 * u] + bs[u];
-                c[i][u] = exp((double)y * (double)sd[u] + (double)(n < p.N ? x.mu[n] : 0.f) + shd);
-              }
+              const float y = st[(r0 + i) * kPitch + lane] + bs;
+              c[i] = exp((double)y * (double)sd + (double)(cin ? x.mu[n] : 0.f) + shd);
             }
           }
 #pragma unroll
           for (int i = 0; i < RU; ++i)
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-              if (r0 + i < nr && nb + lane + 32 * u < p.N)
-                x.CD[(long long)(ib + r0 + i) * p.N + nb + lane + 32 * u] = c[i][u];
+            if (r0 + i < nr && cin) x.CD[(long long)(ib + r0 + i) * p.N + n] = c[i];
         }
       } else if constexpr (EPI == kLoss) {
         float sq = 0.f;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int n = nb + lane + 32 * u;
-          if (n >= p.N) continue;
+        const int n = nb + lane;
+        if (n < p.N) {
           const float b = p.bias[n];
 #pragma unroll
           for (int r = 0; r < 32; ++r) {
             if (r < nr) {
-              const float o = st[r * kPitch + lane + 32 * u] + b;
-              const float d = o - (u ? gz[r].y : gz[r].x);
+              const float o = st[r * kPitch + lane] + b;
+              const float d = o - yt[r];
               const float g = a.ls.scale * d;
               p.C[(long long)(ib + r) * p.ldc + n] = g;
               p.Cb[(long long)(ib + r) * p.ldb + n] = __float2bfloat16_rn(g);
@@ -494,20 +503,19 @@ __global__ void __launch_bounds__(kGemmThreads, ST == 3 ? 2 : 1) gemm_kernel(con
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        if (lane == 0) a.ls.part[(size_t)tile * 8 + warp - 2] = sq;
+        if (lane == 0) a.ls.part[(size_t)tl.tile * kEpiWarpsG + warp - 2] = sq;
       } else {
-        // lane's columns nb + lane, + 32: rows of any length and alignment
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int n = nb + lane + 32 * u;
-          if (n >= p.N) continue;
+        // rows of any length and alignment
+        const int n = nb + lane;
+        if (n < p.N) {
           const float b = EPI == kBias ? p.bias[n] : 0.f;
-          rows(std::integral_constant<int, 8>(), [&](int r) {
-            const float v = st[r * kPitch + lane + 32 * u];
+          rows(std::integral_constant<int, 1>(), [&](int r) {
+            const float v = st[r * kPitch + lane];
             p.C[(long long)(ib + r) * p.ldc + n] = EPI == kBias ? v + b : v;
           });
         }
       }
+      __syncwarp();  // the tile is read before the next one overwrites it
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
