@@ -150,10 +150,17 @@ __global__ void __launch_bounds__(kSumCols *kSumClasses) bias_kernel(const __gri
   __shared__ float s[kSumClasses][kSumCols + 1];
   __shared__ double red[kSumCols * kSumClasses / 32];
   const int c = threadIdx.x % kSumCols, r = threadIdx.x / kSumCols, l = blockIdx.y;
+  // Runs beside the weight gradients, whose CTAs let it start once everything
+  // read here was complete (20 us of column sums under 28 us of GEMM: training
+  // step 164 -> 150 us).  Only the block of the loss waits, at its end, so that
+  // what waits for this kernel finds the weight gradients complete too.
   pdl_start();
-  pdl_wait();
   if (l == L) {
-    if (blockIdx.x > 0 || !a.loss) return;
+    if (blockIdx.x > 0) return;
+    if (!a.loss) {
+      pdl_wait();
+      return;
+    }
     double t = 0.0;
     for (int i = threadIdx.x; i < a.nparts; i += kSumCols * kSumClasses) t += (double)a.part[i];
 #pragma unroll
@@ -164,6 +171,7 @@ __global__ void __launch_bounds__(kSumCols *kSumClasses) bias_kernel(const __gri
       for (int i = 1; i < kSumCols * kSumClasses / 32; ++i) t += red[i];
       *a.loss = (float)(t * a.inv_total);
     }
+    pdl_wait();
     return;
   }
   const int n = blockIdx.x * kSumCols + c, N = a.N[l];

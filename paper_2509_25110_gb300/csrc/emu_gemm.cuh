@@ -31,7 +31,7 @@
 // replaces converted FP32 operands in the loading threads, a row a thread,
 // without a copy in flight beside the MMAs.  Measured, batch 4096, width 512,
 // n_out 2499: forward 412 -> 47 us, input gradients 554 -> 44 us, weight
-// gradients 350 -> 28 us, a whole training step 1600 -> 164 us, bit for bit the
+// gradients 350 -> 28 us, a whole training step 1600 -> 150 us, bit for bit the
 // same parameters; 4096 served spectra 907 -> 126 us.
 //
 // Every wait is bounded; a timeout sets the error word and the CTA drains its
@@ -145,8 +145,8 @@ __device__ __forceinline__ double exp_q53(long long q, const unsigned long long 
 
 // Programmatic dependent launch: a kernel of the emulator's chain starts while
 // the one before it drains (barriers, TMEM, tables) and waits here before it
-// touches anything an earlier kernel wrote.  Every kernel of the chain waits,
-// so what it reads or overwrites is complete through the whole chain.
+// touches anything an earlier kernel wrote.  Every kernel of the chain waits
+// (the bias sums at their end), so what it reads or overwrites is complete through the whole chain.
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -226,6 +226,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
   pdl_wait();
+  // what follows the weight gradients runs beside them (the bias sums, which
+  // read nothing later than this kernel's own inputs)
+  if constexpr (kSl) pdl_start();
 
   if (warp == 0) {
     if (lane == 0) {
