@@ -402,9 +402,9 @@ cudaError_t chain_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cu
 template <int EPI, bool AMN, bool BMN, int NP, bool PS>
 int gemm_ps(const GemmArgs<NP> &a, int grid, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(gemm_kernel<EPI, AMN, BMN, NP, PS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       gemm_smem(PS));
+                                       gemm_smem(EPI, PS));
   if (e != cudaSuccess) return cuda_fail(e, "emu: gemm smem attribute");
-  return ck(chain_launch(gemm_kernel<EPI, AMN, BMN, NP, PS>, dim3(grid), dim3(kGemmThreads), gemm_smem(PS), st, a),
+  return ck(chain_launch(gemm_kernel<EPI, AMN, BMN, NP, PS>, dim3(grid), dim3(kGemmThreads), gemm_smem(EPI, PS), st, a),
             "emu: gemm launch");
 }
 
@@ -528,12 +528,12 @@ int forward_pass(gcamb_emu *e, const float *X, const int *idx, int B, const floa
   return GCAMB_OK;
 }
 
-// 2^(i/64), i < 64, then 2^(j/8192), j < 128, as Q1.63, from the series of
-// exp(x ln 2) in double-double arithmetic (products by fused multiply-add).
-void exp2_tables(unsigned long long *tab) {
+// 2^(j / kExpTab) as Q2.62, from the series of exp(x ln 2) in double-double
+// arithmetic (products by fused multiply-add).
+void exp2_table(unsigned long long *tab) {
   const double ln2h = 0x1.62e42fefa39efp-1, ln2l = 0x1.abc9e3b39803fp-56;
-  for (int i = 0; i < 192; ++i) {
-    const double f = i < 64 ? i / 64.0 : (i - 64) / 8192.0;  // exact
+  for (int i = 0; i < kExpTab; ++i) {
+    const double f = i / (double)kExpTab;  // exact
     const double xh = f * ln2h, xl = std::fma(f, ln2h, -xh) + f * ln2l;
     double sh = 1.0, sl = 0.0;  // Horner: s = 1 + x/n s
     for (int n = 26; n >= 1; --n) {
@@ -546,7 +546,7 @@ void exp2_tables(unsigned long long *tab) {
       sh = uh + ul;
       sl = ul - (sh - uh);
     }
-    const double scale = 9223372036854775808.0;  // 2^63: sh in [1, 2) is an integer of at most 2^64 there
+    const double scale = 4611686018427387904.0;  // 2^62: sh in [1, 2) is an integer there
     tab[i] = (unsigned long long)(sh * scale) + (unsigned long long)(long long)std::nearbyint(sl * scale);
   }
 }
@@ -613,7 +613,7 @@ int gcamb_emu_create(gcamb_grid *g, int n_in, int width, int depth, int max_batc
       (rc = dalloc(&e->v, o)) || (rc = dalloc(&e->mu_x, n_in)) || (rc = dalloc(&e->isd_x, n_in)) ||
       (rc = dalloc(&e->mu_y, e->n_out)) || (rc = dalloc(&e->sd_y, e->n_out)) ||
       (rc = dalloc(&e->loss_part, ((mb + 127) / 128) * ((e->n_out + 127) / 128) * kEpiWarpsG)) ||
-      (rc = dalloc(&e->err, 1)) || (rc = dalloc(&e->exp_tab, 192))) {
+      (rc = dalloc(&e->err, 1)) || (rc = dalloc(&e->exp_tab, kExpTab))) {
     gcamb_emu_destroy(e);
     return rc;
   }
@@ -624,9 +624,9 @@ int gcamb_emu_create(gcamb_grid *g, int n_in, int width, int depth, int max_batc
     return fail(GCAMB_ENOMEM, "emu_create: mapped flags");
   }
   {
-    unsigned long long tab[192];
-    exp2_tables(tab);
-    if ((rc = ck(cudaMemcpy(e->exp_tab, tab, sizeof tab, cudaMemcpyHostToDevice), "emu_create: tables"))) {
+    std::vector<unsigned long long> tab(kExpTab);
+    exp2_table(tab.data());
+    if ((rc = ck(cudaMemcpy(e->exp_tab, tab.data(), kExpTab * sizeof(unsigned long long), cudaMemcpyHostToDevice), "emu_create: tables"))) {
       gcamb_emu_destroy(e);
       return rc;
     }

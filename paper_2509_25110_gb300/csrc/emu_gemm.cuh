@@ -20,9 +20,9 @@
 // Up to 152 tiles: one tile a CTA, six stages (a stage's copy takes about 1.2
 // us from issue to use, and three in flight give an SM 80 GB/s; the last
 // layer's input gradient 38 -> 22 us with six), the epilogue's tiles over the
-// ring.  More tiles: 152 persistent CTAs with four stages, two TMEM accumulators and the
-// epilogue's tiles beside the ring, so that a tile's loads and MMAs run under
-// the epilogue of the one before.  640 tiles of the loss layer (batch 4096,
+// ring.  More tiles: 152 persistent CTAs with four stages (three beside the exp
+// table), two TMEM accumulators and the epilogue's tiles beside the ring, so
+// that a tile's loads and MMAs run under the epilogue of the one before.  640 tiles of the loss layer (batch 4096,
 // n_out 2499) took 46 us with one tile a CTA, two CTAs an SM, whose 2.1 waves
 // ran as three; now 34 us.
 //
@@ -32,7 +32,7 @@
 // without a copy in flight beside the MMAs.  Measured, batch 4096, width 512,
 // n_out 2499: forward 412 -> 47 us, input gradients 554 -> 44 us, weight
 // gradients 350 -> 28 us, a whole training step 1600 -> 150 us, bit for bit the
-// same parameters; 4096 served spectra 907 -> 126 us.
+// same parameters; 4096 served spectra 907 -> 109 us.
 //
 // Every wait is bounded; a timeout sets the error word and the CTA drains its
 // copies and MMAs and frees its TMEM.
@@ -66,9 +66,9 @@ constexpr int kStageG = 32768;
 constexpr int kEpiWarpsG = 16;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarpsG;
 constexpr int kPitch = 34;       // floats per row of the epilogue's tiles (32 x 32 a warp)
-constexpr int gemm_stages(bool ps) { return ps ? 4 : 6; }
-constexpr int gemm_smem(bool ps) {
-  return gemm_stages(ps) * kStageG + 1024 /*align*/ + 256 /*barriers*/ + 192 * 8 /*exp tables*/ +
+constexpr int gemm_stages(int epi, bool ps) { return ps ? (epi == kExp ? 3 : 4) : 6; }
+constexpr int gemm_smem(int epi, bool ps) {
+  return gemm_stages(epi, ps) * kStageG + 1024 /*align*/ + 256 /*barriers*/ + (epi == kExp ? 4096 * 8 : 0) /*exp table*/ +
          (ps ? kEpiWarpsG * 32 * kPitch * 4 : 0);
 }
 
@@ -91,7 +91,7 @@ struct ExpArgs {
   const float *mu, *sd; // [N]
   const float *X, *mu_x;
   int n_in, amp;        // amplitude column of X, or -1
-  const unsigned long long *tab;  // exp2 tables (see exp_q53)
+  const unsigned long long *tab;  // exp2 table (see exp_q53)
 };
 
 struct LossArgs {
@@ -116,31 +116,46 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
 }
 
-// exp(y) for y = q 2^-53, |y| < 690, in 64-bit integers: GB300's FP64 pipe
-// runs at 1/64 of the FP32 rate, so an FP64 exp of every C_l costs more than
-// the network (4096 x 2499: 444 us).  t = y log2(e); exp2 of its fraction is
-// the product of two table entries (2^(i/64), 2^(j/8192), Q1.63) and
-// 1 + z + z^2/2 + z^3/6 of the rest (z < 2^-13.5; the next term is below
-// 2^-58).  Every step keeps at least 2^-52 relative, so the result is within
-// about one unit in the last place of the FP64 one.
-__device__ __forceinline__ double exp_q53(long long q, const unsigned long long *__restrict__ tab) {
-  const unsigned long long kLog2e = 0xB8AA3B295C17F0BCull;                 // log2(e), Q1.63
-  const unsigned long long yu = (unsigned long long)q + (1ull << 63);      // y + 1024, Q11.53
-  // (y + 1024) log2 e in Q.52 less 1024 log2 e
-  const long long t = (long long)(__umul64hi(yu, kLog2e) - (kLog2e >> 1));
-  const int e = (int)(t >> 52);
-  const unsigned long long f = (unsigned long long)t & ((1ull << 52) - 1);
-  const unsigned long long r0 = __umul64hi(tab[f >> 46], tab[64 + ((f >> 39) & 127)]);  // Q2.62
-  const unsigned long long g = (f & ((1ull << 39) - 1)) << 25;             // the rest, Q.77
-  const unsigned long long z = __umul64hi(g, 0xB17217F7D1CF79ACull);       // times ln 2: Q.77
-  const unsigned int zh = (unsigned int)(z >> 32);                         // Q.45
-  const unsigned int z2 = __umulhi(zh, zh);                                // z^2: Q.58; z^2 / 2: Q.59
-  const unsigned int z3 = __umulhi(__umulhi(z2, zh), 0x55555556u);         // z^3 / 6: Q.(59 + 45 - 32) = Q.72
-  const unsigned long long p = z + ((unsigned long long)z2 << 18) + ((unsigned long long)z3 << 5);
-  const unsigned long long r = r0 + (__umul64hi(r0, p) >> 13);             // Q2.62
-  // r in [2^62, 2^63]: round to 53 bits; a carry to 2^63 moves to the exponent
-  const unsigned long long m = (r + (1ull << 9)) >> 10;
-  return __longlong_as_double((long long)(((unsigned long long)(e + 1022) << 52) + m));
+// exp(y) for |y| < 690, q = (y + 1024 ln 2) 2^53, in integers: GB300's FP64
+// pipe runs at 1/64 of the FP32 rate, so an FP64 exp of every C_l costs more
+// than the network (4096 x 2499: 444 us).  k = the steps of ln 2 / 4096 below y
+// (at most 0.006 too few from the rounded factor and q's high half: never
+// above, so that the rest z is no less than 0 and below 2^-12.5); the result is the
+// table's 2^(k mod 4096 / 4096) times 1 + z + z^2 (1/2 + z (1/6 + z/24)), in
+// 32 x 32-bit products, each as wide as its term needs.  Within 0.92 units in
+// the last place over the range (3.9e6 arguments against 113-bit arithmetic).
+// A 64-bit high product for each of y log2(e), two table factors, the rest and
+// the last product made 118 instructions of an exp (and 2.0 units): the served
+// layer 74 us, now 58.
+constexpr int kExpTab = 4096;                                 // 2^(j / 4096), Q2.62
+constexpr unsigned long long kExpLn2 = 0x58B90BFBE8E7BCD6ull;  // ln 2 / 4096 in Q.75 = 1024 ln 2 in Q.53
+constexpr unsigned int kExpLo = 41502639u, kExpSpan = 2893859389u;  // y + 1024 ln 2 in Q.21: 19.79, + 1379.9
+
+__device__ __forceinline__ double exp_q53(unsigned long long q, const unsigned long long *__restrict__ tab) {
+  const unsigned int k = __umulhi((unsigned int)(q >> 32), 3098164009u) >> 8;  // 4096 log2(e) 2^19
+  const unsigned long long t = tab[k & (kExpTab - 1)];
+  const unsigned long long z = (q << 22) - (unsigned long long)k * kExpLn2;  // Q.75
+  const unsigned int zh = (unsigned int)(z >> 32);                           // Q.43
+  const unsigned int w = __umulhi(zh, 87381u) + 0x2AAAAAABu;                 // 1/6 + z/24: Q.32
+  const unsigned int u = (__umulhi(zh, w) >> 11) + 0x80000000u;              // 1/2 + z w: Q.32
+  const unsigned int z2 = (unsigned int)(((unsigned long long)zh * zh) >> 30);  // Q.56
+  const unsigned long long p = z + ((unsigned long long)__umulhi(z2, u) << 19);
+  const unsigned int th = (unsigned int)(t >> 32), tl = (unsigned int)t, ph = (unsigned int)(p >> 32),
+                     pl = (unsigned int)p;
+  const unsigned long long r =
+      t + (((unsigned long long)th * ph + __umulhi(th, pl) + __umulhi(tl, ph)) >> 11);  // Q2.62, below 2^63 (1 + 2^-19)
+  const unsigned int ov = (unsigned int)(r >> 63);
+  const unsigned long long m = (r + (512ull << ov)) >> (10 + ov);  // 53 bits; a carry moves to the exponent
+  return __longlong_as_double((long long)(((unsigned long long)((k >> 12) - 2 + ov) << 52) + m));
+}
+
+// A float below 512 in Q.53 (truncated below 2^-53); any value above: nothing that is used.
+__device__ __forceinline__ long long fix53(float v) {
+  const unsigned int b = __float_as_uint(v);
+  const int e = (int)((b >> 23) & 255u) - 97;
+  const unsigned long long m = e > -97 ? (b & 0x7fffffu) | 0x800000u : 0;
+  const long long q = (long long)(e >= 0 ? m << min(e, 63) : m >> min(-e, 63));
+  return (int)b < 0 ? -q : q;
 }
 
 // Programmatic dependent launch: a kernel of the emulator's chain starts while
@@ -169,7 +184,7 @@ __device__ __forceinline__ uint64_t g_desc(uint32_t saddr) {
 template <int EPI, bool AMN, bool BMN, int NP, bool PS>
 __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_constant__ GemmArgs<NP> a) {
   constexpr bool kSl = EPI == kSliced;
-  constexpr int kStagesG = gemm_stages(PS);
+  constexpr int kStagesG = gemm_stages(EPI, PS);
   constexpr uint32_t kCols = kSl || PS ? 256 : 128;  // TMEM columns: two accumulators, or one
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -220,7 +235,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if constexpr (EPI == kExp)
-    for (int i = threadIdx.x; i < 192; i += kGemmThreads) tab[i] = a.ex.tab[i];
+    for (int i = threadIdx.x; i < kExpTab; i += kGemmThreads) tab[i] = a.ex.tab[i];
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -326,7 +341,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     const int sp = warp & 3, cq = (warp - 2) >> 2;
     const uint32_t taddr = tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(cq * 32);
     // its 32 x 32 tile in shared memory (one tile a CTA: over the ring, which all MMAs have read)
-    float *st = reinterpret_cast<float *>(PS ? reinterpret_cast<unsigned char *>(tab + 192) : smem) +
+    float *st = reinterpret_cast<float *>(PS ? reinterpret_cast<unsigned char *>(tab + (EPI == kExp ? kExpTab : 0)) : smem) +
                 (warp - 2) * 32 * kPitch;
     const int c2 = 2 * (lane & 15), rp = lane >> 4;  // two adjacent columns of rows rp, rp + 2, ..
     int un = 0;
@@ -338,6 +353,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       float acc[32];
       float2 gz[EPI == kDGelu ? 16 : 1];
       float yt[EPI == kLoss ? 32 : 1];
+      // kExp: the lane's column's scale, mean and bias; row `lane`'s amplitude and its mean
+      float xsd = 1.f, xmu = 0.f, xbs = 0.f, xa = 0.f, xm = 0.f;
+      if constexpr (EPI == kExp) {
+        const ExpArgs &x = a.ex;
+        const int n = nb + lane;
+        if (n < p.N) {
+          xsd = x.sd[n];
+          xmu = x.mu[n];
+          xbs = p.bias[n];
+        }
+        if (x.amp >= 0) {
+          xm = x.mu_x[x.amp];
+          xa = lane < nr ? x.X[(size_t)(ib + lane) * x.n_in + x.amp] : xm;
+        }
+      }
       auto load32 = [&](uint32_t ad, uint32_t(&r)[32]) {
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -437,50 +467,44 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           }
         }
       } else if constexpr (EPI == kExp) {
-        // lane's column nb + lane; the amplitude term of row `lane`
+        // lane's column nb + lane; y sd + mu + sh in Q.53 from integers: y's and
+        // sd's mantissas (31 bits) multiply exactly, shifted right by a positive
+        // count where |y sd| < 100
         const ExpArgs &x = a.ex;
         const int n = nb + lane;
         const bool cin = n < p.N;
-        float sd = cin ? x.sd[n] : 1.f;
-        sd = sd > 0.f ? sd : 1.f;
-        float mu = cin ? x.mu[n] : 0.f;
-        const float bs = cin ? p.bias[n] : 0.f;
-        const long long qmu = __double2ll_rn((double)mu * 9007199254740992.0);
+        const float sd = xsd > 0.f ? xsd : 1.f;
+        const unsigned long long qmu = (unsigned long long)fix53(xmu) + kExpLn2;
         const unsigned int sbits = __float_as_uint(sd);
-        const int ms = (int)((sbits & 0x7fffffu) | 0x800000u), es = (int)(sbits >> 23) - 150;
-        if ((sbits >> 23) == 0) mu = __int_as_float(0x7f800000);  // subnormal sd: take the FP64 path
-        double sh = 0.0;
-        if (x.amp >= 0 && lane < nr) sh = (double)x.X[(size_t)(ib + lane) * x.n_in + x.amp] - (double)x.mu_x[x.amp];
-        const float shf_l = (float)sh;
-        const long long qsh_l = __double2ll_rn(sh * 9007199254740992.0);
+        const int ms = (int)((sbits & 0x7fffffu) | 0x800000u) << 7, es = 261 - (int)(sbits >> 23);
+        // columns and rows outside the range (or a subnormal sd): FP64 for the tile
+        const bool badt = __any_sync(0xffffffffu, !(fabsf(xmu) < 300.f) || !(fabsf(xa) < 300.f) ||
+                                                      !(fabsf(xm) < 300.f) || (sbits >> 23) == 0);
+        *reinterpret_cast<long long *>(st + lane * kPitch + 32) = fix53(xa) - fix53(xm);
+        __syncwarp();
         constexpr int RU = 8;  // rows whose chains interleave
         for (int r0 = 0; r0 < nr; r0 += RU) {
           double c[RU];
-          bool bad = false;
+          bool bad = badt;
 #pragma unroll
           for (int i = 0; i < RU; ++i) {
-            const int r = r0 + i;
-            const float shf = __shfl_sync(0xffffffffu, shf_l, r);
-            const long long qsh = __shfl_sync(0xffffffffu, qsh_l, r);
-            const float y = st[r * kPitch + lane] + bs;
-            const float fa = y * sd;
-            bad |= !(fabsf(fa) < 900.f && fabsf(mu) < 900.f && fabsf(shf) < 900.f && fabsf(fa + mu + shf) < 690.f);
+            const float *sr = st + (r0 + i) * kPitch;
+            const float y = sr[lane] + xbs;
             const unsigned int yb = __float_as_uint(y);
-            const int ye = (int)((yb >> 23) & 255u);
-            int my = ye ? (int)((yb & 0x7fffffu) | 0x800000u) : 0;  // a subnormal y adds less than 2^-53
-            my = (yb >> 31) ? -my : my;
-            const long long m = (long long)my * (long long)ms;
-            const int s = ye + es - 97;  // y sd 2^53 = m 2^s
+            const int sg = (int)yb >> 31;
+            const int my = ((int)(((yb << 7) & 0x3fffffffu) | 0x40000000u) ^ sg) - sg;  // a subnormal y: 0 or -2^-53
+            const int rs = min(es - (int)((yb >> 23) & 255u), 63);
             const unsigned long long q =
-                s >= 0 ? (unsigned long long)m << min(s, 63) : (unsigned long long)(m >> min(-s, 63));
-            c[i] = exp_q53((long long)(q + (unsigned long long)qmu + (unsigned long long)qsh), tab);
+                (unsigned long long)(((long long)my * ms) >> (rs & 63)) + qmu + *reinterpret_cast<const unsigned long long *>(sr + 32);
+            bad |= !(fabsf(y * sd) < 100.f) || (unsigned int)(q >> 32) - kExpLo > kExpSpan;
+            c[i] = exp_q53(q, tab);
           }
           if (__any_sync(0xffffffffu, bad)) {  // out of the fixed-point range: FP64
 #pragma unroll
             for (int i = 0; i < RU; ++i) {
-              const double shd = __shfl_sync(0xffffffffu, sh, r0 + i);
-              const float y = st[(r0 + i) * kPitch + lane] + bs;
-              c[i] = exp((double)y * (double)sd + (double)(cin ? x.mu[n] : 0.f) + shd);
+              const double shd = (double)__shfl_sync(0xffffffffu, xa, r0 + i) - (double)xm;
+              const float y = st[(r0 + i) * kPitch + lane] + xbs;
+              c[i] = exp((double)y * (double)sd + (double)xmu + shd);
             }
           }
 #pragma unroll

@@ -1,6 +1,6 @@
 """The emulator's kernels at the edges of their tiling: widths, output counts
-and batches that fill no 128 x 128 tile, more tiles than SMs (three-stage
-rings, two CTAs an SM) and fewer (six stages), K of one chunk, slices of the
+and batches that fill no 128 x 128 tile, more tiles than SMs (persistent
+CTAs) and fewer (one tile a CTA), K of one chunk, slices of the
 batch sum that are not full, gathered batches; and the fixed-point exponential
 of the served spectra over its whole range and beyond it.
 
@@ -36,7 +36,8 @@ def frob_rel(a, b):
 
 @pytest.mark.parametrize("width,depth,lmax,B,gather", [
     (16, 1, 9, 40, False), (33, 2, 130, 127, True), (64, 3, 129, 128, False), (130, 2, 131, 129, True),
-    (128, 1, 300, 257, False), (200, 2, 2500, 1153, True), (512, 2, 40, 2500, False)])
+    (128, 1, 300, 257, False), (200, 2, 2500, 1153, True), (512, 2, 40, 2500, False),
+    (32, 1, 40, 20000, False), (1100, 2, 2500, 130, False)])
 def test_network_at_tile_edges(width, depth, lmax, B, gather):
     g = grid(lmax)
     e = gcamb.emu_create(g, width=width, depth=depth, max_batch=B, seed=1)
@@ -101,3 +102,22 @@ def test_served_exponential(B):
     y, ref = spectra(Xd[:B].contiguous())
     err = np.abs(C.cpu().numpy() / ref - 1.0)
     assert (err <= (2.0 * np.abs(y) + 4.0) * 2.0 ** -52).all(), np.max(err / ((2.0 * np.abs(y) + 4.0) * 2.0 ** -52))
+
+
+@pytest.mark.parametrize("lmax,B,step", [(301, 6600, 2000), (2500, 1025, 128)])
+def test_persistent_ctas_give_the_same_rows(lmax, B, step):
+    """Every row of a batch whose tiles outnumber the SMs against the same rows
+    in batches of one tile a CTA: a row's sums know nothing of the others."""
+    g = grid(lmax)
+    e = gcamb.emu_create(g, width=48, depth=2, max_batch=B, seed=4)
+    rng = np.random.default_rng(10)
+    X = torch.as_tensor(rng.normal(size=(B, 9)).astype(np.float32), device="cuda")
+    out = gcamb.emu_forward(e, X)
+    parts = [gcamb.emu_forward(e, X[i:i + step].contiguous()) for i in range(0, B, step)]
+    gcamb.emu_check(e, X, torch.exp(out.double() + X[:, 8:9].double()), tol=1e-9, min_count=1)
+    C, fb = gcamb.emulate(e, X)
+    Cp = [gcamb.emulate(e, X[i:i + step].contiguous())[0] for i in range(0, B, step)]
+    gcamb.sync()
+    assert int(fb.sum().item()) == 0
+    assert torch.equal(out, torch.cat(parts))
+    assert torch.equal(C, torch.cat(Cp))
