@@ -68,6 +68,14 @@ constexpr int plain_rv(int nv) { return nv == 1 ? 8 : 4; }
 template <typename T>
 constexpr int plain_unroll() { return sizeof(T) == 8 ? 1 : 2; }
 
+// Steps ahead at which a row's line is asked into L2 (0: not), a line a lane:
+// the FP32 kernel's registers hold two steps' loads, which cover half of the
+// DRAM latency (E-mode, 5 sources, l_max 2001: 301 us without, 290 / 278 /
+// 273 / 278 / 282 / 298 at 2 / 3 / 4 / 6 / 8 / 16).  FP64 gains nothing (l_max 500 68.8,
+// 68.4 at 4, l_max 5000 7953, 7910 at 4 and 8622 at 8).
+template <typename T>
+constexpr int plain_ahead() { return sizeof(T) == 8 ? 0 : 4; }
+
 // Tau blocks staged in shared memory at a time (64 KB of sources).
 constexpr int plain_stage_blocks(int nv, size_t esize) { return (int)(65536 / (nv * esize * kPlainKB)); }
 
@@ -159,7 +167,7 @@ __device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, T
 // Measured (one model, before -> after): FP64 l_max 500 93 -> 69 us,
 // l_max 5000 9380 -> 7951 us (its products alone: 7300 us); tensor modes l_max
 // 1500 3105 (four passes and a combining one) -> 1948 us; FP32 E-mode, 5
-// sources, l_max 2001 950 -> 307 us.
+// sources, l_max 2001 950 -> 274 us.
 //
 // Splits: a warp pass covers 4 RV rows (lane group g, slot i: row 4 i + g);
 // the rows / 32 row warps take passes in turn, and the 128 / rows warps that
@@ -339,6 +347,14 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
 #pragma unroll
         for (int i = 0; i < RV; ++i) acc[v][i] = T(0);
       const T *rows = chunk + (size_t)b0 * kTileL * KB + (rsub + rb + grp) * KB + sub * VE;
+      // a lane's row of the pass (4 RV rows) for the lines ahead
+      constexpr int AHEAD = plain_ahead<T>();
+      const T *arow = chunk + (size_t)b0 * kTileL * KB + (rsub + rb + lane) * KB;
+      int an = 0;  // its steps
+      if constexpr (AHEAD > 0) {
+#pragma unroll
+        for (int i = 0; i < RV; ++i) an = (lane >> 2) == i ? ns[i] : an;
+      }
       // steps that all RV row sets need, then the rest (a set's bound is
       // uniform over the warp); UN steps' loads are in flight together
       auto step = [&](int i0, auto un, auto check) {
@@ -374,7 +390,17 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
       };
       constexpr int UN = plain_unroll<T>();
       int st = ts;
-      for (; st + (UN - 1) * TS < nmin; st += UN * TS) step(st, std::integral_constant<int, UN>(), std::false_type());
+      for (; st + (UN - 1) * TS < nmin; st += UN * TS) {
+        if constexpr (AHEAD > 0) {
+#pragma unroll
+          for (int u = 0; u < UN; ++u) {
+            const int sa = st + (AHEAD + u) * TS;
+            if (sa < an)
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(arow + (size_t)(sa / STEPS) * (kTileL * KB) + (sa % STEPS) * SN));
+          }
+        }
+        step(st, std::integral_constant<int, UN>(), std::false_type());
+      }
       for (; st < nmax; st += TS) step(st, std::integral_constant<int, 1>(), std::true_type());
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -488,7 +514,7 @@ int emode_x_lo(const gcamb_grid *g, double *x_lo) {
 // grid, and the warps of a CTA would finish far apart.  By the grid alone, so
 // that a source's sums do not depend on its batch.  Measured at 128 / 64 (32)
 // rows: l_max 500 (count 570) 73 / 69 (74) us; tensor l_max 1500 (2540) 1950 /
-// 2058 (2385); E-mode FP32 l_max 2001 (3063) 307 / 363 (495); l_max 5000
+// 2058 (2385); E-mode FP32 l_max 2001 (3063) 307 / 363 (495) (before its prefetch); l_max 5000
 // (19702) 7951 / 7962 (8334); sampled l_max 2500 (2043) 343 / 293 (302).
 static int plain_rows(const gcamb_grid *g, const Table &t) {
   const double full = t.max_nkb > 0 ? (double)t.nblocks / t.max_nkb : 0.0;
