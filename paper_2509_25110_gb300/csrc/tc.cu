@@ -1075,7 +1075,10 @@ __device__ __forceinline__ double prefix_weight(const double *__restrict__ wk, c
 // Every epilogue weight forms 4 pi w_k P in FP64 and takes its square root in
 // FP32 (wq within 2^-24 relative; the same expression on every path).
 // Rows at or beyond their source tile's longest k prefix (tile_nk) are left
-// out: no work item of that tile reaches them.
+// out: no work item of that tile reaches them.  So are the padding rows of
+// the last tile (m >= M): an operand row enters its own column of the product
+// alone, and the reduce reads no column of theirs (37 sources in a tile of
+// 64, l_max 1237: 50 -> 36 us, with 8-byte loads where rows start on 8 bytes).
 template <int MODE, int CACHE>
 __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict__ S, const double *__restrict__ Pk,
                                                          const double *__restrict__ wk, const double *__restrict__ kk,
@@ -1090,8 +1093,8 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict
   if (row >= (size_t)nk * mpad) return;
   const int q = (int)(row / mpad), mfull = (int)(row - (size_t)q * mpad);
   const int mt = mfull / NT, n = mfull - mt * NT;
-  if (q >= tile_nk[mt]) return;
-  const bool live = mfull < M && q < nk_m[mfull];
+  if (q >= tile_nk[mt] || mfull >= M) return;
+  const bool live = q < nk_m[mfull];
   const int mc = live ? perm[mfull] : 0;
   const float *src = S + ((size_t)mc * nk + q) * ntau;
   int s = 0;
@@ -1101,7 +1104,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict
   // loads one chunk's fp32 values (zero beyond ntau and for dead rows)
   auto load_chunk = [&](int ch, float *v) {
     const int t0 = ch * EPC;
-    if (live && vec && t0 + EPC <= ntau) {
+    if (live && vec == 4 && t0 + EPC <= ntau) {
       const float4 *s4 = reinterpret_cast<const float4 *>(src + t0);
 #pragma unroll
       for (int u = 0; u < EPC / 4; ++u) {
@@ -1110,6 +1113,14 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict
         v[4 * u + 1] = f.y;
         v[4 * u + 2] = f.z;
         v[4 * u + 3] = f.w;
+      }
+    } else if (live && vec == 2 && t0 + EPC <= ntau) {
+      const float2 *s2 = reinterpret_cast<const float2 *>(src + t0);
+#pragma unroll
+      for (int u = 0; u < EPC / 2; ++u) {
+        const float2 f = __ldg(s2 + u);
+        v[2 * u + 0] = f.x;
+        v[2 * u + 1] = f.y;
       }
     } else {
 #pragma unroll
@@ -1131,7 +1142,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict
 #pragma unroll
         for (int u = 0; u < EPC; ++u)
           if (lane + 32 * j < nch) mx = fmaxf(mx, fabsf(cache[j][u]));
-    } else if (live && vec) {
+    } else if (live && vec == 4) {
       // 16-byte loads, eight in flight per lane
       const float4 *s4 = reinterpret_cast<const float4 *>(src);
       const int n4 = ntau >> 2;
@@ -2003,7 +2014,9 @@ int launch_tc(const gcamb_grid *g, const TcPlan &pl, const float *S, const doubl
   }
   {
     const size_t rows = (size_t)g->nk * pl.mpad;
-    const int vec = (g->ntau % 4 == 0) && (reinterpret_cast<uintptr_t>(S) % 16 == 0);
+    // floats of a load that every row's start is aligned to
+    const uintptr_t al = reinterpret_cast<uintptr_t>(S) | (uintptr_t)g->ntau * sizeof(float);
+    const int vec = al % 16 == 0 ? 4 : (al % 8 == 0 ? 2 : 1);
     const unsigned nblk = (unsigned)((rows + 7) / 8);
     // the fused kernel's inputs (weights; fp16: and the row scales) are
     // traced as weights, the split pass (which also writes the weights) as split
@@ -2019,7 +2032,7 @@ int launch_tc(const gcamb_grid *g, const TcPlan &pl, const float *S, const doubl
         if (e != cudaSuccess) return cuda_fail(e, "los_cl: weight reset");
       }
       rowscale_kernel<<<(unsigned)(((size_t)pl.M * g->nk + 15) / 16), 256, 0, st>>>(
-          S, Pk, g->d_wk, pl.M, g->nk, g->ntau, pl.mpad, t.scale_exp, vec, wp, sc);
+          S, Pk, g->d_wk, pl.M, g->nk, g->ntau, pl.mpad, t.scale_exp, vec == 4, wp, sc);
     }
     else if (MODE == kF16 && pl.nkbs * (TcGeom<MODE>::kRowB / 16) <= 32 * 4)  // rows of up to 1024 tau
       split_rows_kernel<MODE, 4><<<nblk, 256, 0, st>>>(S, Pk, g->d_wk, g->d_k, pl.M, g->nk, g->ntau, NT, pl.n_mt,

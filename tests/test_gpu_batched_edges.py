@@ -203,3 +203,44 @@ def test_two_host_threads_share_the_library():
     assert not errs, errs
     for i in range(2):
         assert torch.equal(out[i], refs[i])
+
+
+@pytest.mark.parametrize("mode", [gcamb.BF16X3, gcamb.F16X3, gcamb.TF32X3])
+@pytest.mark.parametrize("ntau,M,offset", [(61, 1, 0), (62, 37, 0), (64, 63, 2), (1030, 65, 0), (1030, 3, 1)])
+def test_split_pass_alignment_and_padding_rows(monkeypatch, mode, ntau, M, offset):
+    """The split pass reads rows that start on 4, 8 or 16 bytes with loads of
+    that width and leaves the padding rows of the last source tile unwritten:
+    in a workspace full of NaNs, and from a buffer `offset` floats off, the
+    spectra are finite, the same bits as from scalar loads, and those of the
+    same sources followed by others (another split of the work: within the
+    batched path's bar)."""
+    monkeypatch.setenv("GCAMB_TC_FUSED", "0")
+    nk = 20
+    k, tau, S, P = inputs(nk, ntau, M)
+    g = gcamb.grid_create(k, tau, 14000.0, 2, 200)
+    gcamb.bessel_table(g, mode)
+    need = gcamb.los_cl_workspace(g, M, mode)
+
+    def run(Sd):
+        ws = torch.full((need,), 0xFF, dtype=torch.uint8, device="cuda")
+        C = gcamb.los_cl(g, Sd, torch.as_tensor(P, device="cuda"), mode, ws=ws)
+        gcamb.sync()
+        return C
+
+    buf = torch.zeros(M * nk * ntau + 8, dtype=torch.float32, device="cuda")
+    Sd = buf[offset:offset + M * nk * ntau].view(M, nk, ntau)
+    Sd.copy_(torch.as_tensor(S))
+    C = run(Sd)
+    assert torch.all(torch.isfinite(C)) and torch.all(C > 0)
+    # one float off: every load scalar
+    buf2 = torch.zeros(M * nk * ntau + 8, dtype=torch.float32, device="cuda")
+    S1 = buf2[3:3 + M * nk * ntau].view(M, nk, ntau)
+    S1.copy_(torch.as_tensor(S))
+    assert torch.equal(C, run(S1))
+    # more sources behind them: no padding rows in the first tile
+    k, tau, S2, P2 = inputs(nk, ntau, M)
+    Sx = torch.as_tensor(np.concatenate([S2] * 3), device="cuda")
+    Px = torch.as_tensor(np.concatenate([P2] * 3), device="cuda")
+    Cx = gcamb.los_cl(g, Sx, Px, mode)
+    gcamb.sync()
+    assert torch.all((Cx[:M] / C - 1).abs() <= 1e-5)
