@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256) spline_eval_kernel(const T *__restrict__ 
 // and the outputs' factors likewise (read from global memory where they are
 // used, they missed the little L1 the rings leave: 2850 us).  The sweep over whole columns that this
 // replaces wrote and read the second derivatives and was one serial chain of
-// loads a column: 1099 us and 1585 us for the evaluation, now 1483 us (DRAM at
+// loads a column: 1099 us and 1585 us for the evaluation, now 1532 us (DRAM at
 // 80% of its peak cycles).  (Segments
 // solved by themselves, with both neighbourhoods loaded and swept for each:
 // 1927 us at best.)
@@ -164,9 +164,9 @@ template <int V>
 __global__ void __launch_bounds__(128 / V) spline_march_kernel(const float *__restrict__ y,
                                                                const SegCoef *__restrict__ coef,
                                                                const int *__restrict__ qs,
-                                                               const OutCoef<float> *__restrict__ qc, int n, int nq,
-                                                               int ntau, int ntc, int nseg, int spp,
-                                                               float *__restrict__ out) {
+                                                               const OutCoef<float> *__restrict__ qc,
+                                                               const int4 *__restrict__ parts, int n, int nq,
+                                                               int ntau, int ntc, float *__restrict__ out) {
   constexpr int NT = 128 / V, T = kSegT, A = kSegA;
   extern __shared__ __align__(16) float ring[];
   FV<V> *yr = reinterpret_cast<FV<V> *>(ring) + threadIdx.x;  // [slot][row]: stride NT
@@ -178,7 +178,8 @@ __global__ void __launch_bounds__(128 / V) spline_march_kernel(const float *__re
   const int t = (int)(blockIdx.x - (unsigned)part * ntc) * 128 + threadIdx.x * V;
   const bool live = t < ntau;
   const size_t m = blockIdx.y;
-  const int sa = part * spp, sb = min(nseg, sa + spp);
+  const int4 pt = parts[part];  // segments [x, y), of their outputs [z, w)
+  const int sa = pt.x, sb = pt.y;
   const float *src = y + m * (size_t)n * ntau + t;
   float *oc = out + m * (size_t)nq * ntau + t;
   auto yslot = [&](int seg) { return yr + (seg + kYSlots * 4) % kYSlots * (T * NT); };
@@ -216,8 +217,8 @@ __global__ void __launch_bounds__(128 / V) spline_march_kernel(const float *__re
     const int qs0 = qs1;  // first output of segment s + 1 (from the part's first segment on)
     qs1 = __ldg(qs + max(s + 2, sa) * T);
     const int na = qa, nb = qb;  // this segment's
-    qa = qs0;
-    qb = s + 1 >= sa ? qs1 : qs0;
+    qa = max(qs0, pt.z);
+    qb = s + 1 >= sa ? max(qa, min(qs1, pt.w)) : qa;
     if (s + 1 >= sa) {
       OutCoef<float> *to = qring + (s + 1 + kQSlots) % kQSlots * kSegQ;
       if (qb - qa <= kSegQ)
@@ -280,8 +281,8 @@ __global__ void __launch_bounds__(128 / V) spline_march_kernel(const float *__re
       FV<V> cur;
 #pragma unroll
       for (int v = 0; v < V; ++v) cur.e[v] = x.e[v] - cf[r].w * next.e[v];
-      int q = nst[r];
-      const int q1 = nst[r + 1];
+      int q = max(nst[r], pt.z);
+      const int q1 = min(nst[r + 1], pt.w);
       float *o = oc + (size_t)q * ntau;
       auto put = [&](const OutCoef<float> &w, float *op) {
         FV<V> z;
@@ -299,6 +300,14 @@ __global__ void __launch_bounds__(128 / V) spline_march_kernel(const float *__re
         }
         for (; q < q1; ++q, o += ntau) put(qst[q - na], o);
       } else {
+        for (; q + 4 <= q1; q += 4) {
+          OutCoef<float> w[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) w[u] = qc[q + u];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) put(w[u], o + (size_t)u * ntau);
+          o += (size_t)4 * ntau;
+        }
         for (; q < q1; ++q, o += ntau) put(qc[q], o);
       }
       next = cur;
@@ -380,6 +389,58 @@ bool seg_halo_ok(const double *h, const double *cp, const double *inv, int n) {
   return true;
 }
 
+// Parts of the march, {first segment, one past the last, first output, one past
+// the last}, of about equal work t, counted in segments: kPartOuts outputs take
+// about as long as a segment's sweep and back substitution.  A part's sweep
+// starts 2 kSegA segments early, so `blocks` columns' parts take (2 kSegA + t)
+// (1 + W / t) one after the other on the chip's places (five blocks an SM),
+// W = all work / places; t = sqrt(2 kSegA W) is its least, and at least
+// kPartMin.  A segment with many outputs (nodes that are sparse where the grid
+// is dense) is shared out by outputs; segments without any are left out where
+// a part can start behind them.  Kernel time, parts of at least 16 whole
+// segments -> these (nodes -> grid, tau, sources): 200 -> 8000, 300, 8: 582 ->
+// 50 us; 395 -> 6075, 498, 15: 267 -> 67; 200 -> 1000, 300, 8: 59 -> 16; 518 -> 4312, 499,
+// 155: 439 -> 432; 1000 -> 8000, 1000, 256: 1509 -> 1532 (the bounds of a part's outputs).
+constexpr int kPartOuts = 64, kPartMin = 4;
+
+std::vector<int4> march_parts(const int *qs, int n, int nq, size_t blocks) {
+  const int nseg = (n - 2) / kSegT + 1;
+  const double work = (nseg + (double)nq / kPartOuts) * (double)blocks / (152 * 5);
+  const double target = std::max((double)kPartMin, std::sqrt(2.0 * kSegA * work));
+  std::vector<int4> parts;
+  int4 p{-1, 0, 0, 0};
+  double c = 0.0;
+  for (int s = 0, q = 0; s < nseg;) {
+    const int q1 = s + 1 < nseg ? qs[(s + 1) * kSegT] : nq;
+    if (p.x < 0) {
+      if (q1 == q) {  // no outputs yet
+        ++s;
+        continue;
+      }
+      p = int4{s, 0, q, 0};
+      c = 0.0;
+    }
+    const double room = (target - c - 1.0) * kPartOuts;
+    const bool last = s + 1 == nseg;
+    if (q1 - q <= room || (c == 0.0 && q1 - q <= kPartOuts)) {  // the whole segment
+      c += 1.0 + (double)(q1 - q) / kPartOuts;
+      q = q1;
+      ++s;
+      if (!last && c < target) continue;
+      p.y = s;
+    } else if (room >= kPartOuts || c == 0.0) {  // as many of its outputs as fit
+      q += std::max(kPartOuts, (int)room);
+      p.y = s + 1;
+    } else {  // up to the segment before
+      p.y = s;
+    }
+    p.w = q;
+    if (p.w > p.z) parts.push_back(p);
+    p.x = -1;
+  }
+  return parts;
+}
+
 }  // namespace
 
 size_t interp_workspace_bytes(int M, int nk_in, int ntau, int nk_out) {
@@ -421,13 +482,11 @@ int launch_interp_sources(const double *k_in, int nk_in, const void *S_in, int M
     if (q == nq - 1)
       for (; jn < n + kSegPad; ++jn) qs[jn] = nq;
   }
-  // segments of intervals, and the parts of the k range: at least 16 segments a
-  // part (its sweep starts three segments early), and enough of them for ten
-  // blocks of 128 columns a resident place (five an SM)
-  const size_t nchunk = ((size_t)ntau + 127) / 128, nseg = ((size_t)n - 2) / kSegT + 1;
-  const size_t want = (152 * 50 + nchunk * M - 1) / (nchunk * M);
-  const size_t spp = std::max<size_t>(16, (nseg + want - 1) / want), nparts = (nseg + spp - 1) / spp;
-  const bool seg = dtype == GCAMB_F32 && nparts * nchunk <= 0x7fffffffULL && seg_halo_ok(h, cp, inv, n);
+  // segments of intervals, and the parts of the k range
+  const size_t nchunk = ((size_t)ntau + 127) / 128;
+  std::vector<int4> parts;
+  if (dtype == GCAMB_F32) parts = march_parts(qs, n, nq, nchunk * M);
+  const bool seg = dtype == GCAMB_F32 && parts.size() * nchunk <= 0x7fffffffULL && seg_halo_ok(h, cp, inv, n);
   if (dtype == GCAMB_F64) {
     std::copy(c64.begin(), c64.end(), reinterpret_cast<double *>(up.data() + L.coef));
     std::copy(q64.begin(), q64.end(), reinterpret_cast<OutCoef<double> *>(up.data() + L.q));
@@ -441,6 +500,8 @@ int launch_interp_sources(const double *k_in, int nk_in, const void *S_in, int M
     }
     OutCoef<float> *qc = reinterpret_cast<OutCoef<float> *>(up.data() + L.q);
     for (int q = 0; q < nq; ++q) qc[q] = {(float)q64[q].s, (float)q64[q].u, (float)q64[q].a, (float)q64[q].b};
+    // the parts (at most nq) behind the factors, whose region is sized for FP64's
+    if (seg) std::copy(parts.begin(), parts.end(), reinterpret_cast<int4 *>(qc + nq));
   }
   char *w = static_cast<char *>(ws);
   // a pageable copy returns once the host data is staged
@@ -453,10 +514,11 @@ int launch_interp_sources(const double *k_in, int nk_in, const void *S_in, int M
   else if (seg) {
     auto go = [&](auto v) {
       constexpr int V = decltype(v)::value;
-      spline_march_kernel<V><<<dim3((unsigned)(nparts * nchunk), (unsigned)M), 128 / V, kSegSmem, st>>>(
+      const auto *qc = reinterpret_cast<const OutCoef<float> *>(w + L.q);
+      spline_march_kernel<V><<<dim3((unsigned)(parts.size() * nchunk), (unsigned)M), 128 / V, kSegSmem, st>>>(
           static_cast<const float *>(S_in), reinterpret_cast<const SegCoef *>(w + L.coef) + kSegPad,
-          reinterpret_cast<const int *>(w + L.qs), reinterpret_cast<const OutCoef<float> *>(w + L.q), n, nq, ntau,
-          (int)nchunk, (int)nseg, (int)spp, static_cast<float *>(S_out));
+          reinterpret_cast<const int *>(w + L.qs), qc, reinterpret_cast<const int4 *>(qc + nq), n, nq, ntau, (int)nchunk,
+          static_cast<float *>(S_out));
     };
     if (ntau % 2 == 0 && (reinterpret_cast<uintptr_t>(S_in) | reinterpret_cast<uintptr_t>(S_out)) % 8 == 0)
       go(std::integral_constant<int, 2>());

@@ -125,3 +125,32 @@ def test_fp32_segments(nk_in, ntau, uneven):
     env = (np.abs(u * cols[..., j]) + np.abs(t * cols[..., j + 1]) +
            h * h / 6.0 * (np.abs(u ** 3 - u) * np.abs(Mo[..., j]) + np.abs(t ** 3 - t) * np.abs(Mo[..., j + 1])))
     assert np.all(np.abs(out - ref) <= 64 * 2.0 ** -24 * np.moveaxis(env, -1, 1) + 1e-30)
+
+
+@pytest.mark.parametrize("nk_in,nk,ntau,lo,hi", [
+    (40, 5000, 3, 1e-4, 0.3),      # segments of 1000 outputs, shared out by outputs
+    (200, 3000, 130, 0.1, 0.12),   # outputs in a few intervals: segments without any
+    (600, 2, 140, 0.15, 0.15001),  # fewer outputs than segments
+    (300, 700, 129, 0.299, 0.3),   # outputs in the last interval alone
+    (301, 1200, 300, 1e-4, 0.004)])
+def test_fp32_parts(nk_in, nk, ntau, lo, hi):
+    """FP32 grids whose nodes are anywhere among the sources' nodes: the march's
+    parts by work.  Bar: that of test_interp_matches_oracle."""
+    k = np.linspace(lo, hi, nk)
+    g = gcamb.grid_create(k, synth.uniform_grid(200.0, 14000.0, max(2, ntau)), 14000.0, 2, 10)
+    rng = np.random.default_rng(nk)
+    k_in = np.linspace(1e-4, 0.3, nk_in)
+    S32 = rng.normal(size=(2, nk_in, g.ntau)).astype(np.float32)
+    ref = ointerp.interp_sources(k_in, S32.astype(np.float64), g.k)
+    buf = torch.full((2, nk, g.ntau), float("nan"), dtype=torch.float32, device="cuda")
+    out = gcamb.interp_sources(g, k_in, torch.as_tensor(S32, device="cuda"), buf).cpu().numpy()
+    gcamb.sync()
+    cols = np.moveaxis(S32.astype(np.float64), 1, -1)
+    Mo = ointerp.natural_second_derivatives(k_in, cols)
+    j = np.clip(np.searchsorted(k_in, g.k, side="right") - 1, 0, nk_in - 2)
+    h = k_in[j + 1] - k_in[j]
+    t = (g.k - k_in[j]) / h
+    u = 1.0 - t
+    env = (np.abs(u * cols[..., j]) + np.abs(t * cols[..., j + 1]) +
+           h * h / 6.0 * (np.abs(u ** 3 - u) * np.abs(Mo[..., j]) + np.abs(t ** 3 - t) * np.abs(Mo[..., j + 1])))
+    assert np.all(np.abs(out - ref) <= 64 * 2.0 ** -24 * np.moveaxis(env, -1, 1) + 1e-30)
