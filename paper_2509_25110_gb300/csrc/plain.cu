@@ -695,6 +695,7 @@ __global__ void __launch_bounds__(256) cl_sum_kernel(const TD *__restrict__ DX, 
   __shared__ double part[kClParts][32];      // this CTA's parts (the first kClParts / cluster size rows)
   __shared__ double gsum[kClGroups][32];     // the first CTA of the cluster: every group's sum
   const int cs = gridDim.y, rank = blockIdx.y;  // cluster size (1, 2, 4, 8) and rank: the cluster spans grid y
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // all that earlier kernels wrote
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = blockIdx.x * 32 + lane;
   const size_t m = blockIdx.z;                            // source within DX
@@ -772,13 +773,16 @@ static cudaError_t launch_cl_sum(const gcamb_grid *g, const void *DX, const void
   cfg.gridDim = dim3(lb, cs, (unsigned)M);
   cfg.blockDim = dim3(256);
   cfg.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = 1;
-  at.val.clusterDim.y = cs;
-  at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = cs;
+  at[0].val.clusterDim.z = 1;
+  // behind the transfer functions' kernel: its launch is done as that one ends
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, cl_sum_kernel<TD, KIND>, static_cast<const TD *>(DX), static_cast<const TD *>(DY),
                             Pk, static_cast<const double *>(g->d_wk), g->nk, g->nl, Cl, px);
 }
