@@ -673,9 +673,9 @@ def run_tensor(args):
         gcamb.sync()
         kms, kn = gcamb.profile_read(gcamb.K_LOS_PLAIN)
         gcamb.profile_enable(False)
-        # four plain launches a step (D0, D1, D2 of S_P; the temperature), each
-        # 2 flop per stored (l, k, tau) table entry per model
-        flops = 4 * 2.0 * info["stored_plain64"] * M
+        # four sums a step (D0, D1, D2 of S_P; the temperature), each 2 flop per
+        # active (l, k, tau) entry per model (rows stop at their own prefix)
+        flops = 4 * 2.0 * info["active"] * M
         peak = gcamb.probe_flops(0 if mode == gcamb.PLAIN64 else 1)
         res[name] = {"models_per_s": M * steps / (ms * 1e-3), "ms_per_step": ms / steps,
                      "projection_ms": kms / steps, "achieved_tflops": flops / (kms / steps * 1e-3) / 1e12,
@@ -777,7 +777,7 @@ def run_tensor(args):
             "warmup": args.warmup, "ms_per_step": r64["ms_per_step"], "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": "tensor_lmax1500", "M": M, "lmax": wl.lmax, "nk": wl.nk, "ntau": wl.ntau,
-                       "stored_entries": info["stored_plain64"],
+                       "active_entries": info["active"],
                        "plain32": {k: v for k, v in res["plain32"].items() if k not in ("cls", "clocks")},
                        "batched_tt_ee_bb": batched,
                        "max_err_vs_oracle": err},

@@ -115,8 +115,8 @@ int gcamb_grid_weights(const gcamb_grid *g, double *wtau, double *wk);
 
 /*
  * Builds (or rebuilds) the grid's table of w_i j_l(k (tau0 - tau_i)) over the
- * active extents, in the layout of `mode`, by an FP64 recurrence on the
- * device (Miller's backward recurrence above x = k(tau0-tau), the forward
+ * active extents, in the layout of `mode`, by a recurrence in 64-bit
+ * integers on the device (Miller's backward recurrence above x = k(tau0-tau), the forward
  * recurrence at and below it).  This is the "calculation of the spherical
  * Bessel-function" inside the line-of-sight loop (Sec. 3.2), hoisted out of
  * it because the table is shared by all sources on the grid.
@@ -660,7 +660,7 @@ int gcamb_probe_flops(int what, double *flops);
  * paper; it documents what the batched path's chain records correct).  One
  * 128 x 128 tile
  *   C[i][n] = sum_{k < K} A[i][k] B[n][k]
- * through the library's tcgen05 GEMM (kind::f16): A[128][K], B[128][K]
+ * by tcgen05 MMAs (kind::f16): A[128][K], B[128][K]
  * device float, row-major, rounded to bf16 by the loaders; C[128][128]
  * device float.  1 <= K <= 2^20.  Asynchronous on `stream`; a device-side
  * timeout is reported by gcamb_sync.  Errors: GCAMB_EINVAL, GCAMB_ECUDA.
