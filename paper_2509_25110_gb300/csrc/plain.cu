@@ -779,10 +779,14 @@ static cudaError_t launch_cl_sum(const gcamb_grid *g, const void *DX, const void
   at[0].val.clusterDim.y = cs;
   at[0].val.clusterDim.z = 1;
   // behind the transfer functions' kernel: its launch is done as that one ends
+  // (not in a caller's capture, where what precedes need not be a kernel)
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool plain_stream = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (!plain_stream) cudaGetLastError();
   cfg.attrs = at;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = plain_stream ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, cl_sum_kernel<TD, KIND>, static_cast<const TD *>(DX), static_cast<const TD *>(DY),
                             Pk, static_cast<const double *>(g->d_wk), g->nk, g->nl, Cl, px);
 }
