@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256) spline_eval_kernel(const T *__restrict__ 
 // and the outputs' factors likewise (read from global memory where they are
 // used, they missed the little L1 the rings leave: 2850 us).  The sweep over whole columns that this
 // replaces wrote and read the second derivatives and was one serial chain of
-// loads a column: 1099 us and 1585 us for the evaluation, now 1532 us (DRAM at
+// loads a column: 1099 us and 1585 us for the evaluation, now 1488 us (DRAM at
 // 80% of its peak cycles).  (Segments
 // solved by themselves, with both neighbourhoods loaded and swept for each:
 // 1927 us at best.)
@@ -399,8 +399,8 @@ bool seg_halo_ok(const double *h, const double *cp, const double *inv, int n) {
 // is dense) is shared out by outputs; segments without any are left out where
 // a part can start behind them.  Kernel time, parts of at least 16 whole
 // segments -> these (nodes -> grid, tau, sources): 200 -> 8000, 300, 8: 582 ->
-// 50 us; 395 -> 6075, 498, 15: 267 -> 67; 200 -> 1000, 300, 8: 59 -> 16; 518 -> 4312, 499,
-// 155: 439 -> 432; 1000 -> 8000, 1000, 256: 1509 -> 1532 (the bounds of a part's outputs).
+// 50 us; 395 -> 6075, 498, 15: 267 -> 67; 200 -> 1000, 300, 8: 59 -> 16;
+// 518 -> 4312, 499, 155: 439 -> 415; 1000 -> 8000, 1000, 256: 1509 -> 1488.
 constexpr int kPartOuts = 64, kPartMin = 4;
 
 std::vector<int4> march_parts(const int *qs, int n, int nq, size_t blocks) {
@@ -420,10 +420,11 @@ std::vector<int4> march_parts(const int *qs, int n, int nq, size_t blocks) {
       p = int4{s, 0, q, 0};
       c = 0.0;
     }
-    const double room = (target - c - 1.0) * kPartOuts;
+    const double room = (target - c - 1.0) * kPartOuts, segc = 1.0 + (double)(q1 - q) / kPartOuts;
     const bool last = s + 1 == nseg;
-    if (q1 - q <= room || (c == 0.0 && q1 - q <= kPartOuts)) {  // the whole segment
-      c += 1.0 + (double)(q1 - q) / kPartOuts;
+    // the whole segment (a small one is not split)
+    if (q1 - q <= room || 4.0 * segc <= target || (c == 0.0 && q1 - q <= kPartOuts)) {
+      c += segc;
       q = q1;
       ++s;
       if (!last && c < target) continue;
