@@ -32,7 +32,7 @@
 // without a copy in flight beside the MMAs.  Measured, batch 4096, width 512,
 // n_out 2499: forward 412 -> 47 us, input gradients 554 -> 44 us, weight
 // gradients 350 -> 28 us, a whole training step 1600 -> 150 us, bit for bit the
-// same parameters; 4096 served spectra 907 -> 109 us.
+// same parameters; 4096 served spectra 907 -> 107 us.
 //
 // Every wait is bounded; a timeout sets the error word and the CTA drains its
 // copies and MMAs and frees its TMEM.
@@ -126,7 +126,7 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
 // the last place over the range (3.9e6 arguments against 113-bit arithmetic).
 // A 64-bit high product for each of y log2(e), two table factors, the rest and
 // the last product made 118 instructions of an exp (and 2.0 units): the served
-// layer 74 us, now 58.
+// layer 74 us, now 52.
 constexpr int kExpTab = 4096;                                 // 2^(j / 4096), Q2.62
 constexpr unsigned long long kExpLn2 = 0x58B90BFBE8E7BCD6ull;  // ln 2 / 4096 in Q.75 = 1024 ln 2 in Q.53
 constexpr unsigned int kExpLo = 41502639u, kExpSpan = 2893859389u;  // y + 1024 ln 2 in Q.21: 19.79, + 1379.9
@@ -198,13 +198,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // tiles blockIdx.x, + gridDim.x, .. (PS; else one)
   const int ntiles = a.p[NP > 1 ? a.np - 1 : 0].tile_end;
+  // The exp layer's last, partial round: a tile's rows (of each warp's 32) shared
+  // out over up to four CTAs, which all compute the tile, cheap beside its exps
+  // (640 tiles on 152 CTAs are 4.2 rounds: 58 -> 52 us).
+  constexpr bool kShare = PS && EPI == kExp;
+  const int full = kShare ? ntiles / (int)gridDim.x * (int)gridDim.x : ntiles, rest = ntiles - full;
+  const int share = rest * 4 <= (int)gridDim.x ? 4 : (rest * 2 <= (int)gridDim.x ? 2 : 1);
+  const int nunits = full + rest * share;
   struct Tile {
     const Prob *p;
     int tile, i0, n0, nkc, per, nsl;  // per: chunks per accumulation, nsl: accumulations
+    int ra, rb;                       // rows [ra, rb) of a warp's 32
   };
   auto get_tile = [&](int t) {
     Tile r;
     int pi = 0;
+    r.ra = 0;
+    r.rb = 32;
+    if (kShare && t >= full) {
+      const int u = t - full;
+      r.ra = 32 / share * (u % share);
+      r.rb = r.ra + 32 / share;
+      t = full + u / share;
+    }
     if constexpr (NP > 1)
       while (pi + 1 < a.np && t >= a.p[pi].tile_end) ++pi;
     r.p = &a.p[pi];
@@ -252,7 +268,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
 #pragma unroll
       for (int s = 0; s < kStagesG; ++s) last[s] = -1;
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      for (int t = blockIdx.x; t < nunits && ok; t += gridDim.x) {
         const Tile tl = get_tile(t);
         const CUtensorMap *ta = &tl.p->ta, *tb = &tl.p->tb;
         for (int kc = 0; kc < tl.nkc; ++kc) {
@@ -294,7 +310,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       int stage = 0, un = 0;  // un: accumulations so far, in buffers 0, 1, 0, ..
       uint32_t ph = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      for (int t = blockIdx.x; t < nunits && ok; t += gridDim.x) {
         const Tile tl = get_tile(t);
         int first = 0;
         for (int kc = 0; kc < tl.nkc; ++kc) {
@@ -346,7 +362,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     const int c2 = 2 * (lane & 15), rp = lane >> 4;  // two adjacent columns of rows rp, rp + 2, ..
     int un = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    for (int t = blockIdx.x; t < nunits; t += gridDim.x) {
       const Tile tl = get_tile(t);
       const Prob &p = *tl.p;
       const int ib = tl.i0 + sp * 32, nr = min(32, p.M - ib), nb = tl.n0 + cq * 32;
@@ -483,7 +499,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         *reinterpret_cast<long long *>(st + lane * kPitch + 32) = fix53(xa) - fix53(xm);
         __syncwarp();
         constexpr int RU = 8;  // rows whose chains interleave
-        for (int r0 = 0; r0 < nr; r0 += RU) {
+        for (int r0 = tl.ra; r0 < min(nr, tl.rb); r0 += RU) {
           double c[RU];
           bool bad = badt;
 #pragma unroll
