@@ -323,7 +323,11 @@ size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 // output node's factors [nq][4], its interval [nq] (int), the intervals' first
 // outputs [n] (int): sized for FP64; the second derivatives [M][n][ntau] in the
 // arithmetic's precision (sized for FP64).  One upload fills the regions
-// before the derivatives.
+// before the derivatives.  The kernels read the regions by 16- and 32-byte
+// loads, a workspace may have any alignment: the regions start at its first
+// multiple of kInterpAlign, within the kInterpAlign bytes of slack in total.
+constexpr size_t kInterpAlign = 256;
+
 struct InterpLayout {
   size_t coef, q, qj, qs, md, total;
   InterpLayout(int M, int n, int ntau, int nq) {
@@ -332,8 +336,13 @@ struct InterpLayout {
     qj = q + a256((size_t)nq * 4 * sizeof(double));
     qs = qj + a256((size_t)nq * sizeof(int));
     md = qs + a256(((size_t)n + kSegPad) * sizeof(int));
-    total = md + a256((size_t)M * n * ntau * sizeof(double));
+    total = md + a256((size_t)M * n * ntau * sizeof(double)) + kInterpAlign;
   }
+};
+
+// The regions up to the derivatives on the host, aligned as on the device.
+struct alignas(kInterpAlign) HostBlock {
+  char b[kInterpAlign];
 };
 
 template <typename T>
@@ -352,9 +361,9 @@ void launch_interp_columns(const InterpLayout &L, char *w, int n, int nq, int nt
         S_in, Md, reinterpret_cast<const int *>(w + L.qj), reinterpret_cast<const OutCoef<T> *>(w + L.q), n, nq, ntau,
         ntc, S_out);
   };
-  // FP32: four columns a thread in 16-byte loads and stores where the rows are aligned
+  // FP32: four columns a thread in 16-byte loads and stores where the rows are aligned (Md's are)
   if (sizeof(T) == 4 && ntau % 4 == 0 &&
-      (reinterpret_cast<uintptr_t>(S_in) | reinterpret_cast<uintptr_t>(S_out) | reinterpret_cast<uintptr_t>(Md)) % 16 == 0)
+      (reinterpret_cast<uintptr_t>(S_in) | reinterpret_cast<uintptr_t>(S_out)) % 16 == 0)
     eval(std::integral_constant<int, sizeof(T) == 4 ? 4 : 1>());
   else
     eval(std::integral_constant<int, 1>());
@@ -458,8 +467,9 @@ int launch_interp_sources(const double *k_in, int nk_in, const void *S_in, int M
   // elimination coefficients (nodes only) and each output node's interval
   std::vector<double> c64(4 * (size_t)n, 0.0);
   std::vector<OutCoef<double>> q64(nq);
-  std::vector<char> up(L.md);
-  int *qj = reinterpret_cast<int *>(up.data() + L.qj), *qs = reinterpret_cast<int *>(up.data() + L.qs);
+  std::vector<HostBlock> blocks(L.md / kInterpAlign);  // zeros
+  char *up = reinterpret_cast<char *>(blocks.data());
+  int *qj = reinterpret_cast<int *>(up + L.qj), *qs = reinterpret_cast<int *>(up + L.qs);
   double *h = c64.data(), *ih = h + n, *cp = ih + n, *inv = cp + n;
   for (int j = 0; j + 1 < n; ++j) {
     h[j] = k_in[j + 1] - k_in[j];
@@ -489,24 +499,24 @@ int launch_interp_sources(const double *k_in, int nk_in, const void *S_in, int M
   if (dtype == GCAMB_F32) parts = march_parts(qs, n, nq, nchunk * M);
   const bool seg = dtype == GCAMB_F32 && parts.size() * nchunk <= 0x7fffffffULL && seg_halo_ok(h, cp, inv, n);
   if (dtype == GCAMB_F64) {
-    std::copy(c64.begin(), c64.end(), reinterpret_cast<double *>(up.data() + L.coef));
-    std::copy(q64.begin(), q64.end(), reinterpret_cast<OutCoef<double> *>(up.data() + L.q));
+    std::copy(c64.begin(), c64.end(), reinterpret_cast<double *>(up + L.coef));
+    std::copy(q64.begin(), q64.end(), reinterpret_cast<OutCoef<double> *>(up + L.q));
   } else {
     if (seg) {
-      SegCoef *sc = reinterpret_cast<SegCoef *>(up.data() + L.coef) + kSegPad;  // zeros around
+      SegCoef *sc = reinterpret_cast<SegCoef *>(up + L.coef) + kSegPad;  // zeros around
       for (int j = 0; j < n; ++j)
         sc[j] = SegCoef{(float)ih[j], j > 0 ? (float)h[j - 1] : 0.f, (float)inv[j], (float)cp[j]};
     } else {
-      std::copy(c64.begin(), c64.end(), reinterpret_cast<float *>(up.data() + L.coef));
+      std::copy(c64.begin(), c64.end(), reinterpret_cast<float *>(up + L.coef));
     }
-    OutCoef<float> *qc = reinterpret_cast<OutCoef<float> *>(up.data() + L.q);
+    OutCoef<float> *qc = reinterpret_cast<OutCoef<float> *>(up + L.q);
     for (int q = 0; q < nq; ++q) qc[q] = {(float)q64[q].s, (float)q64[q].u, (float)q64[q].a, (float)q64[q].b};
     // the parts (at most nq) behind the factors, whose region is sized for FP64's
     if (seg) std::copy(parts.begin(), parts.end(), reinterpret_cast<int4 *>(qc + nq));
   }
-  char *w = static_cast<char *>(ws);
+  char *w = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(ws) + kInterpAlign - 1) & ~(uintptr_t)(kInterpAlign - 1));
   // a pageable copy returns once the host data is staged
-  cudaError_t e = cudaMemcpyAsync(w, up.data(), L.md, cudaMemcpyHostToDevice, st);
+  cudaError_t e = cudaMemcpyAsync(w, up, L.md, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(e, "interp_sources: coefficient upload");
   ProfScope prof(GCAMB_K_INTERP, st);
   if (dtype == GCAMB_F64)

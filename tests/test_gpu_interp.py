@@ -12,6 +12,8 @@ ulp on these grids).  The second-derivative terms can exceed |y| many times
 on uneven nodes, so the bar is not a multiple of the largest |S|.  The
 interpolated sources fed to the batched projection: within 1e-5 of the
 oracle's projection of its own interpolated sources."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -154,3 +156,26 @@ def test_fp32_parts(nk_in, nk, ntau, lo, hi):
     env = (np.abs(u * cols[..., j]) + np.abs(t * cols[..., j + 1]) +
            h * h / 6.0 * (np.abs(u ** 3 - u) * np.abs(Mo[..., j]) + np.abs(t ** 3 - t) * np.abs(Mo[..., j + 1])))
     assert np.all(np.abs(out - ref) <= 64 * 2.0 ** -24 * np.moveaxis(env, -1, 1) + 1e-30)
+
+
+@pytest.mark.parametrize("dtype,nodes,shift", [
+    (torch.float64, "log", 8), (torch.float64, "log", 248), (torch.float32, "even", 4), (torch.float32, "even", 8),
+    (torch.float32, "log", 4), (torch.float32, "log", 8)])
+def test_workspace_of_any_alignment(dtype, nodes, shift):
+    """A slice of a larger buffer as workspace, at the alignment of its
+    scalars: the same bits as an aligned one, and nothing beside the slice is
+    written.  FP32 on even nodes marches, on 30 log-spaced ones it takes the
+    whole-column path."""
+    g = grid()
+    k_in = np.geomspace(1e-4, 0.3, 30) if nodes == "log" else np.linspace(1e-4, 0.3, 100)
+    k_in[0], k_in[-1] = 1e-4, 0.3
+    S = torch.as_tensor(np.random.default_rng(3).normal(size=(2, k_in.size, g.ntau)), dtype=dtype, device="cuda")
+    ref = gcamb.interp_sources(g, k_in, S)
+    b = ctypes.c_size_t()
+    assert gcamb.lib().gcamb_interp_sources_workspace(g.handle, 2, k_in.size, ctypes.byref(b)) == 0
+    buf = torch.full((b.value + 512,), 0x5a, dtype=torch.uint8, device="cuda")
+    out = gcamb.interp_sources(g, k_in, S, ws=buf[shift:shift + b.value])
+    gcamb.sync()
+    assert buf.data_ptr() % 256 == 0
+    assert torch.equal(out, ref)
+    assert (buf[:shift] == 0x5a).all() and (buf[shift + b.value:] == 0x5a).all()
