@@ -695,6 +695,9 @@ __global__ void __launch_bounds__(256) cl_sum_kernel(const TD *__restrict__ DX, 
   __shared__ double part[kClParts][32];      // this CTA's parts (the first kClParts / cluster size rows)
   __shared__ double gsum[kClGroups][32];     // the first CTA of the cluster: every group's sum
   const int cs = gridDim.y, rank = blockIdx.y;  // cluster size (1, 2, 4, 8) and rank: the cluster spans grid y
+  // the first CTA's shared memory is written below: every CTA tells that it runs,
+  // the wait for all of them stands before the write, behind the sums
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");  // all that earlier kernels wrote
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = blockIdx.x * 32 + lane;
@@ -740,6 +743,7 @@ __global__ void __launch_bounds__(256) cl_sum_kernel(const TD *__restrict__ DX, 
     part[lp][lane] = acc;
   }
   __syncthreads();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   const int ng = kClGroups / cs;  // groups of this CTA
   if (warp < ng) {
     double s = part[warp * 8][lane];

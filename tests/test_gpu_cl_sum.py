@@ -43,3 +43,24 @@ def test_cl_matches_numpy(nk, nl, M, dtype):
     # the order of the additions does not depend on the batch
     assert np.array_equal(gcamb.cl(g, X[:1].contiguous(), P[:1].contiguous()).cpu().numpy(), C[:1])
     gcamb.sync()
+
+
+@pytest.mark.parametrize("nk", [1, 2, 7, 8, 9, 40, 63])
+def test_cl_of_few_k(nk):
+    """Fewer k than parts: most CTAs of a cluster have nothing to sum and reach
+    the write into the first one's shared memory at once.  Launched back to
+    back, each result against the numpy sum (bound as above) and against one
+    another."""
+    k = synth.log_grid(1e-4, 0.3, nk) if nk > 1 else np.array([0.01])
+    nl = 777
+    g = gcamb.grid_create(k, synth.uniform_grid(200.0, 14000.0, 8), 14000.0, 2, nl + 1)
+    rng = np.random.default_rng(nk)
+    X = rng.standard_normal((1, nk, nl))
+    P = rng.uniform(0.5, 2.0, (1, nk))
+    d, p = torch.as_tensor(X, device="cuda"), torch.as_tensor(P, device="cuda")
+    out = [gcamb.cl(g, d, p) for _ in range(50)]
+    gcamb.sync()
+    _, wk = gcamb.grid_weights(g)
+    ref = 4.0 * np.pi * (wk[None, :, None] * P[:, :, None] * X * X).sum(1)
+    assert (np.abs(out[0].cpu().numpy() - ref) <= 2.0 * (nk + 3) * 2.0 ** -53 * ref).all()
+    assert all(torch.equal(o, out[0]) for o in out)
