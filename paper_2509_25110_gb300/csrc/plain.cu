@@ -76,8 +76,18 @@ constexpr int plain_unroll() { return sizeof(T) == 8 ? 1 : 2; }
 template <typename T>
 constexpr int plain_ahead() { return sizeof(T) == 8 ? 0 : 4; }
 
-// Tau blocks staged in shared memory at a time (64 KB of sources).
-constexpr int plain_stage_blocks(int nv, size_t esize) { return (int)(65536 / (nv * esize * kPlainKB)); }
+// A row's sum is taken in groups of 32 blocks (2048 nodes), each reduced over
+// the lanes and added to those before it.  The group is the same for every
+// number of sources, so that a source's result does not depend on the batch it
+// came in (a staged chunk holds 128 blocks of one FP64 source, 32 of four).
+constexpr int kPlainGroup = 32;
+
+// Tau blocks staged in shared memory at a time: whole groups, up to 64 KB of
+// sources.  (Staging every group by itself: one FP64 source, 8000 tau 2546 ->
+// 3169 us.)
+constexpr int plain_stage_blocks(int nv, size_t esize) {
+  return (int)(65536 / (nv * esize * kPlainKB)) / kPlainGroup * kPlainGroup;
+}
 
 // x^-1 and x^-2 of one node as sums of two floats (about 2^-45 relative), from
 // x = k dt with k and dt as sums of two floats, in FP32 operations: GB300's
@@ -316,99 +326,104 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
       }
     }
     __syncthreads();
-    // ---- rows
-    for (int rb = rw * 4 * RV; rb < R; rb += WR * 4 * RV) {
-      int ns[RV];  // steps of this chunk that rows rb + 4 i .. + 3 need
-      const int nsc = nbc * STEPS;
-      int nmin = nsc, nmax = 0;
+    // ---- rows, a group of blocks at a time
+#pragma unroll 1
+    for (int gb = 0; gb < nbc; gb += kPlainGroup) {
+      const int b1 = b0 + gb, ng = min(kPlainGroup, nbc - gb);
+      const T *sg = s + gb * KB;
+      for (int rb = rw * 4 * RV; rb < R; rb += WR * 4 * RV) {
+        int ns[RV];  // steps of this group that rows rb + 4 i .. + 3 need
+        const int nsc = ng * STEPS;
+        int nmin = nsc, nmax = 0;
 #pragma unroll
-      for (int i = 0; i < RV; ++i) {
-        const int row = row0 + rb + 4 * i;
-        ns[i] = 0;
-        if (row < a.nl) {
-          ns[i] = nsc;
-          if (a.xthr) {
-            const double xe = a.xthr[row];
-            if (FIELD == kFieldT || xe >= 1.0) {
-              const long long xi = __double_as_longlong(xe);
-              int n = 0;
-              for (int c = 0; c < nsc; c += 32)
-                n += __popc(__ballot_sync(0xffffffffu, c + lane < nsc && xb[b0 * STEPS + c + lane] >= xi));
-              ns[i] = n;
-            }
-          }
-        }
-        nmax = max(nmax, ns[i]);
-        nmin = min(nmin, ns[i]);
-      }
-      T acc[NV][RV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int i = 0; i < RV; ++i) acc[v][i] = T(0);
-      const T *rows = chunk + (size_t)b0 * kTileL * KB + (rsub + rb + grp) * KB + sub * VE;
-      // a lane's row of the pass (4 RV rows) for the lines ahead
-      constexpr int AHEAD = plain_ahead<T>();
-      const T *arow = chunk + (size_t)b0 * kTileL * KB + (rsub + rb + lane) * KB;
-      int an = 0;  // its steps
-      if constexpr (AHEAD > 0) {
-#pragma unroll
-        for (int i = 0; i < RV; ++i) an = (lane >> 2) == i ? ns[i] : an;
-      }
-      // steps that all RV row sets need, then the rest (a set's bound is
-      // uniform over the warp); UN steps' loads are in flight together
-      auto step = [&](int i0, auto un, auto check) {
-        constexpr int UN = decltype(un)::value;
-        V16 j[UN][RV];
-#pragma unroll
-        for (int u = 0; u < UN; ++u) {
-          const int st = i0 + u * TS;
-          const T *blk = rows + (size_t)(st / STEPS) * (kTileL * KB) + (st % STEPS) * SN;
-#pragma unroll
-          for (int i = 0; i < RV; ++i)
-            if (!check || st < ns[i]) j[u][i] = __ldg(reinterpret_cast<const V16 *>(blk + 4 * i * KB));
-        }
-#pragma unroll
-        for (int u = 0; u < UN; ++u) {
-          const int st = i0 + u * TS;
-#pragma unroll
-          for (int v = 0; v < NV; ++v) {
-            const V16 sv = *reinterpret_cast<const V16 *>(s + v * stride + st * SN + sub * VE);
-#pragma unroll
-            for (int i = 0; i < RV; ++i) {
-              if (check && st >= ns[i]) continue;
-              const V16 t = j[u][i];
-              if constexpr (sizeof(T) == 8) {
-                acc[v][i] = fma(t.y, sv.y, fma(t.x, sv.x, acc[v][i]));
-              } else {
-                const float d = __fmaf_rn(t.w, sv.w, __fmaf_rn(t.z, sv.z, __fmaf_rn(t.y, sv.y, __fmul_rn(t.x, sv.x))));
-                acc[v][i] = __fadd_rn(acc[v][i], d);
+        for (int i = 0; i < RV; ++i) {
+          const int row = row0 + rb + 4 * i;
+          ns[i] = 0;
+          if (row < a.nl) {
+            ns[i] = nsc;
+            if (a.xthr) {
+              const double xe = a.xthr[row];
+              if (FIELD == kFieldT || xe >= 1.0) {
+                const long long xi = __double_as_longlong(xe);
+                int n = 0;
+                for (int c = 0; c < nsc; c += 32)
+                  n += __popc(__ballot_sync(0xffffffffu, c + lane < nsc && xb[b1 * STEPS + c + lane] >= xi));
+                ns[i] = n;
               }
             }
           }
+          nmax = max(nmax, ns[i]);
+          nmin = min(nmin, ns[i]);
         }
-      };
-      constexpr int UN = plain_unroll<T>();
-      int st = ts;
-      for (; st + (UN - 1) * TS < nmin; st += UN * TS) {
+        T acc[NV][RV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int i = 0; i < RV; ++i) acc[v][i] = T(0);
+        const T *rows = chunk + (size_t)b1 * kTileL * KB + (rsub + rb + grp) * KB + sub * VE;
+        // a lane's row of the pass (4 RV rows) for the lines ahead
+        constexpr int AHEAD = plain_ahead<T>();
+        const T *arow = chunk + (size_t)b1 * kTileL * KB + (rsub + rb + lane) * KB;
+        int an = 0;  // its steps
         if constexpr (AHEAD > 0) {
 #pragma unroll
-          for (int u = 0; u < UN; ++u) {
-            const int sa = st + (AHEAD + u) * TS;
-            if (sa < an)
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(arow + (size_t)(sa / STEPS) * (kTileL * KB) + (sa % STEPS) * SN));
-          }
+          for (int i = 0; i < RV; ++i) an = (lane >> 2) == i ? ns[i] : an;
         }
-        step(st, std::integral_constant<int, UN>(), std::false_type());
-      }
-      for (; st < nmax; st += TS) step(st, std::integral_constant<int, 1>(), std::true_type());
+        // steps that all RV row sets need, then the rest (a set's bound is
+        // uniform over the warp); UN steps' loads are in flight together
+        auto step = [&](int i0, auto un, auto check) {
+          constexpr int UN = decltype(un)::value;
+          V16 j[UN][RV];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const T t = reduce_group<T, RV>(acc[v], lane);
-        constexpr int LPV = 8 / RV;  // lanes that end with the same value
-        if (sub % LPV == 0) {
-          T *r = res + (ts * NV + v) * R + rb + grp + 4 * (sub / LPV);
-          *r = b0 ? *r + t : t;
+          for (int u = 0; u < UN; ++u) {
+            const int st = i0 + u * TS;
+            const T *blk = rows + (size_t)(st / STEPS) * (kTileL * KB) + (st % STEPS) * SN;
+#pragma unroll
+            for (int i = 0; i < RV; ++i)
+              if (!check || st < ns[i]) j[u][i] = __ldg(reinterpret_cast<const V16 *>(blk + 4 * i * KB));
+          }
+#pragma unroll
+          for (int u = 0; u < UN; ++u) {
+            const int st = i0 + u * TS;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+              const V16 sv = *reinterpret_cast<const V16 *>(sg + v * stride + st * SN + sub * VE);
+#pragma unroll
+              for (int i = 0; i < RV; ++i) {
+                if (check && st >= ns[i]) continue;
+                const V16 t = j[u][i];
+                if constexpr (sizeof(T) == 8) {
+                  acc[v][i] = fma(t.y, sv.y, fma(t.x, sv.x, acc[v][i]));
+                } else {
+                  const float d = __fmaf_rn(t.w, sv.w, __fmaf_rn(t.z, sv.z, __fmaf_rn(t.y, sv.y, __fmul_rn(t.x, sv.x))));
+                  acc[v][i] = __fadd_rn(acc[v][i], d);
+                }
+              }
+            }
+          }
+        };
+        constexpr int UN = plain_unroll<T>();
+        int st = ts;
+        for (; st + (UN - 1) * TS < nmin; st += UN * TS) {
+          if constexpr (AHEAD > 0) {
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+              const int sa = st + (AHEAD + u) * TS;
+              if (sa < an)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(arow + (size_t)(sa / STEPS) * (kTileL * KB) + (sa % STEPS) * SN));
+            }
+          }
+          step(st, std::integral_constant<int, UN>(), std::false_type());
+        }
+        for (; st < nmax; st += TS) step(st, std::integral_constant<int, 1>(), std::true_type());
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const T t = reduce_group<T, RV>(acc[v], lane);
+          constexpr int LPV = 8 / RV;  // lanes that end with the same value
+          if (sub % LPV == 0) {
+            T *r = res + (ts * NV + v) * R + rb + grp + 4 * (sub / LPV);
+            *r = b1 ? *r + t : t;
+          }
         }
       }
     }
@@ -419,21 +434,23 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
         const int pr = row0 - 1, plt = pr / kTileL;
         const T *prow = table + (size_t)a.off[(size_t)q * a.nlt + plt] * (kTileL * KB) + (size_t)b0 * kTileL * KB +
                         (pr - plt * kTileL) * KB;
-        T h[NV];
+        for (int g0 = 0; g0 < nt; g0 += kPlainGroup * KB) {
+          T h[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) h[v] = T(0);
-        for (int t = lane; t < nt; t += 32) {
-          const T j = __ldg(prow + (size_t)(t / KB) * kTileL * KB + t % KB);
+          for (int v = 0; v < NV; ++v) h[v] = T(0);
+          for (int t = g0 + lane; t < min(nt, g0 + kPlainGroup * KB); t += 32) {
+            const T j = __ldg(prow + (size_t)(t / KB) * kTileL * KB + t % KB);
 #pragma unroll
-          for (int v = 0; v < NV; ++v)
-            if (v % 4 != 3) h[v] = fma(j, s[v * stride + t], h[v]);
-        }
+            for (int v = 0; v < NV; ++v)
+              if (v % 4 != 3) h[v] = fma(j, s[v * stride + t], h[v]);
+          }
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          if (v % 4 == 3) continue;
+          for (int v = 0; v < NV; ++v) {
+            if (v % 4 == 3) continue;
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) h[v] += __shfl_xor_sync(0xffffffffu, h[v], o);
-          if (lane == 0) halo[v] += h[v];
+            for (int o = 16; o > 0; o >>= 1) h[v] += __shfl_xor_sync(0xffffffffu, h[v], o);
+            if (lane == 0) halo[v] += h[v];
+          }
         }
       }
     }

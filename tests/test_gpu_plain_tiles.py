@@ -86,3 +86,24 @@ def test_fp32_fields(orc, nk, ntau, lmax, M):
         err = np.abs(a.cpu().numpy() - r)
         left_out = 1e-30 * pre * (np.abs(s) * w).sum(2)[:, :, None]
         assert (err <= tol * A + left_out).all(), np.max(err / (tol * A + left_out + 1e-300))
+
+
+@pytest.mark.parametrize("mode,M,ntau", [(m, M, n) for m, Ms in ((gcamb.PLAIN64, (2, 3, 4, 7)), (gcamb.PLAIN32, (2, 3, 5, 8, 13)))
+                                         for M in Ms for n in (2048, 2113, 4200)])
+def test_long_tau_grids_of_a_batch(mode, M, ntau):
+    """A source's sums are the same bits alone and in a batch, also where its
+    prefix is longer than the chunk of a batch that is staged at a time:
+    temperature, E-mode and tensor fields."""
+    k, tau, S, g = make(4, ntau, 150, M, seed=M + ntau)
+    gcamb.bessel_table(g, mode)
+    d = [torch.as_tensor(s, dtype=torch.float64 if mode == gcamb.PLAIN64 else torch.float32, device="cuda") for s in S]
+
+    def calls(a, b):
+        return [gcamb.los_transfer(g, a, mode), gcamb.los_transfer_e(g, b, mode), *gcamb.los_transfer_tensor(g, a, b, mode)]
+
+    batch = calls(*d)
+    for m in (0, M - 1):
+        one = calls(*(s[m:m + 1].contiguous() for s in d))
+        gcamb.sync()
+        for a, b in zip(one, batch):
+            assert torch.equal(a[0], b[m])
