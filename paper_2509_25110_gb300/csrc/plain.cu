@@ -22,17 +22,68 @@ __device__ __forceinline__ void halve_lanes(T (&v)[V], int lane, int o) {
   }
 }
 
+// FP32 sums over lanes and what follows them are carried as the sum of two
+// floats: their additions are those of the largest numbers (E-mode of 5 sources
+// to l 2001, error against 64 bits 3.7e-8, 5.0e-8 with plain floats, at 278 and
+// 275 us).
+__device__ __forceinline__ float2 add_ff(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x), t = __fsub_rn(s, a.x);
+  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, t)), __fsub_rn(b.x, t));
+  return make_float2(s, __fadd_rn(e, __fadd_rn(a.y, b.y)));
+}
+__device__ __forceinline__ double add_ff(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 shfl_ff(float2 v, int o) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ double shfl_ff(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+// (where the first float is infinite or NaN the second holds nothing)
+__device__ __forceinline__ float round_ff(float2 s) { return fabsf(s.x) <= 3.402823466e38f ? __fadd_rn(s.x, s.y) : s.x; }
+__device__ __forceinline__ double round_ff(double s) { return s; }
+__device__ __forceinline__ double wide(float2 s) {
+  return fabsf(s.x) <= 3.402823466e38f ? (double)s.x + (double)s.y : (double)s.x;
+}
+__device__ __forceinline__ double wide(double s) { return s; }
+__device__ __forceinline__ float2 as_ff(float v) { return make_float2(v, 0.f); }
+__device__ __forceinline__ double as_ff(double v) { return v; }
+template <typename T>
+using PlainSum = std::conditional_t<sizeof(T) == 8, double, float2>;
+
+// halve_lanes on such sums.
+template <int N, int V>
+__device__ __forceinline__ void halve_lanes(float2 (&v)[V], int lane, int o) {
+  const bool up = (lane & o) != 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const float2 send = up ? v[j] : v[j + N], keep = up ? v[j + N] : v[j];
+    v[j] = add_ff(keep, shfl_ff(send, o));
+  }
+}
+
 // Sum over the 8 lanes of a group of each of the RV values a lane holds
 // (RV = 4, 8); lane L of the group returns the total of value L / (8 / RV).
 // The additions of one value are the same for both RV (partners 4, 2, 1).
 template <typename T, int RV>
-__device__ __forceinline__ T reduce_group(T (&v)[RV], int lane) {
+__device__ __forceinline__ PlainSum<T> reduce_group(T (&v)[RV], int lane) {
   static_assert(RV == 4 || RV == 8, "reduce_group: RV in {4, 8}");
-  halve_lanes<T, RV / 2>(v, lane, 4);
-  halve_lanes<T, RV / 4>(v, lane, 2);
-  if constexpr (RV == 8) halve_lanes<T, 1>(v, lane, 1);
-  else v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-  return v[0];
+  if constexpr (sizeof(T) == 8) {
+    halve_lanes<T, RV / 2>(v, lane, 4);
+    halve_lanes<T, RV / 4>(v, lane, 2);
+    if constexpr (RV == 8) halve_lanes<T, 1>(v, lane, 1);
+    else v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+  } else {
+    float2 w[RV / 2];
+    const bool up = (lane & 4) != 0;
+#pragma unroll
+    for (int j = 0; j < RV / 2; ++j) {
+      const T send = up ? v[j] : v[j + RV / 2], keep = up ? v[j + RV / 2] : v[j];
+      w[j] = add_ff(as_ff(keep), as_ff(__shfl_xor_sync(0xffffffffu, send, 4)));
+    }
+    halve_lanes<RV / 4>(w, lane, 2);
+    if constexpr (RV == 8) halve_lanes<1>(w, lane, 1);
+    else w[0] = add_ff(w[0], shfl_ff(w[0], 1));
+    return w[0];
+  }
 }
 
 // What is summed against the table's w_i j_l:
@@ -114,6 +165,13 @@ __device__ __forceinline__ float mul_ff(float v, float2 f) {
   return fabsf(p) <= 3.4e38f ? __fadd_rn(p, e) : p;  // overflow, infinities, NaN: the plain product
 }
 
+// (v.x + v.y) (f.x + f.y), the same way.
+__device__ __forceinline__ float mul_ff(float2 v, float2 f) {
+  const float p = __fmul_rn(v.x, f.x);
+  const float e = __fmaf_rn(v.y, f.x, __fmaf_rn(v.x, f.y, __fmaf_rn(v.x, f.x, -p)));
+  return fabsf(p) <= 3.4e38f ? __fadd_rn(p, e) : p;
+}
+
 // The power series of the tensor kernels at small x for the nodes
 // below the cut, from j_l(x) = x^l s_l(x^2),
 // s_l(y) = sum_n (-y/2)^n / (n! (2l+2n+1)!!) (seven terms: exact to rounding
@@ -140,7 +198,7 @@ __device__ __forceinline__ double sph_series(int l, double y) {
 // j_2(x)/x^2 -> 1/15.  For l >= 3 their eps_l is below
 // c_l x_lo^(l-2)/(2l+1)!!, and x_lo <= 0.2.
 template <typename T>
-__device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, T d2, const T *src) {
+__device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, PlainSum<T> d2, const T *src) {
   if (a.lrow[row] != 2) {
     // c_l from the grid: its square root and the FP64 product per (row,
     // source) took half of the FP32 kernel's time
@@ -148,7 +206,7 @@ __device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, T
     else return mul_ff(d2, a.cl2[row]);
   }
   const double c = a.cl[row];
-  double d = c * (double)d2;
+  double d = c * wide(d2);
   {
     double tail = 0.0;
     for (int i = a.ntau - 1; i >= 0; --i) {
@@ -177,7 +235,7 @@ __device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, T
 // Measured (one model, before -> after): FP64 l_max 500 93 -> 69 us,
 // l_max 5000 9380 -> 7951 us (its products alone: 7300 us); tensor modes l_max
 // 1500 3105 (four passes and a combining one) -> 1948 us; FP32 E-mode, 5
-// sources, l_max 2001 950 -> 274 us.
+// sources, l_max 2001 950 -> 278 us.
 //
 // Splits: a warp pass covers 4 RV rows (lane group g, slot i: row 4 i + g);
 // the rows / 32 row warps take passes in turn, and the 128 / rows warps that
@@ -228,17 +286,18 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
   const double kq = a.kk[q];
   const int stride = (nb < CHB ? nb : CHB) * KB;  // staged nodes per vector
   T *s = reinterpret_cast<T *>(smem_raw);                       // [NV][stride]
-  T *res = s + (size_t)NV * stride;                             // [TS][NV][R]
+  using Sum = PlainSum<T>;
+  Sum *res = reinterpret_cast<Sum *>(s + (size_t)NV * stride);  // [TS][NV][R]
   long long *xb = reinterpret_cast<long long *>(res + (size_t)NV * kTileL);  // [nb STEPS] x of each step's first node
-  T *halo = reinterpret_cast<T *>(xb + nb * STEPS);             // tensor: [NV] sums of row row0 - 1
+  Sum *halo = reinterpret_cast<Sum *>(xb + nb * STEPS);         // tensor: [NV] sums of row row0 - 1
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = lane >> 3, sub = lane & 7;
   const int WR = kPlainWarps / TS, rw = warp % WR, ts = warp / WR;
   // nonnegative doubles order as their bit patterns
   for (int i = tid; i < nb * STEPS; i += kPlainWarps * 32)
     xb[i] = i * SN < a.ntau ? __double_as_longlong(kq * (a.tau0 - a.tau[i * SN])) : -1;
-  for (int i = tid; i < NV * kTileL; i += kPlainWarps * 32) res[i] = T(0);
-  if (HALO && tid < NV) halo[tid] = T(0);
+  for (int i = tid; i < NV * kTileL; i += kPlainWarps * 32) res[i] = as_ff(T(0));
+  if (HALO && tid < NV) halo[tid] = as_ff(T(0));
   const T *chunk = table + (size_t)a.off[e_idx] * (kTileL * KB);
   for (int b0 = 0; b0 < nb; b0 += CHB) {
     const int nbc = min(CHB, nb - b0), nt = nbc * KB, t0 = b0 * KB;
@@ -418,11 +477,11 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
         for (; st < nmax; st += TS) step(st, std::integral_constant<int, 1>(), std::true_type());
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          const T t = reduce_group<T, RV>(acc[v], lane);
+          const Sum t = reduce_group<T, RV>(acc[v], lane);
           constexpr int LPV = 8 / RV;  // lanes that end with the same value
           if (sub % LPV == 0) {
-            T *r = res + (ts * NV + v) * R + rb + grp + 4 * (sub / LPV);
-            *r = b1 ? *r + t : t;
+            Sum *r = res + (ts * NV + v) * R + rb + grp + 4 * (sub / LPV);
+            *r = b1 ? add_ff(*r, t) : t;
           }
         }
       }
@@ -447,9 +506,10 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
             if (v % 4 == 3) continue;
+            Sum hs = as_ff(h[v]);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) h[v] += __shfl_xor_sync(0xffffffffu, h[v], o);
-            if (lane == 0) halo[v] += h[v];
+            for (int o = 16; o > 0; o >>= 1) hs = add_ff(hs, shfl_ff(hs, o));
+            if (lane == 0) halo[v] = add_ff(halo[v], hs);
           }
         }
       }
@@ -458,8 +518,8 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
   __syncthreads();
   // ---- outputs
   auto sum = [&](int v, int r) {
-    T t = res[v * R + r];
-    for (int i = 1; i < TS; ++i) t += res[(i * NV + v) * R + r];
+    Sum t = res[v * R + r];
+    for (int i = 1; i < TS; ++i) t = add_ff(t, res[(i * NV + v) * R + r]);
     return t;
   };
   for (int idx = tid; idx < mc * R; idx += kPlainWarps * 32) {
@@ -468,24 +528,24 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
     if (row >= a.nl) continue;
     const size_t o = ((size_t)(m0 + m) * a.nk + q) * a.nl + row;
     if constexpr (FIELD == kFieldT) {
-      Delta[o] = sum(m, r);
+      Delta[o] = round_ff(sum(m, r));
     } else if constexpr (FIELD == kFieldE) {
-      Delta[o] = emode_row(a, row, kq, sum(m, r), S + ((size_t)(m0 + m) * a.nk + q) * a.ntau);
+      Delta[o] = emode_row<T>(a, row, kq, sum(m, r), S + ((size_t)(m0 + m) * a.nk + q) * a.ntau);
     } else {
       const size_t so = ((size_t)(m0 + m) * a.nk + q) * a.ntau;
       const int l = a.lmin + row;
-      Delta[o] = emode_row(a, row, kq, sum(4 * m + 3, r), ST + so);
+      Delta[o] = emode_row<T>(a, row, kq, sum(4 * m + 3, r), ST + so);
       double ve = 0.0, vb = 0.0;
       if (l >= 2) {
-        const double d0 = (double)sum(4 * m, r), d1 = (double)sum(4 * m + 1, r), d2 = (double)sum(4 * m + 2, r);
+        const double d0 = wide(sum(4 * m, r)), d1 = wide(sum(4 * m + 1, r)), d2 = wide(sum(4 * m + 2, r));
         double p0, p1;  // D0, D1 of row l - 1
         if (row == 0) {
           // j_(l-1) = (2l+1)/x j_l - j_(l+1) (the sums leave out the same nodes)
-          p1 = a.nl > 1 ? (2.0 * l + 1.0) * d2 - (double)sum(4 * m + 1, 1) : 0.0;
-          p0 = a.nl > 1 ? (2.0 * l + 1.0) * d1 - (double)sum(4 * m, 1) : 0.0;
+          p1 = a.nl > 1 ? (2.0 * l + 1.0) * d2 - wide(sum(4 * m + 1, 1)) : 0.0;
+          p0 = a.nl > 1 ? (2.0 * l + 1.0) * d1 - wide(sum(4 * m, 1)) : 0.0;
         } else {
-          p0 = (double)(r > 0 ? sum(4 * m, r - 1) : halo[4 * m]);
-          p1 = (double)(r > 0 ? sum(4 * m + 1, r - 1) : halo[4 * m + 1]);
+          p0 = wide(r > 0 ? sum(4 * m, r - 1) : halo[4 * m]);
+          p1 = wide(r > 0 ? sum(4 * m + 1, r - 1) : halo[4 * m + 1]);
         }
         ve = (double)l * (l - 1) * d2 - 2.0 * d0 + 2.0 * p1;
         vb = 2.0 * p0 - 2.0 * (l - 1) * d1;
@@ -573,8 +633,8 @@ static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, const
   if (FIELD != kFieldT && emode_x_lo(g, &a.x_lo))
     return fail(GCAMB_EINVAL, "los_transfer: eps_cut too large for the l = 2 limit of the polarisation kernels");
   const int stage = t.max_nkb < plain_stage_blocks(NV, sizeof(T)) ? t.max_nkb : plain_stage_blocks(NV, sizeof(T));
-  const size_t smem = (size_t)NV * stage * kPlainKB * sizeof(T) + (size_t)NV * kTileL * sizeof(T) +
-                      (size_t)t.max_nkb * (kPlainKB * sizeof(T) / 128) * sizeof(long long) + NV * sizeof(T);
+  const size_t smem = (size_t)NV * stage * kPlainKB * sizeof(T) + (size_t)NV * kTileL * sizeof(PlainSum<T>) +
+                      (size_t)t.max_nkb * (kPlainKB * sizeof(T) / 128) * sizeof(long long) + NV * sizeof(PlainSum<T>);
   cudaError_t e = cudaFuncSetAttribute(los_plain_kernel<T, MC, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return cuda_fail(e, "los_transfer: smem attribute");

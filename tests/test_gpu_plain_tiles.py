@@ -107,3 +107,27 @@ def test_long_tau_grids_of_a_batch(mode, M, ntau):
         gcamb.sync()
         for a, b in zip(one, batch):
             assert torch.equal(a[0], b[m])
+
+
+@pytest.mark.parametrize("M", [1, 3, 8])
+def test_fp32_lane_sums_are_rounded_once(M):
+    """FP32 sums over lanes, warps and groups of tau are carried as two floats
+    and rounded once.  Sources at one node per lane (every 4th of two steps, a
+    warp each, and of the second group of 2048), so that what a lane adds up
+    is one rounded product t s, with t read back by unit sources: the result is
+    within 2^-24 of the sum of those products, and 2^-44 of their magnitudes
+    (about 20 additions of pairs, each within 2^-47)."""
+    k, tau, S, g = make(3, 2113, 70, M, seed=M)
+    gcamb.bessel_table(g, gcamb.PLAIN32)
+    nodes = np.concatenate([np.arange(0, 64, 4), 2048 + np.arange(0, 64, 4)])
+    U = torch.zeros((nodes.size, k.size, tau.size), dtype=torch.float32, device="cuda")
+    U[torch.arange(nodes.size), :, torch.as_tensor(nodes)] = 1.0
+    t = gcamb.los_transfer(g, U, gcamb.PLAIN32).cpu().numpy()  # [node][q][l]
+    s = np.random.default_rng(M).standard_normal((M, k.size, nodes.size)).astype(np.float32)
+    d = torch.zeros((M, k.size, tau.size), dtype=torch.float32, device="cuda")
+    d[:, :, torch.as_tensor(nodes)] = torch.as_tensor(s, device="cuda")
+    got = gcamb.los_transfer(g, d, gcamb.PLAIN32).cpu().numpy().astype(np.float64)
+    gcamb.sync()
+    p = (t[None] * s.transpose(0, 2, 1)[:, :, :, None]).astype(np.float64)  # [m][node][q][l], products rounded to FP32
+    ref = p.sum(1)
+    assert (np.abs(got - ref) <= 2.0 ** -24 * np.abs(ref) + 2.0 ** -44 * np.abs(p).sum(1) + 1e-40).all()
