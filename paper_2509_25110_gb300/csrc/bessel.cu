@@ -124,11 +124,13 @@ __device__ __forceinline__ double mul_mantissas(unsigned long long a, unsigned l
 // put.order(0) = lmin (a huge order past the last row); put.last(l) is the last
 // row of order <= l.  A sink that can hold FP64 numbers (kRaw) takes the
 // backward orders unscaled, put.raw(r, v), from one pass, and then
-// put.rescale(r, s) for each of them; the others get a second pass.  Returns
-// the number of rows stored (rows 0 .. that - 1).
+// put.rescale(r, s) for each of them; the others get a second pass.  start: this
+// thread's copy, in shared memory, of the Miller start that a set of nodes shares,
+// that of an x not below any of theirs below ltop (0: none).  Returns the number
+// of rows stored (rows 0 .. that - 1).
 template <class Sink>
-__device__ __forceinline__ int bessel_orders(double x, int lmin, int ltop, const double *__restrict__ xs, int nxs,
-                                              Sink &put) {
+__device__ __forceinline__ int bessel_orders(double x, const volatile int *start, int lmin, int ltop,
+                                             const double *__restrict__ xs, int nxs, Sink &put) {
   if (ltop < lmin) return 0;
   const double w = put.weight();
   if (x < 1e-150) {  // j_1 = x/3, j_l < 1e-300 for l >= 2
@@ -219,18 +221,17 @@ __device__ __forceinline__ int bessel_orders(double x, int lmin, int ltop, const
     fb = (double)(long long)(A - kOff);
   }
   // ---- backward from L (here ltop > ls = floor(x) >= 1), to the rows from `row` on
-  int L = miller_start(xs, nxs, ls + 1, x);
+  const int Lg = *start;
+  int L = miller_start(xs, Lg > ls ? Lg + 1 : nxs, ls + 1, x);
   const int top = put.last(L < ltop ? L : ltop);
   if (top < row) return row;
-  {
-    // Neighbouring nodes start at the highest of their orders (a higher start
-    // only lowers the truncation), so that the lanes of a warp come to a row's
-    // order together: one by one, the rows' stores cost more than the steps
-    // added.  Where the orders lie far apart, or the exponent of f (below 1000
-    // from the Miller start) could grow by more than 400, each keeps its own.
-    const int Lw = __reduce_max_sync(__activemask(), L);
-    if ((Lw - L) * (32 - __clz((2 * Lw + 1) / ls)) <= 400) L = Lw;
-  }
+  // Nodes that share a start take it (a higher start only lowers the
+  // truncation), so that the lanes of a warp come to a row's order together: one
+  // by one, the rows' stores cost more than the steps added.  Where the orders
+  // lie far apart, or the exponent of f (below 1000 from the Miller start) could
+  // grow by more than 400, a node keeps its own.  A rule of the nodes' x, not of
+  // which lanes come here together, so that the bits are those of the grid.
+  if (Lg > L && (Lg - L) * (32 - __clz((2 * Lg + 1) / ls)) <= 400) L = Lg;
   // c_L = (2L+1)/x = C 2^(K-64) with C's leading bit set, 32 further bits
   const unsigned __int128 P = N * (unsigned)(2 * L + 1);                          // above 2^96: c_L > 2
   const int sh = 64 - __clzll((long long)(unsigned long long)(P >> 64));          // P >> sh has 64 bits
@@ -628,20 +629,28 @@ __global__ void __launch_bounds__(128) bessel_table_kernel(const double *__restr
   // order, and zeros that this kernel writes one by one are not compressed in
   // DRAM, where the tensor-core kernel reads whole blocks (it took 4% longer).
   const bool fill = (MODE == GCAMB_PLAIN64 || MODE == GCAMB_PLAIN32) && !curved && !kern;
-  if (i >= (fill ? (ntau + KB - 1) / KB * KB : ntau)) return;
+  // a warp's nodes are of one block, so that these are the warp's
   const int32_t *nkb_q = nkb + (size_t)q * nlt;
   const int kbi = i / KB;
   int lt_last = -1;
   while (lt_last + 1 < nlt && nkb_q[lt_last + 1] > kbi) ++lt_last;
   if (lt_last < 0) return;
+  // the highest multipole of the last tile the nodes are active in
+  const int ltop = lrow ? lrow[min((lt_last + 1) * kTileL, nl) - 1] : min(lmin + (lt_last + 1) * kTileL - 1, lmax);
+  // the Miller start they share: that of their first node, x falls along tau
+  // (nodes at ltop and above have no backward part).  Kept in shared memory: held
+  // in a register over the forward part it cost 2% of the sampled tables.
+  __shared__ int starts[128];
+  int *start = starts + threadIdx.x;
+  const int i0 = i & ~31;
+  *start = curved || i0 >= ntau ? 0 : miller_start(xs, nxs, 1, fmin(k[q] * (tau0 - tau[i0]), (double)ltop));
+  if (i >= (fill ? (ntau + KB - 1) / KB * KB : ntau)) return;
   if (i >= ntau) {
     TableSink<MODE> sink{static_cast<char *>(table), off + (size_t)q * nlt, lmin, kbi, i % KB, 0.0, -1, nullptr, nullptr,
                          nullptr, nl};
     for (int r = 0; r < (lt_last + 1) * kTileL; ++r) sink.store(r, 0.0);
     return;
   }
-  // the highest multipole of the last tile this node is active in
-  const int ltop = lrow ? lrow[min((lt_last + 1) * kTileL, nl) - 1] : min(lmin + (lt_last + 1) * kTileL - 1, lmax);
   TableSink<MODE> sink{static_cast<char *>(table), off + (size_t)q * nlt, lmin, kbi, i % KB,
                        ldexp(wtau[i], scale_exp), -1, nullptr, rowof, lrow, nl};
   if (curved) {  // hyperspherical: beta = q / sqrt|K|, chi = sqrt|K| (tau0 - tau)
@@ -653,10 +662,10 @@ __global__ void __launch_bounds__(128) bessel_table_kernel(const double *__restr
     } else {
       const int l0 = lmin > 0 ? lmin - 1 : 0;
       KernelSink<TableSink<MODE>> ks{sink, kern, lmin, 1.0 / x, 1.0 / (x * x), -10, -10, 0.0, 0.0, l0};
-      bessel_orders(x, l0, ltop, xs, nxs, ks);
+      bessel_orders(x, start, l0, ltop, xs, nxs, ks);
     }
   } else {
-    const int n = bessel_orders(k[q] * (tau0 - tau[i]), lmin, ltop, xs, nxs, sink);
+    const int n = bessel_orders(k[q] * (tau0 - tau[i]), start, lmin, ltop, xs, nxs, sink);
     if (fill)
       for (int r = n; r < (lt_last + 1) * kTileL; ++r) sink.store(r, 0.0);
   }
@@ -774,7 +783,9 @@ __global__ void sph_bessel_kernel(const double *__restrict__ x, int n, int lmax,
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   DenseSink s{out + (size_t)i * (lmax + 1)};
-  bessel_orders(x[i], 0, lmax, xs, nxs, s);
+  __shared__ int starts[128];
+  starts[threadIdx.x] = 0;  // an array's values have nothing in common
+  bessel_orders(x[i], starts + threadIdx.x, 0, lmax, xs, nxs, s);
 }
 
 // ------------------------------------------------------------------ table memory

@@ -67,3 +67,16 @@ def test_tables(orc, ntau, eps_cut, boost, mode):
     ref = orc.los_cl(k, tau, 14000.0, 2, lmax, S, want_cl=False)[0][:, :, rows - 2]
     scale = np.abs(ref).reshape(2, -1).max(axis=1)[:, None, None]
     assert (np.abs(D - ref) <= (1e-11 if mode == gcamb.PLAIN64 else 1e-5) * scale).all()
+
+
+@pytest.mark.parametrize("lmax,hi", [(40, 60.0), (700, 900.0), (2200, 2300.0)])
+def test_values_do_not_depend_on_neighbours(lmax, hi):
+    """j_l of a node is the same bits alone and among others, in any order."""
+    rng = np.random.default_rng(lmax)
+    x = torch.as_tensor(rng.uniform(0.2, hi, 300), device="cuda")
+    all_ = gcamb.sph_bessel(x, lmax)
+    p = torch.as_tensor(rng.permutation(300), device="cuda")
+    assert torch.equal(gcamb.sph_bessel(x[p].contiguous(), lmax), all_[p])
+    for i in (0, 17, 299):
+        assert torch.equal(gcamb.sph_bessel(x[i:i + 1].contiguous(), lmax), all_[i:i + 1])
+    gcamb.sync()
