@@ -136,14 +136,16 @@ __device__ __forceinline__ int bessel_orders(double x, const volatile int *start
   if (x < 1e-150) {  // j_1 = x/3, j_l < 1e-300 for l >= 2
     const int r1 = lmin == 0 ? 1 : 0;
     if (lmin == 0) put.store(0, w);
-    if (!(x > 0.0) || ltop < 1 || put.order(r1) != 1) return r1;
+    if (x == 0.0 || ltop < 1 || put.order(r1) != 1) return r1;
     put.store(r1, w * (x / 3.0));
     return r1 + 1;
   }
-  if (x < 1.0) {  // few orders, and (2l+1)/x has no useful bound: FP64
+  // few orders, and (2l+1)/x has no useful bound: FP64 (and for infinities and
+  // NaN, which have no fixed-point form: every order is NaN)
+  if (!(x >= 1.0 && x <= 1.7976931348623157e308)) {
     const double inv = 1.0 / x, j0 = sin(x) / x;
     if (lmin == 0) put.store(0, w * j0);
-    const int L = miller_start(xs, nxs, 1, x);
+    const int L = x < 1.0 ? miller_start(xs, nxs, 1, x) : nxs - 1;
     double fh = 0.0, f = 1.0, dl = 2.0 * L + 1.0;
     for (int l = L; l > 0; --l) {
       const double fm = fma(dl * inv, f, -fh);

@@ -80,3 +80,24 @@ def test_values_do_not_depend_on_neighbours(lmax, hi):
     for i in (0, 17, 299):
         assert torch.equal(gcamb.sph_bessel(x[i:i + 1].contiguous(), lmax), all_[i:i + 1])
     gcamb.sync()
+
+
+@pytest.mark.parametrize("lmax", [0, 1, 2, 7, 300])
+def test_infinite_and_nan_arguments(lmax):
+    """No finite j_l: every order is NaN, and the values beside them are theirs."""
+    x = np.array([0.5, np.nan, 3.0, np.inf, 400.0, -np.nan, 0.0])
+    out = gcamb.sph_bessel(torch.as_tensor(x, device="cuda"), lmax).cpu().numpy()
+    fin = gcamb.sph_bessel(torch.as_tensor(x[[0, 2, 4, 6]], device="cuda"), lmax).cpu().numpy()
+    gcamb.sync()
+    assert np.isnan(out[[1, 3, 5]]).all()
+    assert np.array_equal(out[[0, 2, 4, 6]], fin)
+
+
+def test_arguments_below_zero():
+    """Outside the documented range, as ever: j_0 = 1, j_1 = x/3, the others 0."""
+    x = np.array([-1e-160, -0.25, -5.0])
+    out = gcamb.sph_bessel(torch.as_tensor(x, device="cuda"), 4).cpu().numpy()
+    gcamb.sync()
+    ref = np.zeros((3, 5))
+    ref[:, 0], ref[:, 1] = 1.0, x / 3.0
+    assert np.array_equal(out, ref)
