@@ -100,11 +100,12 @@ __device__ __forceinline__ unsigned __int128 inv_fixed(double x) {
   return n;
 }
 
-// A nonnegative double as g 2^e with the leading bit of g set (0: g = 0).
+// A nonnegative double as g 2^e with the leading bit of g set (0 and subnormal
+// numbers: g = 0).
 __device__ __forceinline__ unsigned long long mantissa(double v, int *e) {
   const long long b = __double_as_longlong(v);
   *e = (int)(b >> 52) - 1086;
-  return b == 0 ? 0 : (unsigned long long)((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << 11;
+  return b >> 52 == 0 ? 0 : (unsigned long long)((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << 11;
 }
 
 // a g 2^e, leading bits of a and g set (or 0), rounded to FP64 (0 below its
@@ -197,7 +198,8 @@ __device__ __forceinline__ int bessel_orders(double x, const volatile int *start
     unsigned long long Am = (unsigned long long)__double2ll_rn(sx * q) + kOff;
     unsigned long long A = (unsigned long long)__double2ll_rn(j1 * q) + kOff;
     int ge;
-    const unsigned long long gm = mantissa(w * inv * (1.0 / q), &ge);
+    const unsigned long long gm = mantissa(w * inv, &ge);
+    ge -= 60;
     // c = (2l+1)/x, 63 + 32 fraction bits; below 2 for every l < ls (3/x of ls = 1 is not used)
     U96 c(3 * N), st(2 * N);
 #pragma unroll 2

@@ -93,6 +93,18 @@ def test_infinite_and_nan_arguments(lmax):
     assert np.array_equal(out[[0, 2, 4, 6]], fin)
 
 
+@pytest.mark.parametrize("x", [1e20, 1e100, 1e285, 1e290, 1e295, 8e299])
+def test_huge_arguments(x):
+    """x far beyond every order: j_l(x) = sin(x - l pi / 2) / x but for l (l+1) / (2x),
+    within 1e-11 of 1/x, up to the documented 1e-300."""
+    lmax = 50
+    out = gcamb.sph_bessel(torch.as_tensor([x], dtype=torch.float64, device="cuda"), lmax).cpu().numpy()[0]
+    gcamb.sync()
+    s, c = np.sin(x), np.cos(x)
+    ref = np.array([(s, -c, -s, c)[l % 4] for l in range(lmax + 1)]) / x
+    assert (np.abs(out - ref) <= 1e-11 / x + 1e-300 * (np.abs(ref) < 1e-300)).all(), (out, ref)
+
+
 def test_arguments_below_zero():
     """Outside the documented range, as ever: j_0 = 1, j_1 = x/3, the others 0."""
     x = np.array([-1e-160, -0.25, -5.0])
