@@ -16,11 +16,13 @@
 // the FP32 rate (two lanes a clock and SM), so a recurrence step of a product,
 // a fused multiply-add and an addition in FP64 takes about ten times as long
 // as the same step in integers:
-//   forward   x j_l + 8 as an unsigned fixed-point number of 60 fraction bits
-//             (|x j_l| < 4 for every l <= x, l <= 20000), (2l+1)/x < 2 as one of 63
+//   forward   x j_l + 8 as an unsigned fixed-point number of 60 fraction bits,
+//             which holds |x j_l| < 8: its maximum over l <= x is 0.85 x^(1/6), 4.41
+//             at x = 20000, the highest order there is; (2l+1)/x < 2 as one of 63
 //             with 32 further bits carried along, the upper half of their
-//             product: an error below 2^-60 a step, where an FP64 step of
-//             values near 1 makes 2^-54;
+//             product: an error below 2^-59 a step (a unit of 2^-60 from the
+//             product, half a one from the factor), where an FP64 step of values
+//             near 1 makes 2^-54;
 //   backward  f_l and f_(l+1) as 64-bit mantissas with a common exponent.
 //             While (2l+1)/x >= 4 (x of a few units) they are renormalised
 //             every step; below, f grows by less than four a step and both
@@ -28,11 +30,11 @@
 //             2^-58 a step, and about 20 x^(1/3) steps.
 // Orders are converted to FP64 (and the row's weight applied) where they are
 // table rows, so a grid of sampled multipoles converts only those.
-// Measured: PLAIN64 table of 130 sampled multipoles to 2500, 2000 k x 1000
-// tau 6667 -> 1328 us; every multipole 7759 -> 3360 (PLAIN64),
-// 9209 -> 3854 (PLAIN32), 13660 -> 8216 (F16X3); l_max 5000, 3000 k x 2000 tau, PLAIN64
-// 41.5 -> 21.8 ms.  What is left is the integer pipes (59% of issue slots) and, for
-// every multipole, the stores.
+// Measured, whole calls: PLAIN64 table of 130 sampled multipoles to 2500, 2000 k x
+// 1000 tau 6880 -> 1404 us; every multipole 8650 -> 3470 (PLAIN64), 9630 -> 3870
+// (PLAIN32), 14190 -> 8660 (F16X3); l_max 5000, 3000 k x 2000 tau, PLAIN64 46.4 ->
+// 22.0 ms.  What is left is the integer pipes (59% of issue slots) and, for every
+// multipole, the stores.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>

@@ -113,3 +113,14 @@ def test_arguments_below_zero():
     ref = np.zeros((3, 5))
     ref[:, 0], ref[:, 1] = 1.0, x / 3.0
     assert np.array_equal(out, ref)
+
+
+@pytest.mark.parametrize("x0", [11900.0, 14990.0, 19900.0])
+def test_highest_orders(orc, x0):
+    """Orders up to the highest, at x where x j_l(x) comes closest to the limit of
+    the fixed-point numbers (4.41 of 8 at x = 20000)."""
+    x = np.concatenate([x0 + np.linspace(0.0, 200.0, 41), [x0 + 97.3]])
+    out = gcamb.sph_bessel(torch.as_tensor(x, device="cuda"), 20000).cpu().numpy()
+    gcamb.sync()
+    assert np.abs(out[:, :int(x0)] * x[:, None]).max() > 4.0
+    check_rows(orc, x, 20000)
