@@ -493,34 +493,44 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         const unsigned long long qmu = (unsigned long long)fix53(xmu) + kExpLn2;
         const unsigned int sbits = __float_as_uint(sd);
         const int ms = (int)((sbits & 0x7fffffu) | 0x800000u) << 7, es = 261 - (int)(sbits >> 23);
-        // columns and rows outside the range (or a subnormal sd): FP64 for the tile
-        const bool badt = __any_sync(0xffffffffu, !(fabsf(xmu) < 300.f) || !(fabsf(xa) < 300.f) ||
-                                                      !(fabsf(xm) < 300.f) || (sbits >> 23) == 0);
+        // Elements out of the fixed-point range take the FP64 exp, each by itself: a
+        // spectrum is the same bits alone and among any others of a batch.
+        const bool badc = !(fabsf(xmu) < 300.f) || !(fabsf(xm) < 300.f) || (sbits >> 23) == 0;  // the column (or a subnormal sd)
+        const unsigned int badr = __ballot_sync(0xffffffffu, !(fabsf(xa) < 300.f));             // rows
+        const bool badt = __any_sync(0xffffffffu, badc) || badr;
         *reinterpret_cast<long long *>(st + lane * kPitch + 32) = fix53(xa) - fix53(xm);
         __syncwarp();
+        // row r's argument in Q.53, and whether it is out of the range
+        auto arg = [&](int r, bool &out) {
+          const float *sr = st + r * kPitch;
+          const float y = sr[lane] + xbs;
+          const unsigned int yb = __float_as_uint(y);
+          const int sg = (int)yb >> 31;
+          const int my = ((int)(((yb << 7) & 0x3fffffffu) | 0x40000000u) ^ sg) - sg;  // a subnormal y: 0 or -2^-53
+          const int rs = min(es - (int)((yb >> 23) & 255u), 63);
+          const unsigned long long q =
+              (unsigned long long)(((long long)my * ms) >> (rs & 63)) + qmu + *reinterpret_cast<const unsigned long long *>(sr + 32);
+          out = !(fabsf(y * sd) < 100.f) || (unsigned int)(q >> 32) - kExpLo > kExpSpan;
+          return q;
+        };
         constexpr int RU = 8;  // rows whose chains interleave
         for (int r0 = tl.ra; r0 < min(nr, tl.rb); r0 += RU) {
           double c[RU];
           bool bad = badt;
 #pragma unroll
           for (int i = 0; i < RU; ++i) {
-            const float *sr = st + (r0 + i) * kPitch;
-            const float y = sr[lane] + xbs;
-            const unsigned int yb = __float_as_uint(y);
-            const int sg = (int)yb >> 31;
-            const int my = ((int)(((yb << 7) & 0x3fffffffu) | 0x40000000u) ^ sg) - sg;  // a subnormal y: 0 or -2^-53
-            const int rs = min(es - (int)((yb >> 23) & 255u), 63);
-            const unsigned long long q =
-                (unsigned long long)(((long long)my * ms) >> (rs & 63)) + qmu + *reinterpret_cast<const unsigned long long *>(sr + 32);
-            bad |= !(fabsf(y * sd) < 100.f) || (unsigned int)(q >> 32) - kExpLo > kExpSpan;
-            c[i] = exp_q53(q, tab);
+            bool out;
+            c[i] = exp_q53(arg(r0 + i, out), tab);
+            bad |= out;
           }
-          if (__any_sync(0xffffffffu, bad)) {  // out of the fixed-point range: FP64
+          if (__any_sync(0xffffffffu, bad)) {
 #pragma unroll
             for (int i = 0; i < RU; ++i) {
               const double shd = (double)__shfl_sync(0xffffffffu, xa, r0 + i) - (double)xm;
+              bool out;
+              arg(r0 + i, out);
               const float y = st[(r0 + i) * kPitch + lane] + xbs;
-              c[i] = exp((double)y * (double)sd + (double)xmu + shd);
+              if (out || badc || (badr >> (r0 + i) & 1u)) c[i] = exp((double)y * (double)sd + (double)xmu + shd);
             }
           }
 #pragma unroll

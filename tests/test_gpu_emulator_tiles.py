@@ -121,3 +121,33 @@ def test_persistent_ctas_give_the_same_rows(lmax, B, step):
     assert int(fb.sum().item()) == 0
     assert torch.equal(out, torch.cat(parts))
     assert torch.equal(C, torch.cat(Cp))
+
+
+@pytest.mark.parametrize("lmax,B", [(130, 64), (2500, 1100)])
+def test_served_spectra_do_not_depend_on_the_batch(lmax, B):
+    """Requests beside ones whose exponent is out of the fixed-point range, in
+    amplitude (rows) and in network output (single elements): the bits they have
+    among others; the ones out of range have theirs alone."""
+    g = grid(lmax)
+    e = gcamb.emu_create(g, width=32, depth=1, max_batch=2048, seed=3)
+    sd = np.geomspace(0.05, 3.0, g.nl).astype(np.float32)
+    gcamb.emu_norm(e, np.zeros(9, np.float32), np.ones(9, np.float32), np.linspace(-30.0, 5.0, g.nl).astype(np.float32), sd)
+    rng = np.random.default_rng(11)
+    X = rng.normal(size=(B, 9)).astype(np.float32)
+    odd = np.arange(5, B, 32)
+    X[odd[::2], 8] = 350.0         # amplitude
+    X[odd[1::2], :8] *= 1e3        # outputs of hundreds: some of its elements
+    Xd = torch.as_tensor(X, device="cuda")
+    ones = torch.ones((B, g.nl), dtype=torch.float64, device="cuda")
+    gcamb.emu_check(e, Xd, ones, tol=float("inf"), min_count=1)
+    C, fb = gcamb.emulate(e, Xd)
+    plain = torch.as_tensor(np.setdiff1d(np.arange(B), odd), device="cuda")
+    Cp, _ = gcamb.emulate(e, Xd[plain].contiguous())
+    Co = [gcamb.emulate(e, Xd[i:i + 1].contiguous())[0] for i in odd[:4]]
+    y = gcamb.emu_forward(e, Xd).double().cpu().numpy() * sd
+    gcamb.sync()
+    assert int(fb.sum().item()) == 0
+    assert (np.abs(y[odd[1::2]]) >= 100.0).any() and (np.abs(y[odd[1::2]]) < 100.0).any()
+    assert torch.equal(C[plain], Cp)
+    for i, c in zip(odd, Co):
+        assert torch.equal(C[int(i)], c[0])
