@@ -383,9 +383,11 @@ __global__ void __launch_bounds__(256) synth_kernel(const float *__restrict__ X,
 
 // ---------------------------------------------------------------- GEMM launcher
 
-// Launch of a kernel of the chain behind the one before it (see pdl_wait).
+// Launch of a kernel of the chain behind the one before it (see pdl_wait); what
+// that one's launch may have left as an error is returned too.
 template <typename... P, typename... A>
 cudaError_t chain_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  if (cudaError_t e = cudaGetLastError()) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;

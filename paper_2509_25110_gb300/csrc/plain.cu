@@ -844,6 +844,7 @@ __global__ void __launch_bounds__(256) cl_sum_kernel(const TD *__restrict__ DX, 
 template <typename TD, int KIND>
 static cudaError_t launch_cl_sum(const gcamb_grid *g, const void *DX, const void *DY, const double *Pk, int M,
                                  double *Cl, cudaStream_t st, const ClPrefix &px = ClPrefix()) {
+  if (cudaError_t e = cudaGetLastError()) return e;  // a launch before this one
   // cluster size: the smallest that gives every SM six CTAs of 256 threads
   // (of the eight that fit), up to the portable eight: with one model even
   // l_max = 5000 has only 157 blocks of 32 multipoles
@@ -864,8 +865,9 @@ static cudaError_t launch_cl_sum(const gcamb_grid *g, const void *DX, const void
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool plain_stream = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-  if (!plain_stream) cudaGetLastError();
+  const bool known = cudaStreamIsCapturing(st, &cap) == cudaSuccess;
+  if (!known) cudaGetLastError();  // another stream's capture: the query's own error
+  const bool plain_stream = known && cap == cudaStreamCaptureStatusNone;
   cfg.attrs = at;
   cfg.numAttrs = plain_stream ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, cl_sum_kernel<TD, KIND>, static_cast<const TD *>(DX), static_cast<const TD *>(DY),
