@@ -402,7 +402,7 @@ bool seg_halo_ok(const double *h, const double *cp, const double *inv, int n) {
 // the last}, of about equal work t, counted in segments: kPartOuts outputs take
 // about as long as a segment's sweep and back substitution.  A part's sweep
 // starts 2 kSegA segments early, so `blocks` columns' parts take (2 kSegA + t)
-// (1 + W / t) one after the other on the chip's places (five blocks an SM),
+// (1 + W / t) one after the other on the chip's places,
 // W = all work / places; t = sqrt(2 kSegA W) is its least, and at least
 // kPartMin.  A segment with many outputs (nodes that are sparse where the grid
 // is dense) is shared out by outputs; segments without any are left out where

@@ -250,7 +250,9 @@ __device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, P
 // later node is below it too): the terms left out are below eps_cut |w S|
 // each.  With x^-1 or x^-2 only rows whose threshold is at least 1 stop:
 // j_l(x) x^-2 rises with x below the threshold (l >= 3 there), so each term
-// left out is below eps_cut |w S| as well.
+// left out is below eps_cut |w S| as well, and c_l / x^2 (below 300) times that
+// in the result; these fields have the thresholds only where that is nothing
+// (kPolRowCut).
 template <typename T, int MC, int FIELD>
 __global__ void __launch_bounds__(kPlainWarps * 32, 4)
     los_plain_kernel(const T *__restrict__ table, const T *__restrict__ S, const T *__restrict__ ST,
@@ -582,6 +584,13 @@ int emode_x_lo(const gcamb_grid *g, double *x_lo) {
   return x <= 0.2 ? 0 : -1;
 }
 
+// Largest eps_cut with which polarisation and tensor rows stop at their own
+// prefix; beyond it they take the whole tile's, whose rows but the lowest lose
+// next to nothing at any eps_cut (E-mode at eps_cut 1e-8, 1e-6, 1e-4, error of the
+// transfers: 2e-12, 2e-10, 2e-8; with rows' own prefixes 3e-8, 1e-6, 3e-4).  At
+// 1e-20 the rows' own prefixes leave out 3e-20 of them, below FP64's rounding.
+constexpr double kPolRowCut = 1e-20;
+
 // Rows per CTA of the plain kernel: a whole 128-row tile, or 64 rows (the
 // CTA's four warps then share out the tau steps in pairs) where the tiles are
 // too few to balance the SMs.  Counted in CTAs of the longest prefix (blocks /
@@ -598,7 +607,7 @@ static int plain_rows(const gcamb_grid *g, const Table &t) {
   return !g->lsampled && full >= 152 * 8 ? 128 : 64;
 }
 
-static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M) {
+static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M, int field) {
   PlainArgs a{};
   a.nkb = t.d_nkb;
   a.off = t.d_off;
@@ -607,10 +616,10 @@ static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M) {
   a.tau = g->d_tau;
   a.wtau = g->d_wtau;
   a.dt2 = reinterpret_cast<const float2 *>(g->d_dt2);
-  // rows stop at their own prefix on flat j_l grids only
   a.cl = g->d_cl;
   a.cl2 = reinterpret_cast<const float2 *>(g->d_cl2);
-  a.xthr = (g->kernel == 0 && !g->curved) ? g->d_xthr : nullptr;
+  // rows stop at their own prefix on flat j_l grids only
+  a.xthr = (g->kernel == 0 && !g->curved && (field == kFieldT || g->eps_cut <= kPolRowCut)) ? g->d_xthr : nullptr;
   a.tau0 = g->tau0;
   a.x_lo = 1e-12;
   a.nk = g->nk;
@@ -629,7 +638,7 @@ template <typename T, int MC, int FIELD>
 static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, const T *ST, int M, T *D, T *DE, T *DB,
                           int nk, int nlt, cudaStream_t st) {
   constexpr int NV = FIELD == kFieldTensor ? 4 * MC : MC;
-  PlainArgs a = plain_args(g, t, M);
+  PlainArgs a = plain_args(g, t, M, FIELD);
   if (FIELD != kFieldT && emode_x_lo(g, &a.x_lo))
     return fail(GCAMB_EINVAL, "los_transfer: eps_cut too large for the l = 2 limit of the polarisation kernels");
   const int stage = t.max_nkb < plain_stage_blocks(NV, sizeof(T)) ? t.max_nkb : plain_stage_blocks(NV, sizeof(T));

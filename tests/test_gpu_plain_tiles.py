@@ -131,3 +131,28 @@ def test_fp32_lane_sums_are_rounded_once(M):
     p = (t[None] * s.transpose(0, 2, 1)[:, :, :, None]).astype(np.float64)  # [m][node][q][l], products rounded to FP32
     ref = p.sum(1)
     assert (np.abs(got - ref) <= 2.0 ** -24 * np.abs(ref) + 2.0 ** -44 * np.abs(p).sum(1) + 1e-40).all()
+
+
+@pytest.mark.parametrize("mode,bar", [(gcamb.PLAIN64, 1e-11), (gcamb.PLAIN32, 1e-6)])
+@pytest.mark.parametrize("eps_cut", [1e-12, 1e-6, 1e-4])
+def test_polarisation_rows_at_large_eps_cut(mode, bar, eps_cut):
+    """Polarisation and tensor rows take their tile's whole prefix at a large
+    eps_cut: only its lowest rows lose terms (a node left out has |j_l| < eps_cut at
+    the lowest multipole, where x < l, and j_l falls by more than a factor of two
+    every few orders above: by 2^-40 and more over 40 orders).  Rows 40.. of every
+    tile against the grid of default eps_cut, within the bars of the other tests of
+    the largest |Delta|."""
+    k, tau, S, _ = make(60, 500, 400, 2, seed=12)
+    d = [torch.as_tensor(s, dtype=torch.float64 if mode == gcamb.PLAIN64 else torch.float32, device="cuda") for s in S]
+
+    def fields(eps):
+        g = gcamb.grid_create(k, tau, 14000.0, 2, 400, eps_cut=eps)
+        gcamb.bessel_table(g, mode)
+        return [gcamb.los_transfer_e(g, d[1], mode), *gcamb.los_transfer_tensor(g, d[0], d[1], mode)]
+
+    rows = torch.arange(399, device="cuda")
+    rows = rows[rows % 128 >= 40]
+    got, ref = fields(eps_cut), fields(0.0)
+    gcamb.sync()
+    for a, r in zip(got, ref):
+        assert ((a - r).abs()[:, :, rows] <= bar * r.abs().max()).all(), float(((a - r).abs()[:, :, rows] / r.abs().max()).max())
