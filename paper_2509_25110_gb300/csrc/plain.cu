@@ -103,6 +103,7 @@ struct PlainArgs {
   const double *xthr;   // [nl] Watson thresholds, or null: every row takes the whole tile's prefix
   double tau0, x_lo;
   int nk, nlt, nl, ntau, M, lmin;
+  int step_round;       // rows' prefixes in steps are rounded up to a multiple of step_round + 1 (1 or a block's)
   int q0;               // last k of the launch
   int rows;             // rows per CTA: 128 or 64
 };
@@ -252,7 +253,7 @@ __device__ __forceinline__ T emode_row(const PlainArgs &a, int row, double kq, P
 // j_l(x) x^-2 rises with x below the threshold (l >= 3 there), so each term
 // left out is below eps_cut |w S| as well, and c_l / x^2 (below 300) times that
 // in the result; these fields have the thresholds only where that is nothing
-// (kPolRowCut).
+// (kRowCut).
 template <typename T, int MC, int FIELD>
 __global__ void __launch_bounds__(kPlainWarps * 32, 4)
     los_plain_kernel(const T *__restrict__ table, const T *__restrict__ S, const T *__restrict__ ST,
@@ -409,7 +410,7 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
                 int n = 0;
                 for (int c = 0; c < nsc; c += 32)
                   n += __popc(__ballot_sync(0xffffffffu, c + lane < nsc && xb[b1 * STEPS + c + lane] >= xi));
-                ns[i] = n;
+                ns[i] = (n + a.step_round) & ~a.step_round;
               }
             }
           }
@@ -584,12 +585,13 @@ int emode_x_lo(const gcamb_grid *g, double *x_lo) {
   return x <= 0.2 ? 0 : -1;
 }
 
-// Largest eps_cut with which polarisation and tensor rows stop at their own
-// prefix; beyond it they take the whole tile's, whose rows but the lowest lose
-// next to nothing at any eps_cut (E-mode at eps_cut 1e-8, 1e-6, 1e-4, error of the
+// Largest eps_cut with which rows stop at the very step of their own prefix.
+// Beyond it temperature rows take whole blocks of 64 nodes, and polarisation and
+// tensor rows the whole tile's prefix, whose rows but the lowest lose next to
+// nothing at any eps_cut (E-mode at eps_cut 1e-8, 1e-6, 1e-4, error of the
 // transfers: 2e-12, 2e-10, 2e-8; with rows' own prefixes 3e-8, 1e-6, 3e-4).  At
 // 1e-20 the rows' own prefixes leave out 3e-20 of them, below FP64's rounding.
-constexpr double kPolRowCut = 1e-20;
+constexpr double kRowCut = 1e-20;
 
 // Rows per CTA of the plain kernel: a whole 128-row tile, or 64 rows (the
 // CTA's four warps then share out the tau steps in pairs) where the tiles are
@@ -619,7 +621,8 @@ static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M, int fiel
   a.cl = g->d_cl;
   a.cl2 = reinterpret_cast<const float2 *>(g->d_cl2);
   // rows stop at their own prefix on flat j_l grids only
-  a.xthr = (g->kernel == 0 && !g->curved && (field == kFieldT || g->eps_cut <= kPolRowCut)) ? g->d_xthr : nullptr;
+  a.xthr = (g->kernel == 0 && !g->curved && (field == kFieldT || g->eps_cut <= kRowCut)) ? g->d_xthr : nullptr;
+  a.step_round = g->eps_cut <= kRowCut ? 0 : kPlainKB * (int)t.lay.esize / 128 - 1;
   a.tau0 = g->tau0;
   a.x_lo = 1e-12;
   a.nk = g->nk;

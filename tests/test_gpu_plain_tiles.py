@@ -156,3 +156,23 @@ def test_polarisation_rows_at_large_eps_cut(mode, bar, eps_cut):
     gcamb.sync()
     for a, r in zip(got, ref):
         assert ((a - r).abs()[:, :, rows] <= bar * r.abs().max()).all(), float(((a - r).abs()[:, :, rows] / r.abs().max()).max())
+
+
+@pytest.mark.parametrize("mode,bar", [(gcamb.PLAIN64, 1e-11), (gcamb.PLAIN32, 1e-6)])
+@pytest.mark.parametrize("eps_cut", [1e-6, 1e-3])
+def test_temperature_rows_at_large_eps_cut(mode, bar, eps_cut):
+    """Temperature rows take whole blocks of 64 nodes at a large eps_cut: a grid of
+    one block, whose first node has x above every multipole, loses nothing."""
+    k = np.array([0.0036, 0.005, 0.02])
+    tau = synth.uniform_grid(200.0, 13990.0, 64)
+    S = np.random.default_rng(5).standard_normal((3, 3, 64))
+    d = torch.as_tensor(S, dtype=torch.float64 if mode == gcamb.PLAIN64 else torch.float32, device="cuda")
+
+    def field(eps):
+        g = gcamb.grid_create(k, tau, 14000.0, 2, 48, eps_cut=eps)
+        gcamb.bessel_table(g, mode)
+        return gcamb.los_transfer(g, d, mode)
+
+    got, ref = field(eps_cut), field(0.0)
+    gcamb.sync()
+    assert ((got - ref).abs() <= bar * ref.abs().max()).all(), float((got - ref).abs().max() / ref.abs().max())
