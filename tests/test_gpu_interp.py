@@ -179,3 +179,19 @@ def test_workspace_of_any_alignment(dtype, nodes, shift):
     assert buf.data_ptr() % 256 == 0
     assert torch.equal(out, ref)
     assert (buf[:shift] == 0x5a).all() and (buf[shift + b.value:] == 0x5a).all()
+
+
+@pytest.mark.parametrize("nk_in,nk,ntau", [(2, 40, 3), (50, 900, 65), (300, 301, 128)])
+def test_fp64_constant_columns_stay_constant(nk_in, nk, ntau):
+    """The weights of an interval's two nodes add up to one: a column of equal
+    powers of two is that value at every node, to the last bit (its second
+    derivatives are zero)."""
+    rng = np.random.default_rng(nk)
+    k = np.sort(rng.uniform(1e-4, 0.3, nk))
+    k_in = np.sort(rng.uniform(1e-4, 0.3, nk_in))
+    k_in[0], k_in[-1] = k[0], k[-1]
+    g = gcamb.grid_create(k, synth.uniform_grid(200.0, 14000.0, ntau), 14000.0, 2, 10)
+    S = np.ones((2, nk_in, ntau)) * 2.0 ** (np.arange(ntau) % 7 - 3)
+    out = gcamb.interp_sources(g, k_in, torch.as_tensor(S, device="cuda")).cpu().numpy()
+    gcamb.sync()
+    assert np.array_equal(out, np.broadcast_to(S[:, :1], out.shape))
