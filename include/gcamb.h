@@ -83,7 +83,10 @@ const char *gcamb_last_error(void);
  *              (k, 128-multipole tile) only the tau-prefix on which Watson's
  *              bound (Abramowitz & Stegun 9.1.63) allows |j_l| >= eps_cut for
  *              some l of the tile is summed.  This prefix is Algorithm 1's
- *              n_min..n_max window.
+ *              n_min..n_max window.  In the plain modes a multipole's sum may
+ *              stop at its own prefix, in whole groups of nodes (polarisation
+ *              and tensor fields: at eps_cut <= 1e-20 only); nodes beyond it
+ *              are not read for it, so a non-finite source there need not show.
  *   out        receives the handle.
  *
  * Computes the quadrature weights and the active extents on the host; the
@@ -274,14 +277,16 @@ int gcamb_cl_interp(const gcamb_grid *g, const double *Cl_s, int M, double *Cl, 
  * Source interpolation onto the grid's k nodes (the step that prepares the
  * sources before the projection, Sec. 3.3): the natural cubic spline in k of
  * every (source, tau) column (second derivatives zero at both ends), solved
- * and evaluated in the sources' precision (FP64 or FP32; in FP32 the nodes more
- * than 24 away from a second derivative may be left out of it where their
- * weight is below 2^-40, so a non-finite value need not reach its whole column).
+ * and evaluated in the sources' precision.  In FP32 the nodes more than 24 away
+ * from a second derivative may be left out of it where they weigh less than
+ * 2^-40 in it (2^-45 on even nodes): less than FP32's rounding of the result,
+ * unless the values there are 2^16 times those here and more, and a non-finite
+ * value need not reach its whole column.
  *   k_in[nk_in]          host, strictly increasing, nk_in >= 2; the grid's k
  *                        range must lie inside [k_in[0], k_in[nk_in-1]]
  *   S_in[M][nk_in][ntau] device, dtype GCAMB_F64 or GCAMB_F32 (ntau: the grid's)
  *   S_out[M][nk][ntau]   device, same dtype
- *   ws, ws_bytes         device workspace of gcamb_interp_sources_workspace bytes
+ *   ws, ws_bytes         device workspace of gcamb_interp_sources_workspace bytes, of any alignment
  * Errors: GCAMB_EINVAL (arguments), GCAMB_ECUDA.
  */
 int gcamb_interp_sources_workspace(const gcamb_grid *g, int M, int nk_in, size_t *bytes);

@@ -414,7 +414,6 @@ int gemm_ps(const GemmArgs<NP> &a, int grid, cudaStream_t st) {
 // (see emu_gemm.cuh).
 template <int EPI, bool AMN, bool BMN, int NP>
 int gemm(const GemmArgs<NP> &a, int tiles, cudaStream_t st) {
-  constexpr int kSms = 152;
   return tiles <= kSms ? gemm_ps<EPI, AMN, BMN, NP, false>(a, tiles, st)
                        : gemm_ps<EPI, AMN, BMN, NP, true>(a, kSms, st);
 }

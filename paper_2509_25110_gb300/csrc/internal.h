@@ -15,6 +15,7 @@ namespace gcamb {
 constexpr int kTileL = 128;      // multipoles per l-tile (UMMA M)
 constexpr int kMaxL = 20000;
 constexpr int kNumModes = 5;
+constexpr int kSms = 152;        // SMs of a GB300
 
 // Table layout of one mode: blocks of [planes][128 rows][kb cols], one block
 // per (k, l-tile, tau-block of kb nodes).  Rows are multipoles, columns tau.

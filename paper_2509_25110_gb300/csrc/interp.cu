@@ -133,9 +133,12 @@ __global__ void __launch_bounds__(256) spline_eval_kernel(const T *__restrict__ 
 // h_(k-1)/den_k between them, and d'_i changes M_j of the back substitution by
 // the product of the c'_k (0.27 a node on even nodes, at most 2/3 and 1/2 on
 // any).  So kSegH nodes decide a second derivative: what is left out is below
-// 2^-40 of the one at that distance (the host checks the products,
-// seg_halo_ok), where FP32 keeps 2^-24.  The k range is also cut into parts
-// whose forward sweeps start kSegH nodes early, in the same way.
+// 2^-40 (2^-45 on even nodes) of the second derivative at that distance (the
+// host checks the products, seg_halo_ok), that is below FP32's rounding of the
+// values here unless those are less than 2^-16 of the ones 24 nodes away.  The k
+// range is also cut into parts whose forward sweeps start kSegH nodes early, in
+// the same way.  (32 nodes and 2^-54: 1512 -> 1596 us, small shapes up to 40%
+// slower.)
 //
 // Bound by HBM: the sources are read once (1 GB of 256 x 1000 x 1000), the
 // outputs written once (8.2 GB on 8000 nodes).  The columns' values arrive by
@@ -403,19 +406,21 @@ bool seg_halo_ok(const double *h, const double *cp, const double *inv, int n) {
 // the last}, of about equal work t, counted in segments: kPartOuts outputs take
 // about as long as a segment's sweep and back substitution.  A part's sweep
 // starts 2 kSegA segments early, so `blocks` columns' parts take (2 kSegA + t)
-// (1 + W / t) one after the other on the chip's places,
-// W = all work / places; t = sqrt(2 kSegA W) is its least, and at least
-// kPartMin.  A segment with many outputs (nodes that are sparse where the grid
+// (1 + W / t) one after the other on the chip's places, W = all work / places;
+// t = sqrt(2 kSegA W) is its least, and at least kPartMin.  Four blocks fit an
+// SM, but W is reckoned with kPartPlaces = 5: parts a little finer leave fewer
+// places idle at the end (four: 1512 -> 1533 us, 21 shapes 0.85 .. 1.17 of the
+// speed, most of them below 1).  A segment with many outputs (nodes that are sparse where the grid
 // is dense) is shared out by outputs; segments without any are left out where
 // a part can start behind them.  Kernel time, parts of at least 16 whole
 // segments -> these (nodes -> grid, tau, sources): 200 -> 8000, 300, 8: 582 ->
 // 50 us; 395 -> 6075, 498, 15: 267 -> 67; 200 -> 1000, 300, 8: 59 -> 16;
 // 518 -> 4312, 499, 155: 439 -> 415; 1000 -> 8000, 1000, 256: 1509 -> 1488.
-constexpr int kPartOuts = 64, kPartMin = 4;
+constexpr int kPartOuts = 64, kPartMin = 4, kPartPlaces = 5;
 
 std::vector<int4> march_parts(const int *qs, int n, int nq, size_t blocks) {
   const int nseg = (n - 2) / kSegT + 1;
-  const double work = (nseg + (double)nq / kPartOuts) * (double)blocks / (152 * 5);
+  const double work = (nseg + (double)nq / kPartOuts) * (double)blocks / (kSms * kPartPlaces);
   const double target = std::max((double)kPartMin, std::sqrt(2.0 * kSegA * work));
   std::vector<int4> parts;
   int4 p{-1, 0, 0, 0};

@@ -606,7 +606,7 @@ constexpr double kRowCut = 1e-20;
 // (19702) 7951 / 7962 (8334); sampled l_max 2500 (2043) 343 / 293 (302).
 static int plain_rows(const gcamb_grid *g, const Table &t) {
   const double full = t.max_nkb > 0 ? (double)t.nblocks / t.max_nkb : 0.0;
-  return !g->lsampled && full >= 152 * 8 ? 128 : 64;
+  return !g->lsampled && full >= kSms * 8 ? 128 : 64;
 }
 
 static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M, int field) {
@@ -665,8 +665,10 @@ static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, const
   return GCAMB_OK;
 }
 
-// Limits of the path: the staged tau-prefix of one chunk of sources (1, 2, 4,
-// FP32 also 8) fits 200 KB, and 65535 chunks.
+// Limits of the path: the whole tau-prefix of a chunk of 1, 2, 4 (FP32 also 8)
+// sources is at most 200 KB, and there are at most 65535 chunks.  The kernel stages
+// 64 KB at a time and takes other chunks; what it would need is less.  The limits
+// are part of the interface: a grid is refused or taken by its size alone.
 static int plain_limits(const Table &t, int M, int mode) {
   const int mc = mode != GCAMB_PLAIN64 && M >= 8 ? 8 : (M >= 4 ? 4 : (M >= 2 ? 2 : 1));
   const size_t smem = (size_t)mc * t.max_nkb * kPlainKB * (mode == GCAMB_PLAIN64 ? 8 : 4);
@@ -862,7 +864,7 @@ static cudaError_t launch_cl_sum(const gcamb_grid *g, const void *DX, const void
   // l_max = 5000 has only 157 blocks of 32 multipoles
   const unsigned lb = (unsigned)((g->nl + 31) / 32);
   unsigned cs = 1;
-  while (cs < 8 && (size_t)lb * M * cs < 152 * 6) cs *= 2;
+  while (cs < 8 && (size_t)lb * M * cs < kSms * 6) cs *= 2;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(lb, cs, (unsigned)M);
   cfg.blockDim = dim3(256);
