@@ -593,20 +593,38 @@ int emode_x_lo(const gcamb_grid *g, double *x_lo) {
 // 1e-20 the rows' own prefixes leave out 3e-20 of them, below FP64's rounding.
 constexpr double kRowCut = 1e-20;
 
+// Full-prefix tiles of the grid: blocks / longest prefix.  (A log-spaced k grid
+// has most of its work in the last few k, so that the number of non-empty tiles
+// says little.)
+static double plain_tiles(const Table &t) { return t.max_nkb > 0 ? (double)t.nblocks / t.max_nkb : 0.0; }
+
 // Rows per CTA of the plain kernel: a whole 128-row tile, or 64 rows (the
 // CTA's four warps then share out the tau steps in pairs) where the tiles are
-// too few to balance the SMs.  Counted in CTAs of the longest prefix (blocks /
-// longest prefix): a log-spaced k grid has most of its work in the last few
-// k, so that the number of non-empty tiles says little.  Sampled multipoles
-// take 64 rows too: the prefixes of one tile's rows then span most of the
-// grid, and the warps of a CTA would finish far apart.  By the grid alone, so
-// that a source's sums do not depend on its batch.  Measured at 128 / 64 (32)
-// rows: l_max 500 (count 570) 73 / 69 (74) us; tensor l_max 1500 (2540) 1950 /
-// 2058 (2385); E-mode FP32 l_max 2001 (3063) 307 / 363 (495) (before its prefetch); l_max 5000
-// (19702) 7951 / 7962 (8334); sampled l_max 2500 (2043) 343 / 293 (302).
+// too few to balance the SMs; FP32, bound by loads rather than a pipe, needs
+// fewer.  Sampled multipoles take 64 rows too: the prefixes of one tile's rows
+// then span most of the grid, and the warps of a CTA would finish far apart.  By
+// the grid alone, so that a source's sums do not depend on its batch.  Measured at
+// 128 / 64 (32) rows: FP64 l_max 500 (570 tiles) 73 / 69 (74) us; tensor l_max 1500
+// (2540) 1950 / 2058 (2385); l_max 5000 (19702) 7951 / 7962 (8334); sampled l_max 2500
+// (2043) 343 / 293 (302); FP32, one and eight sources, 285 tiles 15 / 18 and 29 / 35 us,
+// 570 25 / 29 and 50 / 65, 1899 76 / 89 and 132 / 191, but 122 tiles 13 / 13 and 25 / 23.
 static int plain_rows(const gcamb_grid *g, const Table &t) {
-  const double full = t.max_nkb > 0 ? (double)t.nblocks / t.max_nkb : 0.0;
-  return !g->lsampled && full >= kSms * 8 ? 128 : 64;
+  return !g->lsampled && plain_tiles(t) >= kSms * (t.lay.esize == 8 ? 8 : 2) ? 128 : 64;
+}
+
+// Sources per CTA: the batch in equal chunks of at most `most` (the table is read
+// once per chunk, and FP64 sums of sources that are not there would cost as much
+// as real ones), smaller ones where a grid gives the chip too few CTAs: FP64
+// three an SM, FP32 one and a half, counted in full-prefix CTAs with all rows in
+// use.  FP64, four sources: 300 k x 400 tau sampled to l 500 (403) 114 -> 81 us, 64
+// k x 100 tau to l 64 (63) 19 -> 15 us; two sources at 403: 60 -> 51 us, at 537 no
+// gain.  FP32, 16 sources at 63: 14.8 -> 12.6 us.
+static int plain_sources(const gcamb_grid *g, const Table &t, int M, int most) {
+  const double ctas = plain_tiles(t) * (kTileL / plain_rows(g, t)) * g->nl / ((double)g->nlt * kTileL);
+  const double want = t.lay.esize == 8 ? 3.0 * kSms : 1.5 * kSms;
+  int chunks = (M + most - 1) / most;
+  if (ctas * chunks < want) chunks = ctas * M <= want ? M : (int)std::ceil(want / ctas);
+  return (M + chunks - 1) / chunks;
 }
 
 static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M, int field) {
@@ -677,9 +695,6 @@ static int plain_limits(const Table &t, int M, int mode) {
   return GCAMB_OK;
 }
 
-// Sources per CTA: the batch in equal chunks of at most 4 (FP64) or 8
-// (FP32).  The table is read once per chunk, and FP64 sums of sources
-// that are not there would cost as much as real ones.
 template <int FIELD>
 static int launch_los_plain_f(const gcamb_grid *g, const void *S, int M, int mode, void *Delta, cudaStream_t st) {
   const Table &t = g->tab[mode];
@@ -687,7 +702,7 @@ static int launch_los_plain_f(const gcamb_grid *g, const void *S, int M, int mod
   if (mode == GCAMB_PLAIN64) {
     auto s = static_cast<const double *>(S);
     auto d = static_cast<double *>(Delta);
-    const int chunks = (M + 3) / 4, mc = (M + chunks - 1) / chunks;
+    const int mc = plain_sources(g, t, M, 4);
     auto go = [&](auto c) {
       return launch_plain_t<double, decltype(c)::value, FIELD>(g, t, s, nullptr, M, d, nullptr, nullptr, g->nk, g->nlt,
                                                                st);
@@ -699,7 +714,7 @@ static int launch_los_plain_f(const gcamb_grid *g, const void *S, int M, int mod
   }
   auto s = static_cast<const float *>(S);
   auto d = static_cast<float *>(Delta);
-  const int chunks = (M + 7) / 8, mc = (M + chunks - 1) / chunks;
+  const int mc = plain_sources(g, t, M, 8);
   auto go = [&](auto c) {
     return launch_plain_t<float, decltype(c)::value, FIELD>(g, t, s, nullptr, M, d, nullptr, nullptr, g->nk, g->nlt, st);
   };
