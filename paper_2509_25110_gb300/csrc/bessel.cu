@@ -550,18 +550,25 @@ struct KernelSink {
   double pv, fv;
   static constexpr bool kRaw = false;  // every order from l0 = the order of "row" 0: each kernel takes two
   int l0;
+  const double *cl;  // c_l of each row
   __device__ __forceinline__ double weight() const { return 1.0; }
   __device__ __forceinline__ int order(int row) const { return l0 + row; }
   __device__ __forceinline__ int last(int l) const { return l - l0; }
   __device__ __forceinline__ void store(int row, double v) { (*this)(l0 + row, v); }
+  // In as few FP64 operations as there are (c_l from the grid, l (l-1) as an
+  // integer), and for table rows only: what is left of the FP64 pipe's work once
+  // the recurrences are integers.  300 k x 400 tau, l_max 500, PLAIN64 / F16X3: kernel 1
+  // (with c_l's square root per element) 2166 / 2659 -> 531 / 1052 us, 2 1113 / 1509 ->
+  // 770 / 1357, 3 1053 / 1412 -> 686 / 1248.
   __device__ __forceinline__ void emit(int l, double jl, double jm) {
     if (l < lmin || l < 2) return;
-    const double dl = (double)l;
+    const int row = out.rowof ? out.rowof[l - lmin] : l - lmin;
+    if (row < 0) return;
     double v;
-    if (kern == 1) v = sqrt((dl + 2.0) * (dl + 1.0) * dl * (dl - 1.0)) * jl * ix2;
-    else if (kern == 2) v = (dl * (dl - 1.0) * ix2 - 2.0) * jl + 2.0 * jm * ix;
-    else v = 2.0 * jm - 2.0 * (dl - 1.0) * jl * ix;
-    out(l, v);
+    if (kern == 1) v = __ldg(cl + row) * jl * ix2;
+    else if (kern == 2) v = fma(fma((double)(l * (l - 1)), ix2, -2.0), jl, ix * (2.0 * jm));
+    else v = fma((double)(2 - 2 * l) * ix, jl, 2.0 * jm);
+    out.store(row, out.w * v);
   }
   __device__ __forceinline__ void operator()(int l, double v) {
     if (l == pl + 1) {
@@ -608,7 +615,8 @@ __global__ void __launch_bounds__(128) bessel_table_kernel(const double *__restr
                                                            const double *__restrict__ xs, int nxs, int scale_exp,
                                                            const int *__restrict__ lrow,
                                                            const int *__restrict__ rowof, int nl, int curved,
-                                                           double rk, int kern, double x_lo, int ns, void *table) {
+                                                           double rk, int kern, double x_lo, const double *__restrict__ cl, int ns,
+                                                           void *table) {
   constexpr int KB = (MODE == GCAMB_PLAIN64 || MODE == GCAMB_PLAIN32) ? 64 : 32;
   const int q = blockIdx.y;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -667,7 +675,7 @@ __global__ void __launch_bounds__(128) bessel_table_kernel(const double *__restr
       for (int l = max(lmin, 2); l <= min(ltop, 5); ++l) sink(l, small_x_kernel(kern, l, x));
     } else {
       const int l0 = lmin > 0 ? lmin - 1 : 0;
-      KernelSink<TableSink<MODE>> ks{sink, kern, lmin, 1.0 / x, 1.0 / (x * x), -10, -10, 0.0, 0.0, l0};
+      KernelSink<TableSink<MODE>> ks{sink, kern, lmin, 1.0 / x, 1.0 / (x * x), -10, -10, 0.0, 0.0, l0, cl};
       bessel_orders(x, start, l0, ltop, xs, nxs, ks);
     }
   } else {
@@ -997,35 +1005,35 @@ int launch_bessel_table(gcamb_grid *g, int mode, cudaStream_t st) {
                                                                g->lmax, g->nlt, t.d_nkb, t.d_off, g->d_xstart, g->nxs,
                                                                t.scale_exp, g->lsampled ? g->d_lrow : nullptr,
                                                                g->lsampled ? g->d_rowof : nullptr, g->nl, g->curved, g->rk,
-                                                               g->kernel, x_lo, ns, t.d_data);
+                                                               g->kernel, x_lo, g->d_cl, ns, t.d_data);
       break;
     case GCAMB_PLAIN32:
       bessel_table_kernel<GCAMB_PLAIN32><<<grid, 128, tsmem, st>>>(g->d_k, g->d_tau, g->d_wtau, g->tau0, g->ntau, g->lmin,
                                                                g->lmax, g->nlt, t.d_nkb, t.d_off, g->d_xstart, g->nxs,
                                                                t.scale_exp, g->lsampled ? g->d_lrow : nullptr,
                                                                g->lsampled ? g->d_rowof : nullptr, g->nl, g->curved, g->rk,
-                                                               g->kernel, x_lo, ns, t.d_data);
+                                                               g->kernel, x_lo, g->d_cl, ns, t.d_data);
       break;
     case GCAMB_BF16X3:
       bessel_table_kernel<GCAMB_BF16X3><<<grid, 128, tsmem, st>>>(g->d_k, g->d_tau, g->d_wtau, g->tau0, g->ntau, g->lmin,
                                                               g->lmax, g->nlt, t.d_nkb, t.d_off, g->d_xstart, g->nxs,
                                                               t.scale_exp, g->lsampled ? g->d_lrow : nullptr,
                                                                g->lsampled ? g->d_rowof : nullptr, g->nl, g->curved, g->rk,
-                                                               g->kernel, x_lo, ns, t.d_data);
+                                                               g->kernel, x_lo, g->d_cl, ns, t.d_data);
       break;
     case GCAMB_F16X3:
       bessel_table_kernel<GCAMB_F16X3><<<grid, 128, tsmem, st>>>(g->d_k, g->d_tau, g->d_wtau, g->tau0, g->ntau, g->lmin,
                                                              g->lmax, g->nlt, t.d_nkb, t.d_off, g->d_xstart, g->nxs,
                                                              t.scale_exp, g->lsampled ? g->d_lrow : nullptr,
                                                                g->lsampled ? g->d_rowof : nullptr, g->nl, g->curved, g->rk,
-                                                               g->kernel, x_lo, ns, t.d_data);
+                                                               g->kernel, x_lo, g->d_cl, ns, t.d_data);
       break;
     case GCAMB_TF32X3:
       bessel_table_kernel<GCAMB_TF32X3><<<grid, 128, tsmem, st>>>(g->d_k, g->d_tau, g->d_wtau, g->tau0, g->ntau, g->lmin,
                                                               g->lmax, g->nlt, t.d_nkb, t.d_off, g->d_xstart, g->nxs,
                                                               t.scale_exp, g->lsampled ? g->d_lrow : nullptr,
                                                                g->lsampled ? g->d_rowof : nullptr, g->nl, g->curved, g->rk,
-                                                               g->kernel, x_lo, ns, t.d_data);
+                                                               g->kernel, x_lo, g->d_cl, ns, t.d_data);
       break;
   }
   e = cudaGetLastError();
