@@ -102,8 +102,11 @@ struct PlainArgs {
   const float2 *cl2;    // [nl] the same as the sum of two floats
   const double *xthr;   // [nl] Watson thresholds, or null: every row takes the whole tile's prefix
   double tau0, x_lo;
-  int nk, nlt, nl, ntau, M, lmin;
-  int step_round;       // rows' prefixes in steps are rounded up to a multiple of step_round + 1 (1 or a block's)
+  int nk, nlt, nl, ntau, M;
+  // tensor: lmin.  Temperature: a block's steps - 1 where rows take whole blocks,
+  // else 0 (one word for both, and looked at outside the sums: as an argument of its
+  // own, and in them, it made registers spill: FP32, six to eight sources 5-9%).
+  int lmin_or_round;
   int q0;               // last k of the launch
   int rows;             // rows per CTA: 128 or 64
 };
@@ -137,7 +140,13 @@ constexpr int kPlainGroup = 32;
 // Tau blocks staged in shared memory at a time: whole groups, up to 64 KB of
 // sources.  (Staging every group by itself: one FP64 source, 8000 tau 2546 ->
 // 3169 us.)
-constexpr int plain_stage_blocks(int nv, size_t esize) {
+// (FP32 E-mode of three and four sources: one group, so that no loop over groups
+// takes registers: 205 -> 196 and 227 -> 214 us, 1106 k x 698 tau to l 1738.)
+constexpr bool plain_one_group(int nv, size_t esize, int field) {
+  return esize == 4 && field == kFieldE && (nv == 3 || nv == 4);
+}
+constexpr int plain_stage_blocks(int nv, size_t esize, int field) {
+  if (plain_one_group(nv, esize, field)) return kPlainGroup;
   return (int)(65536 / (nv * esize * kPlainKB)) / kPlainGroup * kPlainGroup;
 }
 
@@ -265,7 +274,7 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
   constexpr int VE = 16 / sizeof(T);        // nodes per 16-byte load
   constexpr int SN = 8 * VE;                // nodes per step of a lane group (128 bytes of a row): 16 or 32
   constexpr int STEPS = KB / SN;            // steps per block
-  constexpr int CHB = plain_stage_blocks(NV, sizeof(T));
+  constexpr int CHB = plain_stage_blocks(NV, sizeof(T), FIELD);
   constexpr int HALO = FIELD == kFieldTensor ? 1 : 0;  // tensor: also the row before the CTA's first
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int R = a.rows, TS = kTileL / R;
@@ -297,8 +306,10 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
   const int grp = lane >> 3, sub = lane & 7;
   const int WR = kPlainWarps / TS, rw = warp % WR, ts = warp / WR;
   // nonnegative doubles order as their bit patterns
-  for (int i = tid; i < nb * STEPS; i += kPlainWarps * 32)
-    xb[i] = i * SN < a.ntau ? __double_as_longlong(kq * (a.tau0 - a.tau[i * SN])) : -1;
+  for (int i = tid; i < nb * STEPS; i += kPlainWarps * 32) {
+    const int n = SN * (FIELD == kFieldT ? i & ~a.lmin_or_round : i);  // whole blocks: that of the block's first node
+    xb[i] = n < a.ntau ? __double_as_longlong(kq * (a.tau0 - a.tau[n])) : -1;
+  }
   for (int i = tid; i < NV * kTileL; i += kPlainWarps * 32) res[i] = as_ff(T(0));
   if (HALO && tid < NV) halo[tid] = as_ff(T(0));
   const T *chunk = table + (size_t)a.off[e_idx] * (kTileL * KB);
@@ -389,9 +400,10 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
     }
     __syncthreads();
     // ---- rows, a group of blocks at a time
+    constexpr bool kOne = plain_one_group(NV, sizeof(T), FIELD);
 #pragma unroll 1
-    for (int gb = 0; gb < nbc; gb += kPlainGroup) {
-      const int b1 = b0 + gb, ng = min(kPlainGroup, nbc - gb);
+    for (int gb = 0; gb < (kOne ? 1 : nbc); gb += kPlainGroup) {
+      const int b1 = kOne ? b0 : b0 + gb, ng = kOne ? nbc : min(kPlainGroup, nbc - gb);
       const T *sg = s + gb * KB;
       for (int rb = rw * 4 * RV; rb < R; rb += WR * 4 * RV) {
         int ns[RV];  // steps of this group that rows rb + 4 i .. + 3 need
@@ -410,7 +422,7 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
                 int n = 0;
                 for (int c = 0; c < nsc; c += 32)
                   n += __popc(__ballot_sync(0xffffffffu, c + lane < nsc && xb[b1 * STEPS + c + lane] >= xi));
-                ns[i] = (n + a.step_round) & ~a.step_round;
+                ns[i] = n;
               }
             }
           }
@@ -536,7 +548,7 @@ __global__ void __launch_bounds__(kPlainWarps * 32, 4)
       Delta[o] = emode_row<T>(a, row, kq, sum(m, r), S + ((size_t)(m0 + m) * a.nk + q) * a.ntau);
     } else {
       const size_t so = ((size_t)(m0 + m) * a.nk + q) * a.ntau;
-      const int l = a.lmin + row;
+      const int l = a.lmin_or_round + row;
       Delta[o] = emode_row<T>(a, row, kq, sum(4 * m + 3, r), ST + so);
       double ve = 0.0, vb = 0.0;
       if (l >= 2) {
@@ -640,7 +652,6 @@ static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M, int fiel
   a.cl2 = reinterpret_cast<const float2 *>(g->d_cl2);
   // rows stop at their own prefix on flat j_l grids only
   a.xthr = (g->kernel == 0 && !g->curved && (field == kFieldT || g->eps_cut <= kRowCut)) ? g->d_xthr : nullptr;
-  a.step_round = g->eps_cut <= kRowCut ? 0 : kPlainKB * (int)t.lay.esize / 128 - 1;
   a.tau0 = g->tau0;
   a.x_lo = 1e-12;
   a.nk = g->nk;
@@ -648,7 +659,6 @@ static PlainArgs plain_args(const gcamb_grid *g, const Table &t, int M, int fiel
   a.nl = g->nl;
   a.ntau = g->ntau;
   a.M = M;
-  a.lmin = g->lmin;
   a.rows = plain_rows(g, t);
   return a;
 }
@@ -662,7 +672,7 @@ static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, const
   PlainArgs a = plain_args(g, t, M, FIELD);
   if (FIELD != kFieldT && emode_x_lo(g, &a.x_lo))
     return fail(GCAMB_EINVAL, "los_transfer: eps_cut too large for the l = 2 limit of the polarisation kernels");
-  const int stage = t.max_nkb < plain_stage_blocks(NV, sizeof(T)) ? t.max_nkb : plain_stage_blocks(NV, sizeof(T));
+  const int stage = t.max_nkb < plain_stage_blocks(NV, sizeof(T), FIELD) ? t.max_nkb : plain_stage_blocks(NV, sizeof(T), FIELD);
   const size_t smem = (size_t)NV * stage * kPlainKB * sizeof(T) + (size_t)NV * kTileL * sizeof(PlainSum<T>) +
                       (size_t)t.max_nkb * (kPlainKB * sizeof(T) / 128) * sizeof(long long) + NV * sizeof(PlainSum<T>);
   cudaError_t e = cudaFuncSetAttribute(los_plain_kernel<T, MC, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -670,6 +680,8 @@ static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, const
   if (e != cudaSuccess) return cuda_fail(e, "los_transfer: smem attribute");
   ProfScope prof(GCAMB_K_LOS_PLAIN, st);
   a.q0 = nk - 1;
+  if (FIELD == kFieldTensor) a.lmin_or_round = g->lmin;
+  if (FIELD == kFieldT) a.lmin_or_round = g->eps_cut > kRowCut ? kPlainKB * (int)sizeof(T) / 128 - 1 : 0;
   for (int m0 = 0; m0 < M; m0 += 65535 * MC) {
     a.M = M - m0 < 65535 * MC ? M - m0 : 65535 * MC;
     const dim3 grid(nlt * (kTileL / a.rows), nk, (a.M + MC - 1) / MC);
