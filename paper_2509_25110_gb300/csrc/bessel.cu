@@ -756,7 +756,7 @@ int curved_extents(gcamb_grid *g, cudaStream_t st) {
     const int ns = curved_stage_orders(g);
     const size_t smem = (size_t)2 * ns * sizeof(double);
     if (smem > 48 * 1024)
-      e = cudaFuncSetAttribute(curved_activity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = cudaFuncSetAttribute(curved_activity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem);
     if (e == cudaSuccess) {
       curved_activity_kernel<<<grid, 128, smem, st>>>(g->d_k, g->d_tau, g->tau0, g->ntau, g->lmin, g->lmax, g->nlt,
                                                       g->rk, g->curved == 2, g->eps_cut,
@@ -990,11 +990,11 @@ int launch_bessel_table(gcamb_grid *g, int mode, cudaStream_t st) {
   const size_t tsmem = (size_t)2 * ns * sizeof(double);
   if (tsmem > 48 * 1024) {
     switch (mode) {
-      case GCAMB_PLAIN64: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_PLAIN64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem); break;
-      case GCAMB_PLAIN32: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_PLAIN32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem); break;
-      case GCAMB_BF16X3: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_BF16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem); break;
-      case GCAMB_F16X3: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_F16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem); break;
-      default: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_TF32X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem); break;
+      case GCAMB_PLAIN64: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_PLAIN64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem); break;
+      case GCAMB_PLAIN32: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_PLAIN32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem); break;
+      case GCAMB_BF16X3: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_BF16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem); break;
+      case GCAMB_F16X3: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_F16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem); break;
+      default: e = cudaFuncSetAttribute(bessel_table_kernel<GCAMB_TF32X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem); break;
     }
     if (e != cudaSuccess) return cuda_fail(e, "bessel_table: smem attribute");
   }

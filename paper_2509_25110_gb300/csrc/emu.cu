@@ -855,8 +855,8 @@ int gcamb_synth_sources(const gcamb_grid *g, const float *X, int M, float *S, do
   int rc = ensure_device_grid(const_cast<gcamb_grid *>(g));
   if (rc) return rc;
   const size_t smem = (2 * (size_t)g->ntau + 512) * sizeof(double);
-  if (smem > 200 * 1024) return fail(GCAMB_EINVAL, "synth_sources: tau grid too long");
-  cudaError_t ea = cudaFuncSetAttribute(synth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > (size_t)kDynSmem) return fail(GCAMB_EINVAL, "synth_sources: tau grid too long");
+  cudaError_t ea = cudaFuncSetAttribute(synth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem);
   if (ea != cudaSuccess) return cuda_fail(ea, "synth_sources: smem attribute");
   dim3 grid((g->nk + 255) / 256, M);
   synth_kernel<<<grid, 256, smem, (cudaStream_t)stream>>>(X, g->d_k, g->d_tau, g->nk, g->ntau, S, Pk);

@@ -16,6 +16,10 @@ constexpr int kTileL = 128;      // multipoles per l-tile (UMMA M)
 constexpr int kMaxL = 20000;
 constexpr int kNumModes = 5;
 constexpr int kSms = 152;        // SMs of a GB300
+// Dynamic shared memory allowed to the kernels that take a call's own amount.
+// The same for every call: the allowance is the process's, and a thread that set
+// it to its own call's amount made another's launch fail.
+constexpr int kDynSmem = 200 * 1024;
 
 // Table layout of one mode: blocks of [planes][128 rows][kb cols], one block
 // per (k, l-tile, tau-block of kb nodes).  Rows are multipoles, columns tau.

@@ -847,8 +847,9 @@ int gcamb_cl_interp(const gcamb_grid *g, const double *Cl_s, int M, double *Cl, 
     cl_spline_pcr_kernel<<<dim3((unsigned)M, ny), 256, 0, st>>>(Cl_s, g->d_lrow, g->d_rowof, d_coef + nl, d_coef + 2 * (size_t)nl, stages, d_j,
                                             d_s, nl, g->lmin, nout, Cl);
   } else if (nl <= kSmemSamples) {
+    static_assert(6 * kSmemSamples * sizeof(double) <= kDynSmem, "samples in shared memory");
     const size_t smem = (size_t)6 * nl * sizeof(double);
-    e = cudaFuncSetAttribute(cl_spline_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(cl_spline_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cl_interp: smem attribute");
     cl_spline_block_kernel<<<M, 256, smem, st>>>(Cl_s, g->d_lrow, g->d_rowof, d_coef, d_j, d_s, nl, g->lmin, nout, Cl);
   } else {

@@ -675,8 +675,9 @@ static int launch_plain_t(const gcamb_grid *g, const Table &t, const T *S, const
   const int stage = t.max_nkb < plain_stage_blocks(NV, sizeof(T), FIELD) ? t.max_nkb : plain_stage_blocks(NV, sizeof(T), FIELD);
   const size_t smem = (size_t)NV * stage * kPlainKB * sizeof(T) + (size_t)NV * kTileL * sizeof(PlainSum<T>) +
                       (size_t)t.max_nkb * (kPlainKB * sizeof(T) / 128) * sizeof(long long) + NV * sizeof(PlainSum<T>);
+  // (at most 64 KB staged, 8 KB of sums and 13 KB of steps: plain_limits)
   cudaError_t e = cudaFuncSetAttribute(los_plain_kernel<T, MC, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+                                       kDynSmem);
   if (e != cudaSuccess) return cuda_fail(e, "los_transfer: smem attribute");
   ProfScope prof(GCAMB_K_LOS_PLAIN, st);
   a.q0 = nk - 1;

@@ -176,3 +176,37 @@ def test_temperature_rows_at_large_eps_cut(mode, bar, eps_cut):
     got, ref = field(eps_cut), field(0.0)
     gcamb.sync()
     assert ((got - ref).abs() <= bar * ref.abs().max()).all(), float((got - ref).abs().max() / ref.abs().max())
+
+
+def test_threads_with_grids_of_different_sizes():
+    """Two host threads whose plain transfers take different amounts of shared
+    memory, on their own streams: every launch succeeds and gives the bits it
+    gives alone."""
+    import threading
+    work = []
+    for ntau in (40, 7000):  # 1 KB and 60 KB
+        k, tau, S, g = make(4, ntau, 40, 1, seed=ntau)
+        gcamb.bessel_table(g, gcamb.PLAIN64)
+        d = torch.as_tensor(S[0], device="cuda")
+        work.append((g, d, gcamb.los_transfer(g, d, gcamb.PLAIN64)))
+    torch.cuda.synchronize()
+    bad = []
+
+    def run(g, d, ref):
+        s = torch.cuda.Stream()
+        out = torch.empty_like(ref)
+        try:
+            for _ in range(3000):
+                gcamb.los_transfer(g, d, gcamb.PLAIN64, out, stream=s)
+            s.synchronize()
+            if not torch.equal(out, ref):
+                bad.append("values")
+        except Exception as e:  # reported below, on the main thread
+            bad.append(repr(e))
+
+    ts = [threading.Thread(target=run, args=w) for w in work]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not bad, bad
